@@ -298,3 +298,87 @@ def tolerance(case):
     if case["kind"] in ("decode", "turn"):
         return {"rel": 8e-3, "max": 0.1}
     return {"rel": 8e-3, "max": 0.3}
+
+
+# ---- the same outputs in 64 bits --------------------------------------------------------------------------
+
+def exact(case, seed):
+    """What run() returns, as dense attention over the visible keys gives it in float64 (torch on the GPU)."""
+    s = prepare(case, seed)
+    wide = lambda t: t.cuda().double()  # noqa: E731
+    scale = case["d"] ** -0.5
+    if case["kind"] in ("decode", "turn"):
+        return exact_cache(case, s, wide, scale)
+    evict, cu = s["evict"].cuda(), s["cu"].tolist()
+    if case.get("layout") == "packed":
+        q, k, v = wide(s["qkv"]).split((case["Hq"], case["Hkv"], case["Hkv"]), dim=1)
+    else:
+        q, k, v = wide(s["q"]), wide(s["k"]), wide(s["v"])
+    if case.get("layout") == "rope":
+        q, k = rotated(q, cu, 1), rotated(k, cu, 1)
+    if case["kind"] in ("score", "dual"):
+        got = attention64(q, k, v, evict, cu, scale)[:2]
+        return got if case["kind"] == "score" else got + attention64(q, k, v, torch.full_like(evict, 2 ** 31 - 1), cu, scale)[:2]
+    out, lse, dq, dk, dv = attention64(q, k, v, evict, cu, scale, s["dout"].cuda())
+    if case.get("layout") == "packed":
+        return out, lse, torch.cat((dq, dk, dv), dim=1)
+    if case.get("layout") == "rope":
+        dq, dk = rotated(dq, cu, -1), rotated(dk, cu, -1)
+    return out, lse, dq, dk, dv
+
+
+def attention64(q, k, v, evict, cu, scale, dout=None, rows=1024):
+    (total, Hq, d), Hkv = q.shape, k.shape[1]
+    G = Hq // Hkv
+    out, lse = torch.empty_like(q), q.new_empty(Hq, total)
+    dq, dk, dv = (None, None, None) if dout is None else (torch.zeros_like(q), torch.zeros_like(k), torch.zeros_like(v))
+    for a, z in zip(cu[:-1], cu[1:]):
+        for i0 in range(a, z, rows):
+            i1 = min(z, i0 + rows)
+            keys = a + torch.nonzero(evict[a:i1] > i0 - a).squeeze(1)          # any of these queries may see them
+            i = torch.arange(i0, i1, device=q.device)
+            hidden = (keys > i[:, None]) | (evict[keys] <= i[:, None] - a)
+            for g in range(Hkv):
+                h = slice(g * G, (g + 1) * G)
+                qq, kk, vv = q[i0:i1, h].transpose(0, 1).reshape(-1, d), k[keys, g], v[keys, g]
+                s = (qq @ kk.T).mul_(scale).view(G, i1 - i0, -1).masked_fill_(hidden, -math.inf)
+                top = torch.logsumexp(s, dim=2)
+                p = s.sub_(top[..., None]).exp_().view(len(qq), -1)
+                o = p @ vv
+                lse[h, i0:i1] = top
+                out[i0:i1, h] = o.view(G, -1, d).transpose(0, 1)
+                if dout is not None:
+                    do = dout[i0:i1, h].double().transpose(0, 1).reshape(-1, d)
+                    dv[:, g].index_add_(0, keys, p.T @ do)
+                    ds = (do @ vv.T).sub_((do * o).sum(1, keepdim=True)).mul_(p).mul_(scale)
+                    dq[i0:i1, h] = (ds @ kk).view(G, -1, d).transpose(0, 1)
+                    dk[:, g].index_add_(0, keys, ds.T @ qq)
+    return out, lse, dq, dk, dv
+
+
+def rotated(x, cu, sign):
+    """Rotary embedding with the position in the trace, halves of the head paired (sign -1: its transpose)."""
+    half = x.shape[-1] // 2
+    at = torch.cat([torch.arange(z - a, device=x.device) for a, z in zip(cu[:-1], cu[1:])]).double()
+    angle = at[:, None] * 10000.0 ** (-torch.arange(half, device=x.device).double() / half)
+    c, n = angle.cos()[:, None], sign * angle.sin()[:, None]
+    lo, hi = x[..., :half], x[..., half:]
+    return torch.cat((lo * c - hi * n, hi * c + lo * n), dim=-1)
+
+
+def exact_cache(case, s, wide, scale):
+    cache, Hkv, d = s["cache"], case["Hkv"], case["d"]
+    steps = case.get("turn", 1)
+    q = wide(s["q"]).view(steps, -1, Hkv, case["Hq"] // Hkv, d)
+    out, lse = torch.empty_like(q), q.new_empty(q.shape[:-1])
+    for b, n in enumerate(cache.n_tokens.tolist()):
+        pages = cache.block_table[b, :-(-n // case["page"])].long()
+        k, v = (wide(c[pages]).reshape(-1, Hkv, d)[:n].transpose(0, 1) for c in (cache.k_cache, cache.v_cache))
+        for t in range(steps):
+            if case["kind"] == "turn":
+                k, v = torch.cat((k, wide(s["k"][t, b])[:, None]), dim=1), torch.cat((v, wide(s["v"][t, b])[:, None]), dim=1)
+            score = q[t, b] @ k.transpose(1, 2) * scale
+            lse[t, b] = torch.logsumexp(score, dim=2)
+            out[t, b] = torch.softmax(score, dim=2) @ v
+    got = [(o.flatten(1, 2), m.flatten(1, 2)) for o, m in zip(out, lse)]
+    return got[0] if case["kind"] == "decode" else (got, cache.n_tokens)
