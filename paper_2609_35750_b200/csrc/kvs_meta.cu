@@ -159,12 +159,15 @@ meta_order_kernel(MetaHeader* hdr, const int32_t* __restrict__ row_cnt, const in
     __shared__ int warp_tot[32];
     const int n = hdr->nblk_total;
     const bool bwd = blockIdx.x == 1;
+    const bool exact = hdr->max_seqlen <= 16 * TILE;
     int32_t* order = bwd ? bwd_order : fwd_order;
     auto key = [&](int i) {
-        // coarse buckets (16 tiles): exact lengths would interleave blocks from all over the batch,
-        // coarse ones keep runs of neighbouring blocks together while still starting the long ones first
-        const int k = bwd ? (col_last[i] - col_first[i] + 1) : row_cnt[i];
-        return min(max(k >> 4, 0), ORDER_BINS - 1);
+        // Coarse buckets (16 tiles): exact lengths would interleave blocks from all over the batch, coarse ones keep runs of
+        // neighbouring blocks together while still starting the long ones first.  Where no trace has more than 16 tiles they
+        // would all fall into one bucket and the longest might start last: there the lengths are exact (96 traces of 60 to
+        // 900 tokens: step 955 -> 894 us; 12 traces of 1500 to 12000 tokens with exact short lengths: 8274 -> 8678 us).
+        const int k = max(bwd ? (col_last[i] - col_first[i] + 1) : row_cnt[i], 0);
+        return min(exact ? k : k >> 4, ORDER_BINS - 1);
     };
     for (int i = threadIdx.x; i < ORDER_BINS; i += blockDim.x) bins[i] = 0;
     __syncthreads();
