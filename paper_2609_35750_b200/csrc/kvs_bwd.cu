@@ -6,7 +6,7 @@
 //              contiguous range of query blocks n .. col_last[n] that can see the key block
 //              (see the comment above bwd_kernel for the pipeline)
 //   post-pass  fp32 dQ accumulator -> bf16 (bf16 gradients only)
-#include "kvs_common.cuh"
+#include "kvs_bwd.cuh"
 
 namespace kvs {
 
@@ -112,8 +112,6 @@ __global__ void bwd_cast_kernel(const float* __restrict__ acc, __nv_bfloat16* __
 // is folded into dS (dS = P (scale dP - scale D)), so dK and dQ leave the tensor core scaled.
 // Rows of a dQ tile past the end of a trace are exactly zero (their P is zero), so the reduce-add
 // of a whole 128-row box is harmless where it overlaps the next trace.
-constexpr int BWD_THREADS = 512;
-
 template <int D>
 struct BwdSmem {
     static constexpr int TB = TILE * D * 2;
@@ -131,19 +129,6 @@ struct BwdSmem {
     static constexpr int TOTAL = OFF_MISC + 16;
     static constexpr int MAX_DYN = 232448;                     // 227 KB
     static constexpr int DYN_BYTES = (TOTAL + 1024 > MAX_DYN) ? MAX_DYN : TOTAL + 1024;
-};
-
-struct BwdParams {
-    int batch, total_tokens, max_seqlen;   // what the caller says meta_buf was built for
-    int Hq, Hkv;
-    float scale, scale_log2;
-    const float* lse;
-    const float* dvec;
-    void* dk;
-    void* dv;
-    long long dkv_ts;       // elements between consecutive tokens of dk and dv
-    int grad_fp32;
-    int32_t* status;
 };
 
 template <int D>
@@ -187,13 +172,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     const bool general = mv.hdr->general != 0;
     if (nm <= 0) {
         // no query sees any key of the block (general metadata only): its gradients are zero
-        const int rows = min(TILE, T - n * TILE);
-        const size_t per_row = (size_t)D * (p.grad_fp32 ? 4 : 2) / 16;          // 16-byte words of one (token, head) row
-        for (int i = tid; i < rows * (int)per_row; i += BWD_THREADS) {
-            const size_t off = (size_t)(tok0 + n * TILE + i / (int)per_row) * (size_t)(p.dkv_ts / D) * per_row + (size_t)g * per_row + i % (int)per_row;
-            reinterpret_cast<uint4*>(p.dk)[off] = make_uint4(0, 0, 0, 0);
-            reinterpret_cast<uint4*>(p.dv)[off] = make_uint4(0, 0, 0, 0);
-        }
+        bwd_zero_rows<D>(p, tok0 + n * TILE, min(TILE, T - n * TILE), g);
         return;
     }
 
@@ -517,26 +496,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
                 uint32_t r[32];
                 tmem_ld32(src + ch * 32, r);
                 tmem_wait_ld();
-                if (kvalid) {
-                    if (p.grad_fp32) {
-                        float4* dst = reinterpret_cast<float4*>(reinterpret_cast<float*>(base) + orow + ch * 32);
-#pragma unroll
-                        for (int e = 0; e < 8; ++e)
-                            dst[e] = make_float4(__uint_as_float(r[e * 4]), __uint_as_float(r[e * 4 + 1]), __uint_as_float(r[e * 4 + 2]),
-                                                 __uint_as_float(r[e * 4 + 3]));
-                    } else {
-                        uint4* dst = reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(base) + orow + ch * 32);
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            uint4 w;
-                            w.x = pack_bf16(__uint_as_float(r[e * 8 + 0]), __uint_as_float(r[e * 8 + 1]));
-                            w.y = pack_bf16(__uint_as_float(r[e * 8 + 2]), __uint_as_float(r[e * 8 + 3]));
-                            w.z = pack_bf16(__uint_as_float(r[e * 8 + 4]), __uint_as_float(r[e * 8 + 5]));
-                            w.w = pack_bf16(__uint_as_float(r[e * 8 + 6]), __uint_as_float(r[e * 8 + 7]));
-                            dst[e] = w;
-                        }
-                    }
-                }
+                if (kvalid) bwd_store_cols(base, orow + ch * 32, r, p.grad_fp32);
             }
         }
     }
@@ -549,25 +509,25 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
 }
 
 template <int D>
-static int launch_bwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tdo,
-                      const CUtensorMap& tdq, const MetaView& mv,
-                      const BwdParams& p, const __nv_bfloat16* dout, const __nv_bfloat16* out, float* dvec, float* dq_acc, long long dq_ts,
-                      WsHeader* hdr, int nb_cap, cudaStream_t st, cudaEvent_t ev0, cudaEvent_t ev1) {
-    {
-        const long long rows = (long long)p.total_tokens * p.Hq;
-        const int rows_per_warp = (32 / (D / 8)) * DOT_ROWS;
-        const long long warps = (rows + rows_per_warp - 1) / rows_per_warp;
-        const int threads = 256;
-        const long long blocks = (warps * 32 + threads - 1) / threads;
-        if (blocks > 0x7fffffffLL) return KVS_ERR_UNSUPPORTED;
-        bwd_dot_kernel<D><<<(unsigned)(blocks > 0 ? blocks : 1), threads, 0, st>>>(dout, out, dvec, dq_acc, dq_ts, p.total_tokens, p.Hq, hdr);
-    }
+static int launch_dot(const __nv_bfloat16* dout, const __nv_bfloat16* out, float* dvec, float* dq_acc, long long dq_ts, int total_tokens, int Hq,
+                      WsHeader* hdr, cudaStream_t st) {
+    const long long rows = (long long)total_tokens * Hq;
+    const int rows_per_warp = (32 / (D / 8)) * DOT_ROWS;
+    const long long warps = (rows + rows_per_warp - 1) / rows_per_warp;
+    const int threads = 256;
+    const long long blocks = (warps * 32 + threads - 1) / threads;
+    if (blocks > 0x7fffffffLL) return KVS_ERR_UNSUPPORTED;
+    bwd_dot_kernel<D><<<(unsigned)(blocks > 0 ? blocks : 1), threads, 0, st>>>(dout, out, dvec, dq_acc, dq_ts, total_tokens, Hq, hdr);
+    return cudaGetLastError() == cudaSuccess ? KVS_OK : KVS_ERR_CUDA;
+}
+
+template <int D>
+static int launch_main(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tdo, const CUtensorMap& tdq,
+                       const MetaView& mv, const BwdParams& p, int nb_cap, cudaStream_t st) {
     auto kern = bwd_kernel<D>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdSmem<D>::DYN_BYTES) != cudaSuccess) return KVS_ERR_CUDA;
     dim3 grid(nb_cap, p.Hkv, 1);
-    if (ev0 && cudaEventRecord(ev0, st) != cudaSuccess) return KVS_ERR_CUDA;
     kern<<<grid, BWD_THREADS, BwdSmem<D>::DYN_BYTES, st>>>(tq, tk, tv, tdo, tdq, mv, p);
-    if (ev1 && cudaEventRecord(ev1, st) != cudaSuccess) return KVS_ERR_CUDA;
     return cudaGetLastError() == cudaSuccess ? KVS_OK : KVS_ERR_CUDA;
 }
 
@@ -582,6 +542,8 @@ extern "C" size_t kvs_attn_bwd_workspace_bytes(int total_tokens, int Hq, int Hkv
 }
 
 namespace {
+bool use_pairs(int batch, int total_tokens, int max_seqlen, int Hkv, int head_dim) { return head_dim == 128; }
+
 // in_ts: elements between consecutive tokens of q and of k, v; g_ts: of dq and of dk, dv (0: tensors of their own)
 int bwd_impl(const void* dout, const void* q, const void* k, const void* v, long long in_ts, const void* out, const float* lse,
              const void* meta_buf, int batch, int total_tokens, int max_seqlen, int Hq, int Hkv, int head_dim,
@@ -604,11 +566,13 @@ int bwd_impl(const void* dout, const void* q, const void* k, const void* v, long
     if (rc != KVS_OK) return rc;
     const MetaLayout L = meta_layout(batch, total_tokens, max_seqlen);
     const MetaView mv = meta_view(meta_buf, L);
+    const bool pair = use_pairs(batch, total_tokens, max_seqlen, Hkv, head_dim);
+    const int q_rows = pair ? TILE / 2 : TILE;       // rows of the boxes of q, dout and dq
     CUtensorMap tq, tk, tv, tdo, tdq;
-    if ((rc = make_tmap_thd(&tq, q, total_tokens, Hq, head_dim, TILE, in_ts)) != KVS_OK) return rc;
+    if ((rc = make_tmap_thd(&tq, q, total_tokens, Hq, head_dim, q_rows, in_ts)) != KVS_OK) return rc;
     if ((rc = make_tmap_thd(&tk, k, total_tokens, Hkv, head_dim, TILE, in_ts)) != KVS_OK) return rc;
     if ((rc = make_tmap_thd(&tv, v, total_tokens, Hkv, head_dim, TILE, in_ts)) != KVS_OK) return rc;
-    if ((rc = make_tmap_thd(&tdo, dout, total_tokens, Hq, head_dim, TILE)) != KVS_OK) return rc;
+    if ((rc = make_tmap_thd(&tdo, dout, total_tokens, Hq, head_dim, q_rows)) != KVS_OK) return rc;
     cudaStream_t st = (cudaStream_t)stream;
     char* ws = (char*)workspace;
     const size_t nq = (size_t)total_tokens * Hq * head_dim;
@@ -627,16 +591,21 @@ int bwd_impl(const void* dout, const void* q, const void* k, const void* v, long
     const long long dq_ts_out = g_ts > 0 ? g_ts : (long long)Hq * head_dim;
     float* dq_acc = grad_dtype == KVS_GRAD_FP32 ? (float*)dq : (float*)(ws + W.dq_acc);
     const long long dq_ts = grad_dtype == KVS_GRAD_FP32 ? dq_ts_out : (long long)Hq * head_dim;
-    if ((rc = make_tmap_f32_thd(&tdq, dq_acc, total_tokens, Hq, head_dim, TILE, dq_ts)) != KVS_OK) return rc;
+    if ((rc = make_tmap_f32_thd(&tdq, dq_acc, total_tokens, Hq, head_dim, q_rows, dq_ts)) != KVS_OK) return rc;
     p.dk = dk;
     p.dv = dv;
     p.dkv_ts = g_ts > 0 ? g_ts : (long long)Hkv * head_dim;
     p.grad_fp32 = grad_dtype == KVS_GRAD_FP32;
     p.status = &((WsHeader*)ws)->status;
-    rc = head_dim == 64 ? launch_bwd<64>(tq, tk, tv, tdo, tdq, mv, p, (const __nv_bfloat16*)dout, (const __nv_bfloat16*)out, (float*)(ws + W.dvec),
-                                         dq_acc, dq_ts, (WsHeader*)ws, L.nb_cap, st, ev0, ev1)
-                        : launch_bwd<128>(tq, tk, tv, tdo, tdq, mv, p, (const __nv_bfloat16*)dout, (const __nv_bfloat16*)out,
-                                          (float*)(ws + W.dvec), dq_acc, dq_ts, (WsHeader*)ws, L.nb_cap, st, ev0, ev1);
+    const __nv_bfloat16 *dout16 = (const __nv_bfloat16*)dout, *out16 = (const __nv_bfloat16*)out;
+    rc = head_dim == 64 ? launch_dot<64>(dout16, out16, (float*)(ws + W.dvec), dq_acc, dq_ts, total_tokens, Hq, (WsHeader*)ws, st)
+                        : launch_dot<128>(dout16, out16, (float*)(ws + W.dvec), dq_acc, dq_ts, total_tokens, Hq, (WsHeader*)ws, st);
+    if (rc != KVS_OK) return rc;
+    if (ev0 && cudaEventRecord(ev0, st) != cudaSuccess) return KVS_ERR_CUDA;
+    rc = pair             ? launch_bwd_pair(tq, tk, tv, tdo, tdq, mv, p, L.nb_cap, st)
+         : head_dim == 64 ? launch_main<64>(tq, tk, tv, tdo, tdq, mv, p, L.nb_cap, st)
+                          : launch_main<128>(tq, tk, tv, tdo, tdq, mv, p, L.nb_cap, st);
+    if (rc == KVS_OK && ev1 && cudaEventRecord(ev1, st) != cudaSuccess) return KVS_ERR_CUDA;
     if (rc != KVS_OK) return rc;
     if (grad_dtype == KVS_GRAD_BF16) {
         const size_t n4 = nq / 4;

@@ -26,13 +26,14 @@ struct MetaHeader {
     int32_t nblk_total;    // sum over traces of ceil(T_b / 128), written on the device
     uint32_t ncls_total;   // sum over traces of nb^2
     int32_t general;       // 1: every key slot carries its own first visible query (kvs_mask_meta_keys); 0: slot j is key j
+    int32_t npair_total;   // sum over traces of ceil(nb_b / 2): pairs of neighbouring key blocks
 };
 
 // Byte offsets of the arrays inside meta_buf; a pure function of the three sizes so that
 // every entry point can recompute it.
 struct MetaLayout {
-    size_t blk_off, cls_off, seq_start, blk_trace, kmin, kmax, fmin, fmax, col_first, col_last, row_cnt, fwd_order, bwd_order, evict, kfirst,
-        tile_class, row_list, total;
+    size_t blk_off, cls_off, seq_start, blk_trace, kmin, kmax, fmin, fmax, col_first, col_last, row_cnt, fwd_order, bwd_order, pair_order, evict,
+        kfirst, tile_class, row_list, total;
     int nb_cap;            // capacity in blocks
     size_t cls_cap;        // capacity in tiles
 };
@@ -66,6 +67,7 @@ __host__ __device__ inline MetaLayout meta_layout(int batch, int total_tokens, i
     L.row_cnt = o;   o = align_up(o + sizeof(int32_t) * nb_cap, 256);
     L.fwd_order = o; o = align_up(o + sizeof(int32_t) * nb_cap, 256);
     L.bwd_order = o; o = align_up(o + sizeof(int32_t) * nb_cap, 256);
+    L.pair_order = o; o = align_up(o + sizeof(int32_t) * nb_cap, 256);
     L.evict = o;     o = align_up(o + sizeof(int32_t) * (size_t)(total_tokens > 0 ? total_tokens : 1), 256);
     L.kfirst = o;    o = align_up(o + sizeof(int32_t) * (size_t)(total_tokens > 0 ? total_tokens : 1), 256);
     L.tile_class = o; o = align_up(o + L.cls_cap, 256);
@@ -90,6 +92,7 @@ struct MetaView {
     const int32_t* row_cnt;     // [nblk] non-empty key blocks of a query block row
     const int32_t* fwd_order;   // [nblk] query blocks, heaviest first
     const int32_t* bwd_order;   // [nblk] key blocks, longest query range first
+    const int32_t* pair_order;  // [npair] first key block of each pair (2p, 2p+1) of a trace, longest query range first
     const int32_t* evict;       // [total_tokens] eviction step of every key slot (copy of evict_at / key_evict)
     const int32_t* kfirst;      // [total_tokens] first query that may see the slot (general metadata only)
     const uint8_t* tile_class;  // [ncls]
@@ -113,6 +116,7 @@ inline MetaView meta_view(const void* buf, const MetaLayout& L) {
     v.row_cnt = (const int32_t*)(p + L.row_cnt);
     v.fwd_order = (const int32_t*)(p + L.fwd_order);
     v.bwd_order = (const int32_t*)(p + L.bwd_order);
+    v.pair_order = (const int32_t*)(p + L.pair_order);
     v.evict = (const int32_t*)(p + L.evict);
     v.kfirst = (const int32_t*)(p + L.kfirst);
     v.tile_class = (const uint8_t*)(p + L.tile_class);
@@ -151,6 +155,22 @@ __device__ __forceinline__ void set_status(int32_t* status, int code) { atomicCA
 __device__ __forceinline__ bool meta_matches(const MetaHeader* hdr, int batch, int total_tokens, int max_seqlen) {
     return hdr->magic == META_MAGIC && hdr->batch == batch && hdr->total_tokens == total_tokens &&
            hdr->max_seqlen == max_seqlen;
+}
+
+// Query blocks that see key block `even` or, where the trace has one, the block after it (none: last < first).
+__device__ __forceinline__ void pair_range(const int32_t* col_first, const int32_t* col_last, int even, bool has_odd, int& first, int& last) {
+    first = col_first[even];
+    last = col_last[even];
+    if (has_odd) {
+        const int f1 = col_first[even + 1], l1 = col_last[even + 1];
+        if (last < first) {
+            first = f1;
+            last = l1;
+        } else if (l1 >= f1) {
+            first = min(first, f1);
+            last = max(last, l1);
+        }
+    }
 }
 
 // ------------------------------------------------------------------------------------------

@@ -149,29 +149,44 @@ __global__ void meta_classify_kernel(MetaHeader* hdr, const int32_t* __restrict_
 
 // ---- kernel 3: work orders, heaviest first (bucket sort, one CTA per order) -------------------
 // blockIdx.x = 0: query blocks by their number of non-empty key blocks (forward);
-// blockIdx.x = 1: key blocks by the length of their query-block range (backward).
+// blockIdx.x = 1: key blocks by the length of their query-block range (backward);
+// blockIdx.x = 2: pairs (2p, 2p+1) of a trace's key blocks by the length of their joint range (backward by CTA pairs).
 // Only the launch order of work depends on it; ties keep their order in the batch.
 constexpr int ORDER_BINS = 4096;
 __global__ void __launch_bounds__(1024)
-meta_order_kernel(MetaHeader* hdr, const int32_t* __restrict__ row_cnt, const int32_t* __restrict__ col_first,
-                  const int32_t* __restrict__ col_last, int32_t* fwd_order, int32_t* bwd_order) {
+meta_order_kernel(MetaHeader* hdr, const int32_t* __restrict__ blk_off, const int32_t* __restrict__ blk_trace,
+                  const int32_t* __restrict__ row_cnt, const int32_t* __restrict__ col_first, const int32_t* __restrict__ col_last,
+                  int32_t* fwd_order, int32_t* bwd_order, int32_t* pair_order) {
     __shared__ int bins[ORDER_BINS];
     __shared__ int warp_tot[32];
     const int n = hdr->nblk_total;
-    const bool bwd = blockIdx.x == 1;
+    const bool bwd = blockIdx.x == 1, pairs = blockIdx.x == 2;
     const bool exact = hdr->max_seqlen <= 16 * TILE;
-    int32_t* order = bwd ? bwd_order : fwd_order;
+    int32_t* order = pairs ? pair_order : bwd ? bwd_order : fwd_order;
     auto key = [&](int i) {
         // Coarse buckets (16 tiles): exact lengths would interleave blocks from all over the batch, coarse ones keep runs of
         // neighbouring blocks together while still starting the long ones first.  Where no trace has more than 16 tiles they
         // would all fall into one bucket and the longest might start last: there the lengths are exact (96 traces of 60 to
         // 900 tokens: step 955 -> 894 us; 12 traces of 1500 to 12000 tokens with exact short lengths: 8274 -> 8678 us).
-        const int k = max(bwd ? (col_last[i] - col_first[i] + 1) : row_cnt[i], 0);
+        int k;
+        if (pairs) {
+            const int b = blk_trace[i];
+            if ((i - blk_off[b]) & 1) return -1;       // the second block of a pair is not an item of its own
+            int first, last;
+            pair_range(col_first, col_last, i, i + 1 < blk_off[b + 1], first, last);
+            k = last - first + 1;
+        } else {
+            k = bwd ? (col_last[i] - col_first[i] + 1) : row_cnt[i];
+        }
+        k = max(k, 0);
         return min(exact ? k : k >> 4, ORDER_BINS - 1);
     };
     for (int i = threadIdx.x; i < ORDER_BINS; i += blockDim.x) bins[i] = 0;
     __syncthreads();
-    for (int i = threadIdx.x; i < n; i += blockDim.x) atomicAdd(&bins[key(i)], 1);
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const int k = key(i);
+        if (k >= 0) atomicAdd(&bins[k], 1);
+    }
     __syncthreads();
     // exclusive scan over the bins in DESCENDING key order: thread t owns 4 consecutive reversed bins
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -205,6 +220,7 @@ meta_order_kernel(MetaHeader* hdr, const int32_t* __restrict__ row_cnt, const in
         bins[ORDER_BINS - 1 - (threadIdx.x * 4 + u)] = run;
         run += c[u];
     }
+    if (pairs && threadIdx.x == blockDim.x - 1) hdr->npair_total = run;
     __syncthreads();
     // Stable scatter by one warp, 32 blocks at a time in index order: blocks with equal keys keep their
     // order in the trace, so CTAs launched together work on neighbouring blocks and share tiles in L2.
@@ -213,9 +229,9 @@ meta_order_kernel(MetaHeader* hdr, const int32_t* __restrict__ row_cnt, const in
             const int i = i0 + lane;
             const int k = (i < n) ? key(i) : -1;
             const unsigned same = __match_any_sync(0xffffffffu, k);
-            if (i < n) order[bins[k] + __popc(same & ((1u << lane) - 1u))] = i;
+            if (k >= 0) order[bins[k] + __popc(same & ((1u << lane) - 1u))] = i;
             __syncwarp();
-            if (i < n && lane == (__ffs(same) - 1)) bins[k] += __popc(same);
+            if (k >= 0 && lane == (__ffs(same) - 1)) bins[k] += __popc(same);
             __syncwarp();
         }
     }
@@ -286,7 +302,8 @@ int launch_mask_meta(const int32_t* key_evict, const int32_t* key_first, int com
     meta_classify_kernel<<<grid, warps_per_cta * 32, 0, st>>>(v.hdr, v.blk_off, v.cls_off, v.seq_start, v.blk_trace, v.kmin, v.kmax,
                                                               v.fmin, v.fmax, (uint8_t*)v.tile_class, (uint16_t*)v.row_list,
                                                               (int32_t*)v.row_cnt);
-    meta_order_kernel<<<2, 1024, 0, st>>>(v.hdr, v.row_cnt, v.col_first, v.col_last, (int32_t*)v.fwd_order, (int32_t*)v.bwd_order);
+    meta_order_kernel<<<3, 1024, 0, st>>>(v.hdr, v.blk_off, v.blk_trace, v.row_cnt, v.col_first, v.col_last, (int32_t*)v.fwd_order,
+                                         (int32_t*)v.bwd_order, (int32_t*)v.pair_order);
     return cudaGetLastError() == cudaSuccess ? KVS_OK : KVS_ERR_CUDA;
 }
 }  // namespace
