@@ -390,21 +390,19 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         const uint32_t lane_sel = (uint32_t)(quad * 32) << 16;
         const int col0 = half * 64;                        // this thread's 64 query columns
         const int kj = n * TILE + row;
-        const int my_ev = (kj < T) ? mv.evict[tok0 + kj] : 0;          // 0: visible to nobody
-        const int my_first = (general && kj < T) ? mv.kfirst[tok0 + kj] : kj;   // first query that may see this key slot
-        const bool key_tail = (n * TILE + TILE > T);
-        const uint8_t* cls_col = mv.tile_class + mv.cls_off[b] + n;   // class of (m, n) at cls_col[m * nb]
+        // queries [my_first, my_end) of the trace see this key; nobody sees a slot past the trace
+        const int my_end = (kj < T) ? min(mv.evict[tok0 + kj], T) : 0;
+        const int my_first = (general && kj < T) ? mv.kfirst[tok0 + kj] : kj;
         const float* sLse = reinterpret_cast<const float*>(sgen + L::OFF_LSE);
         const float* sDv = reinterpret_cast<const float*>(sgen + L::OFF_DVEC);
         uint8_t* sDS_row = sgen + L::OFF_DS + half * BOX_BYTES + row * 128;
         float pv[64];
-        int cls_next = cls_col[(size_t)m_first * nb];      // class of the tile of the next phase_p, fetched early
+        int m = m_first;                                   // query block of the tile of the next phase_p
 
         auto phase_p = [&](int j) {        // P^T(j) = exp2(S^T * c - lse), masked
             const int s = j & 1;
-            const int m = m_first + j % nm;
-            const bool need_mask = (cls_next != KVS_CLASS_FULL) || key_tail || (m * TILE + TILE > T);
-            if (j + 1 < n_iter) cls_next = cls_col[(size_t)(m_first + (j + 1) % nm) * nb];
+            const int lo = my_first - (m * TILE + col0), hi = my_end - (m * TILE + col0);     // columns [lo, hi) see the key
+            m = (m == m_last) ? m_first : m + 1;
             mbar_wait(bar_ldfull(s), (j >> 1) & 1, abort_flag, status);
             mbar_wait(bar_s, j & 1, abort_flag, status);
             tc_fence_after();
@@ -425,12 +423,13 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
                 pv[e4 * 4 + 2] = fast_exp2(x23.x);
                 pv[e4 * 4 + 3] = fast_exp2(x23.y);
             }
-            if (need_mask) {
+            // Only the warps that hold a hidden pair pay for the mask, whatever the class of the tile (a loop of at most one
+            // pass: as an if, its 64 selects are predicated and issued for every tile)
+            const int masked = __any_sync(0xffffffffu, lo > 0 || hi < 64) ? 1 : 0;
+#pragma unroll 1
+            for (int pass = 0; pass < masked; ++pass) {
 #pragma unroll
-                for (int e = 0; e < 64; ++e) {
-                    const int qi = m * TILE + col0 + e;
-                    pv[e] = ((my_first <= qi) && (qi < my_ev) && (qi < T)) ? pv[e] : 0.f;
-                }
+                for (int e = 0; e < 64; ++e) pv[e] = (e >= lo && e < hi) ? pv[e] : 0.f;
             }
             uint32_t pk[32];
 #pragma unroll
@@ -542,7 +541,7 @@ extern "C" size_t kvs_attn_bwd_workspace_bytes(int total_tokens, int Hq, int Hkv
 }
 
 namespace {
-bool use_pairs(int batch, int total_tokens, int max_seqlen, int Hkv, int head_dim) { return head_dim == 128; }
+bool use_pairs(int batch, int total_tokens, int max_seqlen, int Hkv, int head_dim) { return false; }
 
 // in_ts: elements between consecutive tokens of q and of k, v; g_ts: of dq and of dk, dv (0: tensors of their own)
 int bwd_impl(const void* dout, const void* q, const void* k, const void* v, long long in_ts, const void* out, const float* lse,
