@@ -1,7 +1,7 @@
 // Host glue shared by the entry points: error text, tensor maps, device check, status read.
 #include <cudaTypedefs.h>
 
-#include "kvs_common.cuh"
+#include "kvs_bwd.cuh"
 #include <mutex>
 #include <vector>
 
@@ -211,7 +211,7 @@ void plan_trace_ranges(const int32_t* cu, int batch, int total_tokens, int want,
 }
 
 struct ArenaLayout {
-    size_t evict, cu, sticky, meta, slot0, slot_stride, total;      // global part, then HOST_SLOTS equal slots
+    size_t evict, cu, sticky, meta, meta_all, cu_all, slot0, slot_stride, total;      // global part, then HOST_SLOTS equal slots
     size_t q, k, v, dout, out, lse, dq, dk, dv, ws;                  // offsets inside a slot
     size_t meta_stride, ws_bytes;
     int slots, ranges, slot_tokens;
@@ -237,6 +237,10 @@ ArenaLayout arena_layout(int batch, int total_tokens, int max_seqlen, int Hq, in
     A.cu = o;    o = align_up(o + (size_t)(batch + A.ranges) * 4, 256);
     A.sticky = o; o += 256;
     A.meta = o;  o += (size_t)A.ranges * A.meta_stride;
+    // metadata of the whole batch, for the plan of the backward, where the ranges are parts of it
+    const size_t all = A.ranges > 1 ? align_up(kvs_mask_meta_bytes(batch, total_tokens, max_seqlen), 256) : 0;
+    A.meta_all = o; o += all;
+    A.cu_all = o;   o = align_up(o + (A.ranges > 1 ? (size_t)(batch + 1) * 4 : 0), 256);
     A.slot0 = o;
     size_t t = 0;
     A.q = t;     t = align_up(t + nq, 256);
@@ -351,6 +355,18 @@ extern "C" int kvs_attn_fwd_bwd_host(const int32_t* evict_at_host, const int32_t
                            meta, A.meta_stride, stream);
         if (rc != KVS_OK) return rc;
     }
+    BwdWhole whole = {a + A.meta, batch, total_tokens, max_seqlen, Hkv};
+    if (A.ranges > 1) {
+        whole.meta_buf = a + A.meta_all;
+        KVS_CK(cudaMemcpyAsync(a + A.cu_all, cu_seqlens_host, (size_t)(batch + 1) * 4, cudaMemcpyHostToDevice, st));
+        rc = kvs_mask_meta((const int32_t*)(a + A.evict), (const int32_t*)(a + A.cu_all), batch, total_tokens, max_seqlen, a + A.meta_all,
+                           A.cu_all - A.meta_all, stream);
+        if (rc != KVS_OK) return rc;
+    } else {
+        whole.batch = ranges[0].b1 - ranges[0].b0;
+        whole.total_tokens = ranges[0].tokens;
+        whole.max_seqlen = ranges[0].maxlen;
+    }
     KVS_CK(cudaEventRecord(ev_start, st));                 // the internal streams start after what the caller queued before
     KVS_CK(cudaStreamWaitEvent(R.in, ev_start, 0));
     KVS_CK(cudaStreamWaitEvent(R.outs, ev_start, 0));
@@ -398,7 +414,7 @@ extern "C" int kvs_attn_fwd_bwd_host(const int32_t* evict_at_host, const int32_t
         KVS_CK(cudaMemcpy2DAsync((char*)lse_host + ((size_t)kh * G * total_tokens + g.tok0) * 4, (size_t)total_tokens * 4, sl + A.lse,
                                  (size_t)g.tokens * 4, (size_t)g.tokens * 4, (size_t)G, cudaMemcpyDeviceToHost, R.outs));
         KVS_CK(cudaStreamWaitEvent(st, ev_dout(c), 0));
-        rc = kvs_attn_bwd(sl + A.dout, sl + A.q, sl + A.k, sl + A.v, sl + A.out, (const float*)(sl + A.lse), meta, nb, g.tokens, g.maxlen,
+        rc = bwd_of_chunk(whole, sl + A.dout, sl + A.q, sl + A.k, sl + A.v, sl + A.out, (const float*)(sl + A.lse), meta, nb, g.tokens, g.maxlen,
                           G, 1, head_dim, softmax_scale, grad_dtype, sl + A.dq, sl + A.dk, sl + A.dv, sl + A.ws, A.ws_bytes, stream);
         if (rc != KVS_OK) return rc;
         fold_status_kernel<<<1, 1, 0, st>>>((const int32_t*)(sl + A.ws), (int32_t*)(a + A.sticky));

@@ -7,11 +7,18 @@
 //              (see the comment above bwd_kernel for the pipeline)
 //   post-pass  fp32 dQ accumulator -> bf16 (bf16 gradients only)
 #include "kvs_bwd.cuh"
+#include <cstring>
 
 namespace kvs {
 
+constexpr int BWD_SMS = 148;
+constexpr int BWD_MIN_UNIT = 4;             // tiles: a shorter unit is mostly its own start and end
+constexpr int BWD_MAX_SLOTS = 2 * BWD_SMS;  // slots of one CTA each for the dK and dV of cut items, over all KV heads
+
 struct BwdWsLayout {
-    size_t dvec, dq_acc, total;
+    size_t dvec, dq_acc, base;              // base: what is needed without cutting items
+    size_t plan, units, arrived, part, total;
+    int slots, unit_cap;                    // slots of one CTA; entries of the unit list
 };
 
 __host__ __device__ inline BwdWsLayout bwd_ws_layout(int total_tokens, int Hq, int head_dim, int grad_dtype) {
@@ -21,8 +28,190 @@ __host__ __device__ inline BwdWsLayout bwd_ws_layout(int total_tokens, int Hq, i
     o = align_up(o + sizeof(float) * (size_t)total_tokens * Hq, 256);
     L.dq_acc = o;
     if (grad_dtype == KVS_GRAD_BF16) o = align_up(o + sizeof(float) * (size_t)total_tokens * Hq * head_dim, 256);
+    L.base = o;
+    // An item of t tiles cut into units of at least BWD_MIN_UNIT tiles has at most 2 t / BWD_MIN_UNIT of them, and all items
+    // of a batch have at most Hq nb (nb + 1) / 2 tiles (one trace, nothing evicted).
+    const long long nb = ((long long)total_tokens + TILE - 1) / TILE;
+    const long long most = Hq * nb * (nb + 1) / BWD_MIN_UNIT;
+    L.slots = (int)(most < BWD_MAX_SLOTS ? most : BWD_MAX_SLOTS);
+    // key blocks of a batch: short traces have more than total / 128; beyond 4096 more the items are not cut
+    L.unit_cap = (int)((total_tokens < nb + 4096 ? total_tokens : nb + 4096) + L.slots);
+    L.plan = o;    o = align_up(o + sizeof(BwdPlan), 256);
+    L.units = o;   o = align_up(o + sizeof(BwdUnit) * (size_t)L.unit_cap, 256);
+    L.arrived = o; o = align_up(o + sizeof(int32_t) * 2 * (size_t)L.slots, 256);
+    L.part = o;    o = align_up(o + sizeof(float) * 2 * TILE * (size_t)head_dim * L.slots, 256);
     L.total = o;
     return L;
+}
+
+// ---- plan ---------------------------------------------------------------------------------------
+struct BwdPlanArgs {
+    MetaView all, mv;                       // the batch the cut is chosen for; the (part of the) batch whose units are listed
+    int all_batch, all_tokens, all_maxlen, batch, tokens, maxlen;
+    int pairs;                              // items are pairs of key blocks
+    int G, all_Hkv, Hkv;
+    int all_slots, slots;                   // slots there are, of an item's CTAs, over all KV heads
+    BwdPlan* plan;                          // nullptr: none is wanted
+    BwdUnit* units;
+    int32_t* arrived;
+    int arrived_n;
+};
+
+__device__ __forceinline__ int bwd_item(const MetaView& mv, int pairs, int G, int x, int& block) {
+    block = pairs ? mv.pair_order[x] : mv.bwd_order[x];
+    int first = mv.col_first[block], last = mv.col_last[block];
+    if (pairs) pair_range(mv.col_first, mv.col_last, block, block + 1 < mv.blk_off[mv.blk_trace[block] + 1], first, last);
+    return G * max(last - first + 1, 0);
+}
+
+// One CTA of 256 threads, beside the pre-pass.  Chooses the longest unit L among eight candidates (fractions of an SM's, or
+// pair's, share of all tiles, and "no cut") by an estimate of the makespan in tiles, then lists the units.  An item of t
+// tiles becomes ceil(t / L) units of equal length.  The estimate: a unit costs BWD_UNIT_COST tiles beside its own (loads
+// before the first product, the pipeline's first and last tile, the stores), what is left over at the end is half the
+// longest unit, and with up to three waves at least that many average units.
+constexpr float BWD_UNIT_COST = 3.f, BWD_CUT_COST = 2.f;
+__device__ void bwd_plan(const BwdPlanArgs& a) {
+    constexpr int NC = 8;
+    __shared__ int s_units[NC], s_cut[NC], s_longest[NC], s_max, s_len;
+    __shared__ unsigned long long s_total;
+    __shared__ int s_scan[2][8], s_run[2];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (!meta_matches(a.all.hdr, a.all_batch, a.all_tokens, a.all_maxlen) || !meta_matches(a.mv.hdr, a.batch, a.tokens, a.maxlen)) {
+        if (tid == 0) a.plan->n_units = 0;
+        return;
+    }
+    for (int i = tid; i < a.arrived_n; i += 256) a.arrived[i] = 0;
+    if (tid < NC) s_units[tid] = s_cut[tid] = s_longest[tid] = 0;
+    if (tid == 0) {
+        s_total = 0;
+        s_max = 0;
+        s_run[0] = s_run[1] = 0;
+    }
+    __syncthreads();
+    const int n_all = a.pairs ? a.all.hdr->npair_total : a.all.hdr->nblk_total;
+    const int sms = a.pairs ? BWD_SMS / 2 : BWD_SMS;
+    int block;
+    {
+        unsigned long long total = 0;
+        int most = 0;
+        for (int x = tid; x < n_all; x += 256) {
+            const int t = bwd_item(a.all, a.pairs, a.G, x, block);
+            total += t;
+            most = max(most, t);
+        }
+        atomicAdd(&s_total, total);
+        atomicMax(&s_max, most);
+    }
+    __syncthreads();
+    const float share = (float)s_total * a.all_Hkv / sms;          // tiles per SM or pair
+    const int most = max(s_max, 1);
+    int len[NC];
+    const float frac[NC] = {0.25f, 0.5f, 0.75f, 1.0f, 1.25f, 1.6f, 2.2f, 0.f};
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+        const float l = fmaxf(ceilf(share * frac[k]), (float)max(BWD_MIN_UNIT, (most + BWD_MAX_CUT - 1) / BWD_MAX_CUT));
+        len[k] = (k == NC - 1 || l > (float)most) ? most : (int)l;
+    }
+    {
+        int units[NC], cut[NC], longest[NC];
+#pragma unroll
+        for (int k = 0; k < NC; ++k) units[k] = cut[k] = longest[k] = 0;
+        for (int x = tid; x < n_all; x += 256) {
+            const int t = bwd_item(a.all, a.pairs, a.G, x, block);
+#pragma unroll
+            for (int k = 0; k < NC; ++k) {
+                const int c = max((t + len[k] - 1) / len[k], 1);
+                units[k] += c;
+                if (c > 1) cut[k] += c;
+                longest[k] = max(longest[k], (t + c - 1) / c);
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < NC; ++k) {
+            units[k] = __reduce_add_sync(0xffffffffu, units[k]);
+            cut[k] = __reduce_add_sync(0xffffffffu, cut[k]);
+            longest[k] = __reduce_max_sync(0xffffffffu, longest[k]);
+            if (lane == 0) {
+                atomicAdd(&s_units[k], units[k]);
+                atomicAdd(&s_cut[k], cut[k]);
+                atomicMax(&s_longest[k], longest[k]);
+            }
+        }
+    }
+    __syncthreads();
+    if (tid == 0) {
+        float best = 0.f;
+        int at = NC - 1;
+        for (int k = NC - 1; k >= 0; --k) {                        // "no cut" first: it always fits
+            if ((long long)s_cut[k] * a.all_Hkv > a.all_slots) continue;
+            const float units = (float)s_units[k] * a.all_Hkv, longest = (float)s_longest[k];
+            const float waves = ceilf(units / sms);
+            float est = longest + BWD_UNIT_COST;
+            if (waves > 1.f) {
+                est = share + BWD_UNIT_COST * units / sms + 0.5f * longest;
+                if (waves <= 3.f) est = fmaxf(est, waves * (share * sms / units + BWD_UNIT_COST));
+            }
+            if (s_cut[k] > 0) est += BWD_CUT_COST;
+            if (k == NC - 1 || est < best) {
+                best = est;
+                at = k;
+            }
+        }
+        s_len = len[at];
+    }
+    __syncthreads();
+    int longest = s_len;
+    const int n = a.pairs ? a.mv.hdr->npair_total : a.mv.hdr->nblk_total;
+    if (a.mv.hdr != a.all.hdr) {            // a part of the batch has no more cut units than the whole, but its slots are counted too
+        if (tid == 0) s_cut[0] = 0;
+        __syncthreads();
+        int cut = 0;
+        for (int x = tid; x < n; x += 256) {
+            const int c = (bwd_item(a.mv, a.pairs, a.G, x, block) + longest - 1) / longest;
+            if (c > 1) cut += c;
+        }
+        if (cut) atomicAdd(&s_cut[0], cut);
+        __syncthreads();
+        if ((long long)s_cut[0] * a.Hkv > a.slots) longest = most;
+    }
+    // List the units, the item's order kept: prefix sums of the items' units and of their slots
+    for (int x0 = 0; x0 < n; x0 += 256) {
+        const int x = x0 + tid;
+        const int t = x < n ? bwd_item(a.mv, a.pairs, a.G, x, block) : 0;
+        int c = x < n ? max((t + longest - 1) / longest, 1) : 0;
+        int iu = c, is = c > 1 ? c : 0;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, iu, o), s = __shfl_up_sync(0xffffffffu, is, o);
+            if (lane >= o) {
+                iu += u;
+                is += s;
+            }
+        }
+        if (lane == 31) {
+            s_scan[0][warp] = iu;
+            s_scan[1][warp] = is;
+        }
+        __syncthreads();
+        int bu = s_run[0], bs = s_run[1];
+        for (int w = 0; w < warp; ++w) {
+            bu += s_scan[0][w];
+            bs += s_scan[1][w];
+        }
+        const int u0 = bu + iu - c, slot0 = bs + is - (c > 1 ? c : 0);
+        for (int i = 0; i < c; ++i)
+            a.units[u0 + i] = BwdUnit{block, (int)((long long)t * i / c), (int)((long long)t * (i + 1) / c), c > 1 ? (slot0 << 18 | i << 9 | c) : 0};
+        __syncthreads();
+        if (tid == 255) {
+            s_run[0] = bu + iu;
+            s_run[1] = bs + is;
+        }
+        __syncthreads();
+    }
+    if (tid == 0) {
+        a.plan->n_units = s_run[0];
+        a.plan->slots = s_run[1];
+    }
 }
 
 // ---- pre-pass ---------------------------------------------------------------------------------
@@ -33,15 +222,20 @@ constexpr int DOT_ROWS = 4;
 template <int D>
 __global__ void __launch_bounds__(256)
 bwd_dot_kernel(const __nv_bfloat16* __restrict__ dout, const __nv_bfloat16* __restrict__ out,
-               float* __restrict__ dvec, float* __restrict__ dq_acc, long long dq_ts, int total_tokens, int Hq, WsHeader* hdr) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        hdr->magic = WS_MAGIC;
-        hdr->status = KVS_OK;
+               float* __restrict__ dvec, float* __restrict__ dq_acc, long long dq_ts, int total_tokens, int Hq, WsHeader* hdr,
+               const __grid_constant__ BwdPlanArgs plan) {
+    if (blockIdx.x == 0) {                      // the first CTA has no rows
+        if (threadIdx.x == 0) {
+            hdr->magic = WS_MAGIC;
+            hdr->status = KVS_OK;
+        }
+        if (plan.plan) bwd_plan(plan);
+        return;
     }
     constexpr int LPR = D / 8;                  // lanes per row: 16 or 8
     constexpr int RPW = 32 / LPR;               // rows per warp and step
     const long long rows = (long long)total_tokens * Hq;
-    const long long gw = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const long long gw = ((long long)(blockIdx.x - 1) * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     const int sub = lane / LPR, c = lane % LPR;
     const long long row0 = gw * (RPW * DOT_ROWS) + sub;
@@ -155,8 +349,9 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         if (tid == 0 && blockIdx.x == 0 && blockIdx.y == 0) set_status(p.status, KVS_ERR_BAD_META);
         return;
     }
-    if ((int)blockIdx.x >= mv.hdr->nblk_total) return;
-    const int gb = mv.bwd_order[blockIdx.x];
+    BwdUnit unit;
+    if (!bwd_unit_of(p, mv.bwd_order, mv.hdr->nblk_total, blockIdx.x, unit)) return;
+    const int gb = unit.block;
     const int g = blockIdx.y;
     const int G = p.Hq / p.Hkv;
     const int b = mv.blk_trace[gb];
@@ -167,7 +362,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     const int m_first = mv.col_first[gb];           // == n unless the key slots were re-ordered
     const int m_last = mv.col_last[gb];
     const int nm = m_last - m_first + 1;            // query blocks m_first .. m_last can see this key block
-    const int n_iter = G * nm;
+    const int n_iter = (unit.tile1 < 0 ? G * nm : unit.tile1) - unit.tile0;     // tiles of this unit of the G * nm (head, query block) tiles of the key block
     int32_t* status = p.status;
     const bool general = mv.hdr->general != 0;
     if (nm <= 0) {
@@ -175,6 +370,8 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         bwd_zero_rows<D>(p, tok0 + n * TILE, min(TILE, T - n * TILE), g);
         return;
     }
+
+    const int h_start = g * G + unit.tile0 / nm, m_start = m_first + unit.tile0 % nm;
 
     const uint32_t sraw = smem_u32(smem_raw);
     const uint32_t sbase = (sraw + 1023u) & ~1023u;
@@ -238,10 +435,9 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
                 for (int c = 0; c < NBOX; ++c) tma_load_3d(sK + c * BOX_BYTES, &tm_k, c * 64, g, tok0 + n * TILE, bar_kv);
                 for (int c = 0; c < NBOX; ++c) tma_load_3d(sV + c * BOX_BYTES, &tm_v, c * 64, g, tok0 + n * TILE, bar_kv);
             }
+            int h = h_start, m = m_start;
             for (int j = 0; j < n_iter; ++j) {
                 const int s = j & 1;
-                const int h = g * G + j / nm;
-                const int m = m_first + j % nm;
                 const int qtok = tok0 + m * TILE;
                 // Q(j), lse(j), D(j): stage s, free once every MMA of iteration j-2 has completed
                 if (j >= 2) mbar_wait(bar_qfree(s), ((j >> 1) + 1) & 1, abort_flag, status);
@@ -267,6 +463,10 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
                     for (int c = 0; c < NBOX; ++c) tma_load_3d(sDO + c * BOX_BYTES, &tm_do, c * 64, h, qtok, bar_dofull);
                 }
                 __syncwarp();
+                if (++m > m_last) {
+                    m = m_first;
+                    ++h;
+                }
             }
         } else if (warp == 13) {
             // ================= MMA issuer (all lanes walk the loop, one elected lane issues) =================
@@ -345,9 +545,8 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         const int row = quad * 32 + lane;
         const uint32_t lane_sel = (uint32_t)(quad * 32) << 16;
         uint8_t* stg_row = sgen + L::OFF_STG + row * 128;
+        int h = h_start, m = m_start;
         for (int j = 0; j < n_iter; ++j) {
-            const int h = g * G + j / nm;
-            const int m = m_first + j % nm;
             mbar_wait(bar_dq, j & 1, abort_flag, status);
             tc_fence_after();
             uint32_t r[D];
@@ -379,6 +578,10 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
                     bulk_commit();
                 }
             }
+            if (++m > m_last) {
+                m = m_first;
+                ++h;
+            }
         }
         if (tid == 256) bulk_wait<0>();
     } else {
@@ -397,7 +600,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         const float* sDv = reinterpret_cast<const float*>(sgen + L::OFF_DVEC);
         uint8_t* sDS_row = sgen + L::OFF_DS + half * BOX_BYTES + row * 128;
         float pv[64];
-        int m = m_first;                                   // query block of the tile of the next phase_p
+        int m = m_start;                                   // query block of the tile of the next phase_p
 
         auto phase_p = [&](int j) {        // P^T(j) = exp2(S^T * c - lse), masked
             const int s = j & 1;
@@ -486,18 +689,8 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         tc_fence_after();
         const bool kvalid = kj < T;
         const size_t orow = (size_t)(tok0 + kj) * (size_t)p.dkv_ts + (size_t)g * D + half * HALF_D;
-#pragma unroll
-        for (int which = 0; which < 2; ++which) {
-            const uint32_t src = (which == 0 ? tmem_dK : tmem_dV) + lane_sel + half * HALF_D;
-            void* base = which == 0 ? p.dk : p.dv;
-#pragma unroll
-            for (int ch = 0; ch < HALF_D / 32; ++ch) {
-                uint32_t r[32];
-                tmem_ld32(src + ch * 32, r);
-                tmem_wait_ld();
-                if (kvalid) bwd_store_cols(base, orow + ch * 32, r, p.grad_fp32);
-            }
-        }
+        bwd_epilogue<D>(p, unit.cut, g, 1, 0, tmem_dK + lane_sel + half * HALF_D, tmem_dV + lane_sel + half * HALF_D, row, half, kvalid, orow,
+                        reinterpret_cast<volatile int*>(sgen + L::OFF_MISC + 8));
     }
     tc_fence_before();
     __syncthreads();
@@ -509,23 +702,23 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
 
 template <int D>
 static int launch_dot(const __nv_bfloat16* dout, const __nv_bfloat16* out, float* dvec, float* dq_acc, long long dq_ts, int total_tokens, int Hq,
-                      WsHeader* hdr, cudaStream_t st) {
+                      WsHeader* hdr, const BwdPlanArgs& plan, cudaStream_t st) {
     const long long rows = (long long)total_tokens * Hq;
     const int rows_per_warp = (32 / (D / 8)) * DOT_ROWS;
     const long long warps = (rows + rows_per_warp - 1) / rows_per_warp;
     const int threads = 256;
-    const long long blocks = (warps * 32 + threads - 1) / threads;
+    const long long blocks = (warps * 32 + threads - 1) / threads + 1;
     if (blocks > 0x7fffffffLL) return KVS_ERR_UNSUPPORTED;
-    bwd_dot_kernel<D><<<(unsigned)(blocks > 0 ? blocks : 1), threads, 0, st>>>(dout, out, dvec, dq_acc, dq_ts, total_tokens, Hq, hdr);
+    bwd_dot_kernel<D><<<(unsigned)blocks, threads, 0, st>>>(dout, out, dvec, dq_acc, dq_ts, total_tokens, Hq, hdr, plan);
     return cudaGetLastError() == cudaSuccess ? KVS_OK : KVS_ERR_CUDA;
 }
 
 template <int D>
 static int launch_main(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tdo, const CUtensorMap& tdq,
-                       const MetaView& mv, const BwdParams& p, int nb_cap, cudaStream_t st) {
+                       const MetaView& mv, const BwdParams& p, int unit_cap, cudaStream_t st) {
     auto kern = bwd_kernel<D>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdSmem<D>::DYN_BYTES) != cudaSuccess) return KVS_ERR_CUDA;
-    dim3 grid(nb_cap, p.Hkv, 1);
+    dim3 grid(unit_cap, p.Hkv, 1);
     kern<<<grid, BWD_THREADS, BwdSmem<D>::DYN_BYTES, st>>>(tq, tk, tv, tdo, tdq, mv, p);
     return cudaGetLastError() == cudaSuccess ? KVS_OK : KVS_ERR_CUDA;
 }
@@ -540,14 +733,18 @@ extern "C" size_t kvs_attn_bwd_workspace_bytes(int total_tokens, int Hq, int Hkv
     return bwd_ws_layout(total_tokens, Hq, head_dim, grad_dtype).total;
 }
 
+size_t kvs::bwd_base_bytes(int total_tokens, int Hq, int head_dim, int grad_dtype) {
+    return bwd_ws_layout(total_tokens, Hq, head_dim, grad_dtype).base;
+}
+
 namespace {
-bool use_pairs(int batch, int total_tokens, int max_seqlen, int Hkv, int head_dim) { return false; }
+bool use_pairs(int batch, int total_tokens, int max_seqlen, int Hkv, int head_dim) { return head_dim == 128; }
 
 // in_ts: elements between consecutive tokens of q and of k, v; g_ts: of dq and of dk, dv (0: tensors of their own)
 int bwd_impl(const void* dout, const void* q, const void* k, const void* v, long long in_ts, const void* out, const float* lse,
              const void* meta_buf, int batch, int total_tokens, int max_seqlen, int Hq, int Hkv, int head_dim,
              float softmax_scale, int grad_dtype, void* dq, void* dk, void* dv, long long g_ts, void* workspace,
-             size_t workspace_bytes, kvs_stream_t stream, void* event_main_begin, void* event_main_end) {
+             size_t workspace_bytes, kvs_stream_t stream, void* event_main_begin, void* event_main_end, const BwdWhole* part_of = nullptr) {
     cudaEvent_t ev0 = (cudaEvent_t)event_main_begin, ev1 = (cudaEvent_t)event_main_end;
     if (batch < 0 || total_tokens < 0 || max_seqlen < 0 || Hq <= 0 || Hkv <= 0) return KVS_ERR_INVALID_ARG;
     if (head_dim != 64 && head_dim != 128) return KVS_ERR_UNSUPPORTED;
@@ -560,12 +757,13 @@ int bwd_impl(const void* dout, const void* q, const void* k, const void* v, long
     if (((uintptr_t)lse & 3) != 0 || ((uintptr_t)workspace & 255) != 0 || ((uintptr_t)meta_buf & 255) != 0) return KVS_ERR_ALIGNMENT;
     if (softmax_scale < 0.f || softmax_scale != softmax_scale) return KVS_ERR_INVALID_ARG;
     const BwdWsLayout W = bwd_ws_layout(total_tokens, Hq, head_dim, grad_dtype);
-    if (workspace_bytes < W.total) return KVS_ERR_WORKSPACE;
+    if (workspace_bytes < W.base) return KVS_ERR_WORKSPACE;
     int rc = check_device_sm100();
     if (rc != KVS_OK) return rc;
     const MetaLayout L = meta_layout(batch, total_tokens, max_seqlen);
     const MetaView mv = meta_view(meta_buf, L);
-    const bool pair = use_pairs(batch, total_tokens, max_seqlen, Hkv, head_dim);
+    const BwdWhole whole = part_of ? *part_of : BwdWhole{meta_buf, batch, total_tokens, max_seqlen, Hkv};
+    const bool pair = use_pairs(whole.batch, whole.total_tokens, whole.max_seqlen, whole.Hkv, head_dim);
     const int q_rows = pair ? TILE / 2 : TILE;       // rows of the boxes of q, dout and dq
     CUtensorMap tq, tk, tv, tdo, tdq;
     if ((rc = make_tmap_thd(&tq, q, total_tokens, Hq, head_dim, q_rows, in_ts)) != KVS_OK) return rc;
@@ -596,14 +794,49 @@ int bwd_impl(const void* dout, const void* q, const void* k, const void* v, long
     p.dkv_ts = g_ts > 0 ? g_ts : (long long)Hkv * head_dim;
     p.grad_fp32 = grad_dtype == KVS_GRAD_FP32;
     p.status = &((WsHeader*)ws)->status;
+    // Items and their units.  Without room for the plan (a workspace of the base size, or very many very short traces) the
+    // items stay whole.
+    const int ctas = pair ? 2 : 1;
+    const long long both = ((long long)L.nb_cap + batch) / 2;         // sum of ceil(nb_b / 2) over the traces
+    const int items = pair && both < L.nb_cap ? (int)both : L.nb_cap;
+    const int slots = W.slots / ctas;
+    const bool planned = workspace_bytes >= W.total && items + slots / Hkv <= W.unit_cap;
+    BwdPlanArgs pa;
+    memset(&pa, 0, sizeof(pa));
+    if (planned) {
+        const MetaLayout AL = meta_layout(whole.batch, whole.total_tokens, whole.max_seqlen);
+        pa.all = meta_view(whole.meta_buf, AL);
+        pa.mv = mv;
+        pa.all_batch = whole.batch;
+        pa.all_tokens = whole.total_tokens;
+        pa.all_maxlen = whole.max_seqlen < whole.total_tokens ? whole.max_seqlen : whole.total_tokens;
+        pa.batch = batch;
+        pa.tokens = total_tokens;
+        pa.maxlen = p.max_seqlen;
+        pa.pairs = pair;
+        pa.G = Hq / Hkv;
+        pa.all_Hkv = whole.Hkv;
+        pa.Hkv = Hkv;
+        pa.all_slots = bwd_ws_layout(whole.total_tokens, whole.Hkv * pa.G, head_dim, grad_dtype).slots / ctas;
+        pa.slots = slots;
+        pa.plan = (BwdPlan*)(ws + W.plan);
+        pa.units = (BwdUnit*)(ws + W.units);
+        pa.arrived = (int32_t*)(ws + W.arrived);
+        pa.arrived_n = 2 * W.slots;
+    }
+    p.plan = pa.plan;
+    p.units = pa.units;
+    p.arrived = pa.arrived;
+    p.part = (float4*)(ws + W.part);
+    const int unit_cap = planned ? items + slots / Hkv : items;
     const __nv_bfloat16 *dout16 = (const __nv_bfloat16*)dout, *out16 = (const __nv_bfloat16*)out;
-    rc = head_dim == 64 ? launch_dot<64>(dout16, out16, (float*)(ws + W.dvec), dq_acc, dq_ts, total_tokens, Hq, (WsHeader*)ws, st)
-                        : launch_dot<128>(dout16, out16, (float*)(ws + W.dvec), dq_acc, dq_ts, total_tokens, Hq, (WsHeader*)ws, st);
+    rc = head_dim == 64 ? launch_dot<64>(dout16, out16, (float*)(ws + W.dvec), dq_acc, dq_ts, total_tokens, Hq, (WsHeader*)ws, pa, st)
+                        : launch_dot<128>(dout16, out16, (float*)(ws + W.dvec), dq_acc, dq_ts, total_tokens, Hq, (WsHeader*)ws, pa, st);
     if (rc != KVS_OK) return rc;
     if (ev0 && cudaEventRecord(ev0, st) != cudaSuccess) return KVS_ERR_CUDA;
-    rc = pair             ? launch_bwd_pair(tq, tk, tv, tdo, tdq, mv, p, L.nb_cap, st)
-         : head_dim == 64 ? launch_main<64>(tq, tk, tv, tdo, tdq, mv, p, L.nb_cap, st)
-                          : launch_main<128>(tq, tk, tv, tdo, tdq, mv, p, L.nb_cap, st);
+    rc = pair             ? launch_bwd_pair(tq, tk, tv, tdo, tdq, mv, p, unit_cap, st)
+         : head_dim == 64 ? launch_main<64>(tq, tk, tv, tdo, tdq, mv, p, unit_cap, st)
+                          : launch_main<128>(tq, tk, tv, tdo, tdq, mv, p, unit_cap, st);
     if (rc == KVS_OK && ev1 && cudaEventRecord(ev1, st) != cudaSuccess) return KVS_ERR_CUDA;
     if (rc != KVS_OK) return rc;
     if (grad_dtype == KVS_GRAD_BF16) {
@@ -616,6 +849,13 @@ int bwd_impl(const void* dout, const void* q, const void* k, const void* v, long
     return KVS_OK;
 }
 }  // namespace
+
+int kvs::bwd_of_chunk(const BwdWhole& whole, const void* dout, const void* q, const void* k, const void* v, const void* out, const float* lse,
+                      const void* meta_buf, int batch, int total_tokens, int max_seqlen, int Hq, int Hkv, int head_dim, float softmax_scale,
+                      int grad_dtype, void* dq, void* dk, void* dv, void* workspace, size_t workspace_bytes, kvs_stream_t stream) {
+    return bwd_impl(dout, q, k, v, 0, out, lse, meta_buf, batch, total_tokens, max_seqlen, Hq, Hkv, head_dim, softmax_scale, grad_dtype, dq, dk,
+                    dv, 0, workspace, workspace_bytes, stream, nullptr, nullptr, &whole);
+}
 
 extern "C" int kvs_attn_bwd_ex(const void* dout, const void* q, const void* k, const void* v, const void* out, const float* lse,
                                const void* meta_buf, int batch, int total_tokens, int max_seqlen, int Hq, int Hkv, int head_dim,

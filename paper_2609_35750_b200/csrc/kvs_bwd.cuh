@@ -7,6 +7,23 @@ namespace kvs {
 
 constexpr int BWD_THREADS = 512;
 
+// The work of the main kernel, per KV head: units of consecutive tiles of one item (a key block, or a pair of them).  An item
+// is cut into several units where whole items would leave SMs idle (the prompt of a long trace is seen by every query of it,
+// by all heads of the group: on one rollout of 32768 tokens with G = 7 its key blocks take 1792 tiles each, more than an
+// SM's share of the whole work).  The units of an item write their dK and dV to slots of the workspace, and the last of
+// them to finish adds the slots up in their order, so the sums do not depend on which it was.
+struct BwdUnit {
+    int32_t block;          // (first) key block of the item
+    int32_t tile0, tile1;   // tiles [tile0, tile1) of its (head of the group, query block) list
+    int32_t cut;            // 0: the whole item; else first slot << 18 | index of the unit << 9 | units of the item
+};
+struct BwdPlan {
+    int32_t n_units;
+    int32_t slots;          // slots used per KV head
+    int32_t pad[2];
+};
+constexpr int BWD_MAX_CUT = 511;          // units of an item, and the unit's index, are 9 bits each
+
 struct BwdParams {
     int batch, total_tokens, max_seqlen;   // what the caller says meta_buf was built for
     int Hq, Hkv;
@@ -18,13 +35,36 @@ struct BwdParams {
     long long dkv_ts;       // elements between consecutive tokens of dk and dv
     int grad_fp32;
     int32_t* status;
+    const BwdPlan* plan;    // nullptr: whole items in the metadata's order
+    const BwdUnit* units;
+    int32_t* arrived;       // [Hkv][slots][2] units of an item that have written their slot (entry of the item's first slot)
+    float4* part;           // [Hkv][slots] of 2 x rows of the item x D / 4
 };
 
 // head_dim 128 by CTA pairs (kvs_bwd_pair.cu).  k, v: tensor maps with 128-row boxes; q64, do64, dq64: with 64-row boxes
 int launch_bwd_pair(const CUtensorMap& q64, const CUtensorMap& k, const CUtensorMap& v, const CUtensorMap& do64, const CUtensorMap& dq64,
-                    const MetaView& mv, const BwdParams& p, int nb_cap, cudaStream_t st);
+                    const MetaView& mv, const BwdParams& p, int unit_cap, cudaStream_t st);
+
+// The batch a backward over a part of it is planned for: the chunks of the host path cut their items as one call over the
+// whole batch does, so that both give the same sums.
+struct BwdWhole {
+    const void* meta_buf;
+    int batch, total_tokens, max_seqlen, Hkv;
+};
+int bwd_of_chunk(const BwdWhole& whole, const void* dout, const void* q, const void* k, const void* v, const void* out, const float* lse,
+                 const void* meta_buf, int batch, int total_tokens, int max_seqlen, int Hq, int Hkv, int head_dim, float softmax_scale,
+                 int grad_dtype, void* dq, void* dk, void* dv, void* workspace, size_t workspace_bytes, kvs_stream_t stream);
+// what a backward needs without cutting items (status, row sums, fp32 dQ accumulator)
+size_t bwd_base_bytes(int total_tokens, int Hq, int head_dim, int grad_dtype);
 
 #ifdef __CUDACC__
+// the unit of work of CTA (or pair) x; false: there is none.  `tiles` of a whole item: all of its list
+__device__ __forceinline__ bool bwd_unit_of(const BwdParams& p, const int32_t* order, int n_items, int x, BwdUnit& unit) {
+    if (x >= (p.plan ? p.plan->n_units : n_items)) return false;
+    unit = p.plan ? p.units[x] : BwdUnit{order[x], 0, -1, 0};
+    return true;
+}
+
 // rows of zeros for a key block that no query sees (its gradients are zero)
 template <int D>
 __device__ __forceinline__ void bwd_zero_rows(const BwdParams& p, int tok, int rows, int g) {
@@ -56,6 +96,72 @@ __device__ __forceinline__ void bwd_store_cols(void* base, size_t elem, const ui
         }
     }
 }
+
+// Epilogue of the 256 compute threads: thread (row, half) has the columns [half * D/2, +D/2) of its row of dK and dV in
+// tensor memory.  A whole item goes straight to memory.  A unit of a cut item writes them to its slot; the item's last unit
+// adds the slots up in order.  `ctas`: CTAs per item, `cta`: this one's index.
+template <int D>
+__device__ __forceinline__ void bwd_epilogue(const BwdParams& p, int cut, int g, int ctas, int cta, uint32_t tmem_dk, uint32_t tmem_dv, int row,
+                                             int half, bool valid, size_t orow, volatile int* s_last) {
+    constexpr int CH = D / 64;              // 32-column pieces per thread and tensor
+    if (cut == 0) {
+#pragma unroll
+        for (int i = 0; i < 2 * CH; ++i) {
+            uint32_t r[32];
+            tmem_ld32((i < CH ? tmem_dk : tmem_dv) + (i % CH) * 32, r);
+            tmem_wait_ld();
+            if (valid) bwd_store_cols(i < CH ? p.dk : p.dv, orow + (i % CH) * 32, r, p.grad_fp32);
+        }
+        return;
+    }
+    const int first = cut >> 18, index = (cut >> 9) & BWD_MAX_CUT, count = cut & BWD_MAX_CUT;
+    constexpr size_t SLOT = 2 * TILE * D / 4;               // float4s of one CTA's slot: [piece][half][8][128 rows]
+    const size_t slot0 = (size_t)g * p.plan->slots + first;
+    float4* base = p.part + (slot0 * ctas + cta) * SLOT + (size_t)half * 8 * TILE + row;
+    {
+        float4* dst = base + (size_t)index * ctas * SLOT;
+#pragma unroll
+        for (int i = 0; i < 2 * CH; ++i) {
+            uint32_t r[32];
+            tmem_ld32((i < CH ? tmem_dk : tmem_dv) + (i % CH) * 32, r);
+            tmem_wait_ld();
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                dst[(size_t)(i * 16 + e) * TILE] = make_float4(__uint_as_float(r[e * 4]), __uint_as_float(r[e * 4 + 1]), __uint_as_float(r[e * 4 + 2]),
+                                                               __uint_as_float(r[e * 4 + 3]));
+        }
+    }
+    __threadfence();
+    named_bar_sync(2, 256);
+    if (threadIdx.x == 0) *s_last = atomicAdd(&p.arrived[slot0 * 2 + cta], 1) == count - 1;
+    named_bar_sync(2, 256);
+    if (!*s_last) return;
+    __threadfence();
+#pragma unroll
+    for (int i = 0; i < 2 * CH; ++i) {
+        float4 a[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) a[e] = __ldcg(base + (size_t)(i * 16 + e) * TILE);
+        for (int c = 1; c < count; ++c) {
+            const float4* src = base + (size_t)c * ctas * SLOT;
+            float4 b[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) b[e] = __ldcg(src + (size_t)(i * 16 + e) * TILE);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) a[e] = make_float4(a[e].x + b[e].x, a[e].y + b[e].y, a[e].z + b[e].z, a[e].w + b[e].w);
+        }
+        uint32_t r[32];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            r[e * 4] = __float_as_uint(a[e].x);
+            r[e * 4 + 1] = __float_as_uint(a[e].y);
+            r[e * 4 + 2] = __float_as_uint(a[e].z);
+            r[e * 4 + 3] = __float_as_uint(a[e].w);
+        }
+        if (valid) bwd_store_cols(i < CH ? p.dk : p.dv, orow + (i % CH) * 32, r, p.grad_fp32);
+    }
+}
+
 #endif
 
 }  // namespace kvs

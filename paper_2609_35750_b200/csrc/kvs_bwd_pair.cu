@@ -145,8 +145,9 @@ bwd_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         if (tid == 0 && blockIdx.x == 0 && blockIdx.y == 0) set_status(p.status, KVS_ERR_BAD_META);
         return;
     }
-    if ((int)(blockIdx.x >> 1) >= mv.hdr->npair_total) return;
-    const int gb0 = mv.pair_order[blockIdx.x >> 1];
+    BwdUnit unit;
+    if (!bwd_unit_of(p, mv.pair_order, mv.hdr->npair_total, blockIdx.x >> 1, unit)) return;
+    const int gb0 = unit.block;
     const int g = blockIdx.y;
     const int G = p.Hq / p.Hkv;
     const int b = mv.blk_trace[gb0];
@@ -159,13 +160,15 @@ bwd_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     int m_first, m_last;
     pair_range(mv.col_first, mv.col_last, gb0, n0 + 1 < nb, m_first, m_last);
     const int nm = m_last - m_first + 1;            // query blocks m_first .. m_last can see one of the two key blocks
-    const int n_iter = G * nm;
+    const int n_iter = (unit.tile1 < 0 ? G * nm : unit.tile1) - unit.tile0;     // tiles of this unit of the G * nm (head, query block) tiles of the pair
     int32_t* status = p.status;
     const bool general = mv.hdr->general != 0;
     if (nm <= 0) {
         if (exists) bwd_zero_rows<D>(p, tok0 + n * TILE, min(TILE, T - n * TILE), g);
         return;
     }
+
+    const int h_start = g * G + unit.tile0 / nm, m_start = m_first + unit.tile0 % nm;
 
     const uint32_t sraw = smem_u32(smem_raw);
     const uint32_t sbase = (sraw + 1023u) & ~1023u;
@@ -249,7 +252,7 @@ bwd_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 if (lane == 0)
                     for (int c = 0; c < 2; ++c) tma_load_pair(dst + c * HBOX, map, row0, h, tok0 + m * TILE + c * 64, l_full);
             };
-            int h = g * G, m = m_first;
+            int h = h_start, m = m_start;
             if (expects) mbar_expect_tx(bar_kv, 6 * TB);
             if (lane == 0) {
                 // a key block past the end of the trace is read as zeros (a start past the last token is filled)
@@ -381,7 +384,7 @@ bwd_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             // ================= lse and D of the tile's queries =================
             float* sLse = reinterpret_cast<float*>(sgen + L::OFF_LSE);
             float* sDv = reinterpret_cast<float*>(sgen + L::OFF_DVEC);
-            int h = g * G, m = m_first;
+            int h = h_start, m = m_start;
             for (int j = 0; j < n_iter; ++j) {
                 const int s = j & 1;
                 const size_t rowbase = (size_t)h * p.total_tokens + tok0 + m * TILE;
@@ -417,7 +420,7 @@ bwd_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         const int chalf = quad >> 1;                       // columns 64 chalf .. + 63 of d
         uint8_t* stg_row = sgen + L::OFF_STG + chalf * (64 * 128) + row * 128;
         const uint32_t l_drained = map_to(bar_drained, 0);
-        int h = g * G, m = m_first;
+        int h = h_start, m = m_start;
         for (int j = 0; j < n_iter; ++j) {
             mbar_wait(bar_dq, j & 1, abort_flag, status);
             tc_fence_after();
@@ -474,7 +477,7 @@ bwd_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         const uint32_t peer_ds = map_to(sDS + rank * BOX + quad * 4096, rank ^ 1), peer_dss = map_to(bar_dss, rank ^ 1);
         const uint32_t l_sl = map_to(bar_sl, 0), l_p = map_to(bar_p, 0), l_dst = map_to(bar_dst, 0), l_dss = map_to(bar_dss, 0);
         float pv[64];
-        int m = m_first;                                   // query block of the tile of the next phase_p
+        int m = m_start;                                   // query block of the tile of the next phase_p
 
         auto phase_p = [&](int j) {        // P^T(j) = exp2(S^T * c - lse), masked
             const int s = j & 1;
@@ -588,18 +591,8 @@ bwd_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         tc_fence_after();
         const bool kvalid = kj < T;
         const size_t orow = (size_t)(tok0 + kj) * (size_t)p.dkv_ts + (size_t)g * D + half * 64;
-#pragma unroll
-        for (int which = 0; which < 2; ++which) {
-            const uint32_t src = (which == 0 ? tmem_dK : tmem_dV) + lane_sel + half * 64;
-            void* base = which == 0 ? p.dk : p.dv;
-#pragma unroll
-            for (int ch = 0; ch < 2; ++ch) {
-                uint32_t r[32];
-                tmem_ld32(src + ch * 32, r);
-                tmem_wait_ld();
-                if (kvalid) bwd_store_cols(base, orow + ch * 32, r, p.grad_fp32);
-            }
-        }
+        bwd_epilogue<D>(p, unit.cut, g, 2, (int)rank, tmem_dK + lane_sel + half * 64, tmem_dV + lane_sel + half * 64, row, half, kvalid, orow,
+                        reinterpret_cast<volatile int*>(sgen + L::OFF_MISC + 8));
     }
     tc_fence_before();
     __syncthreads();
@@ -613,12 +606,10 @@ bwd_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
 }  // namespace
 
 int launch_bwd_pair(const CUtensorMap& q64, const CUtensorMap& k, const CUtensorMap& v, const CUtensorMap& do64, const CUtensorMap& dq64,
-                    const MetaView& mv, const BwdParams& p, int nb_cap, cudaStream_t st) {
+                    const MetaView& mv, const BwdParams& p, int unit_cap, cudaStream_t st) {
     if (cudaFuncSetAttribute(bwd_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PairSmem::DYN_BYTES) != cudaSuccess)
         return KVS_ERR_CUDA;
-    // sum of ceil(nb_b / 2) over the traces
-    const long long pairs = ((long long)nb_cap + p.batch) / 2;
-    dim3 grid((unsigned)(2 * (pairs < nb_cap ? pairs : nb_cap)), p.Hkv, 1);
+    dim3 grid((unsigned)(2 * unit_cap), p.Hkv, 1);
     bwd_pair_kernel<<<grid, BWD_THREADS, PairSmem::DYN_BYTES, st>>>(q64, k, v, do64, dq64, mv, p);
     return cudaGetLastError() == cudaSuccess ? KVS_OK : KVS_ERR_CUDA;
 }
