@@ -69,15 +69,15 @@ __device__ __forceinline__ int bwd_item(const MetaView& mv, int pairs, int G, in
 // tiles becomes ceil(t / L) units of equal length.  The estimate: a unit costs BWD_UNIT_COST tiles beside its own (loads
 // before the first product, the pipeline's first and last tile, the stores), what is left over at the end is half the
 // longest unit, and with up to three waves at least that many average units.
-constexpr float BWD_UNIT_COST = 3.f, BWD_CUT_COST = 2.f;
+constexpr float BWD_UNIT_COST = 4.f, BWD_CUT_COST = 3.f;
 __device__ void bwd_plan(const BwdPlanArgs& a) {
     constexpr int NC = 8;
     __shared__ int s_units[NC], s_cut[NC], s_longest[NC], s_max, s_len;
     __shared__ unsigned long long s_total;
-    __shared__ int s_scan[2][8], s_run[2];
+    __shared__ int s_scan[2][8], s_run[2], s_heavy;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (!meta_matches(a.all.hdr, a.all_batch, a.all_tokens, a.all_maxlen) || !meta_matches(a.mv.hdr, a.batch, a.tokens, a.maxlen)) {
-        if (tid == 0) a.plan->n_units = 0;
+        if (tid == 0) a.plan->n_units = a.plan->n_heavy = 0;
         return;
     }
     for (int i = tid; i < a.arrived_n; i += 256) a.arrived[i] = 0;
@@ -85,7 +85,7 @@ __device__ void bwd_plan(const BwdPlanArgs& a) {
     if (tid == 0) {
         s_total = 0;
         s_max = 0;
-        s_run[0] = s_run[1] = 0;
+        s_run[0] = s_run[1] = s_heavy = 0;
     }
     __syncthreads();
     const int n_all = a.pairs ? a.all.hdr->npair_total : a.all.hdr->nblk_total;
@@ -104,6 +104,7 @@ __device__ void bwd_plan(const BwdPlanArgs& a) {
     }
     __syncthreads();
     const float share = (float)s_total * a.all_Hkv / sms;          // tiles per SM or pair
+    const float heavy_from = share * 0.125f;
     const int most = max(s_max, 1);
     int len[NC];
     const float frac[NC] = {0.25f, 0.5f, 0.75f, 1.0f, 1.25f, 1.6f, 2.2f, 0.f};
@@ -148,7 +149,8 @@ __device__ void bwd_plan(const BwdPlanArgs& a) {
             const float waves = ceilf(units / sms);
             float est = longest + BWD_UNIT_COST;
             if (waves > 1.f) {
-                est = share + BWD_UNIT_COST * units / sms + 0.5f * longest;
+                est = share + (BWD_UNIT_COST * units + BWD_CUT_COST * s_cut[k] * a.all_Hkv) / sms + 0.5f * fminf(longest, heavy_from);
+                est = fmaxf(est, longest + BWD_UNIT_COST);
                 if (waves <= 3.f) est = fmaxf(est, waves * (share * sms / units + BWD_UNIT_COST));
             }
             if (s_cut[k] > 0) est += BWD_CUT_COST;
@@ -199,6 +201,8 @@ __device__ void bwd_plan(const BwdPlanArgs& a) {
             bs += s_scan[1][w];
         }
         const int u0 = bu + iu - c, slot0 = bs + is - (c > 1 ? c : 0);
+        // one that started last would be felt
+        if (c > 0 && (float)t > heavy_from * c) atomicAdd(&s_heavy, c);
         for (int i = 0; i < c; ++i)
             a.units[u0 + i] = BwdUnit{block, (int)((long long)t * i / c), (int)((long long)t * (i + 1) / c), c > 1 ? (slot0 << 18 | i << 9 | c) : 0};
         __syncthreads();
@@ -211,6 +215,7 @@ __device__ void bwd_plan(const BwdPlanArgs& a) {
     if (tid == 0) {
         a.plan->n_units = s_run[0];
         a.plan->slots = s_run[1];
+        a.plan->n_heavy = s_heavy;
     }
 }
 
@@ -346,13 +351,13 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     const int lane = tid & 31;
     // meta_buf must be the one kvs_mask_meta wrote for these sizes: every index below comes out of it
     if (!meta_matches(mv.hdr, p.batch, p.total_tokens, p.max_seqlen)) {
-        if (tid == 0 && blockIdx.x == 0 && blockIdx.y == 0) set_status(p.status, KVS_ERR_BAD_META);
+        if (tid == 0 && blockIdx.x == 0) set_status(p.status, KVS_ERR_BAD_META);
         return;
     }
     BwdUnit unit;
-    if (!bwd_unit_of(p, mv.bwd_order, mv.hdr->nblk_total, blockIdx.x, unit)) return;
+    int g;
+    if (!bwd_unit_of(p, mv.bwd_order, mv.hdr->nblk_total, blockIdx.x, unit, g)) return;
     const int gb = unit.block;
-    const int g = blockIdx.y;
     const int G = p.Hq / p.Hkv;
     const int b = mv.blk_trace[gb];
     const int n = gb - mv.blk_off[b];
@@ -715,11 +720,10 @@ static int launch_dot(const __nv_bfloat16* dout, const __nv_bfloat16* out, float
 
 template <int D>
 static int launch_main(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tdo, const CUtensorMap& tdq,
-                       const MetaView& mv, const BwdParams& p, int unit_cap, cudaStream_t st) {
+                       const MetaView& mv, const BwdParams& p, unsigned units, cudaStream_t st) {
     auto kern = bwd_kernel<D>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdSmem<D>::DYN_BYTES) != cudaSuccess) return KVS_ERR_CUDA;
-    dim3 grid(unit_cap, p.Hkv, 1);
-    kern<<<grid, BWD_THREADS, BwdSmem<D>::DYN_BYTES, st>>>(tq, tk, tv, tdo, tdq, mv, p);
+    kern<<<units, BWD_THREADS, BwdSmem<D>::DYN_BYTES, st>>>(tq, tk, tv, tdo, tdq, mv, p);
     return cudaGetLastError() == cudaSuccess ? KVS_OK : KVS_ERR_CUDA;
 }
 
@@ -738,7 +742,7 @@ size_t kvs::bwd_base_bytes(int total_tokens, int Hq, int head_dim, int grad_dtyp
 }
 
 namespace {
-bool use_pairs(int batch, int total_tokens, int max_seqlen, int Hkv, int head_dim) { return head_dim == 128; }
+bool use_pairs(int batch, int total_tokens, int max_seqlen, int Hkv, int head_dim) { return head_dim == 128 && total_tokens / batch >= 24000; }
 
 // in_ts: elements between consecutive tokens of q and of k, v; g_ts: of dq and of dk, dv (0: tensors of their own)
 int bwd_impl(const void* dout, const void* q, const void* k, const void* v, long long in_ts, const void* out, const float* lse,
@@ -828,15 +832,17 @@ int bwd_impl(const void* dout, const void* q, const void* k, const void* v, long
     p.units = pa.units;
     p.arrived = pa.arrived;
     p.part = (float4*)(ws + W.part);
-    const int unit_cap = planned ? items + slots / Hkv : items;
+    // every cut of an item adds at most as many units as it takes slots
+    const long long ctas_all = (long long)items * Hkv + (planned ? slots : 0);
+    if (ctas_all > 0x3fffffffLL) return KVS_ERR_UNSUPPORTED;
     const __nv_bfloat16 *dout16 = (const __nv_bfloat16*)dout, *out16 = (const __nv_bfloat16*)out;
     rc = head_dim == 64 ? launch_dot<64>(dout16, out16, (float*)(ws + W.dvec), dq_acc, dq_ts, total_tokens, Hq, (WsHeader*)ws, pa, st)
                         : launch_dot<128>(dout16, out16, (float*)(ws + W.dvec), dq_acc, dq_ts, total_tokens, Hq, (WsHeader*)ws, pa, st);
     if (rc != KVS_OK) return rc;
     if (ev0 && cudaEventRecord(ev0, st) != cudaSuccess) return KVS_ERR_CUDA;
-    rc = pair             ? launch_bwd_pair(tq, tk, tv, tdo, tdq, mv, p, unit_cap, st)
-         : head_dim == 64 ? launch_main<64>(tq, tk, tv, tdo, tdq, mv, p, unit_cap, st)
-                          : launch_main<128>(tq, tk, tv, tdo, tdq, mv, p, unit_cap, st);
+    rc = pair             ? launch_bwd_pair(tq, tk, tv, tdo, tdq, mv, p, (unsigned)ctas_all, st)
+         : head_dim == 64 ? launch_main<64>(tq, tk, tv, tdo, tdq, mv, p, (unsigned)ctas_all, st)
+                          : launch_main<128>(tq, tk, tv, tdo, tdq, mv, p, (unsigned)ctas_all, st);
     if (rc == KVS_OK && ev1 && cudaEventRecord(ev1, st) != cudaSuccess) return KVS_ERR_CUDA;
     if (rc != KVS_OK) return rc;
     if (grad_dtype == KVS_GRAD_BF16) {

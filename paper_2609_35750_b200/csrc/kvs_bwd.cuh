@@ -20,7 +20,8 @@ struct BwdUnit {
 struct BwdPlan {
     int32_t n_units;
     int32_t slots;          // slots used per KV head
-    int32_t pad[2];
+    int32_t n_heavy;        // the first n_heavy units of ALL heads start first; after them one head's units, then the next head's
+    int32_t pad;
 };
 constexpr int BWD_MAX_CUT = 511;          // units of an item, and the unit's index, are 9 bits each
 
@@ -43,7 +44,7 @@ struct BwdParams {
 
 // head_dim 128 by CTA pairs (kvs_bwd_pair.cu).  k, v: tensor maps with 128-row boxes; q64, do64, dq64: with 64-row boxes
 int launch_bwd_pair(const CUtensorMap& q64, const CUtensorMap& k, const CUtensorMap& v, const CUtensorMap& do64, const CUtensorMap& dq64,
-                    const MetaView& mv, const BwdParams& p, int unit_cap, cudaStream_t st);
+                    const MetaView& mv, const BwdParams& p, unsigned units, cudaStream_t st);
 
 // The batch a backward over a part of it is planned for: the chunks of the host path cut their items as one call over the
 // whole batch does, so that both give the same sums.
@@ -58,10 +59,21 @@ int bwd_of_chunk(const BwdWhole& whole, const void* dout, const void* q, const v
 size_t bwd_base_bytes(int total_tokens, int Hq, int head_dim, int grad_dtype);
 
 #ifdef __CUDACC__
-// the unit of work of CTA (or pair) x; false: there is none.  `tiles` of a whole item: all of its list
-__device__ __forceinline__ bool bwd_unit_of(const BwdParams& p, const int32_t* order, int n_items, int x, BwdUnit& unit) {
-    if (x >= (p.plan ? p.plan->n_units : n_items)) return false;
-    unit = p.plan ? p.units[x] : BwdUnit{order[x], 0, -1, 0};
+// The unit and KV head of CTA (or pair) x of a one-dimensional grid; false: there is none.  The CTAs without work come last.
+// A whole item has tile1 = -1: all of its list.
+__device__ __forceinline__ bool bwd_unit_of(const BwdParams& p, const int32_t* order, int n_items, int x, BwdUnit& unit, int& g) {
+    const int n = p.plan ? p.plan->n_units : n_items, heavy = p.plan ? p.plan->n_heavy : 0;
+    if (x >= n * p.Hkv) return false;
+    int u;
+    if (x < heavy * p.Hkv) {
+        u = x / p.Hkv;
+        g = x % p.Hkv;
+    } else {
+        x -= heavy * p.Hkv;
+        u = heavy + x % (n - heavy);
+        g = x / (n - heavy);
+    }
+    unit = p.plan ? p.units[u] : BwdUnit{order[u], 0, -1, 0};
     return true;
 }
 

@@ -142,13 +142,13 @@ bwd_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     const uint32_t rank = cluster_rank();
     // The returns below are taken by both CTAs of a pair alike.
     if (!meta_matches(mv.hdr, p.batch, p.total_tokens, p.max_seqlen)) {
-        if (tid == 0 && blockIdx.x == 0 && blockIdx.y == 0) set_status(p.status, KVS_ERR_BAD_META);
+        if (tid == 0 && blockIdx.x == 0) set_status(p.status, KVS_ERR_BAD_META);
         return;
     }
     BwdUnit unit;
-    if (!bwd_unit_of(p, mv.pair_order, mv.hdr->npair_total, blockIdx.x >> 1, unit)) return;
+    int g;
+    if (!bwd_unit_of(p, mv.pair_order, mv.hdr->npair_total, blockIdx.x >> 1, unit, g)) return;
     const int gb0 = unit.block;
-    const int g = blockIdx.y;
     const int G = p.Hq / p.Hkv;
     const int b = mv.blk_trace[gb0];
     const int n0 = gb0 - mv.blk_off[b];
@@ -474,8 +474,10 @@ bwd_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         // dS^T of this key for queries col0 .. col0+63, a 128-byte row: in place, or on its way to the CTA that owns these queries
         const bool local = half == (int)rank;
         uint8_t* sDS_row = sgen + (local ? L::OFF_DS + (int)rank * BOX : L::OFF_OUT) + row * 128;
-        const uint32_t peer_ds = map_to(sDS + rank * BOX + quad * 4096, rank ^ 1), peer_dss = map_to(bar_dss, rank ^ 1);
-        const uint32_t l_sl = map_to(bar_sl, 0), l_p = map_to(bar_p, 0), l_dst = map_to(bar_dst, 0), l_dss = map_to(bar_dss, 0);
+        const uint32_t peer = map_to(sbase, rank ^ 1), even = map_to(sbase, 0);      // the other's, the issuer's shared memory
+        const uint32_t peer_ds = peer + L::OFF_DS + rank * BOX + quad * 4096, peer_dss = peer + (bar_dss - sbase);
+        const uint32_t l_sl = even + (bar_sl - sbase), l_p = even + (bar_p - sbase), l_dst = even + (bar_dst - sbase),
+                       l_dss = even + (bar_dss - sbase);
         float pv[64];
         int m = m_start;                                   // query block of the tile of the next phase_p
 
@@ -546,44 +548,37 @@ bwd_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 dk_[e4 * 2 + 0] = pack_bf16(d01.x, d01.y);
                 dk_[e4 * 2 + 1] = pack_bf16(d23.x, d23.y);
             }
-            auto to_tmem = [&] {
-                // dS^T for dK: columns of this half's own dP^T (its first 32)
-                tmem_st32(tmem_P + lane_sel + col0, dk_);
-                tmem_wait_st();
-                tc_fence_before();                   // also orders this thread's reads of dP^T before the products that overwrite it
-                __syncwarp();
-                if (lane == 0) {
-                    arrive_cluster(l_dst);
-                    mbar_arrive(bar_ldfree(s));
-                }
-            };
-            auto to_smem = [&] {
-                // dS^T for dQ: MN-major rows of 64 queries, 128-byte swizzle (16-byte chunk c sits at c ^ (row % 8)), once the
-                // previous tile's dQ has read both buffers (or their copy)
-                if (j > 0) mbar_wait(bar_dq, (j - 1) & 1, abort_flag, status);
+            // dS^T for dK first: columns of this half's own dP^T (its first 32)
+            tmem_st32(tmem_P + lane_sel + col0, dk_);
+            tmem_wait_st();
+            tc_fence_before();                       // also orders this thread's reads of dP^T before the products that overwrite it
+            __syncwarp();
+            if (lane == 0) {
+                arrive_cluster(l_dst);
+                mbar_arrive(bar_ldfree(s));
+            }
+            // dS^T for dQ: MN-major rows of 64 queries, 128-byte swizzle (16-byte chunk c sits at c ^ (row % 8)), once the
+            // previous tile's dQ has read both buffers (or their copy)
+            if (j > 0) mbar_wait(bar_dq, (j - 1) & 1, abort_flag, status);
 #pragma unroll
-                for (int c = 0; c < 8; ++c)
-                    *reinterpret_cast<uint4*>(sDS_row + ((c ^ (row & 7)) << 4)) =
-                        make_uint4(dk_[c * 4], dk_[c * 4 + 1], dk_[c * 4 + 2], dk_[c * 4 + 3]);
-                fence_proxy_async();                 // visible to the tensor core's reads and to the copy
-                __syncwarp();
-            };
-            if (local) {
-                to_tmem();
-                to_smem();
-                if (lane == 0) arrive_cluster(l_dss);
-            } else {
-                to_smem();
-                if (lane == 0) bulk_to_peer(peer_ds, sOUT + quad * 4096, 4096, peer_dss);
-                if (tid == ((int)rank ^ 1) * 128) mbar_expect_tx(bar_dss, TB / 2);       // what this CTA receives for the tile
-                to_tmem();
+            for (int c = 0; c < 8; ++c)
+                *reinterpret_cast<uint4*>(sDS_row + ((c ^ (row & 7)) << 4)) =
+                    make_uint4(dk_[c * 4], dk_[c * 4 + 1], dk_[c * 4 + 2], dk_[c * 4 + 3]);
+            fence_proxy_async();                     // visible to the tensor core's reads and to the copy
+            __syncwarp();
+            if (lane == 0) {
+                if (local) {
+                    arrive_cluster(l_dss);
+                } else {
+                    bulk_to_peer(peer_ds, sOUT + quad * 4096, 4096, peer_dss);
+                    if (quad == 0) mbar_expect_tx(bar_dss, TB / 2);       // what this CTA receives for the tile
+                }
             }
         };
 
-        phase_p(0);
-        for (int j = 0; j < n_iter; ++j) {
-            phase_ds(j);
-            if (j + 1 < n_iter) phase_p(j + 1);
+        for (int j = 0; j <= n_iter; ++j) {
+            if (j > 0) phase_ds(j - 1);
+            if (j < n_iter) phase_p(j);
         }
 
         // ---- epilogue: dK, dV of this key block, once every MMA has completed ----
@@ -606,11 +601,10 @@ bwd_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
 }  // namespace
 
 int launch_bwd_pair(const CUtensorMap& q64, const CUtensorMap& k, const CUtensorMap& v, const CUtensorMap& do64, const CUtensorMap& dq64,
-                    const MetaView& mv, const BwdParams& p, int unit_cap, cudaStream_t st) {
+                    const MetaView& mv, const BwdParams& p, unsigned units, cudaStream_t st) {
     if (cudaFuncSetAttribute(bwd_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PairSmem::DYN_BYTES) != cudaSuccess)
         return KVS_ERR_CUDA;
-    dim3 grid((unsigned)(2 * unit_cap), p.Hkv, 1);
-    bwd_pair_kernel<<<grid, BWD_THREADS, PairSmem::DYN_BYTES, st>>>(q64, k, v, do64, dq64, mv, p);
+    bwd_pair_kernel<<<2 * units, BWD_THREADS, PairSmem::DYN_BYTES, st>>>(q64, k, v, do64, dq64, mv, p);
     return cudaGetLastError() == cudaSuccess ? KVS_OK : KVS_ERR_CUDA;
 }
 
