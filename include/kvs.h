@@ -217,7 +217,9 @@ int kvs_rope_qk(const void* q, const void* k, const int32_t* positions, const in
                 int batch, int total_tokens, int Hq, int Hkv, int head_dim, float theta_base,
                 int elem_dtype, int inverse, void* q_out, void* k_out, kvs_stream_t stream);
 
-/* Bytes needed for the backward workspace (row sums, fp32 dQ accumulator, status). */
+/* Bytes of the backward workspace: row sums, fp32 dQ accumulator, status, and the plan and partial sums with which key blocks
+ * with long walks are shared out among CTAs (37 MiB at most).  A workspace without room for the last part is accepted;
+ * every key block is then one CTA's. */
 size_t kvs_attn_bwd_workspace_bytes(int total_tokens, int Hq, int Hkv, int head_dim, int grad_dtype);
 
 /*

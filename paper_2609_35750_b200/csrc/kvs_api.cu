@@ -211,7 +211,7 @@ void plan_trace_ranges(const int32_t* cu, int batch, int total_tokens, int want,
 }
 
 struct ArenaLayout {
-    size_t evict, cu, sticky, meta, meta_all, cu_all, slot0, slot_stride, total;      // global part, then HOST_SLOTS equal slots
+    size_t evict, cu, sticky, meta, meta_all, cu_all, cut, slot0, slot_stride, total;      // global part, then HOST_SLOTS equal slots
     size_t q, k, v, dout, out, lse, dq, dk, dv, ws;                  // offsets inside a slot
     size_t meta_stride, ws_bytes;
     int slots, ranges, slot_tokens;
@@ -231,7 +231,7 @@ ArenaLayout arena_layout(int batch, int total_tokens, int max_seqlen, int Hq, in
     const size_t nq = (size_t)st * G * head_dim * 2, nkv = (size_t)st * head_dim * 2;
     const size_t gq = (size_t)st * G * head_dim * gsz, gkv = (size_t)st * head_dim * gsz;
     A.meta_stride = align_up(kvs_mask_meta_bytes(batch, A.slot_tokens, max_seqlen), 256);
-    A.ws_bytes = kvs_attn_bwd_workspace_bytes(A.slot_tokens, G, 1, head_dim, grad_dtype);
+    A.ws_bytes = bwd_base_bytes(A.slot_tokens, G, head_dim, grad_dtype);
     size_t o = 0;
     A.evict = o; o = align_up(o + (size_t)total_tokens * 4, 256);
     A.cu = o;    o = align_up(o + (size_t)(batch + A.ranges) * 4, 256);
@@ -241,6 +241,7 @@ ArenaLayout arena_layout(int batch, int total_tokens, int max_seqlen, int Hq, in
     const size_t all = A.ranges > 1 ? align_up(kvs_mask_meta_bytes(batch, total_tokens, max_seqlen), 256) : 0;
     A.meta_all = o; o += all;
     A.cu_all = o;   o = align_up(o + (A.ranges > 1 ? (size_t)(batch + 1) * 4 : 0), 256);
+    A.cut = o;      o += bwd_cut_bytes(total_tokens, Hq, head_dim);     // one for all chunks: their backwards follow one another
     A.slot0 = o;
     size_t t = 0;
     A.q = t;     t = align_up(t + nq, 256);
@@ -355,7 +356,7 @@ extern "C" int kvs_attn_fwd_bwd_host(const int32_t* evict_at_host, const int32_t
                            meta, A.meta_stride, stream);
         if (rc != KVS_OK) return rc;
     }
-    BwdWhole whole = {a + A.meta, batch, total_tokens, max_seqlen, Hkv};
+    BwdWhole whole = {a + A.meta, batch, total_tokens, max_seqlen, Hkv, a + A.cut};
     if (A.ranges > 1) {
         whole.meta_buf = a + A.meta_all;
         KVS_CK(cudaMemcpyAsync(a + A.cu_all, cu_seqlens_host, (size_t)(batch + 1) * 4, cudaMemcpyHostToDevice, st));

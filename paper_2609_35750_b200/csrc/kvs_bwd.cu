@@ -1,10 +1,11 @@
 // Backward: dQ, dK, dV of eviction-masked causal attention.
 //
 //   pre-pass   D_i = dout_i . out_i                         (one warp per (token, head))
-//   main       one CTA per (key block n, KV head g), longest key blocks first; K and V tiles stay in
+//   main       one CTA per unit of (key block n, KV head g), longest first; K and V tiles stay in
 //              shared memory; the CTA loops over the G query heads of the group and over the
-//              contiguous range of query blocks n .. col_last[n] that can see the key block
-//              (see the comment above bwd_kernel for the pipeline)
+//              contiguous range of query blocks n .. col_last[n] that can see the key block, or over
+//              a part of that list (see BwdUnit and bwd_plan; the comment above bwd_kernel for the
+//              pipeline).  Long traces at head_dim 128: CTA pairs, kvs_bwd_pair.cu
 //   post-pass  fp32 dQ accumulator -> bf16 (bf16 gradients only)
 #include "kvs_bwd.cuh"
 #include <cstring>
@@ -17,7 +18,8 @@ constexpr int BWD_MAX_SLOTS = 2 * BWD_SMS;  // slots of one CTA each for the dK 
 
 struct BwdWsLayout {
     size_t dvec, dq_acc, base;              // base: what is needed without cutting items
-    size_t plan, units, arrived, part, total;
+    size_t plan, units, arrived, part;      // offsets from there
+    size_t total;
     int slots, unit_cap;                    // slots of one CTA; entries of the unit list
 };
 
@@ -36,11 +38,12 @@ __host__ __device__ inline BwdWsLayout bwd_ws_layout(int total_tokens, int Hq, i
     L.slots = (int)(most < BWD_MAX_SLOTS ? most : BWD_MAX_SLOTS);
     // key blocks of a batch: short traces have more than total / 128; beyond 4096 more the items are not cut
     L.unit_cap = (int)((total_tokens < nb + 4096 ? total_tokens : nb + 4096) + L.slots);
+    o = 0;
     L.plan = o;    o = align_up(o + sizeof(BwdPlan), 256);
     L.units = o;   o = align_up(o + sizeof(BwdUnit) * (size_t)L.unit_cap, 256);
     L.arrived = o; o = align_up(o + sizeof(int32_t) * 2 * (size_t)L.slots, 256);
     L.part = o;    o = align_up(o + sizeof(float) * 2 * TILE * (size_t)head_dim * L.slots, 256);
-    L.total = o;
+    L.total = L.base + o;
     return L;
 }
 
@@ -67,8 +70,11 @@ __device__ __forceinline__ int bwd_item(const MetaView& mv, int pairs, int G, in
 // One CTA of 256 threads, beside the pre-pass.  Chooses the longest unit L among eight candidates (fractions of an SM's, or
 // pair's, share of all tiles, and "no cut") by an estimate of the makespan in tiles, then lists the units.  An item of t
 // tiles becomes ceil(t / L) units of equal length.  The estimate: a unit costs BWD_UNIT_COST tiles beside its own (loads
-// before the first product, the pipeline's first and last tile, the stores), what is left over at the end is half the
-// longest unit, and with up to three waves at least that many average units.
+// before the first product, the pipeline's first and last tile, the stores), a unit of a cut item BWD_CUT_COST more (slot
+// written and read again); no unit is longer than the makespan; units above an eighth of the share start first, over all
+// heads, so what is left over at the end is half of such an eighth at most; and up to three waves take that many average
+// units.  Main kernel, whole items -> cut, us: 1 trace of 1000 tokens with 16 heads on 2: 154 -> 42; 4000 with 32 on 8:
+// 355 -> 180; 16000, head_dim 64: 1199 -> 748; 32768 with 28 on 4 (pairs): 5500 -> 4400; nothing cut: 1 to 3 % slower.
 constexpr float BWD_UNIT_COST = 4.f, BWD_CUT_COST = 3.f;
 __device__ void bwd_plan(const BwdPlanArgs& a) {
     constexpr int NC = 8;
@@ -740,9 +746,17 @@ extern "C" size_t kvs_attn_bwd_workspace_bytes(int total_tokens, int Hq, int Hkv
 size_t kvs::bwd_base_bytes(int total_tokens, int Hq, int head_dim, int grad_dtype) {
     return bwd_ws_layout(total_tokens, Hq, head_dim, grad_dtype).base;
 }
+size_t kvs::bwd_cut_bytes(int total_tokens, int Hq, int head_dim) {
+    const BwdWsLayout L = bwd_ws_layout(total_tokens, Hq, head_dim, KVS_GRAD_FP32);
+    return L.total - L.base;
+}
 
 namespace {
-bool use_pairs(int batch, int total_tokens, int max_seqlen, int Hkv, int head_dim) { return head_dim == 128 && total_tokens / batch >= 24000; }
+// CTA pairs take head_dim 128 where the traces are long, 24000 tokens and more on average.  There the chip runs at its power
+// limit and the pairs' smaller shared-memory and reduce-add traffic counts (main kernel, single CTAs -> pairs: 2 x 65536 tokens
+// of last-4-turns 44.8 -> 42.3 ms, 24576 token-level 17.7 -> 16.8, 50000 summary 12.4 -> 12.1).  Below, a pair's union of two
+// query ranges and its costlier start weigh more (8 x 6000 tokens 2.0 -> 2.3 ms, 128 x 300 0.36 -> 0.54).
+bool use_pairs(int batch, int total_tokens, int head_dim) { return head_dim == 128 && total_tokens / batch >= 24000; }
 
 // in_ts: elements between consecutive tokens of q and of k, v; g_ts: of dq and of dk, dv (0: tensors of their own)
 int bwd_impl(const void* dout, const void* q, const void* k, const void* v, long long in_ts, const void* out, const float* lse,
@@ -766,8 +780,8 @@ int bwd_impl(const void* dout, const void* q, const void* k, const void* v, long
     if (rc != KVS_OK) return rc;
     const MetaLayout L = meta_layout(batch, total_tokens, max_seqlen);
     const MetaView mv = meta_view(meta_buf, L);
-    const BwdWhole whole = part_of ? *part_of : BwdWhole{meta_buf, batch, total_tokens, max_seqlen, Hkv};
-    const bool pair = use_pairs(whole.batch, whole.total_tokens, whole.max_seqlen, whole.Hkv, head_dim);
+    const BwdWhole whole = part_of ? *part_of : BwdWhole{meta_buf, batch, total_tokens, max_seqlen, Hkv, nullptr};
+    const bool pair = use_pairs(whole.batch, whole.total_tokens, head_dim);
     const int q_rows = pair ? TILE / 2 : TILE;       // rows of the boxes of q, dout and dq
     CUtensorMap tq, tk, tv, tdo, tdq;
     if ((rc = make_tmap_thd(&tq, q, total_tokens, Hq, head_dim, q_rows, in_ts)) != KVS_OK) return rc;
@@ -804,7 +818,8 @@ int bwd_impl(const void* dout, const void* q, const void* k, const void* v, long
     const long long both = ((long long)L.nb_cap + batch) / 2;         // sum of ceil(nb_b / 2) over the traces
     const int items = pair && both < L.nb_cap ? (int)both : L.nb_cap;
     const int slots = W.slots / ctas;
-    const bool planned = workspace_bytes >= W.total && items + slots / Hkv <= W.unit_cap;
+    char* cut = whole.cut_buf ? (char*)whole.cut_buf : ws + W.base;
+    const bool planned = (whole.cut_buf || workspace_bytes >= W.total) && items + slots / Hkv <= W.unit_cap;
     BwdPlanArgs pa;
     memset(&pa, 0, sizeof(pa));
     if (planned) {
@@ -823,15 +838,15 @@ int bwd_impl(const void* dout, const void* q, const void* k, const void* v, long
         pa.Hkv = Hkv;
         pa.all_slots = bwd_ws_layout(whole.total_tokens, whole.Hkv * pa.G, head_dim, grad_dtype).slots / ctas;
         pa.slots = slots;
-        pa.plan = (BwdPlan*)(ws + W.plan);
-        pa.units = (BwdUnit*)(ws + W.units);
-        pa.arrived = (int32_t*)(ws + W.arrived);
+        pa.plan = (BwdPlan*)(cut + W.plan);
+        pa.units = (BwdUnit*)(cut + W.units);
+        pa.arrived = (int32_t*)(cut + W.arrived);
         pa.arrived_n = 2 * W.slots;
     }
     p.plan = pa.plan;
     p.units = pa.units;
     p.arrived = pa.arrived;
-    p.part = (float4*)(ws + W.part);
+    p.part = (float4*)(cut + W.part);
     // every cut of an item adds at most as many units as it takes slots
     const long long ctas_all = (long long)items * Hkv + (planned ? slots : 0);
     if (ctas_all > 0x3fffffffLL) return KVS_ERR_UNSUPPORTED;

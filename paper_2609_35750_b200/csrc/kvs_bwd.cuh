@@ -46,17 +46,20 @@ struct BwdParams {
 int launch_bwd_pair(const CUtensorMap& q64, const CUtensorMap& k, const CUtensorMap& v, const CUtensorMap& do64, const CUtensorMap& dq64,
                     const MetaView& mv, const BwdParams& p, unsigned units, cudaStream_t st);
 
-// The batch a backward over a part of it is planned for: the chunks of the host path cut their items as one call over the
-// whole batch does, so that both give the same sums.
+// The batch a backward over a part of it is planned for (the chunks of the host path cut their items as one call over the
+// whole batch does, so that both give the same sums), and the room for its plan and slots, which chunks that follow one
+// another on a stream share.
 struct BwdWhole {
     const void* meta_buf;
     int batch, total_tokens, max_seqlen, Hkv;
+    void* cut_buf;
 };
 int bwd_of_chunk(const BwdWhole& whole, const void* dout, const void* q, const void* k, const void* v, const void* out, const float* lse,
                  const void* meta_buf, int batch, int total_tokens, int max_seqlen, int Hq, int Hkv, int head_dim, float softmax_scale,
                  int grad_dtype, void* dq, void* dk, void* dv, void* workspace, size_t workspace_bytes, kvs_stream_t stream);
-// what a backward needs without cutting items (status, row sums, fp32 dQ accumulator)
+// workspace bytes of a backward: what it needs without cutting items (status, row sums, fp32 dQ accumulator), and the rest
 size_t bwd_base_bytes(int total_tokens, int Hq, int head_dim, int grad_dtype);
+size_t bwd_cut_bytes(int total_tokens, int Hq, int head_dim);
 
 #ifdef __CUDACC__
 // The unit and KV head of CTA (or pair) x of a one-dimensional grid; false: there is none.  The CTAs without work come last.

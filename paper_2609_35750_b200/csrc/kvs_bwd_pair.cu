@@ -548,37 +548,44 @@ bwd_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 dk_[e4 * 2 + 0] = pack_bf16(d01.x, d01.y);
                 dk_[e4 * 2 + 1] = pack_bf16(d23.x, d23.y);
             }
-            // dS^T for dK first: columns of this half's own dP^T (its first 32)
-            tmem_st32(tmem_P + lane_sel + col0, dk_);
-            tmem_wait_st();
-            tc_fence_before();                       // also orders this thread's reads of dP^T before the products that overwrite it
-            __syncwarp();
-            if (lane == 0) {
-                arrive_cluster(l_dst);
-                mbar_arrive(bar_ldfree(s));
-            }
-            // dS^T for dQ: MN-major rows of 64 queries, 128-byte swizzle (16-byte chunk c sits at c ^ (row % 8)), once the
-            // previous tile's dQ has read both buffers (or their copy)
-            if (j > 0) mbar_wait(bar_dq, (j - 1) & 1, abort_flag, status);
-#pragma unroll
-            for (int c = 0; c < 8; ++c)
-                *reinterpret_cast<uint4*>(sDS_row + ((c ^ (row & 7)) << 4)) =
-                    make_uint4(dk_[c * 4], dk_[c * 4 + 1], dk_[c * 4 + 2], dk_[c * 4 + 3]);
-            fence_proxy_async();                     // visible to the tensor core's reads and to the copy
-            __syncwarp();
-            if (lane == 0) {
-                if (local) {
-                    arrive_cluster(l_dss);
-                } else {
-                    bulk_to_peer(peer_ds, sOUT + quad * 4096, 4096, peer_dss);
-                    if (quad == 0) mbar_expect_tx(bar_dss, TB / 2);       // what this CTA receives for the tile
+            auto to_tmem = [&] {
+                // dS^T for dK: columns of this half's own dP^T (its first 32)
+                tmem_st32(tmem_P + lane_sel + col0, dk_);
+                tmem_wait_st();
+                tc_fence_before();                   // also orders this thread's reads of dP^T before the products that overwrite it
+                __syncwarp();
+                if (lane == 0) {
+                    arrive_cluster(l_dst);
+                    mbar_arrive(bar_ldfree(s));
                 }
+            };
+            auto to_smem = [&] {
+                // dS^T for dQ: MN-major rows of 64 queries, 128-byte swizzle (16-byte chunk c sits at c ^ (row % 8)), once the
+                // previous tile's dQ has read both buffers (or their copy)
+                if (j > 0) mbar_wait(bar_dq, (j - 1) & 1, abort_flag, status);
+#pragma unroll
+                for (int c = 0; c < 8; ++c)
+                    *reinterpret_cast<uint4*>(sDS_row + ((c ^ (row & 7)) << 4)) =
+                        make_uint4(dk_[c * 4], dk_[c * 4 + 1], dk_[c * 4 + 2], dk_[c * 4 + 3]);
+                fence_proxy_async();                 // visible to the tensor core's reads and to the copy
+                __syncwarp();
+            };
+            if (local) {
+                to_tmem();
+                to_smem();
+                if (lane == 0) arrive_cluster(l_dss);
+            } else {                                 // what has the longer way first
+                to_smem();
+                if (lane == 0) bulk_to_peer(peer_ds, sOUT + quad * 4096, 4096, peer_dss);
+                if (tid == ((int)rank ^ 1) * 128) mbar_expect_tx(bar_dss, TB / 2);       // what this CTA receives for the tile
+                to_tmem();
             }
         };
 
-        for (int j = 0; j <= n_iter; ++j) {
-            if (j > 0) phase_ds(j - 1);
-            if (j < n_iter) phase_p(j);
+        phase_p(0);
+        for (int j = 0; j < n_iter; ++j) {
+            phase_ds(j);
+            if (j + 1 < n_iter) phase_p(j + 1);
         }
 
         // ---- epilogue: dK, dV of this key block, once every MMA has completed ----
