@@ -51,6 +51,7 @@ __host__ __device__ inline BwdWsLayout bwd_ws_layout(int total_tokens, int Hq, i
 struct BwdPlanArgs {
     MetaView all, mv;                       // the batch the cut is chosen for; the (part of the) batch whose units are listed
     int all_batch, all_tokens, all_maxlen, batch, tokens, maxlen;
+    int all_cap, cap;                       // key blocks that the two have room for
     int pairs;                              // items are pairs of key blocks
     int G, all_Hkv, Hkv;
     int all_slots, slots;                   // slots there are, of an item's CTAs, over all KV heads
@@ -60,77 +61,60 @@ struct BwdPlanArgs {
     int arrived_n;
 };
 
-__device__ __forceinline__ int bwd_item(const MetaView& mv, int pairs, int G, int x, int& block) {
-    block = pairs ? mv.pair_order[x] : mv.bwd_order[x];
-    int first = mv.col_first[block], last = mv.col_last[block];
-    if (pairs) pair_range(mv.col_first, mv.col_last, block, block + 1 < mv.blk_off[mv.blk_trace[block] + 1], first, last);
-    return G * max(last - first + 1, 0);
-}
-
 // One CTA of 256 threads, beside the pre-pass.  Chooses the longest unit L among eight candidates (fractions of an SM's, or
 // pair's, share of all tiles, and "no cut") by an estimate of the makespan in tiles, then lists the units.  An item of t
 // tiles becomes ceil(t / L) units of equal length.  The estimate: a unit costs BWD_UNIT_COST tiles beside its own (loads
 // before the first product, the pipeline's first and last tile, the stores), a unit of a cut item BWD_CUT_COST more (slot
-// written and read again); no unit is longer than the makespan; units above an eighth of the share start first, over all
-// heads, so what is left over at the end is half of such an eighth at most; and up to three waves take that many average
-// units.  Main kernel, whole items -> cut, us: 1 trace of 1000 tokens with 16 heads on 2: 154 -> 42; 4000 with 32 on 8:
+// written and read again); no unit is longer than the makespan; where the longest is over one and a half times what a head
+// has for an SM, those above that start first, over all heads, so what is left over at the end is half of it at most (always
+// doing so costs L2 hits, 2 x 65536 tokens 41.4 -> 42.6 ms, but not on traces of at most 16 tiles: 96 of 60 to 900 472 -> 454 us); and up to three waves take that many average units.  Main kernel, whole items -> cut, us: 1 trace of 1000 tokens with 16 heads on 2: 154 -> 42; 4000 with 32 on 8:
 // 355 -> 180; 16000, head_dim 64: 1199 -> 748; 32768 with 28 on 4 (pairs): 5500 -> 4400; nothing cut: 1 to 3 % slower.
 constexpr float BWD_UNIT_COST = 4.f, BWD_CUT_COST = 3.f;
 __device__ void bwd_plan(const BwdPlanArgs& a) {
     constexpr int NC = 8;
-    __shared__ int s_units[NC], s_cut[NC], s_longest[NC], s_max, s_len;
-    __shared__ unsigned long long s_total;
+    __shared__ int s_units[NC], s_cut[NC], s_longest[NC], s_len;
+    __shared__ float s_heavy_from;
     __shared__ int s_scan[2][8], s_run[2], s_heavy;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (!meta_matches(a.all.hdr, a.all_batch, a.all_tokens, a.all_maxlen) || !meta_matches(a.mv.hdr, a.batch, a.tokens, a.maxlen)) {
+    const MetaHeader* all = a.all.hdr;
+    const MetaHeader* part = a.mv.hdr;
+    const int32_t* all_len = a.pairs ? a.all.pair_len : a.all.bwd_len;
+    const int32_t* len = a.pairs ? a.mv.pair_len : a.mv.bwd_len;
+    const int32_t* order = a.pairs ? a.mv.pair_order : a.mv.bwd_order;
+    // this thread's first item, read beside the headers (the arrays have room for `cap` entries, with or without a value yet)
+    const int all_len0 = tid < a.all_cap ? all_len[tid] : 0;
+    const int len0 = tid < a.cap ? len[tid] : 0, order0 = tid < a.cap ? order[tid] : 0;
+    if (!meta_matches(all, a.all_batch, a.all_tokens, a.all_maxlen) || !meta_matches(part, a.batch, a.tokens, a.maxlen)) {
         if (tid == 0) a.plan->n_units = a.plan->n_heavy = 0;
         return;
     }
+    const int n_all = a.pairs ? all->npair_total : all->nblk_total, n = a.pairs ? part->npair_total : part->nblk_total;
+    const int most = max(a.G * (a.pairs ? all->pair_most : all->blk_most), 1);
+    const int sms = a.pairs ? BWD_SMS / 2 : BWD_SMS;
+    const float share = (float)(a.pairs ? all->pair_tiles : all->blk_tiles) * a.G * a.all_Hkv / sms;          // tiles per SM or pair
     for (int i = tid; i < a.arrived_n; i += 256) a.arrived[i] = 0;
     if (tid < NC) s_units[tid] = s_cut[tid] = s_longest[tid] = 0;
-    if (tid == 0) {
-        s_total = 0;
-        s_max = 0;
-        s_run[0] = s_run[1] = s_heavy = 0;
-    }
+    if (tid == 0) s_run[0] = s_run[1] = s_heavy = 0;
     __syncthreads();
-    const int n_all = a.pairs ? a.all.hdr->npair_total : a.all.hdr->nblk_total;
-    const int sms = a.pairs ? BWD_SMS / 2 : BWD_SMS;
-    int block;
-    {
-        unsigned long long total = 0;
-        int most = 0;
-        for (int x = tid; x < n_all; x += 256) {
-            const int t = bwd_item(a.all, a.pairs, a.G, x, block);
-            total += t;
-            most = max(most, t);
-        }
-        atomicAdd(&s_total, total);
-        atomicMax(&s_max, most);
-    }
-    __syncthreads();
-    const float share = (float)s_total * a.all_Hkv / sms;          // tiles per SM or pair
-    const float heavy_from = share * 0.125f;
-    const int most = max(s_max, 1);
-    int len[NC];
+    int cand[NC];
     const float frac[NC] = {0.25f, 0.5f, 0.75f, 1.0f, 1.25f, 1.6f, 2.2f, 0.f};
 #pragma unroll
     for (int k = 0; k < NC; ++k) {
         const float l = fmaxf(ceilf(share * frac[k]), (float)max(BWD_MIN_UNIT, (most + BWD_MAX_CUT - 1) / BWD_MAX_CUT));
-        len[k] = (k == NC - 1 || l > (float)most) ? most : (int)l;
+        cand[k] = (k == NC - 1 || l > (float)most) ? most : (int)l;
     }
     {
         int units[NC], cut[NC], longest[NC];
 #pragma unroll
         for (int k = 0; k < NC; ++k) units[k] = cut[k] = longest[k] = 0;
         for (int x = tid; x < n_all; x += 256) {
-            const int t = bwd_item(a.all, a.pairs, a.G, x, block);
+            const int t = a.G * (x < 256 ? all_len0 : all_len[x]);
 #pragma unroll
             for (int k = 0; k < NC; ++k) {
-                const int c = max((t + len[k] - 1) / len[k], 1);
+                const int c = t > cand[k] ? (t + cand[k] - 1) / cand[k] : 1;
                 units[k] += c;
                 if (c > 1) cut[k] += c;
-                longest[k] = max(longest[k], (t + c - 1) / c);
+                longest[k] = max(longest[k], c > 1 ? (t + c - 1) / c : t);
             }
         }
 #pragma unroll
@@ -138,7 +122,7 @@ __device__ void bwd_plan(const BwdPlanArgs& a) {
             units[k] = __reduce_add_sync(0xffffffffu, units[k]);
             cut[k] = __reduce_add_sync(0xffffffffu, cut[k]);
             longest[k] = __reduce_max_sync(0xffffffffu, longest[k]);
-            if (lane == 0) {
+            if (lane == 0 && units[k] > 0) {
                 atomicAdd(&s_units[k], units[k]);
                 atomicAdd(&s_cut[k], cut[k]);
                 atomicMax(&s_longest[k], longest[k]);
@@ -146,47 +130,57 @@ __device__ void bwd_plan(const BwdPlanArgs& a) {
         }
     }
     __syncthreads();
-    if (tid == 0) {
-        float best = 0.f;
-        int at = NC - 1;
-        for (int k = NC - 1; k >= 0; --k) {                        // "no cut" first: it always fits
-            if ((long long)s_cut[k] * a.all_Hkv > a.all_slots) continue;
-            const float units = (float)s_units[k] * a.all_Hkv, longest = (float)s_longest[k];
-            const float waves = ceilf(units / sms);
-            float est = longest + BWD_UNIT_COST;
-            if (waves > 1.f) {
-                est = share + (BWD_UNIT_COST * units + BWD_CUT_COST * s_cut[k] * a.all_Hkv) / sms + 0.5f * fminf(longest, heavy_from);
-                est = fmaxf(est, longest + BWD_UNIT_COST);
-                if (waves <= 3.f) est = fmaxf(est, waves * (share * sms / units + BWD_UNIT_COST));
-            }
-            if (s_cut[k] > 0) est += BWD_CUT_COST;
-            if (k == NC - 1 || est < best) {
-                best = est;
-                at = k;
+    if (warp == 0) {                        // lane k: candidate k
+        const int k = lane & (NC - 1);
+        const float units = (float)s_units[k] * a.all_Hkv, longest = (float)s_longest[k], head = share / a.all_Hkv;
+        const float waves = ceilf(units / sms);
+        float est = longest + BWD_UNIT_COST;
+        if (waves > 1.f) {
+            est = share + (BWD_UNIT_COST * units + BWD_CUT_COST * s_cut[k] * a.all_Hkv) / sms + 0.5f * fminf(longest, head);
+            est = fmaxf(est, longest + BWD_UNIT_COST);
+            if (waves <= 3.f) est = fmaxf(est, waves * (share * sms / units + BWD_UNIT_COST));
+        }
+        if (s_cut[k] > 0) est += BWD_CUT_COST;
+        if (k < NC - 1 && (long long)s_cut[k] * a.all_Hkv > a.all_slots) est = INFINITY;          // "no cut" always fits
+        float best = est;
+        int at = k;
+#pragma unroll
+        for (int o = 1; o < NC; o <<= 1) {
+            const float e = __shfl_xor_sync(0xffffffffu, best, o);
+            const int x = __shfl_xor_sync(0xffffffffu, at, o);
+            if (e < best || (e == best && x > at)) {
+                best = e;
+                at = x;
             }
         }
-        s_len = len[at];
+        if (lane == at) {
+            int l = cand[0];
+#pragma unroll
+            for (int c = 1; c < NC; ++c) l = c == at ? cand[c] : l;
+            s_len = l;
+            s_heavy_from = part->max_seqlen <= 16 * TILE ? 0.125f * share : longest > 1.5f * head ? head : INFINITY;
+        }
     }
     __syncthreads();
     int longest = s_len;
-    const int n = a.pairs ? a.mv.hdr->npair_total : a.mv.hdr->nblk_total;
-    if (a.mv.hdr != a.all.hdr) {            // a part of the batch has no more cut units than the whole, but its slots are counted too
+    const float heavy_from = s_heavy_from;
+    if (part != all) {                      // a part of the batch has no more cut units than the whole, but its slots are counted too
         if (tid == 0) s_cut[0] = 0;
         __syncthreads();
         int cut = 0;
         for (int x = tid; x < n; x += 256) {
-            const int c = (bwd_item(a.mv, a.pairs, a.G, x, block) + longest - 1) / longest;
+            const int c = (a.G * len[x] + longest - 1) / longest;
             if (c > 1) cut += c;
         }
         if (cut) atomicAdd(&s_cut[0], cut);
         __syncthreads();
         if ((long long)s_cut[0] * a.Hkv > a.slots) longest = most;
     }
-    // List the units, the item's order kept: prefix sums of the items' units and of their slots
+    // List the units, the items' order kept: prefix sums of the items' units and of their slots
     for (int x0 = 0; x0 < n; x0 += 256) {
         const int x = x0 + tid;
-        const int t = x < n ? bwd_item(a.mv, a.pairs, a.G, x, block) : 0;
-        int c = x < n ? max((t + longest - 1) / longest, 1) : 0;
+        const int t = x >= n ? 0 : a.G * (x0 ? len[x] : len0), block = x >= n ? 0 : (x0 ? order[x] : order0);
+        const int c = x < n ? max((t + longest - 1) / longest, 1) : 0;
         int iu = c, is = c > 1 ? c : 0;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -207,7 +201,6 @@ __device__ void bwd_plan(const BwdPlanArgs& a) {
             bs += s_scan[1][w];
         }
         const int u0 = bu + iu - c, slot0 = bs + is - (c > 1 ? c : 0);
-        // one that started last would be felt
         if (c > 0 && (float)t > heavy_from * c) atomicAdd(&s_heavy, c);
         for (int i = 0; i < c; ++i)
             a.units[u0 + i] = BwdUnit{block, (int)((long long)t * i / c), (int)((long long)t * (i + 1) / c), c > 1 ? (slot0 << 18 | i << 9 | c) : 0};
@@ -826,6 +819,8 @@ int bwd_impl(const void* dout, const void* q, const void* k, const void* v, long
         const MetaLayout AL = meta_layout(whole.batch, whole.total_tokens, whole.max_seqlen);
         pa.all = meta_view(whole.meta_buf, AL);
         pa.mv = mv;
+        pa.all_cap = AL.nb_cap;
+        pa.cap = L.nb_cap;
         pa.all_batch = whole.batch;
         pa.all_tokens = whole.total_tokens;
         pa.all_maxlen = whole.max_seqlen < whole.total_tokens ? whole.max_seqlen : whole.total_tokens;

@@ -27,12 +27,15 @@ struct MetaHeader {
     uint32_t ncls_total;   // sum over traces of nb^2
     int32_t general;       // 1: every key slot carries its own first visible query (kvs_mask_meta_keys); 0: slot j is key j
     int32_t npair_total;   // sum over traces of ceil(nb_b / 2): pairs of neighbouring key blocks
+    uint32_t rows_done;    // CTAs of the classification that are done
+    int32_t blk_most, pair_most;        // query blocks of the longest key block, of the longest pair
+    uint32_t blk_tiles, pair_tiles;     // their sums over all key blocks, over all pairs
 };
 
 // Byte offsets of the arrays inside meta_buf; a pure function of the three sizes so that
 // every entry point can recompute it.
 struct MetaLayout {
-    size_t blk_off, cls_off, seq_start, blk_trace, kmin, kmax, fmin, fmax, col_first, col_last, row_cnt, fwd_order, bwd_order, pair_order, evict,
+    size_t blk_off, cls_off, seq_start, blk_trace, kmin, kmax, fmin, fmax, col_first, col_last, row_cnt, fwd_order, bwd_order, pair_order, bwd_len, pair_len, evict,
         kfirst, tile_class, row_list, total;
     int nb_cap;            // capacity in blocks
     size_t cls_cap;        // capacity in tiles
@@ -68,6 +71,8 @@ __host__ __device__ inline MetaLayout meta_layout(int batch, int total_tokens, i
     L.fwd_order = o; o = align_up(o + sizeof(int32_t) * nb_cap, 256);
     L.bwd_order = o; o = align_up(o + sizeof(int32_t) * nb_cap, 256);
     L.pair_order = o; o = align_up(o + sizeof(int32_t) * nb_cap, 256);
+    L.bwd_len = o;   o = align_up(o + sizeof(int32_t) * nb_cap, 256);
+    L.pair_len = o;  o = align_up(o + sizeof(int32_t) * nb_cap, 256);
     L.evict = o;     o = align_up(o + sizeof(int32_t) * (size_t)(total_tokens > 0 ? total_tokens : 1), 256);
     L.kfirst = o;    o = align_up(o + sizeof(int32_t) * (size_t)(total_tokens > 0 ? total_tokens : 1), 256);
     L.tile_class = o; o = align_up(o + L.cls_cap, 256);
@@ -93,6 +98,8 @@ struct MetaView {
     const int32_t* fwd_order;   // [nblk] query blocks, heaviest first
     const int32_t* bwd_order;   // [nblk] key blocks, longest query range first
     const int32_t* pair_order;  // [npair] first key block of each pair (2p, 2p+1) of a trace, longest query range first
+    const int32_t* bwd_len;     // [nblk] query blocks that see the key block, in the order of bwd_order
+    const int32_t* pair_len;    // [npair] query blocks that see one of the pair, in the order of pair_order
     const int32_t* evict;       // [total_tokens] eviction step of every key slot (copy of evict_at / key_evict)
     const int32_t* kfirst;      // [total_tokens] first query that may see the slot (general metadata only)
     const uint8_t* tile_class;  // [ncls]
@@ -117,6 +124,8 @@ inline MetaView meta_view(const void* buf, const MetaLayout& L) {
     v.fwd_order = (const int32_t*)(p + L.fwd_order);
     v.bwd_order = (const int32_t*)(p + L.bwd_order);
     v.pair_order = (const int32_t*)(p + L.pair_order);
+    v.bwd_len = (const int32_t*)(p + L.bwd_len);
+    v.pair_len = (const int32_t*)(p + L.pair_len);
     v.evict = (const int32_t*)(p + L.evict);
     v.kfirst = (const int32_t*)(p + L.kfirst);
     v.tile_class = (const uint8_t*)(p + L.tile_class);

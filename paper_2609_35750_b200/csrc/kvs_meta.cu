@@ -1,74 +1,115 @@
-// Mask metadata: per key block min/max of evict_at, per-tile class, per-row lists.
-// Integer work only.  Three small kernels on the caller's stream, no host synchronisation.
+// Mask metadata: per key block min/max of evict_at, per-tile class, per-row lists, launch orders.
+// Integer work only, bound by latency: two kernels on the caller's stream, no host synchronisation.
 #include "kvs_common.cuh"
 
 namespace kvs {
 
-// ---- kernel 0: header, per-trace offsets, block -> trace table -----------------------------
-__global__ void meta_prefix_kernel(const int32_t* __restrict__ cu_seqlens, int batch, int total_tokens, int max_seqlen, int general,
-                                   MetaHeader* hdr, int32_t* blk_off, uint32_t* cls_off, int32_t* seq_start,
-                                   int32_t* blk_trace, int nb_cap, unsigned long long cls_cap) {
-    __shared__ int s_bad;
-    if (threadIdx.x == 0) {
-        int bad = 0;
-        long long nblk = 0;
-        unsigned long long ncls = 0;
-        if (cu_seqlens[0] != 0 || cu_seqlens[batch] != total_tokens) bad = 1;
-        for (int b = 0; b < batch; ++b) {
-            long long a = cu_seqlens[b], e = cu_seqlens[b + 1];
-            long long T = e - a;
-            if (T < 0 || T > max_seqlen || a < 0 || e > total_tokens) { bad = 1; T = 0; }
-            long long nb = (T + TILE - 1) / TILE;
-            blk_off[b] = (int32_t)nblk;
-            cls_off[b] = (uint32_t)ncls;
-            seq_start[b] = (int32_t)a;
-            nblk += nb;
-            ncls += (unsigned long long)(nb * nb);
-            if (nblk > nb_cap || ncls > cls_cap) { bad = 1; nblk = 0; ncls = 0; break; }
-        }
-        if (bad) { nblk = 0; ncls = 0; }
-        blk_off[batch] = (int32_t)nblk;
-        cls_off[batch] = (uint32_t)ncls;
-        seq_start[batch] = total_tokens;
-        hdr->magic = META_MAGIC;
-        hdr->status = bad ? KVS_ERR_BAD_EVICT : KVS_OK;
-        hdr->batch = batch;
-        hdr->total_tokens = total_tokens;
-        hdr->max_seqlen = max_seqlen;
-        hdr->nblk_total = (int32_t)nblk;
-        hdr->ncls_total = (uint32_t)ncls;
-        hdr->general = general;
-        s_bad = bad;
-    }
-    __syncthreads();
-    if (s_bad) return;
-    for (int b = 0; b < batch; ++b) {
-        int lo = blk_off[b], hi = blk_off[b + 1];
-        for (int i = lo + threadIdx.x; i < hi; i += blockDim.x) blk_trace[i] = b;
-    }
-}
+constexpr int META_THREADS = 256;
+constexpr int META_WARPS = META_THREADS / 32;
 
-// ---- kernel 1: one warp per key block: min / max over its key slots, validity ---------------
+// ---- kernel 1: offsets, and per key block (one warp each) min / max over its key slots, validity ---------------
+// Every CTA goes through the traces itself, 256 at a time (a scan of their block counts), and keeps what its eight blocks
+// need; the first CTA writes the tables.  A kernel of its own for the offsets, with one thread walking the traces, took 24 us
+// for 96 of them, and another launch.
+//
 // Slot j of a trace holds a key that query i may read iff first[j] <= i < evict[j].  Plain metadata
 // (key_first == nullptr): first[j] = j and evict[j] > j is required.  General metadata: both arrays come
 // from the caller (keys re-ordered, or another visibility rule) and a slot may be visible to nobody.
 // complement != 0: the slots of the EVICTED keys: slot j becomes visible at evict_at[j] and stays (first = evict_at,
 // evict = never), i.e. the causal key set minus what the eviction mask still shows.
-__global__ void meta_minmax_kernel(const int32_t* __restrict__ evict_at, const int32_t* __restrict__ key_first, int complement,
-                                   MetaHeader* hdr,
-                                   const int32_t* __restrict__ blk_off, const int32_t* __restrict__ seq_start,
-                                   const int32_t* __restrict__ blk_trace, int32_t* kmin, int32_t* kmax, int32_t* fmin, int32_t* fmax,
-                                   int32_t* col_first, int32_t* col_last, int32_t* evict_copy, int32_t* first_copy) {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (warp >= hdr->nblk_total) return;
-    const int b = blk_trace[warp];
-    const int n = warp - blk_off[b];
-    const int tok0 = seq_start[b];
-    const int T = seq_start[b + 1] - tok0;
+__global__ void __launch_bounds__(META_THREADS)
+meta_blocks_kernel(const int32_t* __restrict__ evict_at, const int32_t* __restrict__ key_first, int complement,
+                   const int32_t* __restrict__ cu_seqlens, int batch, int total_tokens, int max_seqlen, MetaHeader* hdr, int32_t* blk_off,
+                   uint32_t* cls_off, int32_t* seq_start, int32_t* blk_trace, int nb_cap, unsigned long long cls_cap, int32_t* kmin,
+                   int32_t* kmax, int32_t* fmin, int32_t* fmax, int32_t* col_first, int32_t* col_last, int32_t* row_cnt,
+                   int32_t* evict_copy, int32_t* first_copy) {
+    __shared__ unsigned long long s_cls[META_WARPS];
+    __shared__ long long s_blk[META_WARPS];
+    __shared__ int4 s_mine[META_WARPS];              // trace, its first block, its first token, its length
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const long long blk0 = (long long)blockIdx.x * META_WARPS;
+    const bool writer = blockIdx.x == 0;
+    if (tid < META_WARPS) s_mine[tid].x = -1;
+    bool bad = cu_seqlens[0] != 0 || cu_seqlens[batch] != total_tokens;
+    long long nblk = 0;
+    unsigned long long ncls = 0;
+    for (int b0 = 0; b0 < batch; b0 += META_THREADS) {
+        const int b = b0 + tid;
+        long long a = 0, T = 0;
+        if (b < batch) {
+            a = cu_seqlens[b];
+            T = cu_seqlens[b + 1] - a;
+            if (T < 0 || T > max_seqlen || a < 0 || a + T > total_tokens) {
+                bad = true;
+                T = 0;
+            }
+        }
+        const long long nb = (T + TILE - 1) / TILE;
+        long long ib = nb;
+        unsigned long long ic = (unsigned long long)(nb * nb);
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const long long tb = __shfl_up_sync(0xffffffffu, ib, o);
+            const unsigned long long tc = __shfl_up_sync(0xffffffffu, ic, o);
+            if (lane >= o) {
+                ib += tb;
+                ic += tc;
+            }
+        }
+        __syncthreads();                                  // the previous round's totals have been read
+        if (lane == 31) {
+            s_blk[warp] = ib;
+            s_cls[warp] = ic;
+        }
+        __syncthreads();
+        long long first = nblk + ib - nb;
+        unsigned long long first_cls = ncls + ic - (unsigned long long)(nb * nb);
+#pragma unroll
+        for (int w = 0; w < META_WARPS; ++w) {
+            if (w < warp) {
+                first += s_blk[w];
+                first_cls += s_cls[w];
+            }
+            nblk += s_blk[w];
+            ncls += s_cls[w];
+        }
+        if (b < batch) {
+            const long long lo = max(first, blk0), hi = min(first + nb, blk0 + META_WARPS);
+            for (long long i = lo; i < hi; ++i) s_mine[i - blk0] = make_int4(b, (int)first, (int)a, (int)T);
+            if (writer) {
+                blk_off[b] = (int32_t)first;
+                cls_off[b] = (uint32_t)first_cls;
+                seq_start[b] = (int32_t)a;
+            }
+        }
+    }
+    if (__syncthreads_or(bad) || nblk > nb_cap || ncls > cls_cap) {
+        bad = true;
+        nblk = 0;
+        ncls = 0;
+    }
+    if (writer && tid == 0) {
+        blk_off[batch] = (int32_t)nblk;
+        cls_off[batch] = (uint32_t)ncls;
+        seq_start[batch] = total_tokens;
+        hdr->magic = META_MAGIC;
+        hdr->status = bad ? KVS_ERR_BAD_EVICT : KVS_OK;         // invalid keys are reported by the next kernel
+        hdr->batch = batch;
+        hdr->total_tokens = total_tokens;
+        hdr->max_seqlen = max_seqlen;
+        hdr->nblk_total = (int32_t)nblk;
+        hdr->ncls_total = (uint32_t)ncls;
+        hdr->general = (key_first || complement) ? 1 : 0;
+        hdr->npair_total = 0;
+        hdr->rows_done = 0;
+    }
+    const int4 mine = s_mine[warp];
+    if (blk0 + warp >= nblk || mine.x < 0) return;
+    const int blk = (int)blk0 + warp;
+    const int n = blk - mine.y, tok0 = mine.z, T = mine.w;
     const int nb = (T + TILE - 1) / TILE;
     int mn = INT32_MAX, mx = INT32_MIN, fmn = INT32_MAX, fmx = INT32_MIN;
-    bool bad = false;
+    bool invalid = false;
 #pragma unroll
     for (int t = 0; t < TILE / 32; ++t) {
         const int j = n * TILE + t * 32 + lane;
@@ -78,7 +119,7 @@ __global__ void meta_minmax_kernel(const int32_t* __restrict__ evict_at, const i
             const bool general = complement || key_first;
             evict_copy[tok0 + j] = e;
             if (general) first_copy[tok0 + j] = f;
-            bad |= general ? (f < 0) : (e <= j);
+            invalid |= general ? (f < 0) : (e <= j);
             mn = min(mn, e);
             mx = max(mx, e);
             fmn = min(fmn, f);
@@ -89,152 +130,180 @@ __global__ void meta_minmax_kernel(const int32_t* __restrict__ evict_at, const i
     mx = __reduce_max_sync(0xffffffffu, mx);
     fmn = __reduce_min_sync(0xffffffffu, fmn);
     fmx = __reduce_max_sync(0xffffffffu, fmx);
-    const unsigned any_bad = __ballot_sync(0xffffffffu, bad);
+    const unsigned any_invalid = __ballot_sync(0xffffffffu, invalid);
     if (lane == 0) {
-        kmin[warp] = mn;
-        kmax[warp] = mx;
-        fmin[warp] = fmn;
-        fmax[warp] = fmx;
+        blk_trace[blk] = mine.x;
+        kmin[blk] = mn;
+        kmax[blk] = mx;
+        fmin[blk] = fmn;
+        fmax[blk] = fmx;
         // last query block whose first row q0 = 128 m is still below kmax; first one whose last row reaches fmin
         long long last = ((long long)mx - 1) / TILE;
         if (last > nb - 1) last = nb - 1;
         long long first = fmn / TILE;
         if (first > nb) first = nb;
-        if (first < 0) first = 0;                  // a negative key_first is reported below; never an index
+        if (first < 0) first = 0;                  // a negative key_first is reported; never an index
         if (!key_first && !complement && last < n) last = n;
-        col_first[warp] = (int32_t)first;
-        col_last[warp] = (mx <= 0) ? -1 : (int32_t)last;
-        if (any_bad) set_status(&hdr->status, KVS_ERR_BAD_EVICT);
+        col_first[blk] = (int32_t)first;
+        col_last[blk] = (mx <= 0) ? -1 : (int32_t)last;
+        row_cnt[blk] = any_invalid ? -1 : 0;       // for the next kernel, which puts the count here
     }
 }
 
-// ---- kernel 2: one warp per query block row: classes and the compact non-empty list --------
-__global__ void meta_classify_kernel(MetaHeader* hdr, const int32_t* __restrict__ blk_off, const uint32_t* __restrict__ cls_off,
-                                     const int32_t* __restrict__ seq_start, const int32_t* __restrict__ blk_trace,
-                                     const int32_t* __restrict__ kmin, const int32_t* __restrict__ kmax,
-                                     const int32_t* __restrict__ fmin, const int32_t* __restrict__ fmax,
-                                     uint8_t* tile_class, uint16_t* row_list, int32_t* row_cnt) {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (warp >= hdr->nblk_total) return;
-    const int b = blk_trace[warp];
-    const int base = blk_off[b];
-    const int m = warp - base;
-    const int T = seq_start[b + 1] - seq_start[b];
-    const int nb = (T + TILE - 1) / TILE;
-    const int q0 = m * TILE;
-    const int q1 = min(q0 + TILE - 1, T - 1);
-    uint8_t* cls_row = tile_class + cls_off[b] + (size_t)m * nb;
-    uint16_t* list_row = row_list + cls_off[b] + (size_t)m * nb;
-    int count = 0;
-    for (int n0 = 0; n0 < nb; n0 += 32) {
-        const int n = n0 + lane;
-        int c = KVS_CLASS_EMPTY;
-        if (n < nb) {
-            // f0, f1: the earliest / latest "first query that may see the slot" of the block; for plain
-            // metadata these are the block's first and last valid key, k0 and k1
-            const int f0 = fmin[base + n], f1 = fmax[base + n];
-            const int mn = kmin[base + n], mx = kmax[base + n];
-            if (f0 > q1 || q0 >= mx) c = KVS_CLASS_EMPTY;
-            else if (f1 <= q0 && q1 < mn) c = KVS_CLASS_FULL;
-            else c = KVS_CLASS_PARTIAL;
-            cls_row[n] = (uint8_t)c;
-        }
-        const unsigned live = __ballot_sync(0xffffffffu, c != KVS_CLASS_EMPTY);
-        if (c != KVS_CLASS_EMPTY) list_row[count + __popc(live & ((1u << lane) - 1u))] = (uint16_t)n;
-        count += __popc(live);
-    }
-    if (lane == 0) row_cnt[warp] = count;
-}
-
-// ---- kernel 3: work orders, heaviest first (bucket sort, one CTA per order) -------------------
-// blockIdx.x = 0: query blocks by their number of non-empty key blocks (forward);
-// blockIdx.x = 1: key blocks by the length of their query-block range (backward);
-// blockIdx.x = 2: pairs (2p, 2p+1) of a trace's key blocks by the length of their joint range (backward by CTA pairs).
-// Only the launch order of work depends on it; ties keep their order in the batch.
+// ---- launch orders, heaviest first -----------------------------------------------------------------------------
+// One CTA sorts n items into buckets by length, longest bucket first; items of a bucket keep their order in the batch, so
+// CTAs launched together work on neighbouring blocks and share tiles in L2.
+//   ORDER_ROWS   query blocks by their number of non-empty key blocks (forward)
+//   ORDER_COLS   key blocks by the length of their query-block range (backward)
+//   ORDER_PAIRS  pairs (2p, 2p+1) of a trace's key blocks by the length of their joint range (backward by CTA pairs)
+// Coarse buckets (16 tiles): exact lengths would interleave blocks from all over the batch, coarse ones keep runs of
+// neighbouring blocks together while still starting the long ones first.  Where no trace has more than 16 tiles they
+// would all fall into one bucket and the longest might start last: there the lengths are exact (96 traces of 60 to
+// 900 tokens: step 955 -> 894 us; 12 traces of 1500 to 12000 tokens with exact short lengths: 8274 -> 8678 us).
+enum { ORDER_ROWS, ORDER_COLS, ORDER_PAIRS };
 constexpr int ORDER_BINS = 4096;
-__global__ void __launch_bounds__(1024)
-meta_order_kernel(MetaHeader* hdr, const int32_t* __restrict__ blk_off, const int32_t* __restrict__ blk_trace,
-                  const int32_t* __restrict__ row_cnt, const int32_t* __restrict__ col_first, const int32_t* __restrict__ col_last,
-                  int32_t* fwd_order, int32_t* bwd_order, int32_t* pair_order) {
+constexpr int ORDER_CACHED = 12288;        // lengths kept in shared memory between the passes (16 bits each)
+
+__device__ void meta_order(int what, MetaHeader* hdr, const int32_t* blk_off, const int32_t* blk_trace, const int32_t* row_cnt,
+                           const int32_t* col_first, const int32_t* col_last, int32_t* order, int32_t* len_out) {
     __shared__ int bins[ORDER_BINS];
-    __shared__ int warp_tot[32];
+    __shared__ uint16_t cached[ORDER_CACHED];
+    __shared__ unsigned int s_sum;
+    __shared__ int s_most;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n = hdr->nblk_total;
-    const bool bwd = blockIdx.x == 1, pairs = blockIdx.x == 2;
     const bool exact = hdr->max_seqlen <= 16 * TILE;
-    int32_t* order = pairs ? pair_order : bwd ? bwd_order : fwd_order;
-    auto key = [&](int i) {
-        // Coarse buckets (16 tiles): exact lengths would interleave blocks from all over the batch, coarse ones keep runs of
-        // neighbouring blocks together while still starting the long ones first.  Where no trace has more than 16 tiles they
-        // would all fall into one bucket and the longest might start last: there the lengths are exact (96 traces of 60 to
-        // 900 tokens: step 955 -> 894 us; 12 traces of 1500 to 12000 tokens with exact short lengths: 8274 -> 8678 us).
-        int k;
-        if (pairs) {
-            const int b = blk_trace[i];
-            if ((i - blk_off[b]) & 1) return -1;       // the second block of a pair is not an item of its own
-            int first, last;
-            pair_range(col_first, col_last, i, i + 1 < blk_off[b + 1], first, last);
-            k = last - first + 1;
-        } else {
-            k = bwd ? (col_last[i] - col_first[i] + 1) : row_cnt[i];
-        }
-        k = max(k, 0);
-        return min(exact ? k : k >> 4, ORDER_BINS - 1);
+    const int nbins = exact ? 17 : min((hdr->max_seqlen / TILE >> 4) + 2, ORDER_BINS);
+    auto length = [&](int i) {              // 0xffff: not an item of its own
+        if (what == ORDER_ROWS) return __ldcg(row_cnt + i);
+        if (what == ORDER_COLS) return max(col_last[i] - col_first[i] + 1, 0);
+        const int b = blk_trace[i], lo = blk_off[b], hi = blk_off[b + 1];
+        int first, last;
+        pair_range(col_first, col_last, i, i + 1 < hi, first, last);
+        return ((i - lo) & 1) ? 0xffff : max(last - first + 1, 0);
     };
-    for (int i = threadIdx.x; i < ORDER_BINS; i += blockDim.x) bins[i] = 0;
-    __syncthreads();
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        const int k = key(i);
-        if (k >= 0) atomicAdd(&bins[k], 1);
+    auto bin = [&](int len) { return nbins - 1 - min(exact ? len : len >> 4, nbins - 1); };      // the longest first
+    for (int i = tid; i < nbins; i += META_THREADS) bins[i] = 0;
+    if (tid == 0) {
+        s_sum = 0;
+        s_most = 0;
     }
     __syncthreads();
-    // exclusive scan over the bins in DESCENDING key order: thread t owns 4 consecutive reversed bins
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int c[4], sum = 0;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        c[u] = bins[ORDER_BINS - 1 - (threadIdx.x * 4 + u)];
-        sum += c[u];
+    unsigned int sum = 0;
+    int most = 0;
+    for (int i = tid; i < n; i += META_THREADS) {
+        const int len = length(i);
+        if (i < ORDER_CACHED) cached[i] = (uint16_t)len;
+        if (len == 0xffff) continue;
+        atomicAdd(&bins[bin(len)], 1);
+        sum += len;
+        most = max(most, len);
     }
-    int incl = sum;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
+    sum = __reduce_add_sync(0xffffffffu, sum);
+    most = __reduce_max_sync(0xffffffffu, most);
+    if (lane == 0) {
+        atomicAdd(&s_sum, sum);
+        atomicMax(&s_most, most);
     }
-    if (lane == 31) warp_tot[warp] = incl;
     __syncthreads();
-    if (warp == 0) {
-        int w = warp_tot[lane], wi = w;
+    if (warp != 0) return;
+    // exclusive scan over the bins, then the stable scatter, 32 blocks at a time in index order
+    int run = 0;
+    for (int i0 = 0; i0 < nbins; i0 += 32) {
+        const int c = i0 + lane < nbins ? bins[i0 + lane] : 0;
+        int incl = c;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(0xffffffffu, wi, o);
-            if (lane >= o) wi += t;
+            const int t = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += t;
         }
-        warp_tot[lane] = wi - w;     // exclusive prefix of the warp totals
+        if (i0 + lane < nbins) bins[i0 + lane] = run + incl - c;
+        run += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    __syncwarp();
+    for (int i0 = 0; i0 < n; i0 += 32) {
+        const int i = i0 + lane;
+        const int len = i < n ? (i < ORDER_CACHED ? (int)cached[i] : length(i)) : 0xffff;
+        const int k = len == 0xffff ? -1 : bin(len);
+        const unsigned same = __match_any_sync(0xffffffffu, k);
+        if (k >= 0) {
+            const int at = bins[k] + __popc(same & ((1u << lane) - 1u));
+            order[at] = i;
+            if (len_out) len_out[at] = len;
+        }
+        __syncwarp();
+        if (k >= 0 && lane == (__ffs(same) - 1)) bins[k] += __popc(same);
+        __syncwarp();
+    }
+    if (lane == 0 && what == ORDER_COLS) {
+        hdr->blk_most = s_most;
+        hdr->blk_tiles = s_sum;
+    }
+    if (lane == 0 && what == ORDER_PAIRS) {
+        hdr->npair_total = run;
+        hdr->pair_most = s_most;
+        hdr->pair_tiles = s_sum;
+    }
+}
+
+// ---- kernel 2: one warp per query block row: classes and the compact non-empty list; the orders ----------------------
+// The first two CTAs sort the key blocks and the pairs, the others classify, and the last of those to finish sorts the rows.
+__global__ void __launch_bounds__(META_THREADS)
+meta_classify_kernel(MetaHeader* hdr, const int32_t* __restrict__ blk_off, const uint32_t* __restrict__ cls_off,
+                     const int32_t* __restrict__ seq_start, const int32_t* __restrict__ blk_trace,
+                     const int32_t* __restrict__ kmin, const int32_t* __restrict__ kmax,
+                     const int32_t* __restrict__ fmin, const int32_t* __restrict__ fmax, const int32_t* __restrict__ col_first,
+                     const int32_t* __restrict__ col_last, uint8_t* tile_class, uint16_t* row_list, int32_t* row_cnt, int32_t* fwd_order,
+                     int32_t* bwd_order, int32_t* pair_order, int32_t* bwd_len, int32_t* pair_len) {
+    if (blockIdx.x < 2) {
+        const bool pairs = blockIdx.x == 1;
+        meta_order(pairs ? ORDER_PAIRS : ORDER_COLS, hdr, blk_off, blk_trace, row_cnt, col_first, col_last, pairs ? pair_order : bwd_order,
+                   pairs ? pair_len : bwd_len);
+        return;
+    }
+    __shared__ int s_last;
+    const int row = (blockIdx.x - 2) * META_WARPS + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31;
+    if (row < hdr->nblk_total) {
+        const int b = blk_trace[row];
+        const int base = blk_off[b];
+        const int m = row - base;
+        const int T = seq_start[b + 1] - seq_start[b];
+        const int nb = (T + TILE - 1) / TILE;
+        const int q0 = m * TILE;
+        const int q1 = min(q0 + TILE - 1, T - 1);
+        uint8_t* cls_row = tile_class + cls_off[b] + (size_t)m * nb;
+        uint16_t* list_row = row_list + cls_off[b] + (size_t)m * nb;
+        int count = 0;
+        for (int n0 = 0; n0 < nb; n0 += 32) {
+            const int n = n0 + lane;
+            int c = KVS_CLASS_EMPTY;
+            if (n < nb) {
+                // f0, f1: the earliest / latest "first query that may see the slot" of the block; for plain
+                // metadata these are the block's first and last valid key, k0 and k1
+                const int f0 = fmin[base + n], f1 = fmax[base + n];
+                const int mn = kmin[base + n], mx = kmax[base + n];
+                if (f0 > q1 || q0 >= mx) c = KVS_CLASS_EMPTY;
+                else if (f1 <= q0 && q1 < mn) c = KVS_CLASS_FULL;
+                else c = KVS_CLASS_PARTIAL;
+                cls_row[n] = (uint8_t)c;
+            }
+            const unsigned live = __ballot_sync(0xffffffffu, c != KVS_CLASS_EMPTY);
+            if (c != KVS_CLASS_EMPTY) list_row[count + __popc(live & ((1u << lane) - 1u))] = (uint16_t)n;
+            count += __popc(live);
+        }
+        if (lane == 0) {
+            if (row_cnt[row] < 0) set_status(&hdr->status, KVS_ERR_BAD_EVICT);       // the block's keys, seen by kernel 1
+            row_cnt[row] = count;
+            __threadfence();
+        }
     }
     __syncthreads();
-    int run = warp_tot[warp] + incl - sum;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        bins[ORDER_BINS - 1 - (threadIdx.x * 4 + u)] = run;
-        run += c[u];
-    }
-    if (pairs && threadIdx.x == blockDim.x - 1) hdr->npair_total = run;
+    if (threadIdx.x == 0) s_last = atomicAdd(&hdr->rows_done, 1u) == gridDim.x - 3;
     __syncthreads();
-    // Stable scatter by one warp, 32 blocks at a time in index order: blocks with equal keys keep their
-    // order in the trace, so CTAs launched together work on neighbouring blocks and share tiles in L2.
-    if (warp == 0) {
-        for (int i0 = 0; i0 < n; i0 += 32) {
-            const int i = i0 + lane;
-            const int k = (i < n) ? key(i) : -1;
-            const unsigned same = __match_any_sync(0xffffffffu, k);
-            if (k >= 0) order[bins[k] + __popc(same & ((1u << lane) - 1u))] = i;
-            __syncwarp();
-            if (k >= 0 && lane == (__ffs(same) - 1)) bins[k] += __popc(same);
-            __syncwarp();
-        }
-    }
+    if (!s_last) return;
+    __threadfence();
+    meta_order(ORDER_ROWS, hdr, blk_off, blk_trace, row_cnt, col_first, col_last, fwd_order, nullptr);
 }
 
 // ---- compaction event log -> evict_at ---------------------------------------------------------
@@ -290,20 +359,16 @@ int launch_mask_meta(const int32_t* key_evict, const int32_t* key_first, int com
     if (meta_bytes < L.total) return KVS_ERR_WORKSPACE;
     cudaStream_t st = (cudaStream_t)stream;
     MetaView v = meta_view(meta_buf, L);
-    meta_prefix_kernel<<<1, 256, 0, st>>>(cu_seqlens, batch, total_tokens, max_seqlen, (key_first || complement) ? 1 : 0, v.hdr, (int32_t*)v.blk_off,
-                                          (uint32_t*)v.cls_off, (int32_t*)v.seq_start, (int32_t*)v.blk_trace, L.nb_cap,
-                                          (unsigned long long)L.cls_cap);
-    const int warps_per_cta = 8;
-    const int grid = (L.nb_cap + warps_per_cta - 1) / warps_per_cta;
-    meta_minmax_kernel<<<grid, warps_per_cta * 32, 0, st>>>(key_evict, key_first, complement, v.hdr, v.blk_off, v.seq_start, v.blk_trace,
-                                                            (int32_t*)v.kmin, (int32_t*)v.kmax, (int32_t*)v.fmin, (int32_t*)v.fmax,
-                                                            (int32_t*)v.col_first, (int32_t*)v.col_last, (int32_t*)v.evict,
-                                                            (int32_t*)v.kfirst);
-    meta_classify_kernel<<<grid, warps_per_cta * 32, 0, st>>>(v.hdr, v.blk_off, v.cls_off, v.seq_start, v.blk_trace, v.kmin, v.kmax,
-                                                              v.fmin, v.fmax, (uint8_t*)v.tile_class, (uint16_t*)v.row_list,
-                                                              (int32_t*)v.row_cnt);
-    meta_order_kernel<<<3, 1024, 0, st>>>(v.hdr, v.blk_off, v.blk_trace, v.row_cnt, v.col_first, v.col_last, (int32_t*)v.fwd_order,
-                                         (int32_t*)v.bwd_order, (int32_t*)v.pair_order);
+    const int grid = (L.nb_cap + META_WARPS - 1) / META_WARPS;
+    meta_blocks_kernel<<<grid, META_THREADS, 0, st>>>(key_evict, key_first, complement, cu_seqlens, batch, total_tokens, max_seqlen, v.hdr,
+                                                      (int32_t*)v.blk_off, (uint32_t*)v.cls_off, (int32_t*)v.seq_start, (int32_t*)v.blk_trace,
+                                                      L.nb_cap, (unsigned long long)L.cls_cap, (int32_t*)v.kmin, (int32_t*)v.kmax,
+                                                      (int32_t*)v.fmin, (int32_t*)v.fmax, (int32_t*)v.col_first, (int32_t*)v.col_last,
+                                                      (int32_t*)v.row_cnt, (int32_t*)v.evict, (int32_t*)v.kfirst);
+    meta_classify_kernel<<<grid + 2, META_THREADS, 0, st>>>(v.hdr, v.blk_off, v.cls_off, v.seq_start, v.blk_trace, v.kmin, v.kmax, v.fmin,
+                                                            v.fmax, v.col_first, v.col_last, (uint8_t*)v.tile_class, (uint16_t*)v.row_list,
+                                                            (int32_t*)v.row_cnt, (int32_t*)v.fwd_order, (int32_t*)v.bwd_order,
+                                                            (int32_t*)v.pair_order, (int32_t*)v.bwd_len, (int32_t*)v.pair_len);
     return cudaGetLastError() == cudaSuccess ? KVS_OK : KVS_ERR_CUDA;
 }
 }  // namespace
