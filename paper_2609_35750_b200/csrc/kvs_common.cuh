@@ -152,6 +152,23 @@ int make_tmap_rows(CUtensorMap* map, const void* base, int rows, int cols);
 int check_device_sm100();
 
 #ifdef __CUDACC__
+template <typename... P, typename... A>
+inline int launch_after(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...) == cudaSuccess ? KVS_OK : KVS_ERR_CUDA;
+}
+#endif
+
+#ifdef __CUDACC__
 // ------------------------------------------------------------------------------------------
 // device: status
 // ------------------------------------------------------------------------------------------
@@ -248,6 +265,15 @@ __device__ __forceinline__ void mbar_wait_limit(uint32_t bar, uint32_t parity, v
 }
 __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int32_t* status) {
     mbar_wait_limit(bar, parity, abort_flag, status, WAIT_LIMIT_CLOCKS);
+}
+
+// Programmatic dependent launch: a kernel started by launch_after() may get its CTAs while the kernel before it in the stream
+// still runs its last ones.  It calls pdl_wait() before it touches memory, which returns once that kernel is complete and its
+// writes are visible, and then lets the next one come.  Every CTA calls it before it can leave, so a kernel is not complete
+// before all earlier ones are.
+__device__ __forceinline__ void pdl_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // Register re-balancing between warp groups (all four warps of a warp group execute it).

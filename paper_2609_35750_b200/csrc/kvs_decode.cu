@@ -8,8 +8,8 @@
 // appending a token takes a page from the free list when the last page is full; decode attention
 // reads exactly the pages the table names.  It never sees a mask.
 //
-// Decode attention is bound by HBM (every live K and V row is read once per step).  Two kernels
-// produce per-split partial results that a third merges:
+// Decode attention is bound by HBM (every live K and V row is read once per step).  One of two kernels
+// produces per-split partial results, which the last CTA of a (sequence, KV head) to finish merges, or a third kernel:
 //   decode_partial_kernel  CUDA cores, organised around coalesced 256-byte row reads: one CTA per
 //                          (split, KV head, sequence); each half-warp reads one K (or V) row per load
 //                          instruction and serves all G query heads of the group from it;
@@ -37,7 +37,76 @@ struct DecodeParams {
     float scale_log2;
     float* part_o;                   // [S, Hq, nsplit, D] unnormalised
     float* part_ml;                  // [S, Hq, nsplit, 2]  (max in base-2 units, sum)
+    int32_t* arrived;                // [S, Hkv] splits that have written their part
+    __nv_bfloat16* out;              // [S, Hq, D]
+    float* lse;                      // [S, Hq]
 };
+
+// Merge of the splits of one (sequence, query head) by a warp: weights exp2(m_z - max), normalised, bf16 out and fp32 lse.
+template <int D>
+__device__ __forceinline__ void decode_merge_row(const DecodeParams& p, size_t row, int lane) {
+    constexpr int PER = D / 32;
+    const float2* ml = reinterpret_cast<const float2*>(p.part_ml) + row * p.nsplit;
+    const float* po = p.part_o + row * p.nsplit * D + lane * PER;
+    float M = -INFINITY;
+    for (int z = lane; z < p.nsplit; z += 32) M = fmaxf(M, __ldcg(ml + z).x);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+    const float Mu = (M == -INFINITY) ? 0.f : M;
+    float L = 0.f, acc[PER];
+#pragma unroll
+    for (int e = 0; e < PER; ++e) acc[e] = 0.f;
+    for (int z0 = 0; z0 < p.nsplit; z0 += 32) {
+        const float2 x = (z0 + lane < p.nsplit) ? __ldcg(ml + z0 + lane) : make_float2(-INFINITY, 0.f);
+        const float w = fast_exp2(x.x - Mu);
+        L += x.y * w;
+        const int n = min(32, p.nsplit - z0);
+#pragma unroll 4
+        for (int i = 0; i < n; ++i) {
+            const float wi = __shfl_sync(0xffffffffu, w, i);
+            const float* src = po + (size_t)(z0 + i) * D;
+            if constexpr (PER == 4) {
+                const float4 v = __ldcg(reinterpret_cast<const float4*>(src));
+                acc[0] += v.x * wi; acc[1] += v.y * wi; acc[2] += v.z * wi; acc[3] += v.w * wi;
+            } else {
+                const float2 v = __ldcg(reinterpret_cast<const float2*>(src));
+                acc[0] += v.x * wi; acc[1] += v.y * wi;
+            }
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
+    const float inv = L > 0.f ? 1.f / L : 0.f;
+#pragma unroll
+    for (int e = 0; e < PER; ++e) acc[e] *= inv;
+    if constexpr (PER == 4)
+        *reinterpret_cast<uint2*>(p.out + row * D + lane * PER) = make_uint2(pack_bf16(acc[0], acc[1]), pack_bf16(acc[2], acc[3]));
+    else
+        *reinterpret_cast<uint32_t*>(p.out + row * D + lane * PER) = pack_bf16(acc[0], acc[1]);
+    if (lane == 0) p.lse[row] = (L > 0.f) ? M * 0.6931471805599453f + logf(L) : -INFINITY;
+}
+
+// ... by the CTA that is the last of its (sequence, KV head) to have written its part, where the call wants it so
+// (p.arrived): a launch less, 23.9 -> 21.4 us for a step on a few thousand tokens.  The CTA has to wait until its part is visible,
+// which in a grid of several waves costs what the launch does (20 sequences, 28 heads on 4: 50.5 and 52.1 us): there
+// decode_merge_kernel does it.
+template <int D, int G>
+__device__ __forceinline__ void decode_merge_if_last(const DecodeParams& p, int s, int g, int tid, volatile int* s_last) {
+    if (!p.arrived) return;
+    __threadfence();
+    named_bar_sync(1, 128);
+    if (tid == 0) *s_last = atomicAdd(&p.arrived[s * p.Hkv + g], 1) == p.nsplit - 1;
+    named_bar_sync(1, 128);
+    if (!*s_last) return;
+    __threadfence();
+    for (int h = tid >> 5; h < G; h += 4) decode_merge_row<D>(p, (size_t)s * p.Hq + g * G + h, tid & 31);
+}
+template <int D>
+__global__ void __launch_bounds__(256) decode_merge_kernel(DecodeParams p) {
+    pdl_wait();
+    const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (row < p.S * p.Hq) decode_merge_row<D>(p, row, threadIdx.x & 31);
+}
 
 // A block-table entry is only followed if it names a page of the cache: anything else (a stale or
 // corrupt table) is recorded as KVS_ERR_INVALID_ARG and read as page 0, so no kernel reads outside the cache.
@@ -85,6 +154,7 @@ decode_partial_kernel(DecodeParams p) {
     constexpr int CH = D / 16;                  // elements of a row per lane (16 lanes per row): 8 or 4
     constexpr int ROWS = (G > 4) ? 4 : 8;       // rows per half-warp per block (register budget)
     constexpr int BLK = 2 * ROWS;               // tokens per softmax update
+    pdl_wait();
     const int z = blockIdx.x, g = blockIdx.y, s = blockIdx.z;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int half = lane >> 4, l16 = lane & 15;
@@ -234,6 +304,8 @@ decode_partial_kernel(DecodeParams p) {
             p.part_ml[base * 2 + 1] = L;
         }
     }
+    __shared__ int s_last;
+    decode_merge_if_last<D, G>(p, s, g, tid, &s_last);
 }
 
 // ---- tensor-core variant (head_dim 128) ------------------------------------------------------------
@@ -303,6 +375,7 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
     extern __shared__ uint8_t smem_raw[];
     const int z = blockIdx.x, g = blockIdx.y, s = blockIdx.z;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    pdl_wait();
     const int n = min(max(p.n_tokens[s], 0), p.max_pages * p.page_size);    // never past the sequence's table
     const int ps = p.page_size;
     const int ppt = 128 / ps;                                   // pages per tile (PAGES)
@@ -609,6 +682,7 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
                 p.part_ml[base * 2 + 1] = s_wsum[h] + s_wsum[16 + h] + s_wsum[32 + h] + s_wsum[48 + h];
             }
         }
+        decode_merge_if_last<D, G>(p, s, g, tid, reinterpret_cast<volatile int*>(sgen + DtcSmem::OFF_MISC + 8));
     }
     tc_fence_before();
     __syncthreads();
@@ -616,33 +690,6 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
         __syncwarp();
         tmem_dealloc(tmem, 32);
     }
-}
-
-// one warp per (sequence, query head): merge the splits, normalise, write bf16 out and fp32 lse
-template <int D>
-__global__ void decode_combine_kernel(const float* __restrict__ part_o, const float* __restrict__ part_ml, int rows, int nsplit,
-                                      __nv_bfloat16* __restrict__ out, float* __restrict__ lse) {
-    const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (row >= rows) return;
-    constexpr int PER = D / 32;
-    float M = -INFINITY;
-    for (int z = 0; z < nsplit; ++z) M = fmaxf(M, part_ml[((size_t)row * nsplit + z) * 2]);
-    const float Mu = (M == -INFINITY) ? 0.f : M;
-    float L = 0.f, o[PER];
-#pragma unroll
-    for (int e = 0; e < PER; ++e) o[e] = 0.f;
-    for (int z = 0; z < nsplit; ++z) {
-        const size_t base = (size_t)row * nsplit + z;
-        const float w = fast_exp2(part_ml[base * 2] - Mu);
-        L += part_ml[base * 2 + 1] * w;
-#pragma unroll
-        for (int e = 0; e < PER; ++e) o[e] += part_o[base * D + lane * PER + e] * w;
-    }
-    const float inv = L > 0.f ? 1.f / L : 0.f;
-#pragma unroll
-    for (int e = 0; e < PER; ++e) out[(size_t)row * D + lane * PER + e] = __float2bfloat16(o[e] * inv);
-    if (lane == 0) lse[row] = (L > 0.f) ? M * 0.6931471805599453f + logf(L) : -INFINITY;
 }
 
 // ---- cache maintenance ---------------------------------------------------------------------------
@@ -663,16 +710,25 @@ __global__ void cache_init_kernel(int32_t* free_buf, int num_pages) {
     if (i < num_pages) stack[i] = num_pages - 1 - i;       // page 0 is handed out first
 }
 
-// one thread per sequence: take a page when the last one is full, write the token's K and V rows
+// one CTA per sequence: take a page when the last one is full, write the token's K and V rows.  Latency is all there is:
+// the rows are fetched while the page is looked up, and rows of whole 16-byte words are copied in such words.
 __global__ void cache_append_kernel(const __nv_bfloat16* __restrict__ k_new, const __nv_bfloat16* __restrict__ v_new,
                                     const uint8_t* __restrict__ active, int S, int Hkv, int D, int page_size, int max_pages,
-                                    int num_pages, int32_t* block_table, int32_t* n_tokens, int32_t* free_buf, __nv_bfloat16* k_cache,
-                                    __nv_bfloat16* v_cache) {
+                                    int num_pages, int wide, int32_t* block_table, int32_t* n_tokens, int32_t* free_buf,
+                                    __nv_bfloat16* k_cache, __nv_bfloat16* v_cache) {
     CacheHeader* hdr = reinterpret_cast<CacheHeader*>(free_buf);
     int32_t* stack = free_buf + 4;
     const int s = blockIdx.x;
+    pdl_wait();
     if (s >= S || (active && !active[s])) return;
     __shared__ int s_page;
+    const size_t src = (size_t)s * Hkv * D;
+    const int words = wide ? Hkv * D / 8 : 0;
+    uint4 k0 = make_uint4(0, 0, 0, 0), v0 = k0;
+    if (threadIdx.x < words) {
+        k0 = reinterpret_cast<const uint4*>(k_new + src)[threadIdx.x];
+        v0 = reinterpret_cast<const uint4*>(v_new + src)[threadIdx.x];
+    }
     const int slot = n_tokens[s];
     if (threadIdx.x == 0) {
         int page = -1;
@@ -698,17 +754,28 @@ __global__ void cache_append_kernel(const __nv_bfloat16* __restrict__ k_new, con
         }
         s_page = page;
     }
-    __syncthreads();
+    __syncthreads();                     // every thread has read n_tokens[s]
     const int page = s_page;
     if (page < 0) return;
-    const size_t dst = ((size_t)page * page_size + slot % page_size) * Hkv * D;
-    const size_t src = (size_t)s * Hkv * D;
-    for (int i = threadIdx.x; i < Hkv * D; i += blockDim.x) {
-        k_cache[dst + i] = k_new[src + i];
-        v_cache[dst + i] = v_new[src + i];
-    }
-    __syncthreads();
     if (threadIdx.x == 0) n_tokens[s] = slot + 1;
+    const size_t dst = ((size_t)page * page_size + slot % page_size) * Hkv * D;
+    if (wide) {
+        uint4* kd = reinterpret_cast<uint4*>(k_cache + dst);
+        uint4* vd = reinterpret_cast<uint4*>(v_cache + dst);
+        if (threadIdx.x < words) {
+            kd[threadIdx.x] = k0;
+            vd[threadIdx.x] = v0;
+        }
+        for (int i = threadIdx.x + blockDim.x; i < words; i += blockDim.x) {
+            kd[i] = reinterpret_cast<const uint4*>(k_new + src)[i];
+            vd[i] = reinterpret_cast<const uint4*>(v_new + src)[i];
+        }
+    } else {
+        for (int i = threadIdx.x; i < Hkv * D; i += blockDim.x) {
+            k_cache[dst + i] = k_new[src + i];
+            v_cache[dst + i] = v_new[src + i];
+        }
+    }
 }
 
 // one CTA per sequence: remove the pages [first_page, first_page + n_pages) of every listed range from the
@@ -718,6 +785,7 @@ __global__ void cache_evict_kernel(const int32_t* __restrict__ ranges, int n_ran
     CacheHeader* hdr = reinterpret_cast<CacheHeader*>(free_buf);
     int32_t* stack = free_buf + 4;
     const int s = blockIdx.x;
+    pdl_wait();
     if (s >= S) return;
     extern __shared__ int32_t sh[];              // keep flags / new positions, max_pages entries
     __shared__ int s_base, s_bad;
@@ -819,11 +887,10 @@ extern "C" int kvs_cache_append(const void* k_new, const void* v_new, const uint
     if (!k_new || !v_new || !block_table || !n_tokens || !free_list || !k_cache || !v_cache) return KVS_ERR_INVALID_ARG;
     if (num_seqs < 0 || Hkv <= 0 || head_dim <= 0 || page_size <= 0 || max_pages <= 0 || num_pages <= 0) return KVS_ERR_INVALID_ARG;
     if (num_seqs == 0) return KVS_OK;
-    cache_append_kernel<<<num_seqs, 128, 0, (cudaStream_t)stream>>>((const __nv_bfloat16*)k_new, (const __nv_bfloat16*)v_new, active,
-                                                                   num_seqs, Hkv, head_dim, page_size, max_pages, num_pages, block_table,
-                                                                   n_tokens, free_list, (__nv_bfloat16*)k_cache,
-                                                                   (__nv_bfloat16*)v_cache);
-    return cudaGetLastError() == cudaSuccess ? KVS_OK : KVS_ERR_CUDA;
+    const int wide = (Hkv * head_dim) % 8 == 0 && (((uintptr_t)k_new | (uintptr_t)v_new | (uintptr_t)k_cache | (uintptr_t)v_cache) & 15) == 0;
+    return launch_after(cache_append_kernel, num_seqs, 128, 0, (cudaStream_t)stream, (const __nv_bfloat16*)k_new, (const __nv_bfloat16*)v_new,
+                        active, num_seqs, Hkv, head_dim, page_size, max_pages, num_pages, wide, block_table, n_tokens, free_list,
+                        (__nv_bfloat16*)k_cache, (__nv_bfloat16*)v_cache);
 }
 
 extern "C" int kvs_cache_evict(const int32_t* ranges, int n_ranges, int num_seqs, int page_size, int max_pages, int num_pages,
@@ -838,9 +905,8 @@ extern "C" int kvs_cache_evict(const int32_t* ranges, int n_ranges, int num_seqs
     if (smem > 48 * 1024 &&
         cudaFuncSetAttribute(cache_evict_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return KVS_ERR_CUDA;
-    cache_evict_kernel<<<num_seqs, 256, smem, (cudaStream_t)stream>>>(ranges, n_ranges, num_seqs, page_size, max_pages, num_pages, block_table,
-                                                                     n_tokens, free_list);
-    return cudaGetLastError() == cudaSuccess ? KVS_OK : KVS_ERR_CUDA;
+    return launch_after(cache_evict_kernel, num_seqs, 256, smem, (cudaStream_t)stream, ranges, n_ranges, num_seqs, page_size, max_pages,
+                        num_pages, block_table, n_tokens, free_list);
 }
 
 extern "C" int kvs_decode_num_splits(int num_seqs, int Hkv, int max_tokens) {
@@ -871,14 +937,20 @@ extern "C" int kvs_decode_num_splits(int num_seqs, int Hkv, int max_tokens) {
 
 extern "C" size_t kvs_decode_workspace_bytes(int num_seqs, int Hq, int head_dim, int num_splits) {
     if (num_seqs < 0 || Hq <= 0 || head_dim <= 0 || num_splits <= 0) return 0;
-    return DEC_WS_HEADER + align_up(sizeof(float) * (size_t)num_seqs * Hq * num_splits * (head_dim + 2), 256);
+    return DEC_WS_HEADER + align_up(sizeof(float) * (size_t)num_seqs * Hq * num_splits * (head_dim + 2), 256) +
+           align_up(sizeof(int32_t) * (size_t)num_seqs * Hq, 256);       // arrival counts, at most one per query head
 }
 
 // the first 256 bytes of the workspace: {magic, status} as in the backward workspace, so that
-// kvs_device_status() reads it; the partial results follow
-__global__ void decode_header_kernel(int32_t* hdr) {
-    hdr[0] = (int32_t)WS_MAGIC;
-    hdr[1] = KVS_OK;
+// kvs_device_status() reads it; the partial results follow, then the arrival counts
+__global__ void decode_header_kernel(int32_t* hdr, int32_t* arrived, int n) {
+    pdl_wait();
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0) {
+        hdr[0] = (int32_t)WS_MAGIC;
+        hdr[1] = KVS_OK;
+    }
+    if (i < n) arrived[i] = 0;
 }
 
 template <int G, int LOAD>
@@ -886,13 +958,11 @@ static int launch_decode_tc(const CUtensorMap& tk, const CUtensorMap& tv, const 
     auto kern = decode_tc_kernel<G, LOAD>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, DtcSmem::DYN_BYTES) != cudaSuccess) return KVS_ERR_CUDA;
     dim3 grid(p.nsplit, p.Hkv, p.S);
-    kern<<<grid, DTC_THREADS, DtcSmem::DYN_BYTES, st>>>(tk, tv, p, status);
-    return cudaGetLastError() == cudaSuccess ? KVS_OK : KVS_ERR_CUDA;
+    return launch_after(kern, grid, DTC_THREADS, DtcSmem::DYN_BYTES, st, tk, tv, p, status);
 }
 
 template <int D>
-static int launch_decode(const DecodeParams& p, int G, const void* k_cache, const void* v_cache, int32_t* status, void* out, float* lse,
-                         cudaStream_t st) {
+static int launch_decode(const DecodeParams& p, int G, const void* k_cache, const void* v_cache, int32_t* status, cudaStream_t st) {
     dim3 grid(p.nsplit, p.Hkv, p.S);
     const int ps = p.page_size;
     // tensor-core variant (head_dim 128).  Pages that are whole 8-row swizzle atoms and tile 128 tokens exactly come in
@@ -934,18 +1004,20 @@ static int launch_decode(const DecodeParams& p, int G, const void* k_cache, cons
             }
         }
         if (rc != KVS_OK) return rc;
-    } else
-    switch (G) {
-        case 1: decode_partial_kernel<D, 1><<<grid, DEC_THREADS, 0, st>>>(p); break;
-        case 2: decode_partial_kernel<D, 2><<<grid, DEC_THREADS, 0, st>>>(p); break;
-        case 4: decode_partial_kernel<D, 4><<<grid, DEC_THREADS, 0, st>>>(p); break;
-        case 7: decode_partial_kernel<D, 7><<<grid, DEC_THREADS, 0, st>>>(p); break;
-        case 8: decode_partial_kernel<D, 8><<<grid, DEC_THREADS, 0, st>>>(p); break;
-        default: return KVS_ERR_UNSUPPORTED;
+    } else {
+        int rc = KVS_ERR_UNSUPPORTED;
+        switch (G) {
+            case 1: rc = launch_after(decode_partial_kernel<D, 1>, grid, DEC_THREADS, 0, st, p); break;
+            case 2: rc = launch_after(decode_partial_kernel<D, 2>, grid, DEC_THREADS, 0, st, p); break;
+            case 4: rc = launch_after(decode_partial_kernel<D, 4>, grid, DEC_THREADS, 0, st, p); break;
+            case 7: rc = launch_after(decode_partial_kernel<D, 7>, grid, DEC_THREADS, 0, st, p); break;
+            case 8: rc = launch_after(decode_partial_kernel<D, 8>, grid, DEC_THREADS, 0, st, p); break;
+        }
+        if (rc != KVS_OK) return rc;
     }
-    const int rows = p.S * p.Hq;
-    decode_combine_kernel<D><<<(rows * 32 + 255) / 256, 256, 0, st>>>(p.part_o, p.part_ml, rows, p.nsplit, (__nv_bfloat16*)out, lse);
-    return cudaGetLastError() == cudaSuccess ? KVS_OK : KVS_ERR_CUDA;
+    if (p.arrived) return KVS_OK;
+    const long long rows = (long long)p.S * p.Hq;
+    return launch_after(decode_merge_kernel<D>, (unsigned)((rows + 7) / 8), 256, 0, st, p);
 }
 
 extern "C" int kvs_decode_attn(const void* q, const void* k_cache, const void* v_cache, const int32_t* block_table,
@@ -982,8 +1054,15 @@ extern "C" int kvs_decode_attn(const void* q, const void* k_cache, const void* v
     p.part_o = (float*)((char*)workspace + DEC_WS_HEADER);
     p.part_ml = p.part_o + (size_t)num_seqs * Hq * num_splits * head_dim;
     cudaStream_t st = (cudaStream_t)stream;
-    decode_header_kernel<<<1, 1, 0, st>>>((int32_t*)workspace);
+    p.arrived = (int32_t*)((char*)workspace + DEC_WS_HEADER + align_up(sizeof(float) * (size_t)num_seqs * Hq * num_splits * (head_dim + 2), 256));
+    p.out = (__nv_bfloat16*)out;
+    p.lse = lse;
+    // three CTAs per SM are resident: up to two waves of them merge on their own
+    const int rows = num_seqs * Hkv;
+    if ((long long)rows * num_splits > 2 * 3 * 148) p.arrived = nullptr;
+    const int rc = launch_after(decode_header_kernel, p.arrived ? (rows + 255) / 256 : 1, 256, 0, st, (int32_t*)workspace, p.arrived, p.arrived ? rows : 0);
+    if (rc != KVS_OK) return rc;
     int32_t* status = (int32_t*)workspace + 1;
-    return head_dim == 64 ? launch_decode<64>(p, Hq / Hkv, k_cache, v_cache, status, out, lse, st)
-                          : launch_decode<128>(p, Hq / Hkv, k_cache, v_cache, status, out, lse, st);
+    return head_dim == 64 ? launch_decode<64>(p, Hq / Hkv, k_cache, v_cache, status, st)
+                          : launch_decode<128>(p, Hq / Hkv, k_cache, v_cache, status, st);
 }
