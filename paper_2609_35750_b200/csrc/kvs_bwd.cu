@@ -228,6 +228,7 @@ __global__ void __launch_bounds__(256)
 bwd_dot_kernel(const __nv_bfloat16* __restrict__ dout, const __nv_bfloat16* __restrict__ out,
                float* __restrict__ dvec, float* __restrict__ dq_acc, long long dq_ts, int total_tokens, int Hq, WsHeader* hdr,
                const __grid_constant__ BwdPlanArgs plan) {
+    pdl_wait();
     if (blockIdx.x == 0) {                      // the first CTA has no rows
         if (threadIdx.x == 0) {
             hdr->magic = WS_MAGIC;
@@ -281,6 +282,7 @@ bwd_dot_kernel(const __nv_bfloat16* __restrict__ dout, const __nv_bfloat16* __re
 // ---- post-pass --------------------------------------------------------------------------------
 // acc: contiguous [tokens, row_elems]; dq: rows of row_elems elements, dq_ts elements apart
 __global__ void bwd_cast_kernel(const float* __restrict__ acc, __nv_bfloat16* __restrict__ dq, size_t n4, int row_elems, long long dq_ts) {
+    pdl_wait();
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n4) return;
     const float4 x = reinterpret_cast<const float4*>(acc)[i];
@@ -348,6 +350,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     const int tid = threadIdx.x;
     const int warp = tid >> 5;
     const int lane = tid & 31;
+    pdl_wait();
     // meta_buf must be the one kvs_mask_meta wrote for these sizes: every index below comes out of it
     if (!meta_matches(mv.hdr, p.batch, p.total_tokens, p.max_seqlen)) {
         if (tid == 0 && blockIdx.x == 0) set_status(p.status, KVS_ERR_BAD_META);
@@ -713,8 +716,7 @@ static int launch_dot(const __nv_bfloat16* dout, const __nv_bfloat16* out, float
     const int threads = 256;
     const long long blocks = (warps * 32 + threads - 1) / threads + 1;
     if (blocks > 0x7fffffffLL) return KVS_ERR_UNSUPPORTED;
-    bwd_dot_kernel<D><<<(unsigned)blocks, threads, 0, st>>>(dout, out, dvec, dq_acc, dq_ts, total_tokens, Hq, hdr, plan);
-    return cudaGetLastError() == cudaSuccess ? KVS_OK : KVS_ERR_CUDA;
+    return launch_after(bwd_dot_kernel<D>, (unsigned)blocks, threads, 0, st, dout, out, dvec, dq_acc, dq_ts, total_tokens, Hq, hdr, plan);
 }
 
 template <int D>
@@ -722,8 +724,7 @@ static int launch_main(const CUtensorMap& tq, const CUtensorMap& tk, const CUten
                        const MetaView& mv, const BwdParams& p, unsigned units, cudaStream_t st) {
     auto kern = bwd_kernel<D>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdSmem<D>::DYN_BYTES) != cudaSuccess) return KVS_ERR_CUDA;
-    kern<<<units, BWD_THREADS, BwdSmem<D>::DYN_BYTES, st>>>(tq, tk, tv, tdo, tdq, mv, p);
-    return cudaGetLastError() == cudaSuccess ? KVS_OK : KVS_ERR_CUDA;
+    return launch_after(kern, units, BWD_THREADS, BwdSmem<D>::DYN_BYTES, st, tq, tk, tv, tdo, tdq, mv, p);
 }
 
 }  // namespace kvs
@@ -859,8 +860,9 @@ int bwd_impl(const void* dout, const void* q, const void* k, const void* v, long
         const size_t n4 = nq / 4;
         const size_t blocks = (n4 + 255) / 256;
         if (blocks > 0x7fffffffull) return KVS_ERR_UNSUPPORTED;
-        bwd_cast_kernel<<<(unsigned)blocks, 256, 0, st>>>(dq_acc, (__nv_bfloat16*)dq, n4, Hq * head_dim, dq_ts_out);
-        if (cudaGetLastError() != cudaSuccess) return KVS_ERR_CUDA;
+        if ((rc = launch_after(bwd_cast_kernel, (unsigned)blocks, 256, 0, st, (const float*)dq_acc, (__nv_bfloat16*)dq, n4, Hq * head_dim,
+                               dq_ts_out)) != KVS_OK)
+            return rc;
     }
     return KVS_OK;
 }

@@ -140,6 +140,7 @@ bwd_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     const int warp = tid >> 5;
     const int lane = tid & 31;
     const uint32_t rank = cluster_rank();
+    pdl_wait();
     // The returns below are taken by both CTAs of a pair alike.
     if (!meta_matches(mv.hdr, p.batch, p.total_tokens, p.max_seqlen)) {
         if (tid == 0 && blockIdx.x == 0) set_status(p.status, KVS_ERR_BAD_META);
@@ -611,8 +612,7 @@ int launch_bwd_pair(const CUtensorMap& q64, const CUtensorMap& k, const CUtensor
                     const MetaView& mv, const BwdParams& p, unsigned units, cudaStream_t st) {
     if (cudaFuncSetAttribute(bwd_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PairSmem::DYN_BYTES) != cudaSuccess)
         return KVS_ERR_CUDA;
-    bwd_pair_kernel<<<2 * units, BWD_THREADS, PairSmem::DYN_BYTES, st>>>(q64, k, v, do64, dq64, mv, p);
-    return cudaGetLastError() == cudaSuccess ? KVS_OK : KVS_ERR_CUDA;
+    return launch_after(bwd_pair_kernel, 2 * units, BWD_THREADS, PairSmem::DYN_BYTES, st, q64, k, v, do64, dq64, mv, p);
 }
 
 }  // namespace kvs

@@ -68,6 +68,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     const int tid = threadIdx.x;
     const int warp = tid >> 5;
     const int lane = tid & 31;
+    pdl_wait();
     // meta_buf must be the one kvs_mask_meta wrote for these sizes: every index below comes out of it
     if (!meta_matches(mv.hdr, p.batch, p.total_tokens, p.max_seqlen)) {
         if (tid == 0 && blockIdx.x == 0 && blockIdx.y == 0) set_status(&mv.hdr->status, KVS_ERR_BAD_META);
@@ -514,8 +515,7 @@ static int launch_fwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtens
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem<D>::DYN_BYTES) != cudaSuccess) return KVS_ERR_CUDA;
     const int G = p.Hq / p.Hkv;
     dim3 grid(nb_cap, p.Hkv * ((G + 1) / 2), 1);
-    kern<<<grid, FWD_THREADS, FwdSmem<D>::DYN_BYTES, st>>>(tq, tk, tv, mv, p);
-    return cudaGetLastError() == cudaSuccess ? KVS_OK : KVS_ERR_CUDA;
+    return launch_after(kern, grid, FWD_THREADS, FwdSmem<D>::DYN_BYTES, st, tq, tk, tv, mv, p);
 }
 
 }  // namespace kvs

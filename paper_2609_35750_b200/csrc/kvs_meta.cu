@@ -27,6 +27,7 @@ meta_blocks_kernel(const int32_t* __restrict__ evict_at, const int32_t* __restri
     __shared__ long long s_blk[META_WARPS];
     __shared__ int4 s_mine[META_WARPS];              // trace, its first block, its first token, its length
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    pdl_wait();
     const long long blk0 = (long long)blockIdx.x * META_WARPS;
     const bool writer = blockIdx.x == 0;
     if (tid < META_WARPS) s_mine[tid].x = -1;
@@ -255,6 +256,7 @@ meta_classify_kernel(MetaHeader* hdr, const int32_t* __restrict__ blk_off, const
                      const int32_t* __restrict__ fmin, const int32_t* __restrict__ fmax, const int32_t* __restrict__ col_first,
                      const int32_t* __restrict__ col_last, uint8_t* tile_class, uint16_t* row_list, int32_t* row_cnt, int32_t* fwd_order,
                      int32_t* bwd_order, int32_t* pair_order, int32_t* bwd_len, int32_t* pair_len) {
+    pdl_wait();
     if (blockIdx.x < 2) {
         const bool pairs = blockIdx.x == 1;
         meta_order(pairs ? ORDER_PAIRS : ORDER_COLS, hdr, blk_off, blk_trace, row_cnt, col_first, col_last, pairs ? pair_order : bwd_order,
@@ -360,16 +362,15 @@ int launch_mask_meta(const int32_t* key_evict, const int32_t* key_first, int com
     cudaStream_t st = (cudaStream_t)stream;
     MetaView v = meta_view(meta_buf, L);
     const int grid = (L.nb_cap + META_WARPS - 1) / META_WARPS;
-    meta_blocks_kernel<<<grid, META_THREADS, 0, st>>>(key_evict, key_first, complement, cu_seqlens, batch, total_tokens, max_seqlen, v.hdr,
-                                                      (int32_t*)v.blk_off, (uint32_t*)v.cls_off, (int32_t*)v.seq_start, (int32_t*)v.blk_trace,
-                                                      L.nb_cap, (unsigned long long)L.cls_cap, (int32_t*)v.kmin, (int32_t*)v.kmax,
-                                                      (int32_t*)v.fmin, (int32_t*)v.fmax, (int32_t*)v.col_first, (int32_t*)v.col_last,
-                                                      (int32_t*)v.row_cnt, (int32_t*)v.evict, (int32_t*)v.kfirst);
-    meta_classify_kernel<<<grid + 2, META_THREADS, 0, st>>>(v.hdr, v.blk_off, v.cls_off, v.seq_start, v.blk_trace, v.kmin, v.kmax, v.fmin,
-                                                            v.fmax, v.col_first, v.col_last, (uint8_t*)v.tile_class, (uint16_t*)v.row_list,
-                                                            (int32_t*)v.row_cnt, (int32_t*)v.fwd_order, (int32_t*)v.bwd_order,
-                                                            (int32_t*)v.pair_order, (int32_t*)v.bwd_len, (int32_t*)v.pair_len);
-    return cudaGetLastError() == cudaSuccess ? KVS_OK : KVS_ERR_CUDA;
+    const int rc = launch_after(meta_blocks_kernel, grid, META_THREADS, 0, st, key_evict, key_first, complement, cu_seqlens, batch, total_tokens,
+                                max_seqlen, v.hdr, (int32_t*)v.blk_off, (uint32_t*)v.cls_off, (int32_t*)v.seq_start, (int32_t*)v.blk_trace,
+                                L.nb_cap, (unsigned long long)L.cls_cap, (int32_t*)v.kmin, (int32_t*)v.kmax, (int32_t*)v.fmin,
+                                (int32_t*)v.fmax, (int32_t*)v.col_first, (int32_t*)v.col_last, (int32_t*)v.row_cnt, (int32_t*)v.evict,
+                                (int32_t*)v.kfirst);
+    if (rc != KVS_OK) return rc;
+    return launch_after(meta_classify_kernel, grid + 2, META_THREADS, 0, st, v.hdr, v.blk_off, v.cls_off, v.seq_start, v.blk_trace, v.kmin,
+                        v.kmax, v.fmin, v.fmax, v.col_first, v.col_last, (uint8_t*)v.tile_class, (uint16_t*)v.row_list, (int32_t*)v.row_cnt,
+                        (int32_t*)v.fwd_order, (int32_t*)v.bwd_order, (int32_t*)v.pair_order, (int32_t*)v.bwd_len, (int32_t*)v.pair_len);
 }
 }  // namespace
 
@@ -397,6 +398,7 @@ __global__ void __launch_bounds__(1024)
 reorder_sort_kernel(const int32_t* __restrict__ evict_at, const int32_t* __restrict__ cu_seqlens, int window, int32_t* perm,
                     int32_t* key_first, int32_t* key_evict) {
     __shared__ unsigned long long keys[REORDER_MAX_WINDOW];
+    pdl_wait();
     const int b = blockIdx.y;
     const int tok0 = cu_seqlens[b];
     const int T = cu_seqlens[b + 1] - tok0;
@@ -435,6 +437,7 @@ reorder_sort_kernel(const int32_t* __restrict__ evict_at, const int32_t* __restr
 // dst row r = src row perm[r] (inverse == 0) or dst row perm[r] = src row r (inverse != 0); 16 bytes per lane
 __global__ void permute_rows_kernel(const uint4* __restrict__ src, const int32_t* __restrict__ perm, uint4* __restrict__ dst,
                                     long long n_rows, int row_vec, int inverse) {
+    pdl_wait();
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long r = idx / row_vec;
     const int c = (int)(idx % row_vec);
@@ -455,8 +458,7 @@ extern "C" int kvs_reorder_keys(const int32_t* evict_at, const int32_t* cu_seqle
     if (max_seqlen > total_tokens) max_seqlen = total_tokens;
     const int nwin = (max_seqlen + window - 1) / window;
     dim3 grid(nwin > 0 ? nwin : 1, batch, 1);
-    reorder_sort_kernel<<<grid, 1024, 0, (cudaStream_t)stream>>>(evict_at, cu_seqlens, window, perm, key_first, key_evict);
-    return cudaGetLastError() == cudaSuccess ? KVS_OK : KVS_ERR_CUDA;
+    return launch_after(reorder_sort_kernel, grid, 1024, 0, (cudaStream_t)stream, evict_at, cu_seqlens, window, perm, key_first, key_evict);
 }
 
 extern "C" int kvs_permute_rows(const void* src, const int32_t* perm, void* dst, long long n_rows, long long row_bytes, int inverse,
@@ -469,8 +471,8 @@ extern "C" int kvs_permute_rows(const void* src, const int32_t* perm, void* dst,
     const long long total = n_rows * row_vec;
     const long long blocks = (total + 255) / 256;
     if (blocks > 0x7fffffffLL) return KVS_ERR_UNSUPPORTED;
-    permute_rows_kernel<<<(unsigned)blocks, 256, 0, (cudaStream_t)stream>>>((const uint4*)src, perm, (uint4*)dst, n_rows, row_vec, inverse);
-    return cudaGetLastError() == cudaSuccess ? KVS_OK : KVS_ERR_CUDA;
+    return launch_after(permute_rows_kernel, (unsigned)blocks, 256, 0, (cudaStream_t)stream, (const uint4*)src, perm, (uint4*)dst, n_rows, row_vec,
+                        inverse);
 }
 
 extern "C" int kvs_mask_meta_export(const void* meta_buf, int batch, const int32_t* cu_seqlens_host, int total_tokens,
