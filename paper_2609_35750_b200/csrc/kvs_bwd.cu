@@ -365,7 +365,6 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     const int n = gb - mv.blk_off[b];
     const int tok0 = mv.seq_start[b];
     const int T = mv.seq_start[b + 1] - tok0;
-    const int nb = (T + TILE - 1) / TILE;
     const int m_first = mv.col_first[gb];           // == n unless the key slots were re-ordered
     const int m_last = mv.col_last[gb];
     const int nm = m_last - m_first + 1;            // query blocks m_first .. m_last can see this key block
@@ -638,8 +637,9 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
             const int masked = __any_sync(0xffffffffu, lo > 0 || hi < 64) ? 1 : 0;
 #pragma unroll 1
             for (int pass = 0; pass < masked; ++pass) {
+                const uint32_t seen0 = bit_range(lo, hi), seen1 = bit_range(lo - 32, hi - 32);
 #pragma unroll
-                for (int e = 0; e < 64; ++e) pv[e] = (e >= lo && e < hi) ? pv[e] : 0.f;
+                for (int e = 0; e < 64; ++e) pv[e] = ((e < 32 ? seen0 : seen1) >> (e & 31) & 1u) ? pv[e] : 0.f;
             }
             uint32_t pk[32];
 #pragma unroll

@@ -80,6 +80,12 @@ __device__ __forceinline__ bool bwd_unit_of(const BwdParams& p, const int32_t* o
     return true;
 }
 
+// bits [lo, hi) of a 32-bit word (either end may lie outside it)
+__device__ __forceinline__ uint32_t bit_range(int lo, int hi) {
+    const int l = min(max(lo, 0), 32), h = min(max(hi, 0), 32);
+    return (h >= 32 ? 0xffffffffu : (1u << h) - 1u) & (l >= 32 ? 0u : ~((1u << l) - 1u));
+}
+
 // rows of zeros for a key block that no query sees (its gradients are zero)
 template <int D>
 __device__ __forceinline__ void bwd_zero_rows(const BwdParams& p, int tok, int rows, int g) {

@@ -514,8 +514,9 @@ bwd_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             const int masked = __any_sync(0xffffffffu, lo > 0 || hi < 64) ? 1 : 0;
 #pragma unroll 1
             for (int pass = 0; pass < masked; ++pass) {
+                const uint32_t seen0 = bit_range(lo, hi), seen1 = bit_range(lo - 32, hi - 32);
 #pragma unroll
-                for (int e = 0; e < 64; ++e) pv[e] = (e >= lo && e < hi) ? pv[e] : 0.f;
+                for (int e = 0; e < 64; ++e) pv[e] = ((e < 32 ? seen0 : seen1) >> (e & 31) & 1u) ? pv[e] : 0.f;
             }
             uint32_t pk[32];
 #pragma unroll

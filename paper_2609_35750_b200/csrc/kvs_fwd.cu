@@ -321,29 +321,34 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
                         sv[96 + e] = __uint_as_float(r3[e]);
                     }
                 }
-                
                 if (need_mask) {
-                    const int4* ev4 = reinterpret_cast<const int4*>(sEv + s * TILE);
-                    if (!general) {
+                    // Per warp and 32 keys: seen by all of the warp's 32 rows (nothing to do), hidden from all of them, or
+                    // neither.  Only the last kind is decided element by element.  On a diagonal tile that is one of a warp's
+                    // four groups, where a span of turns leaves it is the warps that its step falls into.
+                    const int q_lo = m * TILE + quad * 32, q_hi = q_lo + 31;
 #pragma unroll
-                        for (int e4 = 0; e4 < TILE / 4; ++e4) {
-                            const int4 ev = ev4[e4];
-                            const int j = n * TILE + e4 * 4;
-                            sv[e4 * 4 + 0] = ((j + 0 <= qi) && (qi < ev.x)) ? sv[e4 * 4 + 0] : -INFINITY;
-                            sv[e4 * 4 + 1] = ((j + 1 <= qi) && (qi < ev.y)) ? sv[e4 * 4 + 1] : -INFINITY;
-                            sv[e4 * 4 + 2] = ((j + 2 <= qi) && (qi < ev.z)) ? sv[e4 * 4 + 2] : -INFINITY;
-                            sv[e4 * 4 + 3] = ((j + 3 <= qi) && (qi < ev.w)) ? sv[e4 * 4 + 3] : -INFINITY;
+                    for (int c = 0; c < 4; ++c) {
+                        const int kev = sEv[s * TILE + c * 32 + lane], kfirst = sKf[s * TILE + c * 32 + lane];
+                        const bool seen = __all_sync(0xffffffffu, kfirst <= q_lo && q_hi < kev);
+                        const bool hidden = __all_sync(0xffffffffu, kfirst > q_hi || kev <= q_lo);
+                        if (hidden) {
+#pragma unroll
+                            for (int e = 0; e < 32; ++e) sv[c * 32 + e] = -INFINITY;
                         }
-                    } else {
-                        const int4* kf4 = reinterpret_cast<const int4*>(sKf + s * TILE);
+                        const int mixed = (seen || hidden) ? 0 : 1;
+#pragma unroll 1
+                        for (int pass = 0; pass < mixed; ++pass) {          // a loop of at most one pass: not predicated
+                            const int4* ev4 = reinterpret_cast<const int4*>(sEv + s * TILE + c * 32);
+                            const int4* kf4 = reinterpret_cast<const int4*>(sKf + s * TILE + c * 32);
 #pragma unroll
-                        for (int e4 = 0; e4 < TILE / 4; ++e4) {
-                            const int4 ev = ev4[e4];
-                            const int4 kf = kf4[e4];
-                            sv[e4 * 4 + 0] = ((kf.x <= qi) && (qi < ev.x)) ? sv[e4 * 4 + 0] : -INFINITY;
-                            sv[e4 * 4 + 1] = ((kf.y <= qi) && (qi < ev.y)) ? sv[e4 * 4 + 1] : -INFINITY;
-                            sv[e4 * 4 + 2] = ((kf.z <= qi) && (qi < ev.z)) ? sv[e4 * 4 + 2] : -INFINITY;
-                            sv[e4 * 4 + 3] = ((kf.w <= qi) && (qi < ev.w)) ? sv[e4 * 4 + 3] : -INFINITY;
+                            for (int e4 = 0; e4 < 8; ++e4) {
+                                const int4 ev = ev4[e4], kf = kf4[e4];
+                                float* x = sv + c * 32 + e4 * 4;
+                                x[0] = ((kf.x <= qi) && (qi < ev.x)) ? x[0] : -INFINITY;
+                                x[1] = ((kf.y <= qi) && (qi < ev.y)) ? x[1] : -INFINITY;
+                                x[2] = ((kf.z <= qi) && (qi < ev.z)) ? x[2] : -INFINITY;
+                                x[3] = ((kf.w <= qi) && (qi < ev.w)) ? x[3] : -INFINITY;
+                            }
                         }
                     }
                 }
