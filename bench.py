@@ -352,7 +352,7 @@ def run_meta_only(args):
     print(json.dumps({"metric": "mask_meta_gbs", "value": gbs, "unit": "GB/s", "steps": len(ms), "warmup": args.warmup,
                       "ms_per_step": float(np.median(ms)), "config": {"workload": w.name, "traces": w.batch, "tokens": w.total_tokens,
                                                                        "key_blocks": nb, "tiles": tiles, "meta_buffer_bytes": nbytes},
-                      "roofline": {"kernel": "mask metadata (4 launches)", "bound": "hbm", "achieved": gbs, "peak": float(peaks["hbm_gbs"]),
+                      "roofline": {"kernel": "mask metadata (2 launches)", "bound": "hbm", "achieved": gbs, "peak": float(peaks["hbm_gbs"]),
                                    "unit": "GB/s", "frac": gbs / float(peaks["hbm_gbs"]), "traffic": None,
                                    "algorithmic_bytes": alg},
                       "status": st, "dtype": "int32", "data": "synthetic"}), flush=True)
@@ -663,7 +663,7 @@ def main():
                      "flops_per_launch": flops_bwd_main},
         "clocks": clocks,
         "e2e": e2e,
-        "gpu_launches": ((8 if grad == B.GRAD_BF16 else 7) + (5 if args.reorder else 0)) * args.steps,
+        "gpu_launches": ((6 if grad == B.GRAD_BF16 else 5) + (5 if args.reorder else 0)) * args.steps,
         "cpu_baseline": cpu_baseline,
         "per_config": per_config,
         "rollout_decode": rollout_decode,

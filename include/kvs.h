@@ -259,7 +259,8 @@ int kvs_attn_bwd_ex(const void* dout, const void* q, const void* k, const void* 
  * whole HBM to its own pool at start-up (a later cudaMalloc fails), or a step loop that must not
  * pay the device-wide synchronisation cudaMalloc/cudaFree imply.  For them the scratch that
  * kvs_attn_bwd takes as `workspace` is a fixed array inside the library, of
- * 256 B + 4 B * KVS_NOALLOC_MAX_ROWS per GPU, resident on every GPU that loads the library.
+ * 256 B + 4 B * KVS_NOALLOC_MAX_ROWS + 38 MiB per GPU (the last for the partial sums of key blocks with long
+ * walks, see kvs_attn_bwd_workspace_bytes), resident on every GPU that loads the library.
  *   - Gradients are fp32 only (dq is accumulated in place, so it needs no scratch); otherwise the
  *     arguments and results are those of kvs_attn_bwd with KVS_GRAD_FP32.
  *   - total_tokens * Hq must not exceed KVS_NOALLOC_MAX_ROWS, else KVS_ERR_WORKSPACE is returned
