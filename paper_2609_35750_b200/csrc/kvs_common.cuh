@@ -215,6 +215,9 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
+__device__ __forceinline__ void mbar_arrive_n(uint32_t bar, uint32_t n) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(n) : "memory");
+}
 __device__ __forceinline__ uint32_t mbar_try_wait(uint32_t bar, uint32_t parity) {
     uint32_t ok;
     asm volatile(
@@ -274,6 +277,30 @@ __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, volatil
 __device__ __forceinline__ void pdl_wait() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Cluster launch control: asks for a CTA of this grid that has not started yet.  It will not start then; its work is the
+// caller's.  The 16-byte answer comes into shared memory and completes 16 bytes on the barrier.  Not to be asked again after a
+// "no".
+__device__ __forceinline__ void ask_for_cta(uint32_t answer, uint32_t bar) {
+    asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(answer), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ bool cta_answer(uint32_t answer, int& x, int& y) {
+    uint32_t ok, cx = 0, cy = 0;
+    asm volatile(
+        "{\n\t.reg .b128 h;\n\t.reg .pred p;\n\t.reg .b32 z, w;\n\t"
+        "mov.b32 %1, 0;\n\tmov.b32 %2, 0;\n\t"
+        "ld.shared.b128 h, [%3];\n\t"
+        "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, h;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t"
+        "@p clusterlaunchcontrol.query_cancel.get_first_ctaid.v4.b32.b128 {%1, %2, z, w}, h;\n\t}"
+        : "=r"(ok), "=&r"(cx), "=&r"(cy)
+        : "r"(answer)
+        : "memory");
+    x = (int)cx;
+    y = (int)cy;
+    return ok != 0;
 }
 
 // Register re-balancing between warp groups (all four warps of a warp group execute it).
