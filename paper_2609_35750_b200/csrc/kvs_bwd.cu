@@ -326,7 +326,8 @@ struct BwdSmem {
     static constexpr int OFF_DVEC = OFF_LSE + 2 * TILE * 4;    // 2 stages x 128 fp32: -D * scale
     static constexpr int OFF_BAR = OFF_DVEC + 2 * TILE * 4;
     static constexpr int OFF_MISC = OFF_BAR + 16 * 8;          // tmem base, abort flag
-    static constexpr int TOTAL = OFF_MISC + 16;
+    static constexpr int OFF_WORK = OFF_MISC + 16;
+    static constexpr int TOTAL = OFF_WORK + (int)sizeof(BwdWork);
     static constexpr int MAX_DYN = 232448;                     // 227 KB
     static constexpr int DYN_BYTES = (TOTAL + 1024 > MAX_DYN) ? MAX_DYN : TOTAL + 1024;
 };
@@ -356,28 +357,29 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         if (tid == 0 && blockIdx.x == 0) set_status(p.status, KVS_ERR_BAD_META);
         return;
     }
-    BwdUnit unit;
-    int g;
-    if (!bwd_unit_of(p, mv.bwd_order, mv.hdr->nblk_total, blockIdx.x, unit, g)) return;
-    const int gb = unit.block;
-    const int G = p.Hq / p.Hkv;
-    const int b = mv.blk_trace[gb];
-    const int n = gb - mv.blk_off[b];
-    const int tok0 = mv.seq_start[b];
-    const int T = mv.seq_start[b + 1] - tok0;
-    const int m_first = mv.col_first[gb];           // == n unless the key slots were re-ordered
-    const int m_last = mv.col_last[gb];
-    const int nm = m_last - m_first + 1;            // query blocks m_first .. m_last can see this key block
-    const int n_iter = (unit.tile1 < 0 ? G * nm : unit.tile1) - unit.tile0;     // tiles of this unit of the G * nm (head, query block) tiles of the key block
-    int32_t* status = p.status;
-    const bool general = mv.hdr->general != 0;
-    if (nm <= 0) {
-        // no query sees any key of the block (general metadata only): its gradients are zero
-        bwd_zero_rows<D>(p, tok0 + n * TILE, min(TILE, T - n * TILE), g);
-        return;
+    BwdWork w;
+    {
+        BwdUnit unit;
+        if (!bwd_unit_of(p, mv.bwd_order, mv.hdr->nblk_total, blockIdx.x, unit, w.g)) return;
+        const int b = mv.blk_trace[unit.block], G = p.Hq / p.Hkv;
+        w.n = unit.block - mv.blk_off[b];
+        w.tok0 = mv.seq_start[b];
+        w.T = mv.seq_start[b + 1] - w.tok0;
+        w.m_first = mv.col_first[unit.block];           // == n unless the key slots were re-ordered
+        w.m_last = mv.col_last[unit.block];
+        w.general = mv.hdr->general != 0;
+        const int nm = w.m_last - w.m_first + 1;        // query blocks m_first .. m_last can see this key block
+        if (nm <= 0) {
+            // no query sees any key of the block (general metadata only): its gradients are zero
+            bwd_zero_rows<D>(p, w.tok0 + w.n * TILE, min(TILE, w.T - w.n * TILE), w.g);
+            return;
+        }
+        w.n_iter = (unit.tile1 < 0 ? G * nm : unit.tile1) - unit.tile0;     // of the G * nm (head, query block) tiles of the key block
+        w.h_start = w.g * G + unit.tile0 / nm;
+        w.m_start = w.m_first + unit.tile0 % nm;
+        w.cut = unit.cut;
     }
-
-    const int h_start = g * G + unit.tile0 / nm, m_start = m_first + unit.tile0 % nm;
+    int32_t* status = p.status;
 
     const uint32_t sraw = smem_u32(smem_raw);
     const uint32_t sbase = (sraw + 1023u) & ~1023u;
@@ -421,10 +423,14 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         tmem_alloc(smem_u32(s_tmem_base), TMEM_COLS);
         tmem_relinquish();
     }
+    if (tid == 0) *reinterpret_cast<BwdWork*>(sgen + L::OFF_WORK) = w;
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *s_tmem_base;
+    const volatile BwdWork* work = reinterpret_cast<const volatile BwdWork*>(sgen + L::OFF_WORK);
+    const int n = work->n, tok0 = work->tok0, T = work->T, m_first = work->m_first, m_last = work->m_last;
+    const int h_start = work->h_start, m_start = work->m_start, n_iter = work->n_iter, g = work->g;
     const uint32_t tmem_S = tmem;
     const uint32_t tmem_P = tmem + 128;
     const uint32_t tmem_dV = tmem + 256;
@@ -601,7 +607,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         const int kj = n * TILE + row;
         // queries [my_first, my_end) of the trace see this key; nobody sees a slot past the trace
         const int my_end = (kj < T) ? min(mv.evict[tok0 + kj], T) : 0;
-        const int my_first = (general && kj < T) ? mv.kfirst[tok0 + kj] : kj;
+        const int my_first = (work->general && kj < T) ? mv.kfirst[tok0 + kj] : kj;
         const float* sLse = reinterpret_cast<const float*>(sgen + L::OFF_LSE);
         const float* sDv = reinterpret_cast<const float*>(sgen + L::OFF_DVEC);
         uint8_t* sDS_row = sgen + L::OFF_DS + half * BOX_BYTES + row * 128;
@@ -696,7 +702,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         tc_fence_after();
         const bool kvalid = kj < T;
         const size_t orow = (size_t)(tok0 + kj) * (size_t)p.dkv_ts + (size_t)g * D + half * HALF_D;
-        bwd_epilogue<D>(p, unit.cut, g, 1, 0, tmem_dK + lane_sel + half * HALF_D, tmem_dV + lane_sel + half * HALF_D, row, half, kvalid, orow,
+        bwd_epilogue<D>(p, work->cut, g, 1, 0, tmem_dK + lane_sel + half * HALF_D, tmem_dV + lane_sel + half * HALF_D, row, half, kvalid, orow,
                         reinterpret_cast<volatile int*>(sgen + L::OFF_MISC + 8));
     }
     tc_fence_before();

@@ -17,6 +17,14 @@ struct BwdUnit {
     int32_t tile0, tile1;   // tiles [tile0, tile1) of its (head of the group, query block) list
     int32_t cut;            // 0: the whole item; else first slot << 18 | index of the unit << 9 | units of the item
 };
+// What the roles of a CTA need of its unit.  They read it from shared memory once they have parted: kept in registers from
+// before, it was spilled around their loops.
+struct BwdWork {
+    int n, tok0, T;                 // key block, first token and length of its trace
+    int m_first, m_last;            // query blocks of the item's list
+    int h_start, m_start, n_iter;   // first (head, query block) tile of the unit, number of tiles
+    int g, cut, general, pad;
+};
 struct BwdPlan {
     int32_t n_units;
     int32_t slots;          // slots used per KV head

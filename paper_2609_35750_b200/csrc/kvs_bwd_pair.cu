@@ -53,7 +53,8 @@ struct PairSmem {
     static constexpr int OFF_DVEC = OFF_LSE + 2 * TILE * 4;   // 2 stages x 128 fp32: -D * scale
     static constexpr int OFF_BAR = OFF_DVEC + 2 * TILE * 4;
     static constexpr int OFF_MISC = OFF_BAR + 20 * 8;     // tmem base, abort flag
-    static constexpr int TOTAL = OFF_MISC + 16;
+    static constexpr int OFF_WORK = OFF_MISC + 16;
+    static constexpr int TOTAL = OFF_WORK + (int)sizeof(BwdWork);
     static constexpr int MAX_DYN = 232448;                // 227 KB
     static constexpr int DYN_BYTES = (TOTAL + 1024 > MAX_DYN) ? MAX_DYN : TOTAL + 1024;
 };
@@ -146,30 +147,28 @@ bwd_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         if (tid == 0 && blockIdx.x == 0) set_status(p.status, KVS_ERR_BAD_META);
         return;
     }
-    BwdUnit unit;
-    int g;
-    if (!bwd_unit_of(p, mv.pair_order, mv.hdr->npair_total, blockIdx.x >> 1, unit, g)) return;
-    const int gb0 = unit.block;
-    const int G = p.Hq / p.Hkv;
-    const int b = mv.blk_trace[gb0];
-    const int n0 = gb0 - mv.blk_off[b];
-    const int n = n0 + (int)rank;                   // this CTA's key block; past the trace when its block count is odd
-    const int tok0 = mv.seq_start[b];
-    const int T = mv.seq_start[b + 1] - tok0;
-    const int nb = (T + TILE - 1) / TILE;
-    const bool exists = n < nb;
-    int m_first, m_last;
-    pair_range(mv.col_first, mv.col_last, gb0, n0 + 1 < nb, m_first, m_last);
-    const int nm = m_last - m_first + 1;            // query blocks m_first .. m_last can see one of the two key blocks
-    const int n_iter = (unit.tile1 < 0 ? G * nm : unit.tile1) - unit.tile0;     // tiles of this unit of the G * nm (head, query block) tiles of the pair
-    int32_t* status = p.status;
-    const bool general = mv.hdr->general != 0;
-    if (nm <= 0) {
-        if (exists) bwd_zero_rows<D>(p, tok0 + n * TILE, min(TILE, T - n * TILE), g);
-        return;
+    BwdWork w;
+    {
+        BwdUnit unit;
+        if (!bwd_unit_of(p, mv.pair_order, mv.hdr->npair_total, blockIdx.x >> 1, unit, w.g)) return;
+        const int b = mv.blk_trace[unit.block], G = p.Hq / p.Hkv;
+        const int n0 = unit.block - mv.blk_off[b];
+        w.n = n0 + (int)rank;                           // this CTA's key block; past the trace when its block count is odd
+        w.tok0 = mv.seq_start[b];
+        w.T = mv.seq_start[b + 1] - w.tok0;
+        pair_range(mv.col_first, mv.col_last, unit.block, (n0 + 1) * TILE < w.T, w.m_first, w.m_last);
+        w.general = mv.hdr->general != 0;
+        const int nm = w.m_last - w.m_first + 1;        // query blocks m_first .. m_last can see one of the two key blocks
+        if (nm <= 0) {
+            if (w.n * TILE < w.T) bwd_zero_rows<D>(p, w.tok0 + w.n * TILE, min(TILE, w.T - w.n * TILE), w.g);
+            return;
+        }
+        w.n_iter = (unit.tile1 < 0 ? G * nm : unit.tile1) - unit.tile0;     // of the G * nm (head, query block) tiles of the pair
+        w.h_start = w.g * G + unit.tile0 / nm;
+        w.m_start = w.m_first + unit.tile0 % nm;
+        w.cut = unit.cut;
     }
-
-    const int h_start = g * G + unit.tile0 / nm, m_start = m_first + unit.tile0 % nm;
+    int32_t* status = p.status;
 
     const uint32_t sraw = smem_u32(smem_raw);
     const uint32_t sbase = (sraw + 1023u) & ~1023u;
@@ -224,11 +223,15 @@ bwd_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         tmem_alloc_pair(smem_u32(s_tmem_base), TMEM_COLS);
         tmem_relinquish_pair();
     }
+    if (tid == 0) *reinterpret_cast<BwdWork*>(sgen + L::OFF_WORK) = w;
     tc_fence_before();
     __syncthreads();
     cluster_sync();                   // the other CTA's barriers and tensor memory are set up too
     tc_fence_after();
     const uint32_t tmem = *s_tmem_base;
+    const volatile BwdWork* work = reinterpret_cast<const volatile BwdWork*>(sgen + L::OFF_WORK);
+    const int n = work->n, tok0 = work->tok0, T = work->T, m_first = work->m_first, m_last = work->m_last;
+    const int h_start = work->h_start, m_start = work->m_start, n_iter = work->n_iter, g = work->g;
     const uint32_t tmem_S = tmem;
     const uint32_t tmem_dQ = tmem + 32;
     const uint32_t tmem_P = tmem + 128;
@@ -257,15 +260,16 @@ bwd_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             if (expects) mbar_expect_tx(bar_kv, 6 * TB);
             if (lane == 0) {
                 // a key block past the end of the trace is read as zeros (a start past the last token is filled)
-                const int tok_own = exists ? tok0 + n * TILE : p.total_tokens;
+                const int tok_own = n * TILE < T ? tok0 + n * TILE : p.total_tokens;
                 for (int c = 0; c < 2; ++c) tma_load_pair(sK + c * BOX, &tm_k, c * 64, g, tok_own, l_kv);
             }
             rows_of(sQR, &tm_q, h, m, bar_qr, l_qr);
             if (lane == 0) {
-                const int tok_own = exists ? tok0 + n * TILE : p.total_tokens;
+                const int tok_own = n * TILE < T ? tok0 + n * TILE : p.total_tokens;
                 for (int c = 0; c < 2; ++c) tma_load_pair(sV + c * BOX, &tm_v, c * 64, g, tok_own, l_kv);
+                const int n0 = n - (int)rank;
                 for (int c = 0; c < 2; ++c)
-                    tma_load_pair(sKC + c * BOX, &tm_k, row0, g, n0 + c < nb ? tok0 + (n0 + c) * TILE : p.total_tokens, l_kv);
+                    tma_load_pair(sKC + c * BOX, &tm_k, row0, g, (n0 + c) * TILE < T ? tok0 + (n0 + c) * TILE : p.total_tokens, l_kv);
             }
             rows_of(sDOR, &tm_do, h, m, bar_dor, l_dor);
             cols_of(sDOC, &tm_do, h, m, bar_doc, l_doc);
@@ -469,7 +473,7 @@ bwd_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         const int kj = n * TILE + row;
         // queries [my_first, my_end) of the trace see this key; nobody sees a slot past the trace
         const int my_end = (kj < T) ? min(mv.evict[tok0 + kj], T) : 0;
-        const int my_first = (general && kj < T) ? mv.kfirst[tok0 + kj] : kj;
+        const int my_first = (work->general && kj < T) ? mv.kfirst[tok0 + kj] : kj;
         const float* sLse = reinterpret_cast<const float*>(sgen + L::OFF_LSE);
         const float* sDv = reinterpret_cast<const float*>(sgen + L::OFF_DVEC);
         // dS^T of this key for queries col0 .. col0+63, a 128-byte row: in place, or on its way to the CTA that owns these queries
@@ -595,7 +599,7 @@ bwd_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         tc_fence_after();
         const bool kvalid = kj < T;
         const size_t orow = (size_t)(tok0 + kj) * (size_t)p.dkv_ts + (size_t)g * D + half * 64;
-        bwd_epilogue<D>(p, unit.cut, g, 2, (int)rank, tmem_dK + lane_sel + half * 64, tmem_dV + lane_sel + half * 64, row, half, kvalid, orow,
+        bwd_epilogue<D>(p, work->cut, g, 2, (int)rank, tmem_dK + lane_sel + half * 64, tmem_dV + lane_sel + half * 64, row, half, kvalid, orow,
                         reinterpret_cast<volatile int*>(sgen + L::OFF_MISC + 8));
     }
     tc_fence_before();
