@@ -81,13 +81,14 @@ __device__ void bwd_plan(const BwdPlanArgs& a) {
     const int32_t* all_len = a.pairs ? a.all.pair_len : a.all.bwd_len;
     const int32_t* len = a.pairs ? a.mv.pair_len : a.mv.bwd_len;
     const int32_t* order = a.pairs ? a.mv.pair_order : a.mv.bwd_order;
-    // this thread's first item, read beside the headers (the arrays have room for `cap` entries, with or without a value yet)
-    const int all_len0 = tid < a.all_cap ? all_len[tid] : 0;
-    const int len0 = tid < a.cap ? len[tid] : 0, order0 = tid < a.cap ? order[tid] : 0;
     if (!meta_matches(all, a.all_batch, a.all_tokens, a.all_maxlen) || !meta_matches(part, a.batch, a.tokens, a.maxlen)) {
         if (tid == 0) a.plan->n_units = a.plan->n_heavy = 0;
         return;
     }
+    // this thread's first item, on its way while the candidates are set up (the arrays have room for `cap` entries, with or
+    // without a value yet)
+    const int all_len0 = tid < a.all_cap ? all_len[tid] : 0;
+    const int len0 = tid < a.cap ? len[tid] : 0, order0 = tid < a.cap ? order[tid] : 0;
     const int n_all = a.pairs ? all->npair_total : all->nblk_total, n = a.pairs ? part->npair_total : part->nblk_total;
     const int most = max(a.G * (a.pairs ? all->pair_most : all->blk_most), 1);
     const int sms = a.pairs ? BWD_SMS / 2 : BWD_SMS;
