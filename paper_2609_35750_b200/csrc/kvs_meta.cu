@@ -163,7 +163,10 @@ meta_blocks_kernel(const int32_t* __restrict__ evict_at, const int32_t* __restri
 // 900 tokens: step 955 -> 894 us; 12 traces of 1500 to 12000 tokens with exact short lengths: 8274 -> 8678 us).
 enum { ORDER_ROWS, ORDER_COLS, ORDER_PAIRS };
 constexpr int ORDER_BINS = 4096;
-constexpr int ORDER_CACHED = 12288;        // lengths kept in shared memory between the passes (16 bits each)
+constexpr int ORDER_CACHED = 12288;        // lengths kept in shared memory between the passes
+// A kept length has 16 bits.  Two of its values stand for something else: a block that is not an item, and a length that they
+// leave no room for (65534 and 65535 blocks, the longest traces there are), which is looked up again.
+constexpr int ORDER_NONE = 0xffff, ORDER_LONG = 0xfffe;
 
 __device__ void meta_order(int what, MetaHeader* hdr, const int32_t* blk_off, const int32_t* blk_trace, const int32_t* row_cnt,
                            const int32_t* col_first, const int32_t* col_last, int32_t* order, int32_t* len_out) {
@@ -175,13 +178,13 @@ __device__ void meta_order(int what, MetaHeader* hdr, const int32_t* blk_off, co
     const int n = hdr->nblk_total;
     const bool exact = hdr->max_seqlen <= 16 * TILE;
     const int nbins = exact ? 17 : min((hdr->max_seqlen / TILE >> 4) + 2, ORDER_BINS);
-    auto length = [&](int i) {              // 0xffff: not an item of its own
+    auto length = [&](int i) {              // -1: not an item of its own
         if (what == ORDER_ROWS) return __ldcg(row_cnt + i);
         if (what == ORDER_COLS) return max(col_last[i] - col_first[i] + 1, 0);
         const int b = blk_trace[i], lo = blk_off[b], hi = blk_off[b + 1];
         int first, last;
         pair_range(col_first, col_last, i, i + 1 < hi, first, last);
-        return ((i - lo) & 1) ? 0xffff : max(last - first + 1, 0);
+        return ((i - lo) & 1) ? -1 : max(last - first + 1, 0);
     };
     auto bin = [&](int len) { return nbins - 1 - min(exact ? len : len >> 4, nbins - 1); };      // the longest first
     for (int i = tid; i < nbins; i += META_THREADS) bins[i] = 0;
@@ -194,8 +197,8 @@ __device__ void meta_order(int what, MetaHeader* hdr, const int32_t* blk_off, co
     int most = 0;
     for (int i = tid; i < n; i += META_THREADS) {
         const int len = length(i);
-        if (i < ORDER_CACHED) cached[i] = (uint16_t)len;
-        if (len == 0xffff) continue;
+        if (i < ORDER_CACHED) cached[i] = (uint16_t)(len < 0 ? ORDER_NONE : min(len, ORDER_LONG));
+        if (len < 0) continue;
         atomicAdd(&bins[bin(len)], 1);
         sum += len;
         most = max(most, len);
@@ -224,8 +227,12 @@ __device__ void meta_order(int what, MetaHeader* hdr, const int32_t* blk_off, co
     __syncwarp();
     for (int i0 = 0; i0 < n; i0 += 32) {
         const int i = i0 + lane;
-        const int len = i < n ? (i < ORDER_CACHED ? (int)cached[i] : length(i)) : 0xffff;
-        const int k = len == 0xffff ? -1 : bin(len);
+        int len = -1;
+        if (i < n) {
+            len = i < ORDER_CACHED ? (int)cached[i] : ORDER_LONG;
+            len = len == ORDER_NONE ? -1 : len == ORDER_LONG ? length(i) : len;
+        }
+        const int k = len < 0 ? -1 : bin(len);
         const unsigned same = __match_any_sync(0xffffffffu, k);
         if (k >= 0) {
             const int at = bins[k] + __popc(same & ((1u << lane) - 1u));
