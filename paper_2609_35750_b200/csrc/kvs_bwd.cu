@@ -730,7 +730,7 @@ template <int D>
 static int launch_main(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tdo, const CUtensorMap& tdq,
                        const MetaView& mv, const BwdParams& p, unsigned units, cudaStream_t st) {
     auto kern = bwd_kernel<D>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdSmem<D>::DYN_BYTES) != cudaSuccess) return KVS_ERR_CUDA;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdSmem<D>::DYN_BYTES) != cudaSuccess) return cuda_refused();
     return launch_after(kern, units, BWD_THREADS, BwdSmem<D>::DYN_BYTES, st, tq, tk, tv, tdo, tdq, mv, p);
 }
 

@@ -616,7 +616,7 @@ bwd_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
 int launch_bwd_pair(const CUtensorMap& q64, const CUtensorMap& k, const CUtensorMap& v, const CUtensorMap& do64, const CUtensorMap& dq64,
                     const MetaView& mv, const BwdParams& p, unsigned units, cudaStream_t st) {
     if (cudaFuncSetAttribute(bwd_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PairSmem::DYN_BYTES) != cudaSuccess)
-        return KVS_ERR_CUDA;
+        return cuda_refused();
     return launch_after(bwd_pair_kernel, 2 * units, BWD_THREADS, PairSmem::DYN_BYTES, st, q64, k, v, do64, dq64, mv, p);
 }
 

@@ -151,6 +151,13 @@ int make_tmap_f32_thd(CUtensorMap* map, const void* base, int total_tokens, int 
 int make_tmap_rows(CUtensorMap* map, const void* base, int rows, int cols);
 int check_device_sm100();
 
+// A refused call leaves no error behind: the runtime keeps the last one until it is asked for, and the next check after a
+// plain launch would report it.
+inline int cuda_refused() {
+    cudaGetLastError();
+    return KVS_ERR_CUDA;
+}
+
 #ifdef __CUDACC__
 template <typename... P, typename... A>
 inline int launch_after(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A&&... args) {
@@ -164,7 +171,7 @@ inline int launch_after(void (*kernel)(P...), dim3 grid, int threads, size_t sme
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...) == cudaSuccess ? KVS_OK : KVS_ERR_CUDA;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...) == cudaSuccess ? KVS_OK : cuda_refused();
 }
 #endif
 

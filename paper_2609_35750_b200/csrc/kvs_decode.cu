@@ -904,7 +904,7 @@ extern "C" int kvs_cache_evict(const int32_t* ranges, int n_ranges, int num_seqs
     const size_t smem = (size_t)max_pages * sizeof(int32_t);
     if (smem > 48 * 1024 &&
         cudaFuncSetAttribute(cache_evict_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return KVS_ERR_CUDA;
+        return cuda_refused();
     return launch_after(cache_evict_kernel, num_seqs, 256, smem, (cudaStream_t)stream, ranges, n_ranges, num_seqs, page_size, max_pages,
                         num_pages, block_table, n_tokens, free_list);
 }
@@ -956,7 +956,7 @@ __global__ void decode_header_kernel(int32_t* hdr, int32_t* arrived, int n) {
 template <int G, int LOAD>
 static int launch_decode_tc(const CUtensorMap& tk, const CUtensorMap& tv, const DecodeParams& p, int32_t* status, cudaStream_t st) {
     auto kern = decode_tc_kernel<G, LOAD>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, DtcSmem::DYN_BYTES) != cudaSuccess) return KVS_ERR_CUDA;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, DtcSmem::DYN_BYTES) != cudaSuccess) return cuda_refused();
     dim3 grid(p.nsplit, p.Hkv, p.S);
     return launch_after(kern, grid, DTC_THREADS, DtcSmem::DYN_BYTES, st, tk, tv, p, status);
 }

@@ -679,7 +679,7 @@ template <int D, bool CHAIN>
 static int launch_fwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const MetaView& mv, const FwdParams& p,
                       int nb_cap, cudaStream_t st) {
     auto kern = fwd_kernel<D, CHAIN>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem<D>::DYN_BYTES) != cudaSuccess) return KVS_ERR_CUDA;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem<D>::DYN_BYTES) != cudaSuccess) return cuda_refused();
     return launch_after(kern, dim3(nb_cap, p.heads, 1), FWD_THREADS, FwdSmem<D>::DYN_BYTES, st, tq, tk, tv, mv, p);
 }
 
