@@ -935,10 +935,14 @@ extern "C" int kvs_decode_num_splits(int num_seqs, int Hkv, int max_tokens) {
     return (int)best;
 }
 
+// header and partial results; the arrival counts (at most one per query head) follow
+static size_t decode_base_bytes(int num_seqs, int Hq, int head_dim, int num_splits) {
+    return DEC_WS_HEADER + align_up(sizeof(float) * (size_t)num_seqs * Hq * num_splits * (head_dim + 2), 256);
+}
+
 extern "C" size_t kvs_decode_workspace_bytes(int num_seqs, int Hq, int head_dim, int num_splits) {
     if (num_seqs < 0 || Hq <= 0 || head_dim <= 0 || num_splits <= 0) return 0;
-    return DEC_WS_HEADER + align_up(sizeof(float) * (size_t)num_seqs * Hq * num_splits * (head_dim + 2), 256) +
-           align_up(sizeof(int32_t) * (size_t)num_seqs * Hq, 256);       // arrival counts, at most one per query head
+    return decode_base_bytes(num_seqs, Hq, head_dim, num_splits) + align_up(sizeof(int32_t) * (size_t)num_seqs * Hq, 256);
 }
 
 // the first 256 bytes of the workspace: {magic, status} as in the backward workspace, so that
@@ -1032,7 +1036,8 @@ extern "C" int kvs_decode_attn(const void* q, const void* k_cache, const void* v
     if (!q || !k_cache || !v_cache || !block_table || !n_tokens || !out || !lse || !workspace) return KVS_ERR_INVALID_ARG;
     if ((((uintptr_t)q | (uintptr_t)k_cache | (uintptr_t)v_cache | (uintptr_t)out) & 15) != 0 || ((uintptr_t)workspace & 255) != 0)
         return KVS_ERR_ALIGNMENT;
-    if (workspace_bytes < kvs_decode_workspace_bytes(num_seqs, Hq, head_dim, num_splits)) return KVS_ERR_WORKSPACE;
+    const size_t base = decode_base_bytes(num_seqs, Hq, head_dim, num_splits);
+    if (workspace_bytes < base) return KVS_ERR_WORKSPACE;
     if (softmax_scale < 0.f || softmax_scale != softmax_scale) return KVS_ERR_INVALID_ARG;
     DecodeParams p;
     p.q = (const __nv_bfloat16*)q;
@@ -1054,12 +1059,13 @@ extern "C" int kvs_decode_attn(const void* q, const void* k_cache, const void* v
     p.part_o = (float*)((char*)workspace + DEC_WS_HEADER);
     p.part_ml = p.part_o + (size_t)num_seqs * Hq * num_splits * head_dim;
     cudaStream_t st = (cudaStream_t)stream;
-    p.arrived = (int32_t*)((char*)workspace + DEC_WS_HEADER + align_up(sizeof(float) * (size_t)num_seqs * Hq * num_splits * (head_dim + 2), 256));
+    p.arrived = (int32_t*)((char*)workspace + base);
     p.out = (__nv_bfloat16*)out;
     p.lse = lse;
-    // three CTAs per SM are resident: up to two waves of them merge on their own
+    // three CTAs per SM are resident: up to two waves of them merge on their own, if the workspace has room for their counts
     const int rows = num_seqs * Hkv;
-    if ((long long)rows * num_splits > 2 * 3 * 148) p.arrived = nullptr;
+    if ((long long)rows * num_splits > 2 * 3 * 148 || workspace_bytes < kvs_decode_workspace_bytes(num_seqs, Hq, head_dim, num_splits))
+        p.arrived = nullptr;
     const int rc = launch_after(decode_header_kernel, p.arrived ? (rows + 255) / 256 : 1, 256, 0, st, (int32_t*)workspace, p.arrived, p.arrived ? rows : 0);
     if (rc != KVS_OK) return rc;
     int32_t* status = (int32_t*)workspace + 1;
