@@ -46,7 +46,7 @@ struct FwdSmem {
     static constexpr int OFF_KV = 2 * TB;                // 2 stages x (K, V)
     static constexpr int OFF_EV = OFF_KV + 4 * TB;       // 2 stages x 128 int32: eviction step of the stage's key slots
     static constexpr int OFF_KF = OFF_EV + 2 * TILE * 4; // 2 stages x 128 int32: first query that may see the slot
-    static constexpr int OFF_FLAG = OFF_KF + 2 * TILE * 4;   // 2 stages x need_mask
+    static constexpr int OFF_FLAG = OFF_KF + 2 * TILE * 4;   // 2 stages x (compare, hidden)
     static constexpr int OFF_BAR = OFF_FLAG + 16;
     static constexpr int OFF_ITEM = OFF_BAR + 32 * 8;    // 2 slots x FwdItem
     static constexpr int OFF_ASK = OFF_ITEM + 2 * 48;    // the answer of the launch control
@@ -259,27 +259,56 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
                     const uint32_t R = ring + i;
                     const int s = R & 1;
                     const int n = list[i];
-                    if (R >= 2) {
-                        mbar_wait(bar_vfree(s), ((R >> 1) + 1) & 1, abort_flag, status);
-                        mbar_wait(bar_evfree(s), ((R >> 1) + 1) & 1, abort_flag, status);
+                    const bool need_mask = (cls[n] != KVS_CLASS_FULL) || (n * TILE + TILE > T);
+                    // What the mask needs comes first: the softmax groups are done with the stage's last one well before its V is
+                    // free, and must not wait for that.
+                    int ev[4] = {0, 0, 0, 0}, kf[4] = {0, 0, 0, 0};       // the intervals of the tile's key slots
+                    if (need_mask) {
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const int j = n * TILE + lane * 4 + u;
+                            ev[u] = (j < T) ? mv.evict[tok0 + j] : 0;                       // 0: visible to nobody
+                            kf[u] = (general && j < T) ? mv.kfirst[tok0 + j] : j;
+                        }
                     }
+                    // What a softmax warp (32 rows, quadrant q) has to do for the keys 32 c .. 32 c + 31: bit 8 c + q of `hidden`:
+                    // none of its rows sees any of them; else bit 8 c + q of `compare`: some key is evicted before the last row,
+                    // bit 8 c + 4 + q: some key is not there yet for the first row.  Found here, beside the loads: votes by the
+                    // softmax warps, with both comparisons where a group was mixed, took 13 % of a forward whose tiles all are
+                    // (24576 tokens, token-level eviction: 11.1 -> 9.2 ms).
+                    uint32_t compare = 0, hidden = 0;
+                    if (need_mask) {
+                        int ev0 = min(min(ev[0], ev[1]), min(ev[2], ev[3])), ev1 = max(max(ev[0], ev[1]), max(ev[2], ev[3]));
+                        int kf0 = min(min(kf[0], kf[1]), min(kf[2], kf[3])), kf1 = max(max(kf[0], kf[1]), max(kf[2], kf[3]));
+#pragma unroll
+                        for (int o = 1; o < 8; o <<= 1) {                 // over the 8 lanes with the group's keys
+                            ev0 = min(ev0, __shfl_xor_sync(0xffffffffu, ev0, o));
+                            ev1 = max(ev1, __shfl_xor_sync(0xffffffffu, ev1, o));
+                            kf0 = min(kf0, __shfl_xor_sync(0xffffffffu, kf0, o));
+                            kf1 = max(kf1, __shfl_xor_sync(0xffffffffu, kf1, o));
+                        }
+                        const int q_lo = m * TILE + (lane & 3) * 32, q_hi = q_lo + 31;
+                        const bool none = kf0 > q_hi || ev1 <= q_lo;
+                        hidden = __ballot_sync(0xffffffffu, none);
+                        compare = __ballot_sync(0xffffffffu, !none && ((lane & 4) ? kf1 > q_lo : ev0 <= q_hi));
+                    }
+                    if (R >= 2) mbar_wait(bar_evfree(s), ((R >> 1) + 1) & 1, abort_flag, status);
+                    if (need_mask) {
+                        *reinterpret_cast<int4*>(sEv + s * TILE + lane * 4) = make_int4(ev[0], ev[1], ev[2], ev[3]);
+                        *reinterpret_cast<int4*>(sKf + s * TILE + lane * 4) = make_int4(kf[0], kf[1], kf[2], kf[3]);
+                    }
+                    if (lane == 0) {
+                        sFlag[2 * s] = (int32_t)compare;
+                        sFlag[2 * s + 1] = (int32_t)hidden;
+                    }
+                    mbar_arrive(bar_evfull(s));
+                    if (R >= 2) mbar_wait(bar_vfree(s), ((R >> 1) + 1) & 1, abort_flag, status);
                     if (lane == 0) {
                         mbar_expect_tx(bar_vfull(s), L::TB);
                         const uint32_t dst = sKV + s * 2 * L::TB;
                         for (int c = 0; c < NBOX; ++c) tma_load_3d(dst + L::TB + c * BOX_BYTES, &tm_v, c * 64, g, tok0 + n * TILE, bar_vfull(s));
                     }
                     if (i + 1 < nlist) load_k(i + 1);
-                    const bool need_mask = (cls[n] != KVS_CLASS_FULL) || (n * TILE + TILE > T);
-                    if (need_mask) {
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            const int j = n * TILE + lane * 4 + u;
-                            sEv[s * TILE + lane * 4 + u] = (j < T) ? mv.evict[tok0 + j] : 0;   // 0: visible to nobody
-                            sKf[s * TILE + lane * 4 + u] = (general && j < T) ? mv.kfirst[tok0 + j] : j;
-                        }
-                    }
-                    if (lane == 0) sFlag[s] = need_mask ? 1 : 0;
-                    mbar_arrive(bar_evfull(s));
                 }
                 if (nlist > 0) {
                     ring += nlist;
@@ -434,7 +463,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         const uint32_t lane_sel = (uint32_t)(quad * 32) << 16;
         const uint32_t tmem_S = tmem + t * 128 + lane_sel;
         const uint32_t tmem_O = tmem + 256 + t * 128 + lane_sel;
-        uint32_t ring = 0, s_phase = 0;                           // key blocks of the CTA so far; phase of this group's next S
+        uint32_t ring = 0, s_count = 0;                           // key blocks of the CTA, S tiles of this group so far
         int items = 0, singles = 0;                               // items with key blocks, those of a single head
         for (int r = 0; CHAIN || r == 0; ++r) {
             int nlist, m, T, tok0, h0, ntile;
@@ -448,13 +477,16 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
             float run_sum = 0.f;
 
             const uint32_t first = ring + (dual ? t : 0), stride = dual ? 2 : 1;
+            // The phase of this group's S follows from the key block's number, up to a constant of the item.  As a bit that every
+            // tile flips it cost 1 % of a long row (3 traces of 9000 to 17000 tokens, nothing evicted: 3.39 -> 3.35 ms).
+            const uint32_t s_shift = dual ? 1 : 0, s_off = CHAIN ? s_count - (first >> s_shift) : 0;
             ring += nlist;
+            if (CHAIN && ring > first) s_count += (ring - first + stride - 1) >> s_shift;
             for (uint32_t R = first; R < ring; R += stride) {
                 const int s = R & 1;
                 mbar_wait(bar_evfull(s), (R >> 1) & 1, abort_flag, status);
-                const bool need_mask = sFlag[s] != 0;
-                mbar_wait(bar_s(t), s_phase, abort_flag, status);
-                s_phase ^= 1;
+                const uint32_t compare = (uint32_t)sFlag[2 * s] >> quad, hidden = (uint32_t)sFlag[2 * s + 1] >> quad;
+                mbar_wait(bar_s(t), ((R >> s_shift) + s_off) & 1, abort_flag, status);
                 tc_fence_after();
                 // raw logits of this row (the softmax scale is positive, so the maximum can be taken before it)
                 float sv[TILE];
@@ -473,33 +505,38 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
                         sv[96 + e] = __uint_as_float(r3[e]);
                     }
                 }
-                if (need_mask) {
-                    // Per warp and 32 keys: seen by all of the warp's 32 rows (nothing to do), hidden from all of them, or
-                    // neither.  Only the last kind is decided element by element.  On a diagonal tile that is one of a warp's
-                    // four groups, where a span of turns leaves it is the warps that its step falls into.
-                    const int q_lo = m * TILE + quad * 32, q_hi = q_lo + 31;
+                if (((compare | hidden) & 0x11111111u) != 0) {
 #pragma unroll
                     for (int c = 0; c < 4; ++c) {
-                        const int kev = sEv[s * TILE + c * 32 + lane], kfirst = sKf[s * TILE + c * 32 + lane];
-                        const bool seen = __all_sync(0xffffffffu, kfirst <= q_lo && q_hi < kev);
-                        const bool hidden = __all_sync(0xffffffffu, kfirst > q_hi || kev <= q_lo);
-                        if (hidden) {
+                        if (hidden >> (8 * c) & 1u) {
 #pragma unroll
                             for (int e = 0; e < 32; ++e) sv[c * 32 + e] = -INFINITY;
                         }
-                        const int mixed = (seen || hidden) ? 0 : 1;
+                        const int by_end = compare >> (8 * c) & 1u, by_start = compare >> (8 * c + 4) & 1u;
 #pragma unroll 1
-                        for (int pass = 0; pass < mixed; ++pass) {          // a loop of at most one pass: not predicated
+                        for (int pass = 0; pass < by_end; ++pass) {          // loops of at most one pass: not predicated
                             const int4* ev4 = reinterpret_cast<const int4*>(sEv + s * TILE + c * 32);
+#pragma unroll
+                            for (int e4 = 0; e4 < 8; ++e4) {
+                                const int4 ev = ev4[e4];
+                                float* x = sv + c * 32 + e4 * 4;
+                                x[0] = (qi < ev.x) ? x[0] : -INFINITY;
+                                x[1] = (qi < ev.y) ? x[1] : -INFINITY;
+                                x[2] = (qi < ev.z) ? x[2] : -INFINITY;
+                                x[3] = (qi < ev.w) ? x[3] : -INFINITY;
+                            }
+                        }
+#pragma unroll 1
+                        for (int pass = 0; pass < by_start; ++pass) {
                             const int4* kf4 = reinterpret_cast<const int4*>(sKf + s * TILE + c * 32);
 #pragma unroll
                             for (int e4 = 0; e4 < 8; ++e4) {
-                                const int4 ev = ev4[e4], kf = kf4[e4];
+                                const int4 kf = kf4[e4];
                                 float* x = sv + c * 32 + e4 * 4;
-                                x[0] = ((kf.x <= qi) && (qi < ev.x)) ? x[0] : -INFINITY;
-                                x[1] = ((kf.y <= qi) && (qi < ev.y)) ? x[1] : -INFINITY;
-                                x[2] = ((kf.z <= qi) && (qi < ev.z)) ? x[2] : -INFINITY;
-                                x[3] = ((kf.w <= qi) && (qi < ev.w)) ? x[3] : -INFINITY;
+                                x[0] = (kf.x <= qi) ? x[0] : -INFINITY;
+                                x[1] = (kf.y <= qi) ? x[1] : -INFINITY;
+                                x[2] = (kf.z <= qi) ? x[2] : -INFINITY;
+                                x[3] = (kf.w <= qi) ? x[3] : -INFINITY;
                             }
                         }
                     }
