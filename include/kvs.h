@@ -368,9 +368,7 @@ int kvs_cache_evict(const int32_t* ranges, int n_ranges, int num_seqs, int page_
                     int32_t* block_table, int32_t* n_tokens, int32_t* free_list, kvs_stream_t stream);
 /* Reads the cache status word.  SYNCHRONISES the stream. */
 int kvs_cache_status(const int32_t* free_list, int* free_pages_host, kvs_stream_t stream);
-/* A split count that fills the GPU for this batch, and the workspace decode attention takes: header, partial results, and 4 bytes
- * per (sequence, query head) with which the splits of a small batch are merged without a further launch.  A workspace without room
- * for the last part is accepted. */
+/* A split count that fills the GPU for this batch, and the workspace decode attention needs. */
 int kvs_decode_num_splits(int num_seqs, int Hkv, int max_tokens);
 size_t kvs_decode_workspace_bytes(int num_seqs, int Hq, int head_dim, int num_splits);
 /*

@@ -9,7 +9,7 @@
 // reads exactly the pages the table names.  It never sees a mask.
 //
 // Decode attention is bound by HBM (every live K and V row is read once per step).  One of two kernels
-// produces per-split partial results, which the last CTA of a (sequence, KV head) to finish merges, or a third kernel:
+// produces per-split partial results, which a third merges:
 //   decode_partial_kernel  CUDA cores, organised around coalesced 256-byte row reads: one CTA per
 //                          (split, KV head, sequence); each half-warp reads one K (or V) row per load
 //                          instruction and serves all G query heads of the group from it;
@@ -33,17 +33,42 @@ struct DecodeParams {
     const int32_t* n_tokens;         // [S]
     int S, Hq, Hkv, page_size, max_pages, num_pages, nsplit;
     int page_shift;                  // log2(page_size) when it is a power of two, else -1
-    int32_t* status;                 // workspace status word: a page id outside [0, num_pages) is recorded there
+    int32_t* status;                 // in the kernels that form partial results: the CTA's own status word in shared memory
+    int32_t* header;                 // of the workspace: {magic, status}
     float scale_log2;
     float* part_o;                   // [S, Hq, nsplit, D] unnormalised
-    float* part_ml;                  // [S, Hq, nsplit, 2]  (max in base-2 units, sum)
-    int32_t* arrived;                // [S, Hkv] splits that have written their part
+    float* part_ml;                  // [S, Hq, nsplit, 2]  (max in base-2 units, sum; see flagged_sum)
     __nv_bfloat16* out;              // [S, Hq, D]
     float* lse;                      // [S, Hq]
 };
 
-// Merge of the splits of one (sequence, query head) by a warp: weights exp2(m_z - max), normalised, bf16 out and fp32 lse.
-template <int D>
+// The status of a call is gathered with its partial results, so that no launch of its own has to reset the workspace's word before
+// any CTA may write to it: a CTA that met an error (a bad page id, a wait that ran out) hands over its sums, which are never
+// negative, with the sign bit set and the kind in the lowest bit.  The first CTA writes {magic, OK}, the merge adds the errors.
+__device__ __forceinline__ float flagged_sum(float sum, int status) {
+    const uint32_t bits = __float_as_uint(sum) & 0x7fffffffu;
+    return __uint_as_float(status == KVS_OK ? bits : (bits & ~1u) | 0x80000000u | (status == KVS_ERR_TIMEOUT ? 1u : 0u));
+}
+__device__ __forceinline__ float sum_and_status(float flagged, int32_t* status) {
+    const uint32_t bits = __float_as_uint(flagged);
+    if (bits >> 31) set_status(status, bits & 1u ? KVS_ERR_TIMEOUT : KVS_ERR_INVALID_ARG);
+    return __uint_as_float(bits & 0x7fffffffu);
+}
+__device__ __forceinline__ void decode_header(const DecodeParams& p) {
+    if ((blockIdx.x | blockIdx.y | blockIdx.z | threadIdx.x) == 0) {
+        p.header[0] = (int32_t)WS_MAGIC;
+        p.header[1] = KVS_OK;
+    }
+}
+
+// Merge of the splits of a (sequence, query head) by a warp: weights exp2(m_z - max), normalised, bf16 out and fp32 lse.  Bound by
+// latency: the loads of PART splits are on their way before the first is used (16, with 4 at a time 47 splits took 5 us more);
+// where there are few splits, PART = 4 leaves room for three times the warps (100 sequences of 64 heads, one split: step 38.0 ->
+// 34.2 us).  A kernel of its own, started by programmatic dependent launch: merging in the last CTA of a (sequence, KV head) to
+// finish, with counts in the workspace, took a launch less but cost every CTA a fence and an atomic and the merge its parallelism
+// (a step in a CUDA graph, merge in the last CTA -> here, us: 1 x 24000 tokens with 8 heads on 1 29.6 -> 20.4, 1 x 2000 with 32
+// on 8 14.2 -> 13.8, 100 x 300 with 8 on 8 and head_dim 64 17.5 -> 13.7; launched one by one the two are within 1 us).
+template <int D, int PART>
 __device__ __forceinline__ void decode_merge_row(const DecodeParams& p, size_t row, int lane) {
     constexpr int PER = D / 32;
     const float2* ml = reinterpret_cast<const float2*>(p.part_ml) + row * p.nsplit;
@@ -59,18 +84,26 @@ __device__ __forceinline__ void decode_merge_row(const DecodeParams& p, size_t r
     for (int z0 = 0; z0 < p.nsplit; z0 += 32) {
         const float2 x = (z0 + lane < p.nsplit) ? __ldcg(ml + z0 + lane) : make_float2(-INFINITY, 0.f);
         const float w = fast_exp2(x.x - Mu);
-        L += x.y * w;
-        const int n = min(32, p.nsplit - z0);
-#pragma unroll 4
-        for (int i = 0; i < n; ++i) {
-            const float wi = __shfl_sync(0xffffffffu, w, i);
-            const float* src = po + (size_t)(z0 + i) * D;
-            if constexpr (PER == 4) {
-                const float4 v = __ldcg(reinterpret_cast<const float4*>(src));
-                acc[0] += v.x * wi; acc[1] += v.y * wi; acc[2] += v.z * wi; acc[3] += v.w * wi;
-            } else {
-                const float2 v = __ldcg(reinterpret_cast<const float2*>(src));
-                acc[0] += v.x * wi; acc[1] += v.y * wi;
+        L += sum_and_status(x.y, p.header + 1) * w;
+        for (int i0 = 0; i0 < min(32, p.nsplit - z0); i0 += PART) {
+            float v[PART][PER];
+#pragma unroll
+            for (int i = 0; i < PART; ++i) {
+                const float* src = po + (size_t)(z0 + i0 + i) * D;
+                const bool there = z0 + i0 + i < p.nsplit;
+                if constexpr (PER == 4) {
+                    const float4 y = there ? __ldcg(reinterpret_cast<const float4*>(src)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    v[i][0] = y.x; v[i][1] = y.y; v[i][2] = y.z; v[i][3] = y.w;
+                } else {
+                    const float2 y = there ? __ldcg(reinterpret_cast<const float2*>(src)) : make_float2(0.f, 0.f);
+                    v[i][0] = y.x; v[i][1] = y.y;
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < PART; ++i) {
+                const float wi = __shfl_sync(0xffffffffu, w, i0 + i);
+#pragma unroll
+                for (int e = 0; e < PER; ++e) acc[e] += v[i][e] * wi;
             }
         }
     }
@@ -85,27 +118,11 @@ __device__ __forceinline__ void decode_merge_row(const DecodeParams& p, size_t r
         *reinterpret_cast<uint32_t*>(p.out + row * D + lane * PER) = pack_bf16(acc[0], acc[1]);
     if (lane == 0) p.lse[row] = (L > 0.f) ? M * 0.6931471805599453f + logf(L) : -INFINITY;
 }
-
-// ... by the CTA that is the last of its (sequence, KV head) to have written its part, where the call wants it so
-// (p.arrived): a launch less, 23.9 -> 21.4 us for a step on a few thousand tokens.  The CTA has to wait until its part is visible,
-// which in a grid of several waves costs what the launch does (20 sequences, 28 heads on 4: 50.5 and 52.1 us): there
-// decode_merge_kernel does it.
-template <int D, int G>
-__device__ __forceinline__ void decode_merge_if_last(const DecodeParams& p, int s, int g, int tid, volatile int* s_last) {
-    if (!p.arrived) return;
-    __threadfence();
-    named_bar_sync(1, 128);
-    if (tid == 0) *s_last = atomicAdd(&p.arrived[s * p.Hkv + g], 1) == p.nsplit - 1;
-    named_bar_sync(1, 128);
-    if (!*s_last) return;
-    __threadfence();
-    for (int h = tid >> 5; h < G; h += 4) decode_merge_row<D>(p, (size_t)s * p.Hq + g * G + h, tid & 31);
-}
-template <int D>
+template <int D, int PART>
 __global__ void __launch_bounds__(256) decode_merge_kernel(DecodeParams p) {
     pdl_wait();
     const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (row < p.S * p.Hq) decode_merge_row<D>(p, row, threadIdx.x & 31);
+    if (row < p.S * p.Hq) decode_merge_row<D, PART>(p, row, threadIdx.x & 31);
 }
 
 // A block-table entry is only followed if it names a page of the cache: anything else (a stale or
@@ -154,7 +171,12 @@ decode_partial_kernel(DecodeParams p) {
     constexpr int CH = D / 16;                  // elements of a row per lane (16 lanes per row): 8 or 4
     constexpr int ROWS = (G > 4) ? 4 : 8;       // rows per half-warp per block (register budget)
     constexpr int BLK = 2 * ROWS;               // tokens per softmax update
+    __shared__ int32_t s_status;
+    p.status = &s_status;
+    if (threadIdx.x == 0) s_status = KVS_OK;
     pdl_wait();
+    decode_header(p);
+    __syncthreads();
     const int z = blockIdx.x, g = blockIdx.y, s = blockIdx.z;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int half = lane >> 4, l16 = lane & 15;
@@ -301,11 +323,9 @@ decode_partial_kernel(DecodeParams p) {
         p.part_o[base * D + c] = o;
         if (c == 0) {
             p.part_ml[base * 2 + 0] = M;
-            p.part_ml[base * 2 + 1] = L;
+            p.part_ml[base * 2 + 1] = flagged_sum(L, s_status);
         }
     }
-    __shared__ int s_last;
-    decode_merge_if_last<D, G>(p, s, g, tid, &s_last);
 }
 
 // ---- tensor-core variant (head_dim 128) ------------------------------------------------------------
@@ -341,7 +361,7 @@ struct DtcSmem {
     static constexpr int OFF_Q = 65536;                // [16 x 128] bf16, two boxes of [16 x 64]
     static constexpr int OFF_P = 65536 + 4096;         // P^T as [16 heads x 128 keys] bf16, two boxes of [16 x 64]
     static constexpr int OFF_BAR = 65536 + 8192;       // 8 mbarriers
-    static constexpr int OFF_MISC = OFF_BAR + 64;      // tmem base, abort flag
+    static constexpr int OFF_MISC = OFF_BAR + 64;      // tmem base, abort flag, status
     static constexpr int OFF_WMAX = OFF_MISC + 64;     // [2 buffers][4 warps][16] fp32
     static constexpr int OFF_WSUM = OFF_WMAX + 512;    // [4 warps][16] fp32
     static constexpr int TOTAL = OFF_WSUM + 256;
@@ -366,7 +386,7 @@ __device__ __forceinline__ void tma_gather4(uint32_t dst, const CUtensorMap* map
 
 template <int G, int LOAD>
 __global__ void __launch_bounds__(DTC_THREADS, 3)
-decode_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v, DecodeParams p, int32_t* status) {
+decode_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v, DecodeParams p) {
     constexpr int D = 128;
     constexpr int BOX = 16384;                  // one 64-column box of a 128-row tile
     constexpr uint32_t IDESC_S = make_idesc(16, 0, 0);
@@ -376,6 +396,7 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
     const int z = blockIdx.x, g = blockIdx.y, s = blockIdx.z;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     pdl_wait();
+    decode_header(p);
     const int n = min(max(p.n_tokens[s], 0), p.max_pages * p.page_size);    // never past the sequence's table
     const int ps = p.page_size;
     const int ppt = 128 / ps;                                   // pages per tile (PAGES)
@@ -395,11 +416,14 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
     const uint32_t bar_kfull = bars, bar_vfull = bars + 8, bar_s = bars + 16, bar_p = bars + 24, bar_done = bars + 32;
     uint32_t* s_tmem = reinterpret_cast<uint32_t*>(sgen + DtcSmem::OFF_MISC);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(sgen + DtcSmem::OFF_MISC + 4);
+    int32_t* status = reinterpret_cast<int32_t*>(sgen + DtcSmem::OFF_MISC + 8);
+    p.status = status;
     float* s_wmax = reinterpret_cast<float*>(sgen + DtcSmem::OFF_WMAX);
     float* s_wsum = reinterpret_cast<float*>(sgen + DtcSmem::OFF_WSUM);
 
     if (tid == 0) {
         *abort_flag = 0;
+        *status = KVS_OK;
         mbar_init(bar_kfull, 1);
         mbar_init(bar_vfull, 1);
         mbar_init(bar_s, 1);
@@ -679,10 +703,9 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
             if (tid == h) {
                 const size_t base = ((size_t)s * p.Hq + g * G + h) * p.nsplit + z;
                 p.part_ml[base * 2 + 0] = m_run[h];
-                p.part_ml[base * 2 + 1] = s_wsum[h] + s_wsum[16 + h] + s_wsum[32 + h] + s_wsum[48 + h];
+                p.part_ml[base * 2 + 1] = flagged_sum(s_wsum[h] + s_wsum[16 + h] + s_wsum[32 + h] + s_wsum[48 + h], *(volatile int32_t*)status);
             }
         }
-        decode_merge_if_last<D, G>(p, s, g, tid, reinterpret_cast<volatile int*>(sgen + DtcSmem::OFF_MISC + 8));
     }
     tc_fence_before();
     __syncthreads();
@@ -935,38 +958,23 @@ extern "C" int kvs_decode_num_splits(int num_seqs, int Hkv, int max_tokens) {
     return (int)best;
 }
 
-// header and partial results; the arrival counts (at most one per query head) follow
-static size_t decode_base_bytes(int num_seqs, int Hq, int head_dim, int num_splits) {
+// the first 256 bytes of the workspace: {magic, status} as in the backward workspace, so that
+// kvs_device_status() reads it; the partial results follow
+extern "C" size_t kvs_decode_workspace_bytes(int num_seqs, int Hq, int head_dim, int num_splits) {
+    if (num_seqs < 0 || Hq <= 0 || head_dim <= 0 || num_splits <= 0) return 0;
     return DEC_WS_HEADER + align_up(sizeof(float) * (size_t)num_seqs * Hq * num_splits * (head_dim + 2), 256);
 }
 
-extern "C" size_t kvs_decode_workspace_bytes(int num_seqs, int Hq, int head_dim, int num_splits) {
-    if (num_seqs < 0 || Hq <= 0 || head_dim <= 0 || num_splits <= 0) return 0;
-    return decode_base_bytes(num_seqs, Hq, head_dim, num_splits) + align_up(sizeof(int32_t) * (size_t)num_seqs * Hq, 256);
-}
-
-// the first 256 bytes of the workspace: {magic, status} as in the backward workspace, so that
-// kvs_device_status() reads it; the partial results follow, then the arrival counts
-__global__ void decode_header_kernel(int32_t* hdr, int32_t* arrived, int n) {
-    pdl_wait();
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i == 0) {
-        hdr[0] = (int32_t)WS_MAGIC;
-        hdr[1] = KVS_OK;
-    }
-    if (i < n) arrived[i] = 0;
-}
-
 template <int G, int LOAD>
-static int launch_decode_tc(const CUtensorMap& tk, const CUtensorMap& tv, const DecodeParams& p, int32_t* status, cudaStream_t st) {
+static int launch_decode_tc(const CUtensorMap& tk, const CUtensorMap& tv, const DecodeParams& p, cudaStream_t st) {
     auto kern = decode_tc_kernel<G, LOAD>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, DtcSmem::DYN_BYTES) != cudaSuccess) return cuda_refused();
     dim3 grid(p.nsplit, p.Hkv, p.S);
-    return launch_after(kern, grid, DTC_THREADS, DtcSmem::DYN_BYTES, st, tk, tv, p, status);
+    return launch_after(kern, grid, DTC_THREADS, DtcSmem::DYN_BYTES, st, tk, tv, p);
 }
 
 template <int D>
-static int launch_decode(const DecodeParams& p, int G, const void* k_cache, const void* v_cache, int32_t* status, cudaStream_t st) {
+static int launch_decode(const DecodeParams& p, int G, const void* k_cache, const void* v_cache, cudaStream_t st) {
     dim3 grid(p.nsplit, p.Hkv, p.S);
     const int ps = p.page_size;
     // tensor-core variant (head_dim 128).  Pages that are whole 8-row swizzle atoms and tile 128 tokens exactly come in
@@ -988,11 +996,11 @@ static int launch_decode(const DecodeParams& p, int G, const void* k_cache, cons
             if ((rc = make_tmap_thd(&tk, k_cache, p.num_pages * ps, p.Hkv, 128, ps)) != KVS_OK) return rc;
             if ((rc = make_tmap_thd(&tv, v_cache, p.num_pages * ps, p.Hkv, 128, ps)) != KVS_OK) return rc;
             switch (G) {
-                case 1: rc = launch_decode_tc<1, DTC_PAGES>(tk, tv, p, status, st); break;
-                case 2: rc = launch_decode_tc<2, DTC_PAGES>(tk, tv, p, status, st); break;
-                case 4: rc = launch_decode_tc<4, DTC_PAGES>(tk, tv, p, status, st); break;
-                case 7: rc = launch_decode_tc<7, DTC_PAGES>(tk, tv, p, status, st); break;
-                default: rc = launch_decode_tc<8, DTC_PAGES>(tk, tv, p, status, st); break;
+                case 1: rc = launch_decode_tc<1, DTC_PAGES>(tk, tv, p, st); break;
+                case 2: rc = launch_decode_tc<2, DTC_PAGES>(tk, tv, p, st); break;
+                case 4: rc = launch_decode_tc<4, DTC_PAGES>(tk, tv, p, st); break;
+                case 7: rc = launch_decode_tc<7, DTC_PAGES>(tk, tv, p, st); break;
+                default: rc = launch_decode_tc<8, DTC_PAGES>(tk, tv, p, st); break;
             }
         } else {
             // the K cache as (Hkv * d, rows): a gather names four rows and a 64-column slice of one KV head (V is
@@ -1000,11 +1008,11 @@ static int launch_decode(const DecodeParams& p, int G, const void* k_cache, cons
             if ((long long)p.num_pages * ps > 0x7fffffffLL) return KVS_ERR_UNSUPPORTED;
             if ((rc = make_tmap_rows(&tk, k_cache, p.num_pages * ps, p.Hkv * 128)) != KVS_OK) return rc;
             switch (G) {
-                case 1: rc = launch_decode_tc<1, DTC_ROWS>(tk, tv, p, status, st); break;
-                case 2: rc = launch_decode_tc<2, DTC_ROWS>(tk, tv, p, status, st); break;
-                case 4: rc = launch_decode_tc<4, DTC_ROWS>(tk, tv, p, status, st); break;
-                case 7: rc = launch_decode_tc<7, DTC_ROWS>(tk, tv, p, status, st); break;
-                default: rc = launch_decode_tc<8, DTC_ROWS>(tk, tv, p, status, st); break;
+                case 1: rc = launch_decode_tc<1, DTC_ROWS>(tk, tv, p, st); break;
+                case 2: rc = launch_decode_tc<2, DTC_ROWS>(tk, tv, p, st); break;
+                case 4: rc = launch_decode_tc<4, DTC_ROWS>(tk, tv, p, st); break;
+                case 7: rc = launch_decode_tc<7, DTC_ROWS>(tk, tv, p, st); break;
+                default: rc = launch_decode_tc<8, DTC_ROWS>(tk, tv, p, st); break;
             }
         }
         if (rc != KVS_OK) return rc;
@@ -1019,9 +1027,9 @@ static int launch_decode(const DecodeParams& p, int G, const void* k_cache, cons
         }
         if (rc != KVS_OK) return rc;
     }
-    if (p.arrived) return KVS_OK;
     const long long rows = (long long)p.S * p.Hq;
-    return launch_after(decode_merge_kernel<D>, (unsigned)((rows + 7) / 8), 256, 0, st, p);
+    const unsigned blocks = (unsigned)((rows + 7) / 8);
+    return p.nsplit <= 4 ? launch_after(decode_merge_kernel<D, 4>, blocks, 256, 0, st, p) : launch_after(decode_merge_kernel<D, 16>, blocks, 256, 0, st, p);
 }
 
 extern "C" int kvs_decode_attn(const void* q, const void* k_cache, const void* v_cache, const int32_t* block_table,
@@ -1036,8 +1044,7 @@ extern "C" int kvs_decode_attn(const void* q, const void* k_cache, const void* v
     if (!q || !k_cache || !v_cache || !block_table || !n_tokens || !out || !lse || !workspace) return KVS_ERR_INVALID_ARG;
     if ((((uintptr_t)q | (uintptr_t)k_cache | (uintptr_t)v_cache | (uintptr_t)out) & 15) != 0 || ((uintptr_t)workspace & 255) != 0)
         return KVS_ERR_ALIGNMENT;
-    const size_t base = decode_base_bytes(num_seqs, Hq, head_dim, num_splits);
-    if (workspace_bytes < base) return KVS_ERR_WORKSPACE;
+    if (workspace_bytes < kvs_decode_workspace_bytes(num_seqs, Hq, head_dim, num_splits)) return KVS_ERR_WORKSPACE;
     if (softmax_scale < 0.f || softmax_scale != softmax_scale) return KVS_ERR_INVALID_ARG;
     DecodeParams p;
     p.q = (const __nv_bfloat16*)q;
@@ -1052,23 +1059,15 @@ extern "C" int kvs_decode_attn(const void* q, const void* k_cache, const void* v
     p.page_shift = (page_size & (page_size - 1)) == 0 ? __builtin_ctz((unsigned)page_size) : -1;
     p.max_pages = max_pages;
     p.num_pages = num_pages;
-    p.status = (int32_t*)workspace + 1;
+    p.status = nullptr;
+    p.header = (int32_t*)workspace;
     p.nsplit = num_splits;
     const float s = softmax_scale == 0.f ? 1.0f / sqrtf((float)head_dim) : softmax_scale;
     p.scale_log2 = s * 1.4426950408889634f;
     p.part_o = (float*)((char*)workspace + DEC_WS_HEADER);
     p.part_ml = p.part_o + (size_t)num_seqs * Hq * num_splits * head_dim;
     cudaStream_t st = (cudaStream_t)stream;
-    p.arrived = (int32_t*)((char*)workspace + base);
     p.out = (__nv_bfloat16*)out;
     p.lse = lse;
-    // three CTAs per SM are resident: up to two waves of them merge on their own, if the workspace has room for their counts
-    const int rows = num_seqs * Hkv;
-    if ((long long)rows * num_splits > 2 * 3 * 148 || workspace_bytes < kvs_decode_workspace_bytes(num_seqs, Hq, head_dim, num_splits))
-        p.arrived = nullptr;
-    const int rc = launch_after(decode_header_kernel, p.arrived ? (rows + 255) / 256 : 1, 256, 0, st, (int32_t*)workspace, p.arrived, p.arrived ? rows : 0);
-    if (rc != KVS_OK) return rc;
-    int32_t* status = (int32_t*)workspace + 1;
-    return head_dim == 64 ? launch_decode<64>(p, Hq / Hkv, k_cache, v_cache, status, st)
-                          : launch_decode<128>(p, Hq / Hkv, k_cache, v_cache, status, st);
+    return head_dim == 64 ? launch_decode<64>(p, Hq / Hkv, k_cache, v_cache, st) : launch_decode<128>(p, Hq / Hkv, k_cache, v_cache, st);
 }

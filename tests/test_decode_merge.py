@@ -1,7 +1,7 @@
-"""The two ways in which decode attention merges its splits (needs a B200): the last CTA of a (sequence, KV head) in small grids
-whose workspace has room for the arrival counts, a kernel of its own otherwise.  Both add the same partial results in the same
-order, so they agree bit for bit; and both are compared with the definition in fp64.  Bounds: weights and outputs are rounded to
-bf16 (2^-9 relative each), and |out| is below 4 on these inputs, so 2e-2 as in the other decode tests."""
+"""The merge of the splits of decode attention (needs a B200): grids below and above one wave, one split, more splits than a warp
+has lanes and than there are tiles, sequences without a token; against the definition in fp64, and a workspace that still holds
+another call's results.  Bounds: weights and outputs are rounded to bf16 (2^-9 relative each), and |out| is below 4 on these
+inputs, so 2e-2 as in the other decode tests."""
 import numpy as np
 import pytest
 import torch
@@ -35,35 +35,31 @@ def _cache(lens, page, Hkv, d, seed):
 
 
 def _bytes(S, Hq, d, splits):
-    up = lambda x: -(-x // 256) * 256  # noqa: E731
-    partial = 256 + up(4 * S * Hq * splits * (d + 2))
-    assert int(B.load().kvs_decode_workspace_bytes(S, Hq, d, splits)) == partial + up(4 * S * Hq)
-    return partial, partial + up(4 * S * Hq)
+    least = 256 + -(-4 * S * Hq * splits * (d + 2) // 256) * 256
+    assert int(B.load().kvs_decode_workspace_bytes(S, Hq, d, splits)) == least
+    return least
 
 
 @pytest.mark.parametrize("S,lens,page,Hkv,G,d,splits", [
-    (37, (0, 1, 900), 16, 8, 4, 128, 3),        # 888 CTAs: the largest grid that merges on its own
-    (48, (0, 1, 700), 16, 8, 4, 128, 3),        # 1152
-    (112, (0, 5, 300), 1, 8, 2, 128, 1),        # 896 CTAs, a single split
-    (64, (0, 3, 400), 4, 4, 7, 128, 4),         # 1024, pages of 4
-    (120, (0, 1, 257), 16, 4, 2, 64, 2),        # 960, head_dim 64
+    (48, (0, 1, 700), 16, 8, 4, 128, 3),        # 1152 CTAs
+    (112, (0, 5, 300), 1, 8, 2, 128, 1),        # a single split
+    (64, (0, 3, 400), 4, 4, 7, 128, 4),         # the most splits that are merged 4 at a time
+    (64, (0, 3, 900), 4, 4, 1, 128, 5),         # ... 16 at a time
+    (120, (0, 1, 257), 16, 4, 2, 64, 2),
     (2, (5000, 1), 1, 2, 7, 128, 40),           # more splits than a warp has lanes
     (3, (4000, 0, 33), 16, 2, 8, 128, 64),      # ... and more than there are tiles
     (2, (3000, 10), 16, 3, 1, 64, 33),
+    (5, (2100, 0), 16, 2, 4, 64, 17),
 ])
-def test_both_merges_give_the_definition(S, lens, page, Hkv, G, d, splits):
+def test_merge_gives_the_definition(S, lens, page, Hkv, G, d, splits):
     lens = [lens[s % len(lens)] for s in range(S)]
     cache, live = _cache(lens, page, Hkv, d, S + splits)
     q = torch.randn((S, Hkv * G, d), generator=torch.Generator(device="cuda").manual_seed(1), device="cuda", dtype=torch.bfloat16)
-    got = []
-    for room in _bytes(S, Hkv * G, d, splits):
-        ws = torch.full((room,), 0xa5, dtype=torch.uint8, device="cuda")
-        for _ in range(2):                       # the counts of the call before are no longer zero
-            got.append(cache.decode(q, num_splits=splits, workspace=ws))
-        assert B.kvs_device_status(ws) == B.KVS_OK
-    for out, lse in got[1:]:
-        assert torch.equal(out, got[0][0]) and torch.equal(lse, got[0][1])
-    out, lse = got[0]
+    ws = torch.full((_bytes(S, Hkv * G, d, splits),), 0xff, dtype=torch.uint8, device="cuda")      # NaN in every partial result
+    out, lse = cache.decode(q, num_splits=splits, workspace=ws)
+    assert B.kvs_device_status(ws) == B.KVS_OK
+    again = cache.decode(q, num_splits=splits, workspace=ws)
+    assert torch.equal(out, again[0]) and torch.equal(lse, again[1])
     for s, n in enumerate(lens):
         if n == 0:
             assert (out[s] == 0).all() and (lse[s] == -float("inf")).all()
@@ -77,8 +73,28 @@ def test_both_merges_give_the_definition(S, lens, page, Hkv, G, d, splits):
 def test_workspace_limits():
     cache, _ = _cache([300], 16, 2, 128, 0)
     q = torch.randn((1, 8, 128), device="cuda", dtype=torch.bfloat16)
-    least, _ = _bytes(1, 8, 128, 2)
+    least = _bytes(1, 8, 128, 2)
     with pytest.raises(B.KvsError) as e:
         cache.decode(q, num_splits=2, workspace=torch.empty(least - 1, dtype=torch.uint8, device="cuda"))
     assert e.value.code == B.KVS_ERR_WORKSPACE
     cache.decode(q, num_splits=2, workspace=torch.empty(least, dtype=torch.uint8, device="cuda"))
+
+
+@pytest.mark.parametrize("page,G,d", [(16, 4, 128), (1, 7, 128), (1, 1, 128), (16, 2, 64)])
+@pytest.mark.parametrize("splits", [1, 5, 40])
+def test_bad_page_is_reported_and_the_next_call_is_clean(page, G, d, splits):
+    # page ids outside the cache are not followed (page 0 is read instead); the status comes with the partial results
+    cache, _ = _cache([2000, 700, 0], page, 2, d, splits)
+    q = torch.randn((3, 2 * G, d), device="cuda", dtype=torch.bfloat16)
+    ws = torch.full((_bytes(3, 2 * G, d, splits),), 0xff, dtype=torch.uint8, device="cuda")
+    last = (2000 - 1) // page
+    good = int(cache.block_table[0, last])
+    for bad in (-1, cache.num_pages, 2 ** 31 - 1):
+        cache.block_table[0, last] = bad
+        cache.decode(q, num_splits=splits, workspace=ws)
+        assert B.kvs_device_status(ws) == B.KVS_ERR_INVALID_ARG
+        out, lse = cache.decode(q, num_splits=splits, workspace=ws)
+        assert torch.isfinite(out).all() and torch.isfinite(lse[:2]).all()
+        cache.block_table[0, last] = good
+        cache.decode(q, num_splits=splits, workspace=ws)
+        assert B.kvs_device_status(ws) == B.KVS_OK
