@@ -1,8 +1,8 @@
 // Forward: eviction-masked causal attention.
 //
-// One item per (query block, pair of query heads of one GQA group), and a CTA per item or a chain of items.  The two heads share every K/V
-// tile (identical key-block list and element mask), so each tile is fetched once for two 128-row
-// query tiles.  The last head of an odd group (and every head when there is no grouping) gets an item
+// One item per (query block, pair of query heads of one GQA group), and a CTA per item or a chain of
+// items.  The two heads share every K/V tile (identical key-block list and element mask), so each tile
+// is fetched once for two 128-row query tiles.  The last head of an odd group (and every head when there is no grouping) gets an item
 // of its own, in which the two softmax groups take alternate key blocks of that one head as two
 // independent streams, merged at the end.  384 threads in three warp groups:
 //   warps 0-3   softmax of tile 0 (one query row per thread)        } registers re-balanced with
@@ -18,8 +18,9 @@
 // Per key block i the tensor pipe runs  O0 += P0 V, S0(i+1) = Q0 K^T, O1 += P1 V, S1(i+1) = Q1 K^T
 // while the two softmax groups alternate, so the exponentials of one tile overlap the MMAs of the
 // other.  A row's probabilities are handed over in two parts (the first P_SPLIT keys, then the
-// rest), so most of P V overlaps the last exponentials of the row.  EMPTY tiles are never visited (the CTA walks the row's non-empty list); the element mask
-// is evaluated on PARTIAL or ragged tiles only.  O is rescaled lazily: a row keeps its reference
+// rest), so most of P V overlaps the last exponentials of the row.  EMPTY tiles are never visited (the
+// CTA walks the row's non-empty list); the element mask is evaluated on PARTIAL or ragged tiles only,
+// and there only by the warps and for the 32 keys that need it.  O is rescaled lazily: a row keeps its reference
 // maximum until the running maximum exceeds it by more than 8 (base-2), so exp2 arguments stay
 // below 2^8 and the rescale of O in tensor memory is rare.
 #include "kvs_common.cuh"
@@ -606,7 +607,6 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
                 }
                 const float2 t01 = __fadd2_rn(ts[0], ts[1]), t23 = __fadd2_rn(ts[2], ts[3]);
                 const float tile_sum = (t01.x + t01.y) + (t23.x + t23.y);
-                
                 run_sum += tile_sum;
                 {
                     uint32_t r2[16];
@@ -659,39 +659,39 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
                 ++singles;
             }
             if (!dual || t == 0) {
-            const float inv = (run_sum > 0.f && nlist > 0) ? 1.f / run_sum : 0.f;
-            __nv_bfloat16* orow = p.out + ((size_t)(tok0 + qi) * p.Hq + h) * D;
+                const float inv = (run_sum > 0.f && nlist > 0) ? 1.f / run_sum : 0.f;
+                __nv_bfloat16* orow = p.out + ((size_t)(tok0 + qi) * p.Hq + h) * D;
 #pragma unroll
-            for (int c = 0; c < D / 32; ++c) {
-                uint32_t r[32];
-                tmem_ld32(tmem_O + c * 32, r);
-                tmem_wait_ld();
-                if (nlist == 0) {      // only a bad evict_at (already reported by the metadata pass) gets here
+                for (int c = 0; c < D / 32; ++c) {
+                    uint32_t r[32];
+                    tmem_ld32(tmem_O + c * 32, r);
+                    tmem_wait_ld();
+                    if (nlist == 0) {      // only a bad evict_at (already reported by the metadata pass) gets here
 #pragma unroll
-                    for (int e = 0; e < 32; ++e) r[e] = 0u;
-                }
-                if (dual && nlist > 0) {
+                        for (int e = 0; e < 32; ++e) r[e] = 0u;
+                    }
+                    if (dual && nlist > 0) {
 #pragma unroll
-                    for (int e = 0; e < 32; ++e) {
-                        float o = __uint_as_float(r[e]) * a0;
-                        if (a1 > 0.f) o = fmaf(x_o[(c * 32 + e) * TILE + row], a1, o);
-                        r[e] = __float_as_uint(o);
+                        for (int e = 0; e < 32; ++e) {
+                            float o = __uint_as_float(r[e]) * a0;
+                            if (a1 > 0.f) o = fmaf(x_o[(c * 32 + e) * TILE + row], a1, o);
+                            r[e] = __float_as_uint(o);
+                        }
+                    }
+                    if (valid) {
+                        uint4* dst = reinterpret_cast<uint4*>(orow + c * 32);
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            uint4 w;
+                            w.x = pack_bf16(__uint_as_float(r[e * 8 + 0]) * inv, __uint_as_float(r[e * 8 + 1]) * inv);
+                            w.y = pack_bf16(__uint_as_float(r[e * 8 + 2]) * inv, __uint_as_float(r[e * 8 + 3]) * inv);
+                            w.z = pack_bf16(__uint_as_float(r[e * 8 + 4]) * inv, __uint_as_float(r[e * 8 + 5]) * inv);
+                            w.w = pack_bf16(__uint_as_float(r[e * 8 + 6]) * inv, __uint_as_float(r[e * 8 + 7]) * inv);
+                            dst[e] = w;
+                        }
                     }
                 }
-                if (valid) {
-                    uint4* dst = reinterpret_cast<uint4*>(orow + c * 32);
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        uint4 w;
-                        w.x = pack_bf16(__uint_as_float(r[e * 8 + 0]) * inv, __uint_as_float(r[e * 8 + 1]) * inv);
-                        w.y = pack_bf16(__uint_as_float(r[e * 8 + 2]) * inv, __uint_as_float(r[e * 8 + 3]) * inv);
-                        w.z = pack_bf16(__uint_as_float(r[e * 8 + 4]) * inv, __uint_as_float(r[e * 8 + 5]) * inv);
-                        w.w = pack_bf16(__uint_as_float(r[e * 8 + 6]) * inv, __uint_as_float(r[e * 8 + 7]) * inv);
-                        dst[e] = w;
-                    }
-                }
-            }
-            if (valid) p.lse[(size_t)h * p.total_tokens + tok0 + qi] = ref_max * 0.6931471805599453f + logf(run_sum);
+                if (valid) p.lse[(size_t)h * p.total_tokens + tok0 + qi] = ref_max * 0.6931471805599453f + logf(run_sum);
             }
             if (nlist > 0) {
                 tc_fence_before();
@@ -720,11 +720,18 @@ static int launch_fwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtens
     return launch_after(kern, dim3(nb_cap, p.heads, 1), FWD_THREADS, FwdSmem<D>::DYN_BYTES, st, tq, tk, tv, mv, p);
 }
 
-// Items are chained where traces are short (2048 tokens on average) and the grid is more than two waves of CTAs: forward alone,
-// a CTA per item -> chained, us: 96 traces of 60 to 900 tokens 307 -> 259, 40 of 50 to 900 262 -> 217, 20 of 100 to 2000 with
-// head_dim 64 156 -> 137.  One trace of 7000 tokens 203 -> 204; rows of 70 tiles 17.3 -> 17.9 ms; one of 300 tokens 18.4 -> 19.8.
+// Items are chained where rows are short and the grid is a few waves of CTAs.  A chained CTA saves the start and the end of an
+// item; its loop over items costs 2 to 4 % of a tile.  Forward, a CTA per item -> chained, us (32 heads on 8; of the same batch
+// with last-4-turns eviction and with none): 131 x 500 tokens 751 -> 615, 725 -> 589; 32 x 2000 946 -> 841, 1260 -> 1167;
+// 14 x 4500 1333 -> 1272, 2123 -> 2111; 9 x 7000 1639 -> 1597, 2955 -> 2987; 5 x 12000 2210 -> 2209, 4519 -> 4637: with nothing
+// evicted they meet at 5000 tokens.  Longer traces need more waves, or a CTA has an item in hand while others have nothing left:
+// 4 x 1000 (3.8 waves) 64.5 -> 62.7, but 1 x 3000 (2.6) 72.2 -> 75.8, 2 x 3000 (5.2) 117 -> 118; 1 x 1000 (0.9) 22.5 -> 24.3.
+// The mean length is what is known here that a caller cannot overstate.  A long trace among many short ones is chained with them
+// (32768 + 60 x 300: 2938 -> 2984; 16000 + 100 x 300: 1118 -> 1098).
 static bool chain_items(int batch, int total_tokens, int nb_cap, int heads) {
-    return total_tokens / batch <= 2048 && (long long)nb_cap * heads > 2 * 148;
+    const long long ctas = (long long)nb_cap * heads;
+    const int mean = total_tokens / batch;
+    return (mean <= 2048 && ctas > 2 * 148) || (mean <= 4096 && ctas > 6 * 148);
 }
 
 }  // namespace kvs

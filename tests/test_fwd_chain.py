@@ -18,9 +18,10 @@ LENS = [int(x) for x in np.random.default_rng(1).permutation(np.concatenate([np.
 
 
 def _chained(lens, Hq, Hkv):
-    """The condition of the dispatch: traces of 2048 tokens or less on average, more than two waves of CTAs."""
-    blocks = sum(lens) // 128 + len(lens)
-    return sum(lens) // len(lens) <= 2048 and blocks * Hkv * ((Hq // Hkv + 1) // 2) > 2 * 148
+    """The condition of the dispatch: traces of 2048 tokens or less on average and more than two waves of CTAs, or 4096 and six."""
+    ctas = (sum(lens) // 128 + len(lens)) * Hkv * ((Hq // Hkv + 1) // 2)
+    mean = sum(lens) // len(lens)
+    return (mean <= 2048 and ctas > 2 * 148) or (mean <= 4096 and ctas > 6 * 148)
 
 
 def _evict(lens, rule, seed):
@@ -125,3 +126,20 @@ def test_chained_key_slots(Hq, Hkv, d):
     out, lse = B.kvs_attn_fwd(q, B.kvs_permute_rows(k, perm), B.kvs_permute_rows(v, perm), meta, len(LENS), longest)
     j = torch.arange(longest, device="cuda")
     _compare(LENS, cu, out, lse, lambda b, z: _definition(q[z], k[z], v[z], j[:LENS[b]], ev[z]))
+
+
+def test_chained_longer_traces():
+    Hq, Hkv, d, lens = 9, 3, 128, [4096, 2111, 4095, 3000, 4001, 4000, 3999, 3500, 2900]      # pairs and single heads
+    assert _chained(lens, Hq, Hkv) and sum(lens) // len(lens) > 2048
+    ev = torch.from_numpy(_evict(lens, "mixed", 3)).cuda()
+    cu = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    q, k, v = _inputs(lens, Hq, Hkv, d, 4)
+    meta = B.kvs_mask_meta(ev, torch.from_numpy(cu).cuda(), max(lens))
+    out, lse = B.kvs_attn_fwd(q, k, v, meta, len(lens), max(lens))
+    assert B.kvs_device_status(meta) == B.KVS_OK
+    for b, T in enumerate(lens):
+        z = slice(int(cu[b]), int(cu[b]) + T)
+        assert not _chained([T], Hq, Hkv)
+        one = B.kvs_mask_meta(ev[z].contiguous(), torch.tensor([0, T], dtype=torch.int32, device="cuda"), T)
+        o, m = B.kvs_attn_fwd(q[z].contiguous(), k[z].contiguous(), v[z].contiguous(), one, 1, T)
+        assert torch.equal(o, out[z]) and torch.equal(m, lse[:, z]), (b, T)
