@@ -67,8 +67,11 @@ struct BwdPlanArgs {
 // before the first product, the pipeline's first and last tile, the stores), a unit of a cut item BWD_CUT_COST more (slot
 // written and read again); no unit is longer than the makespan; where the longest is over one and a half times what a head
 // has for an SM, those above that start first, over all heads, so what is left over at the end is half of it at most (always
-// doing so costs L2 hits, 2 x 65536 tokens 41.4 -> 42.6 ms, but not on traces of at most 16 tiles: 96 of 60 to 900 472 -> 454 us); and up to three waves take that many average units.  Main kernel, whole items -> cut, us: 1 trace of 1000 tokens with 16 heads on 2: 154 -> 42; 4000 with 32 on 8:
-// 355 -> 180; 16000, head_dim 64: 1199 -> 748; 32768 with 28 on 4 (pairs): 5500 -> 4400; nothing cut: 1 to 3 % slower.
+// doing so costs L2 hits, 2 x 65536 tokens 41.4 -> 42.6 ms, but not on traces of at most 16 tiles: 96 of 60 to 900
+// 472 -> 454 us); and up to three waves take that many average units.
+// Main kernel, whole items -> cut, us: 1 trace of 1000 tokens with 16 heads on 2 154 -> 42; 4000 with 32 on 8 355 -> 180; 16000,
+// head_dim 64 1199 -> 748; 20 of 100 to 2000, head_dim 64 229 -> 161; 32768 with 28 on 4 (pairs) 5500 -> 4400.  Where nothing is
+// cut, the list and the registers of the slots cost 1 % at head_dim 64 and 9 % at 128 (96 of 60 to 900: 316 -> 319, 447 -> 494).
 constexpr float BWD_UNIT_COST = 4.f, BWD_CUT_COST = 3.f;
 __device__ void bwd_plan(const BwdPlanArgs& a) {
     constexpr int NC = 8;
@@ -753,11 +756,21 @@ size_t kvs::bwd_cut_bytes(int total_tokens, int Hq, int head_dim) {
 }
 
 namespace {
-// CTA pairs take head_dim 128 where the traces are long, 24000 tokens and more on average.  There the chip runs at its power
-// limit and the pairs' smaller shared-memory and reduce-add traffic counts (main kernel, single CTAs -> pairs: 2 x 65536 tokens
-// of last-4-turns 44.8 -> 42.3 ms, 24576 token-level 17.7 -> 16.8, 50000 summary 12.4 -> 12.1).  Below, a pair's union of two
-// query ranges and its costlier start weigh more (8 x 6000 tokens 2.0 -> 2.3 ms, 128 x 300 0.36 -> 0.54).
-bool use_pairs(int batch, int total_tokens, int head_dim) { return head_dim == 128 && total_tokens / batch >= 24000; }
+// CTA pairs take head_dim 128 where the traces are long: they read and stage less, and on long walks the chip runs at its power
+// limit.  On short ones a pair's union of two query ranges and its costlier start weigh more, the more so the fewer heads share
+// a key block.  Main kernel, single CTAs -> pairs, us (by tokens a trace, 48000 a batch, with nothing evicted 24000 to 32000; last-
+// 4-turns, summary, nothing evicted, token-level):
+//   32 heads on 8,  6000: 2844 -> 3064, 1980 -> 2307,  3694 ->  3441,  5932 ->  5832
+//                  12000: 5293 -> 5120, 3437 -> 3440,  6040 ->  5495, 11404 -> 10971
+//                  16000: 6687 -> 6436, 4443 -> 4403, 10129 ->  8952, 15039 -> 14283
+//                  24000: 9750 -> 9072, 6520 -> 6232, 11745 -> 10639, 22404 -> 21227
+//   16 on 16,      16000: 3506 -> 3463, 2410 -> 2515,  5152 ->  4734,  7524 ->  7429
+//                  24000: 5060 -> 4838, 3456 -> 3427,  6000 ->  5501, 11329 -> 10872
+// (28 on 4 and 16 on 2 are like 32 on 8.)  The mean length is what is known here that a caller cannot overstate, and no batch of
+// short traces reaches it; a long trace with short ones beside it stays with single CTAs (40000 + 1 token: 11.7 instead of 10.8 ms).
+bool use_pairs(int batch, int total_tokens, int G, int head_dim) {
+    return head_dim == 128 && total_tokens / batch >= (G > 1 ? 16000 : 24000);
+}
 
 // in_ts: elements between consecutive tokens of q and of k, v; g_ts: of dq and of dk, dv (0: tensors of their own)
 int bwd_impl(const void* dout, const void* q, const void* k, const void* v, long long in_ts, const void* out, const float* lse,
@@ -782,7 +795,7 @@ int bwd_impl(const void* dout, const void* q, const void* k, const void* v, long
     const MetaLayout L = meta_layout(batch, total_tokens, max_seqlen);
     const MetaView mv = meta_view(meta_buf, L);
     const BwdWhole whole = part_of ? *part_of : BwdWhole{meta_buf, batch, total_tokens, max_seqlen, Hkv, nullptr};
-    const bool pair = use_pairs(whole.batch, whole.total_tokens, head_dim);
+    const bool pair = use_pairs(whole.batch, whole.total_tokens, Hq / Hkv, head_dim);
     const int q_rows = pair ? TILE / 2 : TILE;       // rows of the boxes of q, dout and dq
     CUtensorMap tq, tk, tv, tdo, tdq;
     if ((rc = make_tmap_thd(&tq, q, total_tokens, Hq, head_dim, q_rows, in_ts)) != KVS_OK) return rc;

@@ -70,10 +70,10 @@ def test_cut_items_equal_whole_items(lens, Hq, Hkv, d, rule):
     assert torch.equal(got[1], again[1]) and torch.equal(got[2], again[2])        # the slots are added in a fixed order
 
 
-@pytest.mark.parametrize("T,rule", [(24000, "turns"), (24064, "tokens"), (24193, "turns"), (24321, "causal")])
+@pytest.mark.parametrize("T,rule", [(24000, "turns"), (24064, "tokens"), (24193, "turns"), (24321, "causal"), (16000, "tokens"), (16129, "turns")])
 def test_pairs_equal_single_ctas(T, rule):
     # a long trace alone is taken by CTA pairs; with a one-token trace behind it the mean length is below their line and
-    # single CTAs take the same keys.  Block counts: 188 (even, last block half full), 188 (full), 190, 191 (odd, one row)
+    # single CTAs take the same keys.  Block counts: 188 (even, last block half full), 188 (full), 190, 191 (odd, one row), 125, 127
     Hq, Hkv, d = 4, 2, 128
     x = _inputs([T], Hq, Hkv, d, rule)
     out, lse, got = _backward(x, [T], False)
