@@ -260,7 +260,9 @@ int kvs_attn_bwd_ex(const void* dout, const void* q, const void* k, const void* 
  * pay the device-wide synchronisation cudaMalloc/cudaFree imply.  For them the scratch that
  * kvs_attn_bwd takes as `workspace` is a fixed array inside the library, of
  * 256 B + 4 B * KVS_NOALLOC_MAX_ROWS + 38 MiB per GPU (the last for the partial sums of key blocks with long
- * walks, see kvs_attn_bwd_workspace_bytes), resident on every GPU that loads the library.
+ * walks, see kvs_attn_bwd_workspace_bytes).  The CUDA runtime places it on a GPU when the first call there looks
+ * its address up (44 MiB less free memory), or, with CUDA_MODULE_LOADING=EAGER, when the library's first kernel is
+ * loaded; a pool that takes all free memory has to be set up after that.
  *   - Gradients are fp32 only (dq is accumulated in place, so it needs no scratch); otherwise the
  *     arguments and results are those of kvs_attn_bwd with KVS_GRAD_FP32.
  *   - total_tokens * Hq must not exceed KVS_NOALLOC_MAX_ROWS, else KVS_ERR_WORKSPACE is returned

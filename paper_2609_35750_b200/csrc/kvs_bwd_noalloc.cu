@@ -8,7 +8,8 @@ namespace {
 
 // Room for the workspace header plus one fp32 row sum per (token, query head), total_tokens * Hq <= KVS_NOALLOC_MAX_ROWS
 // (4 MiB), and for the units and slots of cut items at any such size (37 MiB of slots at head_dim 128), so that the sums are
-// those of kvs_attn_bwd.  Every GPU that loads the library holds these 42 MiB until the process exits.
+// those of kvs_attn_bwd.  A GPU holds these 42 MiB from the first call there until the process exits (measured: 44 MiB less
+// free memory after it, none before); with CUDA_MODULE_LOADING=EAGER from the first kernel of the library on.
 constexpr size_t kScratchBytes = 256 + sizeof(float) * (size_t)KVS_NOALLOC_MAX_ROWS + ((size_t)38 << 20);
 static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
 
