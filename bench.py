@@ -640,6 +640,8 @@ def main():
     flops_bwd_main = 10.0 * d * Hq * pairs
     achieved = flops_bwd_main / (ms_bwd_main * 1e-3) / 1e12
     peak = float(peaks["bf16_tflops_sustained"])      # the kernel is timed inside a long step
+    # the main kernel that the library takes for this batch: CTA pairs on long traces at head_dim 128
+    bwd_main = "bwd_pair_kernel" if d == 128 and Tt // w.batch >= (16000 if Hq > Hkv else 24000) else "bwd_kernel"
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
         "ms_per_step": ms_total_max / args.steps, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
@@ -656,7 +658,7 @@ def main():
         "breakdown_ms": {"mask_meta": ms_meta, "fwd": ms_fwd, "bwd_main": ms_bwd_main,
                          "bwd_pre_post": ms_total_max / args.steps - ms_meta - ms_fwd - ms_bwd_main,
                          "fwd_tflops": 4.0 * d * Hq * pairs / (ms_fwd * 1e-3) / 1e12, "bwd_main_tflops": achieved},
-        "roofline": {"kernel": "bwd_kernel (dQ/dK/dV main)", "bound": "tensor", "achieved": achieved, "peak": peak,
+        "roofline": {"kernel": f"{bwd_main} (dQ/dK/dV main)", "bound": "tensor", "achieved": achieved, "peak": peak,
                      "unit": "TFLOP/s", "frac": achieved / peak, "traffic": load_traffic(w.name),
                      "frac_of_burst_peak": achieved / float(peaks["bf16_tflops"]),
                      "peak_source": f"{peaks['_source']} cuBLAS bf16, sustained (kernel timed inside a long step)",
