@@ -62,12 +62,12 @@ __device__ __forceinline__ void decode_header(const DecodeParams& p) {
 }
 
 // Merge of the splits of a (sequence, query head) by a warp: weights exp2(m_z - max), normalised, bf16 out and fp32 lse.  Bound by
-// latency: the loads of PART splits are on their way before the first is used (16, with 4 at a time 47 splits took 5 us more);
-// where there are few splits, PART = 4 leaves room for three times the warps (100 sequences of 64 heads, one split: step 38.0 ->
+// latency: the loads of PART splits are on their way before the first is used (16: with 4 at a time 47 splits took 7 us more);
+// where there are few splits, PART = 4 leaves room for twice the warps (100 sequences of 64 heads, one split: step 38.0 ->
 // 34.8 us).  A kernel of its own, started by programmatic dependent launch: merging in the last CTA of a (sequence, KV head) to
-// finish, with counts in the workspace, took a launch less but cost every CTA a fence and an atomic and the merge its parallelism
-// (a step in a CUDA graph, merge in the last CTA -> here, us: 1 x 24000 tokens with 8 heads on 1 29.6 -> 20.4, 1 x 2000 with 32
-// on 8 14.2 -> 13.8, 100 x 300 with 8 on 8 and head_dim 64 17.5 -> 13.7; launched one by one the two are within 1 us).
+// finish, with counts in the workspace, cost every CTA a fence and an atomic and the merge its parallelism (a step in a CUDA
+// graph, merge in the last CTA -> here, us: 1 x 24000 tokens with 8 heads on 1 29.6 -> 15.0, 1 x 2000 with 32 on 8 14.2 -> 12.7,
+// 100 x 300 with 8 on 8 and head_dim 64 17.4 -> 13.5; launched call by call 30.4 -> 15.8, 14.6 -> 13.3, 17.9 -> 13.8).
 template <int D, int PART>
 __device__ __forceinline__ void decode_merge_row(const DecodeParams& p, size_t row, int lane) {
     constexpr int PER = D / 32;
