@@ -267,8 +267,9 @@ __device__ __forceinline__ void mbar_wait_limit(uint32_t bar, uint32_t parity, v
         if (mbar_try_wait_hint(bar, parity, KVS_WAIT_HINT_NS)) return;
         if (*abort_flag) return;
         if (clock64() - t0 > limit_clocks) {
+            set_status(status, KVS_ERR_TIMEOUT);      // before the flag: who sees that may read this (decode hands it over)
+            __threadfence_block();
             *abort_flag = 1;
-            set_status(status, KVS_ERR_TIMEOUT);
             return;
         }
     }
