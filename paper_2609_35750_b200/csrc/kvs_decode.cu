@@ -38,8 +38,6 @@ struct DecodeParams {
     float scale_log2;
     float* part_o;                   // [S, Hq, nsplit, D] unnormalised
     float* part_ml;                  // [S, Hq, nsplit, 2]  (max in base-2 units, sum; see flagged_sum)
-    __nv_bfloat16* out;              // [S, Hq, D]
-    float* lse;                      // [S, Hq]
 };
 
 // The status of a call is gathered with its partial results, so that no launch of its own has to reset the workspace's word before
@@ -68,8 +66,16 @@ __device__ __forceinline__ void decode_header(const DecodeParams& p) {
 // finish, with counts in the workspace, cost every CTA a fence and an atomic and the merge its parallelism (a step in a CUDA
 // graph, merge in the last CTA -> here, us: 1 x 24000 tokens with 8 heads on 1 29.6 -> 15.0, 1 x 2000 with 32 on 8 14.2 -> 12.7,
 // 100 x 300 with 8 on 8 and head_dim 64 17.4 -> 13.5; launched call by call 30.4 -> 15.8, 14.6 -> 13.3, 17.9 -> 13.8).
+struct MergeParams {
+    const float* part_o;
+    const float* part_ml;
+    __nv_bfloat16* out;
+    float* lse;
+    int32_t* header;
+    int rows, nsplit;
+};
 template <int D, int PART>
-__device__ __forceinline__ void decode_merge_row(const DecodeParams& p, size_t row, int lane) {
+__device__ __forceinline__ void decode_merge_row(const MergeParams& p, size_t row, int lane) {
     constexpr int PER = D / 32;
     const float2* ml = reinterpret_cast<const float2*>(p.part_ml) + row * p.nsplit;
     const float* po = p.part_o + row * p.nsplit * D + lane * PER;
@@ -119,10 +125,10 @@ __device__ __forceinline__ void decode_merge_row(const DecodeParams& p, size_t r
     if (lane == 0) p.lse[row] = (L > 0.f) ? M * 0.6931471805599453f + logf(L) : -INFINITY;
 }
 template <int D, int PART>
-__global__ void __launch_bounds__(256) decode_merge_kernel(DecodeParams p) {
+__global__ void __launch_bounds__(256) decode_merge_kernel(MergeParams p) {
     pdl_wait();
     const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (row < p.S * p.Hq) decode_merge_row<D, PART>(p, row, threadIdx.x & 31);
+    if (row < p.rows) decode_merge_row<D, PART>(p, row, threadIdx.x & 31);
 }
 
 // A block-table entry is only followed if it names a page of the cache: anything else (a stale or
@@ -974,7 +980,7 @@ static int launch_decode_tc(const CUtensorMap& tk, const CUtensorMap& tv, const 
 }
 
 template <int D>
-static int launch_decode(const DecodeParams& p, int G, const void* k_cache, const void* v_cache, cudaStream_t st) {
+static int launch_decode(const DecodeParams& p, int G, const void* k_cache, const void* v_cache, __nv_bfloat16* out, float* lse, cudaStream_t st) {
     dim3 grid(p.nsplit, p.Hkv, p.S);
     const int ps = p.page_size;
     // tensor-core variant (head_dim 128).  Pages that are whole 8-row swizzle atoms and tile 128 tokens exactly come in
@@ -1027,9 +1033,8 @@ static int launch_decode(const DecodeParams& p, int G, const void* k_cache, cons
         }
         if (rc != KVS_OK) return rc;
     }
-    const long long rows = (long long)p.S * p.Hq;
-    const unsigned blocks = (unsigned)((rows + 7) / 8);
-    return p.nsplit <= 4 ? launch_after(decode_merge_kernel<D, 4>, blocks, 256, 0, st, p) : launch_after(decode_merge_kernel<D, 16>, blocks, 256, 0, st, p);
+    const MergeParams m = {p.part_o, p.part_ml, out, lse, p.header, p.S * p.Hq, p.nsplit};
+    return launch_after(p.nsplit <= 4 ? decode_merge_kernel<D, 4> : decode_merge_kernel<D, 16>, (m.rows + 7) / 8, 256, 0, st, m);
 }
 
 extern "C" int kvs_decode_attn(const void* q, const void* k_cache, const void* v_cache, const int32_t* block_table,
@@ -1067,7 +1072,6 @@ extern "C" int kvs_decode_attn(const void* q, const void* k_cache, const void* v
     p.part_o = (float*)((char*)workspace + DEC_WS_HEADER);
     p.part_ml = p.part_o + (size_t)num_seqs * Hq * num_splits * head_dim;
     cudaStream_t st = (cudaStream_t)stream;
-    p.out = (__nv_bfloat16*)out;
-    p.lse = lse;
-    return head_dim == 64 ? launch_decode<64>(p, Hq / Hkv, k_cache, v_cache, st) : launch_decode<128>(p, Hq / Hkv, k_cache, v_cache, st);
+    return head_dim == 64 ? launch_decode<64>(p, Hq / Hkv, k_cache, v_cache, (__nv_bfloat16*)out, lse, st)
+                          : launch_decode<128>(p, Hq / Hkv, k_cache, v_cache, (__nv_bfloat16*)out, lse, st);
 }
