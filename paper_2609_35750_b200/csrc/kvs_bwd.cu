@@ -340,7 +340,8 @@ template <int D>
 __global__ void __launch_bounds__(BWD_THREADS, 1)
 bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
            const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_do,
-           const __grid_constant__ CUtensorMap tm_dq, MetaView mv, BwdParams p) {
+           const __grid_constant__ CUtensorMap tm_dq, const __grid_constant__ MetaView mv,
+           const __grid_constant__ BwdParams p) {
     using L = BwdSmem<D>;
     constexpr int NBOX = D / 64;
     constexpr int BOX_BYTES = TILE * 128;
@@ -704,9 +705,9 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         // ---- epilogue: dK, dV of this key block, once every MMA has completed ----
         mbar_wait(bar_qfree((n_iter - 1) & 1), ((n_iter - 1) >> 1) & 1, abort_flag, status);
         tc_fence_after();
-        const bool kvalid = kj < T;
-        const size_t orow = (size_t)(tok0 + kj) * (size_t)p.dkv_ts + (size_t)g * D + half * HALF_D;
-        bwd_epilogue<D>(p, work->cut, g, 1, 0, tmem_dK + lane_sel + half * HALF_D, tmem_dV + lane_sel + half * HALF_D, row, half, kvalid, orow,
+        // through the memory of K and V, which nothing reads any more
+        bwd_epilogue<D>(p, work->cut, g, 1, 0, tmem_dK + lane_sel + half * HALF_D, tmem_dV + lane_sel + half * HALF_D, row, half,
+                        tok0 + n * TILE + quad * 32, T - n * TILE - quad * 32, sgen + L::OFF_K + warp * (L::TB / 4),
                         reinterpret_cast<volatile int*>(sgen + L::OFF_MISC + 8));
     }
     tc_fence_before();

@@ -105,41 +105,25 @@ __device__ __forceinline__ void bwd_zero_rows(const BwdParams& p, int tok, int r
     }
 }
 
-// 32 fp32 columns of a dK or dV row from registers to memory, as fp32 or bf16
-__device__ __forceinline__ void bwd_store_cols(void* base, size_t elem, const uint32_t (&r)[32], int grad_fp32) {
-    if (grad_fp32) {
-        float4* dst = reinterpret_cast<float4*>(reinterpret_cast<float*>(base) + elem);
-#pragma unroll
-        for (int e = 0; e < 8; ++e)
-            dst[e] = make_float4(__uint_as_float(r[e * 4]), __uint_as_float(r[e * 4 + 1]), __uint_as_float(r[e * 4 + 2]), __uint_as_float(r[e * 4 + 3]));
-    } else {
-        uint4* dst = reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(base) + elem);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            uint4 w;
-            w.x = pack_bf16(__uint_as_float(r[e * 8 + 0]), __uint_as_float(r[e * 8 + 1]));
-            w.y = pack_bf16(__uint_as_float(r[e * 8 + 2]), __uint_as_float(r[e * 8 + 3]));
-            w.z = pack_bf16(__uint_as_float(r[e * 8 + 4]), __uint_as_float(r[e * 8 + 5]));
-            w.w = pack_bf16(__uint_as_float(r[e * 8 + 6]), __uint_as_float(r[e * 8 + 7]));
-            dst[e] = w;
-        }
-    }
-}
-
 // Epilogue of the 256 compute threads: thread (row, half) has the columns [half * D/2, +D/2) of its row of dK and dV in
-// tensor memory.  A whole item goes straight to memory.  A unit of a cut item writes them to its slot; the item's last unit
+// tensor memory.  A whole item goes straight to memory (`tok`: first token of this warp's 32 rows, `rows`: how many of them the
+// trace has; `stage`: 32 x D/2 fp32 of shared memory of this warp's own).  A unit of a cut item writes them to its slot; the item's last unit
 // adds the slots up in order.  `ctas`: CTAs per item, `cta`: this one's index.
 template <int D>
 __device__ __forceinline__ void bwd_epilogue(const BwdParams& p, int cut, int g, int ctas, int cta, uint32_t tmem_dk, uint32_t tmem_dv, int row,
-                                             int half, bool valid, size_t orow, volatile int* s_last) {
+                                             int half, int tok, int rows, uint8_t* stage, volatile int* s_last) {
     constexpr int CH = D / 64;              // 32-column pieces per thread and tensor
+    using Rows = RowStage<D / 2>;
+    const int lane = threadIdx.x & 31;
+    const size_t elem = (size_t)tok * (size_t)p.dkv_ts + (size_t)g * D + half * (D / 2);
     if (cut == 0) {
 #pragma unroll
         for (int i = 0; i < 2 * CH; ++i) {
             uint32_t r[32];
             tmem_ld32((i < CH ? tmem_dk : tmem_dv) + (i % CH) * 32, r);
             tmem_wait_ld();
-            if (valid) bwd_store_cols(i < CH ? p.dk : p.dv, orow + (i % CH) * 32, r, p.grad_fp32);
+            Rows::put(stage, lane, i % CH, r, p.grad_fp32);
+            if (i % CH == CH - 1) Rows::flush(stage, lane, i < CH ? p.dk : p.dv, elem, (size_t)p.dkv_ts, rows, p.grad_fp32);
         }
         return;
     }
@@ -187,7 +171,8 @@ __device__ __forceinline__ void bwd_epilogue(const BwdParams& p, int cut, int g,
             r[e * 4 + 2] = __float_as_uint(a[e].z);
             r[e * 4 + 3] = __float_as_uint(a[e].w);
         }
-        if (valid) bwd_store_cols(i < CH ? p.dk : p.dv, orow + (i % CH) * 32, r, p.grad_fp32);
+        Rows::put(stage, lane, i % CH, r, p.grad_fp32);
+        if (i % CH == CH - 1) Rows::flush(stage, lane, i < CH ? p.dk : p.dv, elem, (size_t)p.dkv_ts, rows, p.grad_fp32);
     }
 }
 

@@ -128,7 +128,8 @@ __host__ __device__ constexpr uint32_t pair_idesc(int m, int n, int a_mn_major, 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(BWD_THREADS, 1)
 bwd_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                 const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_do,
-                const __grid_constant__ CUtensorMap tm_dq, MetaView mv, BwdParams p) {
+                const __grid_constant__ CUtensorMap tm_dq, const __grid_constant__ MetaView mv,
+                const __grid_constant__ BwdParams p) {
     using L = PairSmem;
     constexpr uint32_t TMEM_COLS = 512;
     constexpr uint32_t IDESC_ST = pair_idesc(256, 128, 0, 0);    // K-major x K-major, N = 128 queries
@@ -597,9 +598,9 @@ bwd_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         // ---- epilogue: dK, dV of this key block, once every MMA has completed ----
         mbar_wait(bar_done, 0, abort_flag, status);
         tc_fence_after();
-        const bool kvalid = kj < T;
-        const size_t orow = (size_t)(tok0 + kj) * (size_t)p.dkv_ts + (size_t)g * D + half * 64;
-        bwd_epilogue<D>(p, work->cut, g, 2, (int)rank, tmem_dK + lane_sel + half * 64, tmem_dV + lane_sel + half * 64, row, half, kvalid, orow,
+        // through the memory of K and V, which nothing reads any more
+        bwd_epilogue<D>(p, work->cut, g, 2, (int)rank, tmem_dK + lane_sel + half * 64, tmem_dV + lane_sel + half * 64, row, half,
+                        tok0 + n * TILE + quad * 32, T - n * TILE - quad * 32, sgen + L::OFF_K + warp * (TB / 4),
                         reinterpret_cast<volatile int*>(sgen + L::OFF_MISC + 8));
     }
     tc_fence_before();

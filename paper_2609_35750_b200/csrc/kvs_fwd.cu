@@ -45,7 +45,8 @@ struct FwdSmem {
     static constexpr int TB = TILE * D * 2;
     static constexpr int OFF_Q = 0;                      // 2 query tiles
     static constexpr int OFF_KV = 2 * TB;                // 2 stages x (K, V)
-    static constexpr int OFF_EV = OFF_KV + 4 * TB;       // 2 stages x 128 int32: eviction step of the stage's key slots
+    static constexpr int OFF_STG = OFF_KV + 4 * TB;      // chained: 32 rows x 32 columns of out per softmax warp
+    static constexpr int OFF_EV = OFF_STG + 8 * 2048;    // 2 stages x 128 int32: eviction step of the stage's key slots
     static constexpr int OFF_KF = OFF_EV + 2 * TILE * 4; // 2 stages x 128 int32: first query that may see the slot
     static constexpr int OFF_FLAG = OFF_KF + 2 * TILE * 4;   // 2 stages x (compare, hidden)
     static constexpr int OFF_BAR = OFF_FLAG + 16;
@@ -73,7 +74,7 @@ struct FwdParams {
 template <int D, bool CHAIN>
 __global__ void __launch_bounds__(FWD_THREADS, 1)
 fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
-           const __grid_constant__ CUtensorMap tm_v, MetaView mv, FwdParams p) {
+           const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ MetaView mv, const __grid_constant__ FwdParams p) {
     using L = FwdSmem<D>;
     constexpr int NBOX = D / 64;             // 64-column TMA boxes per tile row
     constexpr int BOX_BYTES = TILE * 128;    // 128 rows x 128 bytes
@@ -660,7 +661,13 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
             }
             if (!dual || t == 0) {
                 const float inv = (run_sum > 0.f && nlist > 0) ? 1.f / run_sum : 0.f;
-                __nv_bfloat16* orow = p.out + ((size_t)(tok0 + qi) * p.Hq + h) * D;
+                // Through shared memory to memory as whole rows: the whole row through the query tile, which no product reads any
+                // more, or, where the next item's comes there, in pieces of 64 bytes through memory of its own.
+                constexpr int COLS = CHAIN ? 32 : D;
+                using Rows = RowStage<COLS>;
+                uint8_t* stage = sgen + (CHAIN ? L::OFF_STG + warp * 2048 : L::OFF_Q + warp * (L::TB / 4));
+                __nv_bfloat16* orow = p.out + ((size_t)(tok0 + m * TILE + quad * 32) * p.Hq + h) * D;
+                const int rows = T - m * TILE - quad * 32;
 #pragma unroll
                 for (int c = 0; c < D / 32; ++c) {
                     uint32_t r[32];
@@ -678,18 +685,11 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
                             r[e] = __float_as_uint(o);
                         }
                     }
-                    if (valid) {
-                        uint4* dst = reinterpret_cast<uint4*>(orow + c * 32);
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            uint4 w;
-                            w.x = pack_bf16(__uint_as_float(r[e * 8 + 0]) * inv, __uint_as_float(r[e * 8 + 1]) * inv);
-                            w.y = pack_bf16(__uint_as_float(r[e * 8 + 2]) * inv, __uint_as_float(r[e * 8 + 3]) * inv);
-                            w.z = pack_bf16(__uint_as_float(r[e * 8 + 4]) * inv, __uint_as_float(r[e * 8 + 5]) * inv);
-                            w.w = pack_bf16(__uint_as_float(r[e * 8 + 6]) * inv, __uint_as_float(r[e * 8 + 7]) * inv);
-                            dst[e] = w;
-                        }
-                    }
+                    for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) * inv);
+                    Rows::put(stage, lane, c % (COLS / 32), r, 0);
+                    if ((c + 1) % (COLS / 32) == 0)
+                        Rows::flush(stage, lane, orow, CHAIN ? c * 32 : 0, (size_t)p.Hq * D, rows, 0);
                 }
                 if (valid) p.lse[(size_t)h * p.total_tokens + tok0 + qi] = ref_max * 0.6931471805599453f + logf(run_sum);
             }
