@@ -13,6 +13,7 @@
 namespace kvs {
 
 constexpr int BWD_SMS = 148;
+constexpr uint32_t BWD_LATE = 3;              // tiles left of a unit when the CTA asks for the next one
 constexpr int BWD_MIN_UNIT = 4;             // tiles: a shorter unit is mostly its own start and end
 constexpr int BWD_MAX_SLOTS = 2 * BWD_SMS;  // slots of one CTA each for the dK and dV of cut items, over all KV heads
 
@@ -304,8 +305,8 @@ __global__ void bwd_cast_kernel(const float* __restrict__ acc, __nv_bfloat16* __
 //               reduce-add into the fp32 accumulator (global `red` instructions are processed at
 //               about one thread per clock per SM, which alone would exceed the MMA time of a tile)
 //   warp 12     producer (TMA for K, V, Q, dO; plain loads for lse and D)
-//   warp 13     MMA issuer;   warps 14-15 idle (they only complete the warp group)
-// Registers are re-balanced per warp group with setmaxnreg (compute 144, drain 136, the rest 88).
+//   warp 13     MMA issuer;   warp 14  list of units;   warp 15 idle (it only completes the warp group)
+// Registers are re-balanced per warp group with setmaxnreg (compute 144, drain 144, the rest 80).
 //
 // Tensor memory (512 columns):  [0,128) S^T fp32, then P^T bf16 in [0,32) and [64,96)
 //                               [128,256) dP^T fp32, then dQ fp32
@@ -314,6 +315,13 @@ __global__ void bwd_cast_kernel(const float* __restrict__ acc, __nv_bfloat16* __
 //     dP^T(j) = V dO^T,  dV(j) += P^T dO,  S^T(j+1) = K Q^T,  dQ(j) = dS K,  dK(j) += dS^T Q
 // while the compute warps run  dS(j), P(j+1)  and the drain warps empty dQ(j).  The softmax scale
 // is folded into dS (dS = P (scale dP - scale D)), so dK and dQ leave the tensor core scaled.
+// A CTA goes on with units of CTAs that have not started (cluster launch control).  Barriers run on across units, so that the
+// next unit's K, V, Q and dO arrive and its first products run while the compute warps write out the last one's dK and dV and
+// the last dQ is added; only what the last products read is waited for.  With a CTA per unit the launch, the chain of metadata
+// loads, the set-up, the first loads, the write-out and the wait for the last adds stood beside the tiles: 12 of 138 us a unit on
+// 12 traces of 1500 to 12000 tokens, 13 of 56 on 96 of 60 to 900.  Main kernel, a CTA per unit -> chained, us: 123 traces of 199
+// to 350, 16 heads on 4, head_dim 64 211 -> 189; 40 of 100 to 1000, 4 on 4, head_dim 64 60.7 -> 51.3; 20 of 500 to 2000, 32 on 8
+// 645 -> 610; 3 of 14000 with nothing evicted 12350 -> 11880.
 // Rows of a dQ tile past the end of a trace are exactly zero (their P is zero), so the reduce-add
 // of a whole 128-row box is harmless where it overlaps the next trace.
 template <int D>
@@ -329,9 +337,10 @@ struct BwdSmem {
     static constexpr int OFF_LSE = OFF_STG + 2 * STG_BYTES;    // 2 stages x 128 fp32: -lse * log2 e
     static constexpr int OFF_DVEC = OFF_LSE + 2 * TILE * 4;    // 2 stages x 128 fp32: -D * scale
     static constexpr int OFF_BAR = OFF_DVEC + 2 * TILE * 4;
-    static constexpr int OFF_MISC = OFF_BAR + 16 * 8;          // tmem base, abort flag
-    static constexpr int OFF_WORK = OFF_MISC + 16;
-    static constexpr int TOTAL = OFF_WORK + (int)sizeof(BwdWork);
+    static constexpr int OFF_MISC = OFF_BAR + 22 * 8;          // tmem base, abort flag
+    static constexpr int OFF_ASK = OFF_MISC + 16;              // the answer of the launch control
+    static constexpr int OFF_WORK = OFF_ASK + 16;              // 2 slots
+    static constexpr int TOTAL = OFF_WORK + 2 * (int)sizeof(BwdWork);
     static constexpr int MAX_DYN = 232448;                     // 227 KB
     static constexpr int DYN_BYTES = (TOTAL + 1024 > MAX_DYN) ? MAX_DYN : TOTAL + 1024;
 };
@@ -362,28 +371,8 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         if (tid == 0 && blockIdx.x == 0) set_status(p.status, KVS_ERR_BAD_META);
         return;
     }
-    BwdWork w;
-    {
-        BwdUnit unit;
-        if (!bwd_unit_of(p, mv.bwd_order, mv.hdr->nblk_total, blockIdx.x, unit, w.g)) return;
-        const int b = mv.blk_trace[unit.block], G = p.Hq / p.Hkv;
-        w.n = unit.block - mv.blk_off[b];
-        w.tok0 = mv.seq_start[b];
-        w.T = mv.seq_start[b + 1] - w.tok0;
-        w.m_first = mv.col_first[unit.block];           // == n unless the key slots were re-ordered
-        w.m_last = mv.col_last[unit.block];
-        w.general = mv.hdr->general != 0;
-        const int nm = w.m_last - w.m_first + 1;        // query blocks m_first .. m_last can see this key block
-        if (nm <= 0) {
-            // no query sees any key of the block (general metadata only): its gradients are zero
-            bwd_zero_rows<D>(p, w.tok0 + w.n * TILE, min(TILE, w.T - w.n * TILE), w.g);
-            return;
-        }
-        w.n_iter = (unit.tile1 < 0 ? G * nm : unit.tile1) - unit.tile0;     // of the G * nm (head, query block) tiles of the key block
-        w.h_start = w.g * G + unit.tile0 / nm;
-        w.m_start = w.m_first + unit.tile0 % nm;
-        w.cut = unit.cut;
-    }
+    const int n_items = mv.hdr->nblk_total;
+    if (!bwd_has_unit(p, n_items, blockIdx.x)) return;
     int32_t* status = p.status;
 
     const uint32_t sraw = smem_u32(smem_raw);
@@ -405,6 +394,11 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     const uint32_t bar_dofull = bars + 8 * 7, bar_dofree = bars + 8 * 8, bar_s = bars + 8 * 9, bar_dp = bars + 8 * 10,
                    bar_p = bars + 8 * 11, bar_dq = bars + 8 * 13, bar_drained = bars + 8 * 14,
                    bar_dss = bars + 8 * 15;
+    auto bar_work = [&](int s) { return bars + 8 * (16 + s); };      // unit written
+    auto bar_workfree = [&](int s) { return bars + 8 * (18 + s); };  // unit done by the producer, MMA, 4 drain and 8 compute warps
+    const uint32_t bar_ask = bars + 8 * 12;                           // the launch control has answered
+    const uint32_t bar_late = bars + 8 * 20;                          // the MMA warp is near the end of a unit
+    volatile BwdWork* s_work = reinterpret_cast<volatile BwdWork*>(sgen + L::OFF_WORK);
 
     if (tid == 0) {
         *abort_flag = 0;
@@ -413,6 +407,8 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
             mbar_init(bar_qfull(s), 1);
             mbar_init(bar_ldfull(s), 32);
             mbar_init(bar_qfree(s), 1);
+            mbar_init(bar_work(s), 1);
+            mbar_init(bar_workfree(s), 14);
         }
         mbar_init(bar_dofull, 1);
         mbar_init(bar_dofree, 1);
@@ -422,68 +418,152 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         mbar_init(bar_dss, 8);
         mbar_init(bar_dq, 1);
         mbar_init(bar_drained, 4);
+        mbar_init(bar_ask, 1);
+        mbar_init(bar_late, 1);
         fence_mbar_init();
     }
     if (warp == 13) {
         tmem_alloc(smem_u32(s_tmem_base), TMEM_COLS);
         tmem_relinquish();
     }
-    if (tid == 0) *reinterpret_cast<BwdWork*>(sgen + L::OFF_WORK) = w;
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *s_tmem_base;
-    const volatile BwdWork* work = reinterpret_cast<const volatile BwdWork*>(sgen + L::OFF_WORK);
-    const int n = work->n, tok0 = work->tok0, T = work->T, m_first = work->m_first, m_last = work->m_last;
-    const int h_start = work->h_start, m_start = work->m_start, n_iter = work->n_iter, g = work->g;
+    // The r-th unit of the CTA; false: there is none.  A role reads what it needs of it and arrives at the end of it.
+    auto take = [&](int r) {
+        mbar_wait(bar_work(r & 1), (r >> 1) & 1, abort_flag, status);
+        return s_work[r & 1].n_iter >= 0 && !*abort_flag;
+    };
+    auto done = [&](int r) {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_workfree(r & 1));
+    };
     const uint32_t tmem_S = tmem;
     const uint32_t tmem_P = tmem + 128;
     const uint32_t tmem_dV = tmem + 256;
     const uint32_t tmem_dK = tmem + 384;
 
     if (warp >= 12) {
-        reg_dec<88>();
+        reg_dec<80>();
         if (warp == 12) {
             // ================= producer =================
             float* sLse = reinterpret_cast<float*>(sgen + L::OFF_LSE);
             float* sDv = reinterpret_cast<float*>(sgen + L::OFF_DVEC);
-            if (lane == 0) {
-                mbar_expect_tx(bar_kv, 2 * L::TB);
-                for (int c = 0; c < NBOX; ++c) tma_load_3d(sK + c * BOX_BYTES, &tm_k, c * 64, g, tok0 + n * TILE, bar_kv);
-                for (int c = 0; c < NBOX; ++c) tma_load_3d(sV + c * BOX_BYTES, &tm_v, c * 64, g, tok0 + n * TILE, bar_kv);
-            }
-            int h = h_start, m = m_start;
-            for (int j = 0; j < n_iter; ++j) {
-                const int s = j & 1;
-                const int qtok = tok0 + m * TILE;
-                // Q(j), lse(j), D(j): stage s, free once every MMA of iteration j-2 has completed
-                if (j >= 2) mbar_wait(bar_qfree(s), ((j >> 1) + 1) & 1, abort_flag, status);
-                if (lane == 0) {
-                    mbar_expect_tx(bar_qfull(s), L::TB);
-                    for (int c = 0; c < NBOX; ++c) tma_load_3d(sQ + s * L::TB + c * BOX_BYTES, &tm_q, c * 64, h, qtok, bar_qfull(s));
+            uint32_t J = 0;                                     // tiles of the CTA so far
+            for (int r = 0; take(r); ++r) {
+                const volatile BwdWork* work = s_work + (r & 1);
+                const int tok0 = work->tok0, T = work->T, m_first = work->m_first, m_last = work->m_last, g = work->g;
+                const uint32_t end = J + work->n_iter;
+                int h = work->h_start, m = work->m_start;
+                auto load_q = [&](uint32_t J, int h, int qtok) {
+                    // Q(J): stage s, free once every MMA of tile J-2 has completed
+                    const int s = J & 1;
+                    if (J >= 2) mbar_wait(bar_qfree(s), ((J >> 1) + 1) & 1, abort_flag, status);
+                    if (lane == 0) {
+                        mbar_expect_tx(bar_qfull(s), L::TB);
+                        for (int c = 0; c < NBOX; ++c) tma_load_3d(sQ + s * L::TB + c * BOX_BYTES, &tm_q, c * 64, h, qtok, bar_qfull(s));
+                    }
+                };
+                if (J < end) {
+                    load_q(J, h, tok0 + m * TILE);
+                    // K is last read by the last unit's last dQ product, V before that
+                    if (J > 0) mbar_wait(bar_dq, (J - 1) & 1, abort_flag, status);
+                    if (lane == 0) {
+                        const int ktok = tok0 + work->n * TILE;
+                        mbar_expect_tx(bar_kv, 2 * L::TB);
+                        for (int c = 0; c < NBOX; ++c) tma_load_3d(sK + c * BOX_BYTES, &tm_k, c * 64, g, ktok, bar_kv);
+                        for (int c = 0; c < NBOX; ++c) tma_load_3d(sV + c * BOX_BYTES, &tm_v, c * 64, g, ktok, bar_kv);
+                    }
                 }
-                const size_t rowbase = (size_t)h * p.total_tokens + qtok;
+                for (const uint32_t first = J; J < end; ++J) {
+                    const int s = J & 1;
+                    const int qtok = tok0 + m * TILE;
+                    if (J != first) load_q(J, h, qtok);
+                    // lse(J), D(J): beside Q
+                    const size_t rowbase = (size_t)h * p.total_tokens + qtok;
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int i = lane * 4 + u;
-                    const bool qv = (m * TILE + i) < T;
-                    // stored negated (they are subtracted with one fused multiply-add); -inf makes P vanish
-                    // for the rows past the end of the trace
-                    sLse[s * TILE + i] = qv ? p.lse[rowbase + i] * -1.4426950408889634f : -INFINITY;
-                    sDv[s * TILE + i] = qv ? p.dvec[rowbase + i] * -p.scale : 0.f;
+                    for (int u = 0; u < 4; ++u) {
+                        const int i = lane * 4 + u;
+                        const bool qv = (m * TILE + i) < T;
+                        // stored negated (they are subtracted with one fused multiply-add); -inf makes P vanish
+                        // for the rows past the end of the trace
+                        sLse[s * TILE + i] = qv ? p.lse[rowbase + i] * -1.4426950408889634f : -INFINITY;
+                        sDv[s * TILE + i] = qv ? p.dvec[rowbase + i] * -p.scale : 0.f;
+                    }
+                    mbar_arrive(bar_ldfull(s));
+                    // dO(J): single buffer, free once dP(J-1) and dV(J-1) have completed
+                    if (lane == 0) {
+                        if (J >= 1) mbar_wait(bar_dofree, (J - 1) & 1, abort_flag, status);
+                        mbar_expect_tx(bar_dofull, L::TB);
+                        for (int c = 0; c < NBOX; ++c) tma_load_3d(sDO + c * BOX_BYTES, &tm_do, c * 64, h, qtok, bar_dofull);
+                    }
+                    __syncwarp();
+                    if (++m > m_last) {
+                        m = m_first;
+                        ++h;
+                    }
                 }
-                mbar_arrive(bar_ldfull(s));
-                // dO(j): single buffer, free once dP(j-1) and dV(j-1) have completed
+                done(r);
+            }
+            if (*abort_flag) {                            // a wait gave up: let the copies in flight land, then leave
+                const long long t0 = clock64();
+                while (clock64() - t0 < 2000000) {}
+            }
+        } else if (warp == 14) {
+            // ================= list of units =================
+            // The first one is the CTA's own; after it units of CTAs of the grid that have not started, asked for a few tiles
+            // before the end of the one before: what is asked for and found (about 3 us) lies beside those tiles, and the last
+            // units still go to whoever is free first.
+            int x = blockIdx.x;
+            bool ok = true;
+            for (int r = 0; ; ++r) {
+                if (r > 0) {
+                    mbar_wait(bar_late, (r - 1) & 1, abort_flag, status);
+                    if (*abort_flag) break;               // nothing is asked for that would not be waited for
+                    if (lane == 0) {
+                        mbar_expect_tx(bar_ask, 16);
+                        ask_for_cta(sbase + L::OFF_ASK, bar_ask);
+                    }
+                    mbar_wait(bar_ask, (r - 1) & 1, abort_flag, status);
+                    int y;
+                    ok = cta_answer(sbase + L::OFF_ASK, x, y) && !*abort_flag;
+                    fence_proxy_async();                  // the answer is read before the next one comes over it
+                    __syncwarp();
+                }
+                BwdWork w;
+                w.n = w.tok0 = w.T = w.m_first = w.m_last = w.h_start = w.m_start = w.g = w.cut = w.general = w.pad = 0;
+                w.n_iter = -1;
+                BwdUnit unit;
+                if (ok && bwd_unit_of(p, mv.bwd_order, n_items, x, unit, w.g)) {
+                    const int b = mv.blk_trace[unit.block], G = p.Hq / p.Hkv;
+                    w.n = unit.block - mv.blk_off[b];
+                    w.tok0 = mv.seq_start[b];
+                    w.T = mv.seq_start[b + 1] - w.tok0;
+                    w.m_first = mv.col_first[unit.block];           // == n unless the key slots were re-ordered
+                    w.m_last = mv.col_last[unit.block];
+                    w.general = mv.hdr->general != 0;
+                    const int nm = w.m_last - w.m_first + 1;        // query blocks m_first .. m_last can see this key block
+                    if (nm <= 0) {
+                        w.n_iter = 0;                               // no query sees any key of the block (general metadata only)
+                    } else {
+                        w.n_iter = (unit.tile1 < 0 ? G * nm : unit.tile1) - unit.tile0;     // of the G * nm (head, query block) tiles
+                        w.h_start = w.g * G + unit.tile0 / nm;
+                        w.m_start = w.m_first + unit.tile0 % nm;
+                    }
+                    w.cut = unit.cut;
+                }
+                const int slot = r & 1;
+                if (r >= 2) mbar_wait(bar_workfree(slot), ((r >> 1) + 1) & 1, abort_flag, status);
                 if (lane == 0) {
-                    if (j >= 1) mbar_wait(bar_dofree, (j - 1) & 1, abort_flag, status);
-                    mbar_expect_tx(bar_dofull, L::TB);
-                    for (int c = 0; c < NBOX; ++c) tma_load_3d(sDO + c * BOX_BYTES, &tm_do, c * 64, h, qtok, bar_dofull);
+                    volatile int* dst = reinterpret_cast<volatile int*>(s_work + slot);
+                    const int* src = reinterpret_cast<const int*>(&w);
+#pragma unroll
+                    for (int i = 0; i < (int)(sizeof(BwdWork) / 4); ++i) dst[i] = src[i];
+                    mbar_arrive(bar_work(slot));
                 }
                 __syncwarp();
-                if (++m > m_last) {
-                    m = m_first;
-                    ++h;
-                }
+                if (w.n_iter < 0 || *abort_flag) break;
             }
         } else if (warp == 13) {
             // ================= MMA issuer (all lanes walk the loop, one elected lane issues) =================
@@ -495,110 +575,134 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
             const uint64_t dDS_k = smem_desc(sDS, 16, 1024);
             const uint64_t dQ_mn = smem_desc(sQ, BOX_BYTES, 1024), dDO_mn = smem_desc(sDO, BOX_BYTES, 1024);
             constexpr uint64_t STAGE = (uint64_t)(L::TB >> 4);
-            mbar_wait(bar_kv, 0, abort_flag, status);
-            mbar_wait(bar_qfull(0), 0, abort_flag, status);
-            tc_fence_after();
-#pragma unroll
-            for (int kk = 0; kk < D / 16; ++kk) {
-                const uint64_t off = (uint64_t)(((kk >> 2) * BOX_BYTES + (kk & 3) * 32) >> 4);
-                if (leader) mma_ss(tmem_S, dK_k + off, dQ_k + off, IDESC_ST, kk > 0);
-            }
-            if (leader) mma_commit(bar_s);
-            for (int j = 0; j < n_iter; ++j) {
-                const int s = j & 1;
-                const uint32_t ph = j & 1;
-                const uint64_t so = s ? STAGE : 0;
-                // dP^T(j) = V dO^T  (its columns hold dQ(j-1) until the drain warps have read it)
-                mbar_wait(bar_dofull, ph, abort_flag, status);
-                if (j > 0) mbar_wait(bar_drained, (j - 1) & 1, abort_flag, status);
-                tc_fence_after();
-#pragma unroll
-                for (int kk = 0; kk < D / 16; ++kk) {
-                    const uint64_t off = (uint64_t)(((kk >> 2) * BOX_BYTES + (kk & 3) * 32) >> 4);
-                    if (leader) mma_ss(tmem_P, dV_k + off, dDO_k + off, IDESC_ST, kk > 0);
+            uint32_t J = 0;                                     // tiles of the CTA so far
+            int loads = 0;                                      // units with tiles so far
+            for (int r = 0; take(r); ++r) {
+                const uint32_t first = J, end = J + s_work[r & 1].n_iter;
+                if (first == end) {
+                    if (lane == 0) mbar_arrive(bar_late);
+                    done(r);
+                    continue;
                 }
-                if (leader) mma_commit(bar_dp);
-                // dV(j) += P^T dO
-                mbar_wait(bar_p, ph, abort_flag, status);
+                mbar_wait(bar_kv, loads & 1, abort_flag, status);
+                ++loads;
+                mbar_wait(bar_qfull(J & 1), (J >> 1) & 1, abort_flag, status);
                 tc_fence_after();
+                {
+                    const uint64_t so = J & 1 ? STAGE : 0;
 #pragma unroll
-                for (int kk = 0; kk < TILE / 16; ++kk)
-                    if (leader) mma_ts(tmem_dV, tmem_S + (kk >> 2) * 64 + (kk & 3) * 8, dDO_mn + (uint64_t)(kk * 128), IDESC_KV,
-                           (j > 0) || (kk > 0));
-                if (leader) mma_commit(bar_dofree);
-                // S^T(j+1) = K Q^T
-                if (j + 1 < n_iter) {
-                    const uint64_t so1 = s ? 0 : STAGE;
-                    mbar_wait(bar_qfull(s ^ 1), ((j + 1) >> 1) & 1, abort_flag, status);
+                    for (int kk = 0; kk < D / 16; ++kk) {
+                        const uint64_t off = (uint64_t)(((kk >> 2) * BOX_BYTES + (kk & 3) * 32) >> 4);
+                        if (leader) mma_ss(tmem_S, dK_k + off, dQ_k + so + off, IDESC_ST, kk > 0);
+                    }
+                }
+                if (leader) mma_commit(bar_s);
+                for (; J < end; ++J) {
+                    const int s = J & 1;
+                    const uint32_t ph = J & 1;
+                    const uint64_t so = s ? STAGE : 0;
+                    if (lane == 0 && (J + BWD_LATE == end || (J == first && end - first < BWD_LATE))) mbar_arrive(bar_late);
+                    // dP^T(J) = V dO^T  (its columns hold dQ(J-1) until the drain warps have read it)
+                    mbar_wait(bar_dofull, ph, abort_flag, status);
+                    if (J > 0) mbar_wait(bar_drained, (J - 1) & 1, abort_flag, status);
                     tc_fence_after();
 #pragma unroll
                     for (int kk = 0; kk < D / 16; ++kk) {
                         const uint64_t off = (uint64_t)(((kk >> 2) * BOX_BYTES + (kk & 3) * 32) >> 4);
-                        if (leader) mma_ss(tmem_S, dK_k + off, dQ_k + so1 + off, IDESC_ST, kk > 0);
+                        if (leader) mma_ss(tmem_P, dV_k + off, dDO_k + off, IDESC_ST, kk > 0);
                     }
-                    if (leader) mma_commit(bar_s);
-                }
-                // dQ(j) = dS K, then dK(j) += dS^T Q.  Both read dS from shared memory: the same swizzled buffer
-                // is the MN-major A operand of dQ (queries contiguous) and, read as [keys x queries] rows, the
-                // K-major A operand of dK; dQ goes first so that the drain can start while dK still runs.
-                mbar_wait(bar_dss, ph, abort_flag, status);
-                tc_fence_after();
+                    if (leader) mma_commit(bar_dp);
+                    // dV(J) += P^T dO.  A unit's first one overwrites the last unit's dV (and dK later on): the compute warps
+                    // have read both out before they write this tile's P.
+                    mbar_wait(bar_p, ph, abort_flag, status);
+                    tc_fence_after();
 #pragma unroll
-                for (int kk = 0; kk < TILE / 16; ++kk)
-                    if (leader) mma_ss(tmem_P, dDS_mn + (uint64_t)(kk * 128), dK_mn + (uint64_t)(kk * 128), IDESC_DQ, kk > 0);
-                if (leader) mma_commit(bar_dq);
+                    for (int kk = 0; kk < TILE / 16; ++kk)
+                        if (leader) mma_ts(tmem_dV, tmem_S + (kk >> 2) * 64 + (kk & 3) * 8, dDO_mn + (uint64_t)(kk * 128), IDESC_KV,
+                               (J != first) || (kk > 0));
+                    if (leader) mma_commit(bar_dofree);
+                    // S^T(J+1) = K Q^T
+                    if (J + 1 < end) {
+                        const uint64_t so1 = s ? 0 : STAGE;
+                        mbar_wait(bar_qfull(s ^ 1), ((J + 1) >> 1) & 1, abort_flag, status);
+                        tc_fence_after();
 #pragma unroll
-                for (int kk = 0; kk < TILE / 16; ++kk) {
-                    const uint64_t off = (uint64_t)(((kk >> 2) * BOX_BYTES + (kk & 3) * 32) >> 4);
-                    if (leader) mma_ss(tmem_dK, dDS_k + off, dQ_mn + so + (uint64_t)(kk * 128), IDESC_KV, (j > 0) || (kk > 0));
+                        for (int kk = 0; kk < D / 16; ++kk) {
+                            const uint64_t off = (uint64_t)(((kk >> 2) * BOX_BYTES + (kk & 3) * 32) >> 4);
+                            if (leader) mma_ss(tmem_S, dK_k + off, dQ_k + so1 + off, IDESC_ST, kk > 0);
+                        }
+                        if (leader) mma_commit(bar_s);
+                    }
+                    // dQ(J) = dS K, then dK(J) += dS^T Q.  Both read dS from shared memory: the same swizzled buffer
+                    // is the MN-major A operand of dQ (queries contiguous) and, read as [keys x queries] rows, the
+                    // K-major A operand of dK; dQ goes first so that the drain can start while dK still runs.
+                    mbar_wait(bar_dss, ph, abort_flag, status);
+                    tc_fence_after();
+#pragma unroll
+                    for (int kk = 0; kk < TILE / 16; ++kk)
+                        if (leader) mma_ss(tmem_P, dDS_mn + (uint64_t)(kk * 128), dK_mn + (uint64_t)(kk * 128), IDESC_DQ, kk > 0);
+                    if (leader) mma_commit(bar_dq);
+#pragma unroll
+                    for (int kk = 0; kk < TILE / 16; ++kk) {
+                        const uint64_t off = (uint64_t)(((kk >> 2) * BOX_BYTES + (kk & 3) * 32) >> 4);
+                        if (leader) mma_ss(tmem_dK, dDS_k + off, dQ_mn + so + (uint64_t)(kk * 128), IDESC_KV, (J != first) || (kk > 0));
+                    }
+                    if (leader) mma_commit(bar_qfree(s));
                 }
-                if (leader) mma_commit(bar_qfree(s));
+                done(r);
             }
         }
     } else if (warp >= 8) {
         // ================= drain warps: dQ(j), query rows on lanes =================
-        reg_inc<136>();
+        reg_inc<144>();
         const int quad = warp & 3;
         const int row = quad * 32 + lane;
         const uint32_t lane_sel = (uint32_t)(quad * 32) << 16;
         uint8_t* stg_row = sgen + L::OFF_STG + row * 128;
-        int h = h_start, m = m_start;
-        for (int j = 0; j < n_iter; ++j) {
-            mbar_wait(bar_dq, j & 1, abort_flag, status);
-            tc_fence_after();
-            uint32_t r[D];
-#pragma unroll
-            for (int ch = 0; ch < D / 32; ++ch) {
-                uint32_t t[32];
-                tmem_ld32(tmem_P + lane_sel + ch * 32, t);
-#pragma unroll
-                for (int e = 0; e < 32; ++e) r[ch * 32 + e] = t[e];
-            }
-            tmem_wait_ld();
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar_drained);      // the columns may be overwritten from here on
-            // chunks of 32 head-dim columns through two staging buffers
-#pragma unroll
-            for (int ch = 0; ch < D / 32; ++ch) {
-                const int buf = ch & 1;
-                if (tid == 256) bulk_wait_read<1>();      // the reduce that last read this buffer has finished reading
-                named_bar_sync(1, 128);
-#pragma unroll
-                for (int c = 0; c < 8; ++c)
-                    *reinterpret_cast<uint4*>(stg_row + buf * L::STG_BYTES + ((c ^ (row & 7)) << 4)) =
-                        make_uint4(r[ch * 32 + c * 4], r[ch * 32 + c * 4 + 1], r[ch * 32 + c * 4 + 2], r[ch * 32 + c * 4 + 3]);
-                fence_proxy_async();
-                named_bar_sync(1, 128);
-                if (tid == 256) {
-                    tma_reduce_add_3d(&tm_dq, ch * 32, h, tok0 + m * TILE, sSTG + buf * L::STG_BYTES);
-                    bulk_commit();
+        uint32_t J = 0;                                         // tiles of the CTA so far
+        for (int r = 0; take(r); ++r) {
+            const volatile BwdWork* work = s_work + (r & 1);
+            const int tok0 = work->tok0, m_first = work->m_first, m_last = work->m_last;
+            const uint32_t end = J + work->n_iter;
+            int h = work->h_start, m = work->m_start;
+            for (; J < end; ++J) {
+                mbar_wait(bar_dq, J & 1, abort_flag, status);
+                tc_fence_after();
+                uint32_t o[D];
+    #pragma unroll
+                for (int ch = 0; ch < D / 32; ++ch) {
+                    uint32_t t[32];
+                    tmem_ld32(tmem_P + lane_sel + ch * 32, t);
+    #pragma unroll
+                    for (int e = 0; e < 32; ++e) o[ch * 32 + e] = t[e];
+                }
+                tmem_wait_ld();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar_drained);      // the columns may be overwritten from here on
+                // chunks of 32 head-dim columns through two staging buffers
+    #pragma unroll
+                for (int ch = 0; ch < D / 32; ++ch) {
+                    const int buf = ch & 1;
+                    if (tid == 256) bulk_wait_read<1>();      // the reduce that last read this buffer has finished reading
+                    named_bar_sync(1, 128);
+    #pragma unroll
+                    for (int c = 0; c < 8; ++c)
+                        *reinterpret_cast<uint4*>(stg_row + buf * L::STG_BYTES + ((c ^ (row & 7)) << 4)) =
+                            make_uint4(o[ch * 32 + c * 4], o[ch * 32 + c * 4 + 1], o[ch * 32 + c * 4 + 2], o[ch * 32 + c * 4 + 3]);
+                    fence_proxy_async();
+                    named_bar_sync(1, 128);
+                    if (tid == 256) {
+                        tma_reduce_add_3d(&tm_dq, ch * 32, h, tok0 + m * TILE, sSTG + buf * L::STG_BYTES);
+                        bulk_commit();
+                    }
+                }
+                if (++m > m_last) {
+                    m = m_first;
+                    ++h;
                 }
             }
-            if (++m > m_last) {
-                m = m_first;
-                ++h;
-            }
+            done(r);
         }
         if (tid == 256) bulk_wait<0>();
     } else {
@@ -609,20 +713,32 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         const int row = quad * 32 + lane;                  // TMEM lane: key row of S^T, dP^T
         const uint32_t lane_sel = (uint32_t)(quad * 32) << 16;
         const int col0 = half * 64;                        // this thread's 64 query columns
-        const int kj = n * TILE + row;
-        // queries [my_first, my_end) of the trace see this key; nobody sees a slot past the trace
-        const int my_end = (kj < T) ? min(mv.evict[tok0 + kj], T) : 0;
-        const int my_first = (work->general && kj < T) ? mv.kfirst[tok0 + kj] : kj;
         const float* sLse = reinterpret_cast<const float*>(sgen + L::OFF_LSE);
         const float* sDv = reinterpret_cast<const float*>(sgen + L::OFF_DVEC);
         uint8_t* sDS_row = sgen + L::OFF_DS + half * BOX_BYTES + row * 128;
         float pv[64];
-        int m = m_start;                                   // query block of the tile of the next phase_p
+        uint32_t J = 0;                                         // tiles of the CTA so far
+        for (int r = 0; take(r); ++r) {
+        const volatile BwdWork* work = s_work + (r & 1);
+        const uint32_t end = J + work->n_iter;
+        if (J == end) {                                         // a key block that no query sees: its gradients are zero
+            bwd_zero_rows<D>(p, work->tok0 + work->n * TILE, min(TILE, work->T - work->n * TILE), work->g, 256);
+            done(r);
+            continue;
+        }
+        // queries [my_first, my_end) of the trace see this key; nobody sees a slot past the trace
+        int my_end = 0, my_first = work->n * TILE + row;
+        if (my_first < work->T) {
+            const int at = work->tok0 + my_first;
+            my_end = min(mv.evict[at], work->T);
+            if (work->general) my_first = mv.kfirst[at];
+        }
+        int m = work->m_start;                             // query block of the tile of the next phase_p
 
-        auto phase_p = [&](int j) {        // P^T(j) = exp2(S^T * c - lse), masked
+        auto phase_p = [&](uint32_t j) {        // P^T(j) = exp2(S^T * c - lse), masked
             const int s = j & 1;
             const int lo = my_first - (m * TILE + col0), hi = my_end - (m * TILE + col0);     // columns [lo, hi) see the key
-            m = (m == m_last) ? m_first : m + 1;
+            m = (m == work->m_last) ? work->m_first : m + 1;       // read again, not kept: registers are short here
             mbar_wait(bar_ldfull(s), (j >> 1) & 1, abort_flag, status);
             mbar_wait(bar_s, j & 1, abort_flag, status);
             tc_fence_after();
@@ -662,7 +778,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
             if (lane == 0) mbar_arrive(bar_p);
         };
 
-        auto phase_ds = [&](int j) {       // dS^T(j) = P^T (scale dP^T - scale D)
+        auto phase_ds = [&](uint32_t j) {       // dS^T(j) = P^T (scale dP^T - scale D)
             const int s = j & 1;
             mbar_wait(bar_dp, j & 1, abort_flag, status);
             tc_fence_after();
@@ -696,19 +812,21 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
             if (lane == 0) mbar_arrive(bar_dss);
         };
 
-        phase_p(0);
-        for (int j = 0; j < n_iter; ++j) {
-            phase_ds(j);
-            if (j + 1 < n_iter) phase_p(j + 1);
+        phase_p(J);
+        for (; J < end; ++J) {
+            phase_ds(J);
+            if (J + 1 < end) phase_p(J + 1);
         }
 
         // ---- epilogue: dK, dV of this key block, once every MMA has completed ----
-        mbar_wait(bar_qfree((n_iter - 1) & 1), ((n_iter - 1) >> 1) & 1, abort_flag, status);
+        mbar_wait(bar_qfree((end - 1) & 1), ((end - 1) >> 1) & 1, abort_flag, status);
         tc_fence_after();
-        // through the memory of K and V, which nothing reads any more
-        bwd_epilogue<D>(p, work->cut, g, 1, 0, tmem_dK + lane_sel + half * HALF_D, tmem_dV + lane_sel + half * HALF_D, row, half,
-                        tok0 + n * TILE + quad * 32, T - n * TILE - quad * 32, sgen + L::OFF_K + warp * (L::TB / 4),
+        // through the memory of dS, which nothing reads any more; the next unit's tiles are on their way into the others
+        bwd_epilogue<D>(p, work->cut, work->g, 1, 0, tmem_dK + lane_sel + half * HALF_D, tmem_dV + lane_sel + half * HALF_D, row, half,
+                        work->tok0 + work->n * TILE + quad * 32, work->T - work->n * TILE - quad * 32, sgen + L::OFF_DS + warp * 4096,
                         reinterpret_cast<volatile int*>(sgen + L::OFF_MISC + 8));
+        done(r);
+        }
     }
     tc_fence_before();
     __syncthreads();

@@ -88,6 +88,8 @@ __device__ __forceinline__ bool bwd_unit_of(const BwdParams& p, const int32_t* o
     return true;
 }
 
+__device__ __forceinline__ bool bwd_has_unit(const BwdParams& p, int n_items, int x) { return x < (p.plan ? p.plan->n_units : n_items) * p.Hkv; }
+
 // bits [lo, hi) of a 32-bit word (either end may lie outside it)
 __device__ __forceinline__ uint32_t bit_range(int lo, int hi) {
     const int l = min(max(lo, 0), 32), h = min(max(hi, 0), 32);
@@ -96,9 +98,9 @@ __device__ __forceinline__ uint32_t bit_range(int lo, int hi) {
 
 // rows of zeros for a key block that no query sees (its gradients are zero)
 template <int D>
-__device__ __forceinline__ void bwd_zero_rows(const BwdParams& p, int tok, int rows, int g) {
+__device__ __forceinline__ void bwd_zero_rows(const BwdParams& p, int tok, int rows, int g, int threads = BWD_THREADS) {
     const int per_row = D * (p.grad_fp32 ? 4 : 2) / 16;          // 16-byte words of one (token, head) row
-    for (int i = threadIdx.x; i < rows * per_row; i += BWD_THREADS) {
+    for (int i = threadIdx.x; i < rows * per_row; i += threads) {
         const size_t off = (size_t)(tok + i / per_row) * (size_t)(p.dkv_ts / D) * per_row + (size_t)g * per_row + i % per_row;
         reinterpret_cast<uint4*>(p.dk)[off] = make_uint4(0, 0, 0, 0);
         reinterpret_cast<uint4*>(p.dv)[off] = make_uint4(0, 0, 0, 0);
@@ -107,23 +109,33 @@ __device__ __forceinline__ void bwd_zero_rows(const BwdParams& p, int tok, int r
 
 // Epilogue of the 256 compute threads: thread (row, half) has the columns [half * D/2, +D/2) of its row of dK and dV in
 // tensor memory.  A whole item goes straight to memory (`tok`: first token of this warp's 32 rows, `rows`: how many of them the
-// trace has; `stage`: 32 x D/2 fp32 of shared memory of this warp's own).  A unit of a cut item writes them to its slot; the item's last unit
+// trace has; `stage`: 4 KB of shared memory of this warp's own).  A unit of a cut item writes them to its slot; the item's last unit
 // adds the slots up in order.  `ctas`: CTAs per item, `cta`: this one's index.
 template <int D>
 __device__ __forceinline__ void bwd_epilogue(const BwdParams& p, int cut, int g, int ctas, int cta, uint32_t tmem_dk, uint32_t tmem_dv, int row,
                                              int half, int tok, int rows, uint8_t* stage, volatile int* s_last) {
     constexpr int CH = D / 64;              // 32-column pieces per thread and tensor
-    using Rows = RowStage<D / 2>;
     const int lane = threadIdx.x & 31;
     const size_t elem = (size_t)tok * (size_t)p.dkv_ts + (size_t)g * D + half * (D / 2);
+    // piece i (32 columns) of this thread's row of dK, then dV: fp32 leaves piece by piece, bf16 with the whole half row
+    auto put = [&](int i, const uint32_t (&r)[32]) {
+        void* base = i < CH ? p.dk : p.dv;
+        if (p.grad_fp32) {
+            RowStage<32>::put_f32(stage, lane, r);
+            RowStage<32>::template flush<4>(stage, lane, reinterpret_cast<char*>(base) + (elem + (i % CH) * 32) * 4, (size_t)p.dkv_ts, rows);
+        } else {
+            RowStage<D / 2>::put_bf16(stage, lane, i % CH, r);
+            if (i % CH == CH - 1)
+                RowStage<D / 2>::template flush<2>(stage, lane, reinterpret_cast<char*>(base) + elem * 2, (size_t)p.dkv_ts, rows);
+        }
+    };
     if (cut == 0) {
 #pragma unroll
         for (int i = 0; i < 2 * CH; ++i) {
             uint32_t r[32];
             tmem_ld32((i < CH ? tmem_dk : tmem_dv) + (i % CH) * 32, r);
             tmem_wait_ld();
-            Rows::put(stage, lane, i % CH, r, p.grad_fp32);
-            if (i % CH == CH - 1) Rows::flush(stage, lane, i < CH ? p.dk : p.dv, elem, (size_t)p.dkv_ts, rows, p.grad_fp32);
+            put(i, r);
         }
         return;
     }
@@ -171,8 +183,7 @@ __device__ __forceinline__ void bwd_epilogue(const BwdParams& p, int cut, int g,
             r[e * 4 + 2] = __float_as_uint(a[e].z);
             r[e * 4 + 3] = __float_as_uint(a[e].w);
         }
-        Rows::put(stage, lane, i % CH, r, p.grad_fp32);
-        if (i % CH == CH - 1) Rows::flush(stage, lane, i < CH ? p.dk : p.dv, elem, (size_t)p.dkv_ts, rows, p.grad_fp32);
+        put(i, r);
     }
 }
 

@@ -476,45 +476,42 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
 template <int COLS>
 struct RowStage {
     __device__ static __forceinline__ int chunk(int r, int c, int chunks) { return c ^ (chunks >= 8 ? r & 7 : (r >> 1) & 3); }
-    // 32 fp32 columns (piece i of the row) of this lane's row
-    __device__ static __forceinline__ void put(uint8_t* stage, int lane, int i, const uint32_t (&r)[32], int grad_fp32) {
-        if (grad_fp32) {
-            uint8_t* row = stage + lane * (COLS * 4);
+    // 32 fp32 columns of this lane's row, all of a piece
+    __device__ static __forceinline__ void put_f32(uint8_t* stage, int lane, const uint32_t (&r)[32]) {
+        uint8_t* row = stage + lane * (COLS * 4);
 #pragma unroll
-            for (int e = 0; e < 8; ++e)
-                *reinterpret_cast<uint4*>(row + (chunk(lane, i * 8 + e, COLS / 4) << 4)) = make_uint4(r[e * 4], r[e * 4 + 1], r[e * 4 + 2], r[e * 4 + 3]);
-        } else {
-            uint8_t* row = stage + lane * (COLS * 2);
+        for (int e = 0; e < 8; ++e)
+            *reinterpret_cast<uint4*>(row + (chunk(lane, e, COLS / 4) << 4)) = make_uint4(r[e * 4], r[e * 4 + 1], r[e * 4 + 2], r[e * 4 + 3]);
+    }
+    // ... as bf16, columns 32 i .. of the piece
+    __device__ static __forceinline__ void put_bf16(uint8_t* stage, int lane, int i, const uint32_t (&r)[32]) {
+        uint8_t* row = stage + lane * (COLS * 2);
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                uint4 w;
-                w.x = pack_bf16(__uint_as_float(r[e * 8 + 0]), __uint_as_float(r[e * 8 + 1]));
-                w.y = pack_bf16(__uint_as_float(r[e * 8 + 2]), __uint_as_float(r[e * 8 + 3]));
-                w.z = pack_bf16(__uint_as_float(r[e * 8 + 4]), __uint_as_float(r[e * 8 + 5]));
-                w.w = pack_bf16(__uint_as_float(r[e * 8 + 6]), __uint_as_float(r[e * 8 + 7]));
-                *reinterpret_cast<uint4*>(row + (chunk(lane, i * 4 + e, COLS / 8) << 4)) = w;
-            }
+        for (int e = 0; e < 4; ++e) {
+            uint4 w;
+            w.x = pack_bf16(__uint_as_float(r[e * 8 + 0]), __uint_as_float(r[e * 8 + 1]));
+            w.y = pack_bf16(__uint_as_float(r[e * 8 + 2]), __uint_as_float(r[e * 8 + 3]));
+            w.z = pack_bf16(__uint_as_float(r[e * 8 + 4]), __uint_as_float(r[e * 8 + 5]));
+            w.w = pack_bf16(__uint_as_float(r[e * 8 + 6]), __uint_as_float(r[e * 8 + 7]));
+            *reinterpret_cast<uint4*>(row + (chunk(lane, i * 4 + e, COLS / 8) << 4)) = w;
         }
     }
-    // the first `rows` rows to memory: row r at element elem + r * stride of base
+    // the piece's first `rows` rows to memory, `stride` elements of BYTES bytes apart
     template <int BYTES>
-    __device__ static __forceinline__ void flush_as(const uint8_t* stage, int lane, char* dst, size_t stride, int rows) {
+    __device__ static __forceinline__ void flush(const uint8_t* stage, int lane, char* dst, size_t stride, int rows) {
         constexpr int CHUNKS = COLS * BYTES / 16, STEP = 32 / CHUNKS;
         const int c = lane % CHUNKS;
+        __syncwarp();
 #pragma unroll
         for (int r0 = 0; r0 < 32; r0 += STEP) {
             const int r = r0 + lane / CHUNKS;
             const uint4 w = *reinterpret_cast<const uint4*>(stage + r * (COLS * BYTES) + (chunk(r, c, CHUNKS) << 4));
             if (r < rows) *reinterpret_cast<uint4*>(dst + (size_t)r * stride * BYTES + c * 16) = w;
         }
-    }
-    __device__ static __forceinline__ void flush(const uint8_t* stage, int lane, void* base, size_t elem, size_t stride, int rows, int grad_fp32) {
-        __syncwarp();
-        if (grad_fp32) flush_as<4>(stage, lane, reinterpret_cast<char*>(base) + elem * 4, stride, rows);
-        else flush_as<2>(stage, lane, reinterpret_cast<char*>(base) + elem * 2, stride, rows);
         __syncwarp();
     }
 };
+
 #endif  // __CUDACC__
 
 }  // namespace kvs

@@ -687,9 +687,9 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
                     }
 #pragma unroll
                     for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) * inv);
-                    Rows::put(stage, lane, c % (COLS / 32), r, 0);
+                    Rows::put_bf16(stage, lane, c % (COLS / 32), r);
                     if ((c + 1) % (COLS / 32) == 0)
-                        Rows::flush(stage, lane, orow, CHAIN ? c * 32 : 0, (size_t)p.Hq * D, rows, 0);
+                        Rows::template flush<2>(stage, lane, reinterpret_cast<char*>(orow + (CHAIN ? c * 32 : 0)), (size_t)p.Hq * D, rows);
                 }
                 if (valid) p.lse[(size_t)h * p.total_tokens + tok0 + qi] = ref_max * 0.6931471805599453f + logf(run_sum);
             }
