@@ -1,4 +1,5 @@
-"""Thin ctypes binding of libkvs.so: same names as the C ABI, argument marshalling only.
+"""Thin binding of libkvs.so: same names as the C ABI, argument marshalling only.  The calls of a step and of a generated
+token go through native functions (csrc/kvs_native.cpp), the others through ctypes.
 
 Every step of the path runs in the library's CUDA kernels.  PyTorch is used here for
 device memory and streams.  There is no CPU fallback: if the library is missing or
@@ -7,6 +8,7 @@ the tensors are not on a CUDA device the calls raise.
 from __future__ import annotations
 
 import ctypes
+import importlib
 import os
 from typing import Optional, Tuple
 
@@ -69,6 +71,7 @@ SIGNATURES = {
 }
 
 _lib = None
+_native = None          # the extension module, bound to the functions of _lib
 
 
 class KvsError(RuntimeError):
@@ -78,8 +81,8 @@ class KvsError(RuntimeError):
 
 
 def load() -> ctypes.CDLL:
-    """Loads libkvs.so (built by paper_2609_35750_b200.build).  Raises if absent."""
-    global _lib
+    """Loads libkvs.so and the native calls (built by paper_2609_35750_b200.build).  Raises if either is absent."""
+    global _lib, _native
     if _lib is None:
         path = LIB_PATH
         if not os.path.exists(path):
@@ -90,7 +93,9 @@ def load() -> ctypes.CDLL:
             fn = getattr(lib, name)
             fn.restype = res
             fn.argtypes = args
-        _lib = lib
+        native = importlib.import_module("._kvs_native", __package__)
+        native.bind({name: ctypes.cast(getattr(lib, name), ctypes.c_void_p).value for name in SIGNATURES}, KvsError)
+        _lib, _native = lib, native
     return _lib
 
 
@@ -106,8 +111,7 @@ def _check(code: int, where: str) -> None:
 def _stream(stream: Optional[torch.cuda.Stream]) -> int:
     if stream is not None:
         return int(stream.cuda_stream)
-    # The handle of torch.cuda.current_stream() without the Stream object around it, which took a third of a call's host
-    # time (a turn of 16 tokens is 33 calls and bound by it).
+    # the handle of torch.cuda.current_stream() without the Stream object around it
     return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
@@ -144,28 +148,15 @@ def kvs_evict_at_from_events(events: torch.Tensor, cu_seqlens: torch.Tensor, tot
 def kvs_mask_meta(evict_at: torch.Tensor, cu_seqlens: torch.Tensor, max_seqlen: int,
                   meta_buf: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """evict_at int32 [Ttot], cu_seqlens int32 [batch+1] (device).  Returns meta_buf (uint8)."""
-    batch = cu_seqlens.numel() - 1
-    total = evict_at.numel()
-    need = kvs_mask_meta_bytes(batch, total, max_seqlen)
-    if meta_buf is None:
-        meta_buf = torch.empty(need, dtype=torch.uint8, device=evict_at.device)
-    _check(load().kvs_mask_meta(_dev(evict_at, "evict_at", torch.int32), _dev(cu_seqlens, "cu_seqlens", torch.int32),
-                                batch, total, max_seqlen, _dev(meta_buf, "meta_buf", torch.uint8),
-                                meta_buf.numel(), _stream(stream)), "kvs_mask_meta")
-    return meta_buf
+    load()
+    return _native.mask_meta(0, None, evict_at, cu_seqlens, max_seqlen, meta_buf, stream)
 
 
 def kvs_mask_meta_keys(key_first: torch.Tensor, key_evict: torch.Tensor, cu_seqlens: torch.Tensor, max_seqlen: int,
                        meta_buf: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """Metadata for key slots with their own visibility interval [key_first, key_evict) (int32 [Ttot], device)."""
-    batch = cu_seqlens.numel() - 1
-    total = key_evict.numel()
-    if meta_buf is None:
-        meta_buf = torch.empty(kvs_mask_meta_bytes(batch, total, max_seqlen), dtype=torch.uint8, device=key_evict.device)
-    _check(load().kvs_mask_meta_keys(_dev(key_first, "key_first", torch.int32), _dev(key_evict, "key_evict", torch.int32),
-                                     _dev(cu_seqlens, "cu_seqlens", torch.int32), batch, total, max_seqlen,
-                                     _dev(meta_buf, "meta_buf", torch.uint8), meta_buf.numel(), _stream(stream)), "kvs_mask_meta_keys")
-    return meta_buf
+    load()
+    return _native.mask_meta(1, key_first, key_evict, cu_seqlens, max_seqlen, meta_buf, stream)
 
 
 def kvs_reorder_keys(evict_at: torch.Tensor, cu_seqlens: torch.Tensor, max_seqlen: int, window: int, perm=None, key_first=None,
@@ -184,15 +175,8 @@ def kvs_reorder_keys(evict_at: torch.Tensor, cu_seqlens: torch.Tensor, max_seqle
 
 def kvs_permute_rows(src: torch.Tensor, perm: torch.Tensor, dst: Optional[torch.Tensor] = None, inverse: bool = False, stream=None):
     """dst[s] = src[perm[s]] (inverse False) or dst[perm[s]] = src[s] (inverse True) along the leading dimension."""
-    if dst is None:
-        dst = torch.empty_like(src)
-    n = src.shape[0]
-    row_bytes = (src.numel() // max(n, 1)) * src.element_size()
-    if not src.is_cuda or not src.is_contiguous() or not dst.is_contiguous() or dst.shape != src.shape or dst.dtype != src.dtype:
-        raise ValueError("src and dst must be contiguous CUDA tensors of the same shape and dtype")
-    _check(load().kvs_permute_rows(src.data_ptr(), _dev(perm, "perm", torch.int32), dst.data_ptr(), n, row_bytes, 1 if inverse else 0,
-                                   _stream(stream)), "kvs_permute_rows")
-    return dst
+    load()
+    return _native.permute_rows(src, perm, dst, inverse, stream)
 
 
 def kvs_mask_meta_export(meta_buf: torch.Tensor, cu_seqlens_host, total_tokens: int, max_seqlen: int, stream=None):
@@ -213,107 +197,46 @@ def kvs_mask_meta_export(meta_buf: torch.Tensor, cu_seqlens_host, total_tokens: 
 def kvs_attn_fwd(q, k, v, meta_buf, batch: int, max_seqlen: int, softmax_scale: float = 0.0,
                  out: Optional[torch.Tensor] = None, lse: Optional[torch.Tensor] = None, stream=None):
     """q [Ttot,Hq,d], k, v [Ttot,Hkv,d] bf16 (device).  Returns (out bf16 [Ttot,Hq,d], lse fp32 [Hq,Ttot])."""
-    total, Hq, d = q.shape
-    Hkv = k.shape[1]
-    if out is None:
-        out = torch.empty_like(q)
-    if lse is None:
-        lse = torch.empty((Hq, total), dtype=torch.float32, device=q.device)
-    _check(load().kvs_attn_fwd(_dev(q, "q", torch.bfloat16), _dev(k, "k", torch.bfloat16), _dev(v, "v", torch.bfloat16),
-                               _dev(meta_buf, "meta_buf", torch.uint8), batch, total, max_seqlen, Hq, Hkv, d,
-                               float(softmax_scale), _dev(out, "out", torch.bfloat16), _dev(lse, "lse", torch.float32),
-                               _stream(stream)), "kvs_attn_fwd")
-    return out, lse
+    load()
+    return _native.attn_fwd(q, k, v, meta_buf, batch, max_seqlen, softmax_scale, out, lse, stream)
 
 
 def kvs_mask_meta_evicted(key_evict: torch.Tensor, cu_seqlens: torch.Tensor, max_seqlen: int,
                           meta_buf: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """Metadata for the keys the eviction mask no longer shows (visible from their eviction step on)."""
-    batch = cu_seqlens.numel() - 1
-    total = key_evict.numel()
-    if meta_buf is None:
-        meta_buf = torch.empty(kvs_mask_meta_bytes(batch, total, max_seqlen), dtype=torch.uint8, device=key_evict.device)
-    _check(load().kvs_mask_meta_evicted(_dev(key_evict, "key_evict", torch.int32), _dev(cu_seqlens, "cu_seqlens", torch.int32),
-                                        batch, total, max_seqlen, _dev(meta_buf, "meta_buf", torch.uint8), meta_buf.numel(),
-                                        _stream(stream)), "kvs_mask_meta_evicted")
-    return meta_buf
+    load()
+    return _native.mask_meta(2, None, key_evict, cu_seqlens, max_seqlen, meta_buf, stream)
 
 
 def kvs_attn_fwd_dual(q, k, v, meta_student, meta_evicted, batch: int, max_seqlen: int, softmax_scale: float = 0.0,
                       out_student=None, lse_student=None, out_teacher=None, lse_teacher=None, stream=None):
     """Student (eviction mask) and teacher (every key seen or evicted: the full causal context) forward.
     Returns (out_student, lse_student, out_teacher, lse_teacher)."""
-    total, Hq, d = q.shape
-    Hkv = k.shape[1]
-    if out_student is None:
-        out_student = torch.empty_like(q)
-    if out_teacher is None:
-        out_teacher = torch.empty_like(q)
-    if lse_student is None:
-        lse_student = torch.empty((Hq, total), dtype=torch.float32, device=q.device)
-    if lse_teacher is None:
-        lse_teacher = torch.empty((Hq, total), dtype=torch.float32, device=q.device)
-    _check(load().kvs_attn_fwd_dual(_dev(q, "q", torch.bfloat16), _dev(k, "k", torch.bfloat16), _dev(v, "v", torch.bfloat16),
-                                    _dev(meta_student, "meta_student", torch.uint8), _dev(meta_evicted, "meta_evicted", torch.uint8),
-                                    batch, total, max_seqlen, Hq, Hkv, d, float(softmax_scale),
-                                    _dev(out_student, "out_student", torch.bfloat16), _dev(lse_student, "lse_student", torch.float32),
-                                    _dev(out_teacher, "out_teacher", torch.bfloat16), _dev(lse_teacher, "lse_teacher", torch.float32),
-                                    _stream(stream)), "kvs_attn_fwd_dual")
-    return out_student, lse_student, out_teacher, lse_teacher
+    load()
+    return _native.attn_fwd_dual(q, k, v, meta_student, meta_evicted, batch, max_seqlen, softmax_scale, out_student, lse_student,
+                                 out_teacher, lse_teacher, stream)
 
 
 def kvs_attn_fwd_packed(qkv, meta_buf, batch: int, max_seqlen: int, Hq: int, Hkv: int, softmax_scale: float = 0.0,
                         out=None, lse=None, stream=None):
     """qkv bf16 [Ttot, Hq + 2 Hkv, d] (q heads, k heads, v heads).  Returns (out [Ttot,Hq,d], lse [Hq,Ttot])."""
-    total, H, d = qkv.shape
-    if H != Hq + 2 * Hkv:
-        raise ValueError("qkv must have Hq + 2 Hkv heads")
-    if out is None:
-        out = torch.empty((total, Hq, d), dtype=torch.bfloat16, device=qkv.device)
-    if lse is None:
-        lse = torch.empty((Hq, total), dtype=torch.float32, device=qkv.device)
-    _check(load().kvs_attn_fwd_packed(_dev(qkv, "qkv", torch.bfloat16), _dev(meta_buf, "meta_buf", torch.uint8), batch, total,
-                                      max_seqlen, Hq, Hkv, d, float(softmax_scale), _dev(out, "out", torch.bfloat16),
-                                      _dev(lse, "lse", torch.float32), _stream(stream)), "kvs_attn_fwd_packed")
-    return out, lse
+    load()
+    return _native.attn_fwd_packed(qkv, meta_buf, batch, max_seqlen, Hq, Hkv, softmax_scale, out, lse, stream)
 
 
 def kvs_attn_bwd_packed(dout, qkv, out, lse, meta_buf, batch: int, max_seqlen: int, Hq: int, Hkv: int, softmax_scale: float = 0.0,
                         grad_dtype: int = GRAD_FP32, dqkv=None, workspace=None, stream=None):
     """Returns dqkv [Ttot, Hq + 2 Hkv, d] (bf16 or fp32): dq, dk, dv in the head order of qkv."""
-    total, H, d = qkv.shape
-    gdt = torch.float32 if grad_dtype == GRAD_FP32 else torch.bfloat16
-    if dqkv is None:
-        dqkv = torch.empty(qkv.shape, dtype=gdt, device=qkv.device)
-    if workspace is None:
-        workspace = torch.empty(kvs_attn_bwd_workspace_bytes(total, Hq, Hkv, d, grad_dtype), dtype=torch.uint8, device=qkv.device)
-    _check(load().kvs_attn_bwd_packed(_dev(dout, "dout", torch.bfloat16), _dev(qkv, "qkv", torch.bfloat16),
-                                      _dev(out, "out", torch.bfloat16), _dev(lse, "lse", torch.float32),
-                                      _dev(meta_buf, "meta_buf", torch.uint8), batch, total, max_seqlen, Hq, Hkv, d,
-                                      float(softmax_scale), grad_dtype, _dev(dqkv, "dqkv", gdt),
-                                      _dev(workspace, "workspace", torch.uint8), workspace.numel(), _stream(stream)),
-           "kvs_attn_bwd_packed")
-    return dqkv
+    load()
+    return _native.attn_bwd_packed(dout, qkv, out, lse, meta_buf, batch, max_seqlen, Hq, Hkv, softmax_scale, grad_dtype, dqkv, workspace, stream)
 
 
 def kvs_rope_qk(q, k, cu_seqlens=None, positions=None, theta_base: float = 10000.0, inverse: bool = False, q_out=None, k_out=None,
                 stream=None):
     """Rotary embedding of q and/or k (bf16 or fp32, [Ttot, H, d]); inverse=True applies the transposed rotation (for
     gradients).  positions int32 [Ttot] or None for the trace-local index (cu_seqlens then required).  Returns (q_out, k_out)."""
-    ref = q if q is not None else k
-    total, _, d = ref.shape
-    dt = GRAD_FP32 if ref.dtype == torch.float32 else GRAD_BF16
-    if q is not None and q_out is None:
-        q_out = torch.empty_like(q)
-    if k is not None and k_out is None:
-        k_out = torch.empty_like(k)
-    ptr = lambda t, n: _dev(t, n, ref.dtype) if t is not None else None
-    _check(load().kvs_rope_qk(ptr(q, "q"), ptr(k, "k"), _dev(positions, "positions", torch.int32) if positions is not None else None,
-                              _dev(cu_seqlens, "cu_seqlens", torch.int32) if cu_seqlens is not None else None,
-                              (cu_seqlens.numel() - 1) if cu_seqlens is not None else 0, total,
-                              q.shape[1] if q is not None else 0, k.shape[1] if k is not None else 0, d, float(theta_base), dt,
-                              1 if inverse else 0, ptr(q_out, "q_out"), ptr(k_out, "k_out"), _stream(stream)), "kvs_rope_qk")
-    return q_out, k_out
+    load()
+    return _native.rope_qk(q, k, cu_seqlens, positions, theta_base, inverse, q_out, k_out, stream)
 
 
 def kvs_host_chunk_plan(cu_seqlens, max_seqlen: int, Hkv: int):
@@ -339,6 +262,9 @@ def kvs_attn_bwd(dout, q, k, v, out, lse, meta_buf, batch: int, max_seqlen: int,
     """Returns (dq, dk, dv) in bf16 or fp32 according to grad_dtype.  main_events: two timing
     events (already recorded once, so that their handles exist) to be recorded around the
     main kernel; this routes through kvs_attn_bwd_ex."""
+    load()
+    if main_events is None:
+        return _native.attn_bwd(dout, q, k, v, out, lse, meta_buf, batch, max_seqlen, softmax_scale, grad_dtype, dq, dk, dv, workspace, stream)
     total, Hq, d = q.shape
     Hkv = k.shape[1]
     gdt = torch.float32 if grad_dtype == GRAD_FP32 else torch.bfloat16
@@ -356,13 +282,10 @@ def kvs_attn_bwd(dout, q, k, v, out, lse, meta_buf, batch: int, max_seqlen: int,
             _dev(meta_buf, "meta_buf", torch.uint8), batch, total, max_seqlen, Hq, Hkv, d,
             float(softmax_scale), grad_dtype, _dev(dq, "dq", gdt), _dev(dk, "dk", gdt), _dev(dv, "dv", gdt),
             _dev(workspace, "workspace", torch.uint8), workspace.numel(), _stream(stream))
-    if main_events is None:
-        _check(load().kvs_attn_bwd(*args), "kvs_attn_bwd")
-    else:
-        e0, e1 = (int(e.cuda_event) for e in main_events)
-        if not e0 or not e1:
-            raise ValueError("main_events must have been recorded once before the call")
-        _check(load().kvs_attn_bwd_ex(*args, e0, e1), "kvs_attn_bwd_ex")
+    e0, e1 = (int(e.cuda_event) for e in main_events)
+    if not e0 or not e1:
+        raise ValueError("main_events must have been recorded once before the call")
+    _check(load().kvs_attn_bwd_ex(*args, e0, e1), "kvs_attn_bwd_ex")
     return dq, dk, dv
 
 
@@ -451,11 +374,9 @@ class PagedCache:
         _check(load().kvs_cache_init(self.free_list.data_ptr(), num_pages, _stream(None)), "kvs_cache_init")
 
     def append(self, k_new: torch.Tensor, v_new: torch.Tensor, active: Optional[torch.Tensor] = None, stream=None) -> None:
-        _check(load().kvs_cache_append(_dev(k_new, "k_new", torch.bfloat16), _dev(v_new, "v_new", torch.bfloat16),
-                                       _dev(active, "active", torch.uint8) if active is not None else None,
-                                       self.num_seqs, self.Hkv, self.d, self.page_size, self.max_pages, self.num_pages,
-                                       self.block_table.data_ptr(), self.n_tokens.data_ptr(), self.free_list.data_ptr(),
-                                       self.k_cache.data_ptr(), self.v_cache.data_ptr(), _stream(stream)), "kvs_cache_append")
+        load()
+        _native.cache_append(k_new, v_new, active, self.num_seqs, self.Hkv, self.d, self.page_size, self.max_pages, self.num_pages,
+                             self.block_table, self.n_tokens, self.free_list, self.k_cache, self.v_cache, stream)
 
     def evict(self, ranges: torch.Tensor, stream=None) -> None:
         """ranges int32 [n, 3] rows (sequence, first_page_slot, n_pages) (device)."""
@@ -473,19 +394,6 @@ class PagedCache:
     def decode(self, q: torch.Tensor, softmax_scale: float = 0.0, num_splits: int = 0, out=None, lse=None, workspace=None,
                max_tokens: Optional[int] = None, stream=None):
         """q bf16 [num_seqs, Hq, d] -> (out bf16 [num_seqs, Hq, d], lse fp32 [num_seqs, Hq])."""
-        S, Hq, d = q.shape
-        if num_splits <= 0:
-            num_splits = int(load().kvs_decode_num_splits(S, self.Hkv, max_tokens or self.max_pages * self.page_size))
-        need = int(load().kvs_decode_workspace_bytes(S, Hq, d, num_splits))
-        if workspace is None:
-            workspace = torch.empty(need, dtype=torch.uint8, device=q.device)
-        if out is None:
-            out = torch.empty_like(q)
-        if lse is None:
-            lse = torch.empty((S, Hq), dtype=torch.float32, device=q.device)
-        _check(load().kvs_decode_attn(_dev(q, "q", torch.bfloat16), self.k_cache.data_ptr(), self.v_cache.data_ptr(),
-                                      self.block_table.data_ptr(), self.n_tokens.data_ptr(), S, Hq, self.Hkv, d, self.page_size,
-                                      self.max_pages, self.num_pages, float(softmax_scale), num_splits, _dev(out, "out", torch.bfloat16),
-                                      _dev(lse, "lse", torch.float32), _dev(workspace, "workspace", torch.uint8),
-                                      workspace.numel(), _stream(stream)), "kvs_decode_attn")
-        return out, lse
+        load()
+        return _native.decode(q, softmax_scale, num_splits, out, lse, workspace, max_tokens or self.max_pages * self.page_size, self.Hkv,
+                              self.page_size, self.max_pages, self.num_pages, self.block_table, self.n_tokens, self.k_cache, self.v_cache, stream)

@@ -1,4 +1,4 @@
-"""Builds libkvs.so (the C-ABI library) in-tree with nvcc for sm_100a.
+"""Builds libkvs.so (the C-ABI library, nvcc for sm_100a) and _kvs_native.so (the native calls of the binding, g++) in-tree.
 
     python -m paper_2609_35750_b200.build [--force]
 """
@@ -12,6 +12,8 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 LIB = os.path.join(HERE, "libkvs.so")
+NATIVE = os.path.join(HERE, "_kvs_native.so")
+NATIVE_SOURCE = os.path.join(CSRC, "kvs_native.cpp")
 SOURCES = ["kvs_api.cu", "kvs_meta.cu", "kvs_fwd.cu", "kvs_fwd_dual.cu", "kvs_bwd.cu", "kvs_bwd_pair.cu", "kvs_bwd_noalloc.cu", "kvs_decode.cu", "kvs_rope.cu"]
 HEADERS = [os.path.join(CSRC, "kvs_common.cuh"), os.path.join(CSRC, "kvs_bwd.cuh"), os.path.join(INCLUDE, "kvs.h")]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -25,12 +27,25 @@ def _nvcc() -> str:
     return "nvcc"
 
 
+def native_command() -> list:
+    import sysconfig
+
+    import torch
+    from torch.utils.cpp_extension import include_paths, library_paths
+    cuda = os.path.dirname(os.path.dirname(_nvcc())) if os.path.sep in _nvcc() else "/usr/local/cuda"
+    dirs = include_paths() + [sysconfig.get_paths()["include"], os.path.join(cuda, "include"), INCLUDE]
+    return (["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch.compiled_with_cxx11_abi()] +
+            ["-I" + d for d in dirs] + [NATIVE_SOURCE, "-o", NATIVE] + ["-L" + d for d in library_paths()] +
+            ["-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda"])
+
+
+def _older(target: str, deps: list) -> bool:
+    return not os.path.exists(target) or any(os.path.getmtime(d) > os.path.getmtime(target) for d in deps)
+
+
 def needs_build() -> bool:
-    if not os.path.exists(LIB):
-        return True
-    t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, s) for s in SOURCES] + HEADERS
-    return any(os.path.getmtime(d) > t for d in deps)
+    return (_older(LIB, [os.path.join(CSRC, s) for s in SOURCES] + HEADERS) or
+            _older(NATIVE, [NATIVE_SOURCE, os.path.join(INCLUDE, "kvs.h")]))
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -44,6 +59,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         obj = os.path.join(objdir, s.replace(".cu", ".o"))
         cmd = [nvcc] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) + ["-c", os.path.join(CSRC, s), "-o", obj]
         procs.append((s, obj, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
+    native = subprocess.Popen(native_command(), stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
     objs = []
     for s, obj, p in procs:
         out, _ = p.communicate()
@@ -56,6 +72,9 @@ def build(force: bool = False, verbose: bool = False) -> str:
     r = subprocess.run(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
     if r.returncode != 0:
         raise RuntimeError(f"link failed:\n{r.stdout}")
+    out, _ = native.communicate()
+    if native.returncode != 0:
+        raise RuntimeError(f"g++ failed on {os.path.basename(NATIVE_SOURCE)}:\n{out}")
     return LIB
 
 
