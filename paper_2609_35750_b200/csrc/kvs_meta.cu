@@ -7,6 +7,81 @@ namespace kvs {
 constexpr int META_THREADS = 256;
 constexpr int META_WARPS = META_THREADS / 32;
 
+// ---- parts of the kernels ---------------------------------------------------------------------------------------
+// What a key block's slots say, found by a warp; lane 0 has `first`, `last`: the query blocks that can see the block.
+struct BlockStat {
+    int mn, mx, fmn, fmx, first, last;
+    bool invalid;
+};
+__device__ __forceinline__ BlockStat meta_block_stat(const int32_t* evict_at, const int32_t* key_first, int complement, int n, int tok0, int T,
+                                                     int32_t* evict_copy, int32_t* first_copy) {
+    const int lane = threadIdx.x & 31, nb = (T + TILE - 1) / TILE;
+    BlockStat r = {INT32_MAX, INT32_MIN, INT32_MAX, INT32_MIN, 0, 0, false};
+    const bool general = complement || key_first;
+#pragma unroll
+    for (int t = 0; t < TILE / 32; ++t) {
+        const int j = n * TILE + t * 32 + lane;
+        if (j < T) {
+            const int e = complement ? INT32_MAX : evict_at[tok0 + j];
+            const int f = complement ? evict_at[tok0 + j] : (key_first ? key_first[tok0 + j] : j);
+            evict_copy[tok0 + j] = e;
+            if (general) first_copy[tok0 + j] = f;
+            r.invalid |= general ? (f < 0) : (e <= j);
+            r.mn = min(r.mn, e);
+            r.mx = max(r.mx, e);
+            r.fmn = min(r.fmn, f);
+            r.fmx = max(r.fmx, f);
+        }
+    }
+    r.mn = __reduce_min_sync(0xffffffffu, r.mn);
+    r.mx = __reduce_max_sync(0xffffffffu, r.mx);
+    r.fmn = __reduce_min_sync(0xffffffffu, r.fmn);
+    r.fmx = __reduce_max_sync(0xffffffffu, r.fmx);
+    r.invalid = __any_sync(0xffffffffu, r.invalid);
+    // last query block whose first row q0 = 128 m is still below kmax; first one whose last row reaches fmin
+    long long last = ((long long)r.mx - 1) / TILE;
+    if (last > nb - 1) last = nb - 1;
+    long long first = r.fmn / TILE;
+    if (first > nb) first = nb;
+    if (first < 0) first = 0;                  // a negative key_first is reported; never an index
+    if (!general && last < n) last = n;
+    r.first = (int)first;
+    r.last = (r.mx <= 0) ? -1 : (int)last;
+    return r;
+}
+
+// A warp's query block row m of a trace of T tokens: the classes of its tiles and the list of the non-empty ones, whose number
+// is returned.  kmin .. fmax: of the trace's key blocks.
+__device__ __forceinline__ int meta_classify_row(int m, int T, const int32_t* kmin, const int32_t* kmax, const int32_t* fmin, const int32_t* fmax,
+                                                 uint8_t* cls_row, uint16_t* list_row) {
+    const int lane = threadIdx.x & 31, nb = (T + TILE - 1) / TILE;
+    const int q0 = m * TILE, q1 = min(q0 + TILE - 1, T - 1);
+    int count = 0;
+    for (int n0 = 0; n0 < nb; n0 += 32) {
+        const int n = n0 + lane;
+        int c = KVS_CLASS_EMPTY;
+        if (n < nb) {
+            // f0, f1: the earliest / latest "first query that may see the slot" of the block; for plain
+            // metadata these are the block's first and last valid key, k0 and k1
+            const int f0 = fmin[n], f1 = fmax[n];
+            const int mn = kmin[n], mx = kmax[n];
+            if (f0 > q1 || q0 >= mx) c = KVS_CLASS_EMPTY;
+            else if (f1 <= q0 && q1 < mn) c = KVS_CLASS_FULL;
+            else c = KVS_CLASS_PARTIAL;
+            cls_row[n] = (uint8_t)c;
+        }
+        const unsigned live = __ballot_sync(0xffffffffu, c != KVS_CLASS_EMPTY);
+        if (c != KVS_CLASS_EMPTY) list_row[count + __popc(live & ((1u << lane) - 1u))] = (uint16_t)n;
+        count += __popc(live);
+    }
+    return count;
+}
+
+// The bucket of a length in a launch order (see meta_order), of nbins
+__device__ __forceinline__ bool meta_exact(int max_seqlen) { return max_seqlen <= 16 * TILE; }
+__device__ __forceinline__ int meta_bins(int max_seqlen, int most) { return meta_exact(max_seqlen) ? 17 : min((max_seqlen / TILE >> 4) + 2, most); }
+__device__ __forceinline__ int meta_bin(int len, bool exact, int nbins) { return nbins - 1 - min(exact ? len : len >> 4, nbins - 1); }   // the longest first
+
 // ---- kernel 1: offsets, and per key block (one warp each) min / max over its key slots, validity ---------------
 // Every CTA goes through the traces itself, 256 at a time (a scan of their block counts), and keeps what its eight blocks
 // need; the first CTA writes the tables.  A kernel of its own for the offsets, with one thread walking the traces, took 24 us
@@ -108,46 +183,16 @@ meta_blocks_kernel(const int32_t* __restrict__ evict_at, const int32_t* __restri
     if (blk0 + warp >= nblk || mine.x < 0) return;
     const int blk = (int)blk0 + warp;
     const int n = blk - mine.y, tok0 = mine.z, T = mine.w;
-    const int nb = (T + TILE - 1) / TILE;
-    int mn = INT32_MAX, mx = INT32_MIN, fmn = INT32_MAX, fmx = INT32_MIN;
-    bool invalid = false;
-#pragma unroll
-    for (int t = 0; t < TILE / 32; ++t) {
-        const int j = n * TILE + t * 32 + lane;
-        if (j < T) {
-            const int e = complement ? INT32_MAX : evict_at[tok0 + j];
-            const int f = complement ? evict_at[tok0 + j] : (key_first ? key_first[tok0 + j] : j);
-            const bool general = complement || key_first;
-            evict_copy[tok0 + j] = e;
-            if (general) first_copy[tok0 + j] = f;
-            invalid |= general ? (f < 0) : (e <= j);
-            mn = min(mn, e);
-            mx = max(mx, e);
-            fmn = min(fmn, f);
-            fmx = max(fmx, f);
-        }
-    }
-    mn = __reduce_min_sync(0xffffffffu, mn);
-    mx = __reduce_max_sync(0xffffffffu, mx);
-    fmn = __reduce_min_sync(0xffffffffu, fmn);
-    fmx = __reduce_max_sync(0xffffffffu, fmx);
-    const unsigned any_invalid = __ballot_sync(0xffffffffu, invalid);
+    const BlockStat st = meta_block_stat(evict_at, key_first, complement, n, tok0, T, evict_copy, first_copy);
     if (lane == 0) {
         blk_trace[blk] = mine.x;
-        kmin[blk] = mn;
-        kmax[blk] = mx;
-        fmin[blk] = fmn;
-        fmax[blk] = fmx;
-        // last query block whose first row q0 = 128 m is still below kmax; first one whose last row reaches fmin
-        long long last = ((long long)mx - 1) / TILE;
-        if (last > nb - 1) last = nb - 1;
-        long long first = fmn / TILE;
-        if (first > nb) first = nb;
-        if (first < 0) first = 0;                  // a negative key_first is reported; never an index
-        if (!key_first && !complement && last < n) last = n;
-        col_first[blk] = (int32_t)first;
-        col_last[blk] = (mx <= 0) ? -1 : (int32_t)last;
-        row_cnt[blk] = any_invalid ? -1 : 0;       // for the next kernel, which puts the count here
+        kmin[blk] = st.mn;
+        kmax[blk] = st.mx;
+        fmin[blk] = st.fmn;
+        fmax[blk] = st.fmx;
+        col_first[blk] = st.first;
+        col_last[blk] = st.last;
+        row_cnt[blk] = st.invalid ? -1 : 0;        // for the next kernel, which puts the count here
     }
 }
 
@@ -176,8 +221,8 @@ __device__ void meta_order(int what, MetaHeader* hdr, const int32_t* blk_off, co
     __shared__ int s_most, s_items;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n = hdr->nblk_total;
-    const bool exact = hdr->max_seqlen <= 16 * TILE;
-    const int nbins = exact ? 17 : min((hdr->max_seqlen / TILE >> 4) + 2, ORDER_BINS);
+    const bool exact = meta_exact(hdr->max_seqlen);
+    const int nbins = meta_bins(hdr->max_seqlen, ORDER_BINS);
     auto length = [&](int i) {              // -1: not an item of its own
         if (what == ORDER_ROWS) return __ldcg(row_cnt + i);
         if (what == ORDER_COLS) return max(col_last[i] - col_first[i] + 1, 0);
@@ -186,7 +231,7 @@ __device__ void meta_order(int what, MetaHeader* hdr, const int32_t* blk_off, co
         pair_range(col_first, col_last, i, i + 1 < hi, first, last);
         return ((i - lo) & 1) ? -1 : max(last - first + 1, 0);
     };
-    auto bin = [&](int len) { return nbins - 1 - min(exact ? len : len >> 4, nbins - 1); };      // the longest first
+    auto bin = [&](int len) { return meta_bin(len, exact, nbins); };
     // Every warp has a run of the items and a column of the bins, so that all of them can scatter: by one warp alone the
     // metadata of 128 traces of 32768 tokens took 493 us, 172 like this.  Fewer columns where the bins have no room for eight
     // (traces of a million tokens), one for the few items of a small batch, whose sort is a matter of latency.
@@ -290,29 +335,8 @@ meta_classify_kernel(MetaHeader* hdr, const int32_t* __restrict__ blk_off, const
         const int base = blk_off[b];
         const int m = row - base;
         const int T = seq_start[b + 1] - seq_start[b];
-        const int nb = (T + TILE - 1) / TILE;
-        const int q0 = m * TILE;
-        const int q1 = min(q0 + TILE - 1, T - 1);
-        uint8_t* cls_row = tile_class + cls_off[b] + (size_t)m * nb;
-        uint16_t* list_row = row_list + cls_off[b] + (size_t)m * nb;
-        int count = 0;
-        for (int n0 = 0; n0 < nb; n0 += 32) {
-            const int n = n0 + lane;
-            int c = KVS_CLASS_EMPTY;
-            if (n < nb) {
-                // f0, f1: the earliest / latest "first query that may see the slot" of the block; for plain
-                // metadata these are the block's first and last valid key, k0 and k1
-                const int f0 = fmin[base + n], f1 = fmax[base + n];
-                const int mn = kmin[base + n], mx = kmax[base + n];
-                if (f0 > q1 || q0 >= mx) c = KVS_CLASS_EMPTY;
-                else if (f1 <= q0 && q1 < mn) c = KVS_CLASS_FULL;
-                else c = KVS_CLASS_PARTIAL;
-                cls_row[n] = (uint8_t)c;
-            }
-            const unsigned live = __ballot_sync(0xffffffffu, c != KVS_CLASS_EMPTY);
-            if (c != KVS_CLASS_EMPTY) list_row[count + __popc(live & ((1u << lane) - 1u))] = (uint16_t)n;
-            count += __popc(live);
-        }
+        const size_t at = cls_off[b] + (size_t)m * ((T + TILE - 1) / TILE);
+        const int count = meta_classify_row(m, T, kmin + base, kmax + base, fmin + base, fmax + base, tile_class + at, row_list + at);
         if (lane == 0) {
             if (row_cnt[row] < 0) set_status(&hdr->status, KVS_ERR_BAD_EVICT);       // the block's keys, seen by kernel 1
             row_cnt[row] = count;
@@ -325,6 +349,155 @@ meta_classify_kernel(MetaHeader* hdr, const int32_t* __restrict__ blk_off, const
     if (!s_last) return;
     __threadfence();
     meta_order(ORDER_ROWS, hdr, blk_off, blk_trace, row_cnt, col_first, col_last, fwd_order, nullptr);
+}
+
+// ---- small batches: all of it by one CTA ---------------------------------------------------------------------------
+// The two kernels above are latency: a launch, two chains of loads and a sort each.  For up to META_SMALL blocks everything
+// between the input and the tables stays in shared memory of one CTA of 32 warps, and an item's place in an order is counted,
+// not sorted for (the same order: by bucket, then by index).  (Figures: see the dispatch in launch_mask_meta.)
+constexpr int META_SMALL = 64, META_SMALL_BATCH = 1024, META_SMALL_THREADS = 1024;
+__global__ void __launch_bounds__(META_SMALL_THREADS)
+meta_small_kernel(const int32_t* __restrict__ evict_at, const int32_t* __restrict__ key_first, int complement,
+                  const int32_t* __restrict__ cu_seqlens, int batch, int total_tokens, int max_seqlen, MetaView v, int nb_cap,
+                  unsigned long long cls_cap) {
+    // per block: trace, block of the trace, first token and length of the trace, first tile of the row
+    __shared__ int s_trace[META_SMALL], s_n[META_SMALL], s_tok0[META_SMALL], s_T[META_SMALL], s_at[META_SMALL];
+    __shared__ int s_kmin[META_SMALL], s_kmax[META_SMALL], s_fmin[META_SMALL], s_fmax[META_SMALL], s_first[META_SMALL], s_last[META_SMALL];
+    __shared__ int s_len[3][META_SMALL];               // the items' lengths in the three orders, -1: not an item
+    __shared__ int s_nblk, s_ncls, s_bad;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (tid < META_SMALL) s_len[0][tid] = s_len[1][tid] = s_len[2][tid] = -1;
+    if (tid == 0) s_bad = 0;
+    pdl_wait();
+    if (warp == 0) {                                   // the offsets: the traces, 32 at a time
+        bool bad = cu_seqlens[0] != 0 || cu_seqlens[batch] != total_tokens;
+        long long nblk = 0, ncls = 0;
+        for (int b0 = 0; b0 < batch; b0 += 32) {
+            const int b = b0 + lane;
+            long long a = 0, T = 0;
+            if (b < batch) {
+                a = cu_seqlens[b];
+                T = cu_seqlens[b + 1] - a;
+                if (T < 0 || T > max_seqlen || a < 0 || a + T > total_tokens) {
+                    bad = true;
+                    T = 0;
+                }
+            }
+            const long long nb = (T + TILE - 1) / TILE;
+            long long ib = nb, ic = nb * nb;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const long long tb = __shfl_up_sync(0xffffffffu, ib, o), tc = __shfl_up_sync(0xffffffffu, ic, o);
+                if (lane >= o) {
+                    ib += tb;
+                    ic += tc;
+                }
+            }
+            const long long first = nblk + ib - nb, cls = ncls + ic - nb * nb;
+            nblk += __shfl_sync(0xffffffffu, ib, 31);
+            ncls += __shfl_sync(0xffffffffu, ic, 31);
+            if (b < batch) {
+                ((int32_t*)v.blk_off)[b] = (int32_t)first;
+                ((uint32_t*)v.cls_off)[b] = (uint32_t)cls;
+                ((int32_t*)v.seq_start)[b] = (int32_t)a;
+                for (long long i = 0; i < nb && first + i < META_SMALL; ++i) {
+                    s_trace[first + i] = b;
+                    s_n[first + i] = (int)i;
+                    s_tok0[first + i] = (int)a;
+                    s_T[first + i] = (int)T;
+                    s_at[first + i] = (int)(cls + i * nb);
+                }
+            }
+        }
+        bad = __any_sync(0xffffffffu, bad) || nblk > nb_cap || (unsigned long long)ncls > cls_cap;
+        if (lane == 0) {
+            s_nblk = bad ? 0 : (int)nblk;
+            s_ncls = bad ? 0 : (int)ncls;
+            if (bad) s_bad = 1;
+            ((int32_t*)v.blk_off)[batch] = s_nblk;
+            ((uint32_t*)v.cls_off)[batch] = (uint32_t)s_ncls;
+            ((int32_t*)v.seq_start)[batch] = total_tokens;
+        }
+    }
+    __syncthreads();
+    const int nblk = s_nblk;
+    for (int i = warp; i < nblk; i += META_SMALL_THREADS / 32) {
+        const BlockStat st = meta_block_stat(evict_at, key_first, complement, s_n[i], s_tok0[i], s_T[i], (int32_t*)v.evict, (int32_t*)v.kfirst);
+        if (lane == 0) {
+            ((int32_t*)v.blk_trace)[i] = s_trace[i];
+            ((int32_t*)v.kmin)[i] = s_kmin[i] = st.mn;
+            ((int32_t*)v.kmax)[i] = s_kmax[i] = st.mx;
+            ((int32_t*)v.fmin)[i] = s_fmin[i] = st.fmn;
+            ((int32_t*)v.fmax)[i] = s_fmax[i] = st.fmx;
+            ((int32_t*)v.col_first)[i] = s_first[i] = st.first;
+            ((int32_t*)v.col_last)[i] = s_last[i] = st.last;
+            s_len[ORDER_COLS][i] = max(st.last - st.first + 1, 0);
+            if (st.invalid) s_bad = 1;
+        }
+    }
+    __syncthreads();
+    for (int i = warp; i < nblk; i += META_SMALL_THREADS / 32) {
+        const int base = i - s_n[i];
+        const int count = meta_classify_row(s_n[i], s_T[i], s_kmin + base, s_kmax + base, s_fmin + base, s_fmax + base,
+                                            (uint8_t*)v.tile_class + s_at[i], (uint16_t*)v.row_list + s_at[i]);
+        if (lane == 0) {
+            ((int32_t*)v.row_cnt)[i] = s_len[ORDER_ROWS][i] = count;
+            if (s_n[i] % 2 == 0) {
+                int first, last;
+                pair_range(s_first, s_last, i, (s_n[i] + 1) * TILE < s_T[i], first, last);
+                s_len[ORDER_PAIRS][i] = max(last - first + 1, 0);
+            }
+        }
+    }
+    __syncthreads();
+    // A quarter warp per item: its place is the number of items before it
+    const bool exact = meta_exact(max_seqlen);
+    const int nbins = meta_bins(max_seqlen, 1 << 30);
+    for (int x = tid >> 3; x < 3 * META_SMALL; x += META_SMALL_THREADS / 8) {
+        const int what = x / META_SMALL, i = x % META_SMALL, len = s_len[what][i];
+        const int mine = meta_bin(max(len, 0), exact, nbins);
+        int before = 0;
+        if (len >= 0)
+            for (int j = lane & 7; j < nblk; j += 8) {
+                const int other = s_len[what][j], k = meta_bin(max(other, 0), exact, nbins);
+                if (other >= 0 && (k < mine || (k == mine && j < i))) ++before;
+            }
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+        if (len >= 0 && (lane & 7) == 0) {
+            int32_t* order = (int32_t*)(what == ORDER_ROWS ? v.fwd_order : what == ORDER_COLS ? v.bwd_order : v.pair_order);
+            order[before] = i;
+            if (what == ORDER_COLS) ((int32_t*)v.bwd_len)[before] = len;
+            if (what == ORDER_PAIRS) ((int32_t*)v.pair_len)[before] = len;
+        }
+    }
+    if (warp == 0) {
+        MetaHeader h;
+        int most[3], items[3];
+        unsigned int sum[3];
+#pragma unroll
+        for (int what = 0; what < 3; ++what) {
+            const int a = s_len[what][lane], b = s_len[what][lane + 32];
+            most[what] = max(__reduce_max_sync(0xffffffffu, max(a, b)), 0);
+            sum[what] = __reduce_add_sync(0xffffffffu, (unsigned)(max(a, 0) + max(b, 0)));
+            items[what] = __popc(__ballot_sync(0xffffffffu, a >= 0)) + __popc(__ballot_sync(0xffffffffu, b >= 0));
+        }
+        h.magic = META_MAGIC;
+        h.status = s_bad ? KVS_ERR_BAD_EVICT : KVS_OK;
+        h.batch = batch;
+        h.total_tokens = total_tokens;
+        h.max_seqlen = max_seqlen;
+        h.nblk_total = nblk;
+        h.ncls_total = (uint32_t)s_ncls;
+        h.general = (key_first || complement) ? 1 : 0;
+        h.npair_total = items[ORDER_PAIRS];
+        h.rows_done = 0;
+        h.blk_most = most[ORDER_COLS];
+        h.pair_most = most[ORDER_PAIRS];
+        h.blk_tiles = sum[ORDER_COLS];
+        h.pair_tiles = sum[ORDER_PAIRS];
+        if (lane == 0) *v.hdr = h;
+    }
 }
 
 // ---- compaction event log -> evict_at ---------------------------------------------------------
@@ -380,6 +553,9 @@ int launch_mask_meta(const int32_t* key_evict, const int32_t* key_first, int com
     if (meta_bytes < L.total) return KVS_ERR_WORKSPACE;
     cudaStream_t st = (cudaStream_t)stream;
     MetaView v = meta_view(meta_buf, L);
+    if (L.nb_cap <= META_SMALL && batch <= META_SMALL_BATCH)
+        return launch_after(meta_small_kernel, 1, META_SMALL_THREADS, 0, st, key_evict, key_first, complement, cu_seqlens, batch, total_tokens,
+                            max_seqlen, v, L.nb_cap, (unsigned long long)L.cls_cap);
     const int grid = (L.nb_cap + META_WARPS - 1) / META_WARPS;
     const int rc = launch_after(meta_blocks_kernel, grid, META_THREADS, 0, st, key_evict, key_first, complement, cu_seqlens, batch, total_tokens,
                                 max_seqlen, v.hdr, (int32_t*)v.blk_off, (uint32_t*)v.cls_off, (int32_t*)v.seq_start, (int32_t*)v.blk_trace,
