@@ -536,10 +536,11 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
                 w.n_iter = -1;
                 BwdUnit unit;
                 if (ok && bwd_unit_of(p, mv.bwd_order, n_items, x, unit, w.g)) {
-                    const int b = mv.blk_trace[unit.block], G = p.Hq / p.Hkv;
-                    w.n = unit.block - mv.blk_off[b];
-                    w.tok0 = mv.seq_start[b];
-                    w.T = mv.seq_start[b + 1] - w.tok0;
+                    const int4 me = mv.info[unit.block];
+                    const int G = p.Hq / p.Hkv;
+                    w.n = me.z;
+                    w.tok0 = me.x;
+                    w.T = me.y;
                     w.m_first = mv.col_first[unit.block];           // == n unless the key slots were re-ordered
                     w.m_last = mv.col_last[unit.block];
                     w.general = mv.hdr->general != 0;

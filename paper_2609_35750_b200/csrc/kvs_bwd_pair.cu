@@ -152,11 +152,11 @@ bwd_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     {
         BwdUnit unit;
         if (!bwd_unit_of(p, mv.pair_order, mv.hdr->npair_total, blockIdx.x >> 1, unit, w.g)) return;
-        const int b = mv.blk_trace[unit.block], G = p.Hq / p.Hkv;
-        const int n0 = unit.block - mv.blk_off[b];
+        const int4 me = mv.info[unit.block];
+        const int G = p.Hq / p.Hkv, n0 = me.z;
         w.n = n0 + (int)rank;                           // this CTA's key block; past the trace when its block count is odd
-        w.tok0 = mv.seq_start[b];
-        w.T = mv.seq_start[b + 1] - w.tok0;
+        w.tok0 = me.x;
+        w.T = me.y;
         pair_range(mv.col_first, mv.col_last, unit.block, (n0 + 1) * TILE < w.T, w.m_first, w.m_last);
         w.general = mv.hdr->general != 0;
         const int nm = w.m_last - w.m_first + 1;        // query blocks m_first .. m_last can see one of the two key blocks

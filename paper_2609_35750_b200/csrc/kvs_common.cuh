@@ -35,7 +35,7 @@ struct MetaHeader {
 // Byte offsets of the arrays inside meta_buf; a pure function of the three sizes so that
 // every entry point can recompute it.
 struct MetaLayout {
-    size_t blk_off, cls_off, seq_start, blk_trace, kmin, kmax, fmin, fmax, col_first, col_last, row_cnt, fwd_order, bwd_order, pair_order, bwd_len, pair_len, evict,
+    size_t blk_off, cls_off, seq_start, blk_trace, info, kmin, kmax, fmin, fmax, col_first, col_last, row_cnt, fwd_order, bwd_order, pair_order, bwd_len, pair_len, evict,
         kfirst, tile_class, row_list, total;
     int nb_cap;            // capacity in blocks
     size_t cls_cap;        // capacity in tiles
@@ -61,6 +61,7 @@ __host__ __device__ inline MetaLayout meta_layout(int batch, int total_tokens, i
     L.cls_off = o;   o = align_up(o + sizeof(uint32_t) * (batch + 1), 256);
     L.seq_start = o; o = align_up(o + sizeof(int32_t) * (batch + 1), 256);
     L.blk_trace = o; o = align_up(o + sizeof(int32_t) * nb_cap, 256);
+    L.info = o;      o = align_up(o + 4 * sizeof(int32_t) * nb_cap, 256);
     L.kmin = o;      o = align_up(o + sizeof(int32_t) * nb_cap, 256);
     L.kmax = o;      o = align_up(o + sizeof(int32_t) * nb_cap, 256);
     L.fmin = o;      o = align_up(o + sizeof(int32_t) * nb_cap, 256);
@@ -88,6 +89,7 @@ struct MetaView {
     const uint32_t* cls_off;    // [batch+1] first tile of each trace's class matrix
     const int32_t* seq_start;   // [batch+1] copy of cu_seqlens
     const int32_t* blk_trace;   // [nblk] trace of a global block
+    const int4* info;           // [nblk] first token and length of the block's trace, block of the trace, first tile of its row
     const int32_t* kmin;        // [nblk] min / max over the block's key slots of the eviction step
     const int32_t* kmax;        // [nblk]
     const int32_t* fmin;        // [nblk] min / max over the block's key slots of the first query that may see the slot
@@ -114,6 +116,7 @@ inline MetaView meta_view(const void* buf, const MetaLayout& L) {
     v.cls_off = (const uint32_t*)(p + L.cls_off);
     v.seq_start = (const int32_t*)(p + L.seq_start);
     v.blk_trace = (const int32_t*)(p + L.blk_trace);
+    v.info = (const int4*)(p + L.info);
     v.kmin = (const int32_t*)(p + L.kmin);
     v.kmax = (const int32_t*)(p + L.kmax);
     v.fmin = (const int32_t*)(p + L.fmin);

@@ -100,12 +100,12 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     auto item_of = [&](int x, int y) {
         FwdItem it;
         const int gb = mv.fwd_order[x];
-        const int b = mv.blk_trace[gb];
+        const int4 me = mv.info[gb];
         it.nlist = mv.row_cnt[gb];
-        it.m = gb - mv.blk_off[b];
-        it.tok0 = mv.seq_start[b];
-        it.T = mv.seq_start[b + 1] - it.tok0;
-        it.at = (long long)(mv.cls_off[b] + (size_t)it.m * ((it.T + TILE - 1) / TILE));
+        it.tok0 = me.x;
+        it.T = me.y;
+        it.m = me.z;
+        it.at = (long long)(uint32_t)me.w;
         it.g = y / pairs_per_group;
         it.h0 = it.g * G + 2 * (y % pairs_per_group);
         // An odd group ends with a single head.  Its item still runs both softmax groups: they take alternate key blocks of

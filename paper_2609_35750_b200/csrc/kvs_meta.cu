@@ -95,17 +95,18 @@ __device__ __forceinline__ int meta_bin(int len, bool exact, int nbins) { return
 __global__ void __launch_bounds__(META_THREADS)
 meta_blocks_kernel(const int32_t* __restrict__ evict_at, const int32_t* __restrict__ key_first, int complement,
                    const int32_t* __restrict__ cu_seqlens, int batch, int total_tokens, int max_seqlen, MetaHeader* hdr, int32_t* blk_off,
-                   uint32_t* cls_off, int32_t* seq_start, int32_t* blk_trace, int nb_cap, unsigned long long cls_cap, int32_t* kmin,
+                   uint32_t* cls_off, int32_t* seq_start, int32_t* blk_trace, int4* info, int nb_cap, unsigned long long cls_cap, int32_t* kmin,
                    int32_t* kmax, int32_t* fmin, int32_t* fmax, int32_t* col_first, int32_t* col_last, int32_t* row_cnt,
                    int32_t* evict_copy, int32_t* first_copy) {
     __shared__ unsigned long long s_cls[META_WARPS];
     __shared__ long long s_blk[META_WARPS];
-    __shared__ int4 s_mine[META_WARPS];              // trace, its first block, its first token, its length
+    __shared__ int s_trace[META_WARPS];
+    __shared__ int4 s_mine[META_WARPS];              // the block's info
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     pdl_wait();
     const long long blk0 = (long long)blockIdx.x * META_WARPS;
     const bool writer = blockIdx.x == 0;
-    if (tid < META_WARPS) s_mine[tid].x = -1;
+    if (tid < META_WARPS) s_trace[tid] = -1;
     bool bad = cu_seqlens[0] != 0 || cu_seqlens[batch] != total_tokens;
     long long nblk = 0;
     unsigned long long ncls = 0;
@@ -151,7 +152,10 @@ meta_blocks_kernel(const int32_t* __restrict__ evict_at, const int32_t* __restri
         }
         if (b < batch) {
             const long long lo = max(first, blk0), hi = min(first + nb, blk0 + META_WARPS);
-            for (long long i = lo; i < hi; ++i) s_mine[i - blk0] = make_int4(b, (int)first, (int)a, (int)T);
+            for (long long i = lo; i < hi; ++i) {
+                s_trace[i - blk0] = b;
+                s_mine[i - blk0] = make_int4((int)a, (int)T, (int)(i - first), (int)(uint32_t)(first_cls + (i - first) * nb));
+            }
             if (writer) {
                 blk_off[b] = (int32_t)first;
                 cls_off[b] = (uint32_t)first_cls;
@@ -180,12 +184,13 @@ meta_blocks_kernel(const int32_t* __restrict__ evict_at, const int32_t* __restri
         hdr->rows_done = 0;
     }
     const int4 mine = s_mine[warp];
-    if (blk0 + warp >= nblk || mine.x < 0) return;
+    if (blk0 + warp >= nblk || s_trace[warp] < 0) return;
     const int blk = (int)blk0 + warp;
-    const int n = blk - mine.y, tok0 = mine.z, T = mine.w;
+    const int n = mine.z, tok0 = mine.x, T = mine.y;
     const BlockStat st = meta_block_stat(evict_at, key_first, complement, n, tok0, T, evict_copy, first_copy);
     if (lane == 0) {
-        blk_trace[blk] = mine.x;
+        blk_trace[blk] = s_trace[warp];
+        info[blk] = mine;
         kmin[blk] = st.mn;
         kmax[blk] = st.mx;
         fmin[blk] = st.fmn;
@@ -314,8 +319,7 @@ __device__ void meta_order(int what, MetaHeader* hdr, const int32_t* blk_off, co
 // ---- kernel 2: one warp per query block row: classes and the compact non-empty list; the orders ----------------------
 // The first two CTAs sort the key blocks and the pairs, the others classify, and the last of those to finish sorts the rows.
 __global__ void __launch_bounds__(META_THREADS)
-meta_classify_kernel(MetaHeader* hdr, const int32_t* __restrict__ blk_off, const uint32_t* __restrict__ cls_off,
-                     const int32_t* __restrict__ seq_start, const int32_t* __restrict__ blk_trace,
+meta_classify_kernel(MetaHeader* hdr, const int32_t* __restrict__ blk_off, const int32_t* __restrict__ blk_trace, const int4* __restrict__ info,
                      const int32_t* __restrict__ kmin, const int32_t* __restrict__ kmax,
                      const int32_t* __restrict__ fmin, const int32_t* __restrict__ fmax, const int32_t* __restrict__ col_first,
                      const int32_t* __restrict__ col_last, uint8_t* tile_class, uint16_t* row_list, int32_t* row_cnt, int32_t* fwd_order,
@@ -331,12 +335,10 @@ meta_classify_kernel(MetaHeader* hdr, const int32_t* __restrict__ blk_off, const
     const int row = (blockIdx.x - 2) * META_WARPS + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (row < hdr->nblk_total) {
-        const int b = blk_trace[row];
-        const int base = blk_off[b];
-        const int m = row - base;
-        const int T = seq_start[b + 1] - seq_start[b];
-        const size_t at = cls_off[b] + (size_t)m * ((T + TILE - 1) / TILE);
-        const int count = meta_classify_row(m, T, kmin + base, kmax + base, fmin + base, fmax + base, tile_class + at, row_list + at);
+        const int4 me = info[row];
+        const int base = row - me.z;
+        const size_t at = (uint32_t)me.w;
+        const int count = meta_classify_row(me.z, me.y, kmin + base, kmax + base, fmin + base, fmax + base, tile_class + at, row_list + at);
         if (lane == 0) {
             if (row_cnt[row] < 0) set_status(&hdr->status, KVS_ERR_BAD_EVICT);       // the block's keys, seen by kernel 1
             row_cnt[row] = count;
@@ -425,6 +427,7 @@ meta_small_kernel(const int32_t* __restrict__ evict_at, const int32_t* __restric
         const BlockStat st = meta_block_stat(evict_at, key_first, complement, s_n[i], s_tok0[i], s_T[i], (int32_t*)v.evict, (int32_t*)v.kfirst);
         if (lane == 0) {
             ((int32_t*)v.blk_trace)[i] = s_trace[i];
+            ((int4*)v.info)[i] = make_int4(s_tok0[i], s_T[i], s_n[i], s_at[i]);
             ((int32_t*)v.kmin)[i] = s_kmin[i] = st.mn;
             ((int32_t*)v.kmax)[i] = s_kmax[i] = st.mx;
             ((int32_t*)v.fmin)[i] = s_fmin[i] = st.fmn;
@@ -559,11 +562,11 @@ int launch_mask_meta(const int32_t* key_evict, const int32_t* key_first, int com
     const int grid = (L.nb_cap + META_WARPS - 1) / META_WARPS;
     const int rc = launch_after(meta_blocks_kernel, grid, META_THREADS, 0, st, key_evict, key_first, complement, cu_seqlens, batch, total_tokens,
                                 max_seqlen, v.hdr, (int32_t*)v.blk_off, (uint32_t*)v.cls_off, (int32_t*)v.seq_start, (int32_t*)v.blk_trace,
-                                L.nb_cap, (unsigned long long)L.cls_cap, (int32_t*)v.kmin, (int32_t*)v.kmax, (int32_t*)v.fmin,
+                                (int4*)v.info, L.nb_cap, (unsigned long long)L.cls_cap, (int32_t*)v.kmin, (int32_t*)v.kmax, (int32_t*)v.fmin,
                                 (int32_t*)v.fmax, (int32_t*)v.col_first, (int32_t*)v.col_last, (int32_t*)v.row_cnt, (int32_t*)v.evict,
                                 (int32_t*)v.kfirst);
     if (rc != KVS_OK) return rc;
-    return launch_after(meta_classify_kernel, grid + 2, META_THREADS, 0, st, v.hdr, v.blk_off, v.cls_off, v.seq_start, v.blk_trace, v.kmin,
+    return launch_after(meta_classify_kernel, grid + 2, META_THREADS, 0, st, v.hdr, v.blk_off, v.blk_trace, v.info, v.kmin,
                         v.kmax, v.fmin, v.fmax, v.col_first, v.col_last, (uint8_t*)v.tile_class, (uint16_t*)v.row_list, (int32_t*)v.row_cnt,
                         (int32_t*)v.fwd_order, (int32_t*)v.bwd_order, (int32_t*)v.pair_order, (int32_t*)v.bwd_len, (int32_t*)v.pair_len);
 }
