@@ -98,9 +98,6 @@ __device__ void bwd_plan(const BwdPlanArgs& a) {
     const int sms = a.pairs ? BWD_SMS / 2 : BWD_SMS;
     const float share = (float)(a.pairs ? all->pair_tiles : all->blk_tiles) * a.G * a.all_Hkv / sms;          // tiles per SM or pair
     for (int i = tid; i < a.arrived_n; i += 256) a.arrived[i] = 0;
-    if (tid < NC) s_units[tid] = s_cut[tid] = s_longest[tid] = 0;
-    if (tid == 0) s_run[0] = s_run[1] = s_heavy = 0;
-    __syncthreads();
     int cand[NC];
     const float frac[NC] = {0.25f, 0.5f, 0.75f, 1.0f, 1.25f, 1.6f, 2.2f, 0.f};
 #pragma unroll
@@ -108,6 +105,79 @@ __device__ void bwd_plan(const BwdPlanArgs& a) {
         const float l = fmaxf(ceilf(share * frac[k]), (float)max(BWD_MIN_UNIT, (most + BWD_MAX_CUT - 1) / BWD_MAX_CUT));
         cand[k] = (k == NC - 1 || l > (float)most) ? most : (int)l;
     }
+    // What a warp makes of the candidates' numbers (lane k: those of candidate k): the longest unit, and from which length on
+    // units of all heads start first.
+    auto choose = [&](int n_units, int n_cut, int n_longest, int& length, float& heavy) {
+        const int k = lane & (NC - 1);
+        const float units = (float)n_units * a.all_Hkv, longest = (float)n_longest, head = share / a.all_Hkv;
+        const float waves = ceilf(units / sms);
+        float est = longest + BWD_UNIT_COST;
+        if (waves > 1.f) {
+            est = share + (BWD_UNIT_COST * units + BWD_CUT_COST * n_cut * a.all_Hkv) / sms + 0.5f * fminf(longest, head);
+            est = fmaxf(est, longest + BWD_UNIT_COST);
+            if (waves <= 3.f) est = fmaxf(est, waves * (share * sms / units + BWD_UNIT_COST));
+        }
+        if (n_cut > 0) est += BWD_CUT_COST;
+        if (k < NC - 1 && (long long)n_cut * a.all_Hkv > a.all_slots) est = INFINITY;          // "no cut" always fits
+        float best = est;
+        int at = k;
+#pragma unroll
+        for (int o = 1; o < NC; o <<= 1) {
+            const float e = __shfl_xor_sync(0xffffffffu, best, o);
+            const int x = __shfl_xor_sync(0xffffffffu, at, o);
+            if (e < best || (e == best && x > at)) {
+                best = e;
+                at = x;
+            }
+        }
+        length = cand[0];
+#pragma unroll
+        for (int c = 1; c < NC; ++c) length = c == at ? cand[c] : length;
+        heavy = part->max_seqlen <= 16 * TILE ? 0.125f * share : __shfl_sync(0xffffffffu, longest, at) > 1.5f * head ? head : INFINITY;
+    };
+    auto unit_of = [&](int block, int t, int c, int i, int slot0) {      // the i-th of an item's c units
+        return BwdUnit{block, (int)((long long)t * i / c), (int)((long long)t * (i + 1) / c), c > 1 ? (slot0 << 18 | i << 9 | c) : 0};
+    };
+    if (n_all <= 32 && part == all) {       // a few items: one warp, an item a lane, no synchronisation of the CTA
+        if (warp != 0) return;
+        const int t = lane < n_all ? a.G * all_len0 : 0;
+        int my_units = 0, my_cut = 0, my_longest = 0;
+#pragma unroll
+        for (int k = 0; k < NC; ++k) {
+            const int c = lane >= n_all ? 0 : t > cand[k] ? (t + cand[k] - 1) / cand[k] : 1;
+            const int units = __reduce_add_sync(0xffffffffu, c), cut = __reduce_add_sync(0xffffffffu, c > 1 ? c : 0);
+            const int longest = __reduce_max_sync(0xffffffffu, c > 1 ? (t + c - 1) / c : t);
+            if ((lane & (NC - 1)) == k) {
+                my_units = units;
+                my_cut = cut;
+                my_longest = longest;
+            }
+        }
+        int longest;
+        float heavy_from;
+        choose(my_units, my_cut, my_longest, longest, heavy_from);
+        const int c = lane < n_all ? max((t + longest - 1) / longest, 1) : 0;
+        int iu = c, is = c > 1 ? c : 0;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, iu, o), s = __shfl_up_sync(0xffffffffu, is, o);
+            if (lane >= o) {
+                iu += u;
+                is += s;
+            }
+        }
+        for (int i = 0; i < c; ++i) a.units[iu - c + i] = unit_of(order0, t, c, i, is - (c > 1 ? c : 0));
+        const int heavy = __reduce_add_sync(0xffffffffu, (float)t > heavy_from * c ? c : 0);
+        if (lane == 31) {
+            a.plan->n_units = iu;
+            a.plan->slots = is;
+            a.plan->n_heavy = heavy;
+        }
+        return;
+    }
+    if (tid < NC) s_units[tid] = s_cut[tid] = s_longest[tid] = 0;
+    if (tid == 0) s_run[0] = s_run[1] = s_heavy = 0;
+    __syncthreads();
     {
         int units[NC], cut[NC], longest[NC];
 #pragma unroll
@@ -137,33 +207,12 @@ __device__ void bwd_plan(const BwdPlanArgs& a) {
     __syncthreads();
     if (warp == 0) {                        // lane k: candidate k
         const int k = lane & (NC - 1);
-        const float units = (float)s_units[k] * a.all_Hkv, longest = (float)s_longest[k], head = share / a.all_Hkv;
-        const float waves = ceilf(units / sms);
-        float est = longest + BWD_UNIT_COST;
-        if (waves > 1.f) {
-            est = share + (BWD_UNIT_COST * units + BWD_CUT_COST * s_cut[k] * a.all_Hkv) / sms + 0.5f * fminf(longest, head);
-            est = fmaxf(est, longest + BWD_UNIT_COST);
-            if (waves <= 3.f) est = fmaxf(est, waves * (share * sms / units + BWD_UNIT_COST));
-        }
-        if (s_cut[k] > 0) est += BWD_CUT_COST;
-        if (k < NC - 1 && (long long)s_cut[k] * a.all_Hkv > a.all_slots) est = INFINITY;          // "no cut" always fits
-        float best = est;
-        int at = k;
-#pragma unroll
-        for (int o = 1; o < NC; o <<= 1) {
-            const float e = __shfl_xor_sync(0xffffffffu, best, o);
-            const int x = __shfl_xor_sync(0xffffffffu, at, o);
-            if (e < best || (e == best && x > at)) {
-                best = e;
-                at = x;
-            }
-        }
-        if (lane == at) {
-            int l = cand[0];
-#pragma unroll
-            for (int c = 1; c < NC; ++c) l = c == at ? cand[c] : l;
-            s_len = l;
-            s_heavy_from = part->max_seqlen <= 16 * TILE ? 0.125f * share : longest > 1.5f * head ? head : INFINITY;
+        int length;
+        float heavy;
+        choose(s_units[k], s_cut[k], s_longest[k], length, heavy);
+        if (lane == 0) {
+            s_len = length;
+            s_heavy_from = heavy;
         }
     }
     __syncthreads();
@@ -208,7 +257,7 @@ __device__ void bwd_plan(const BwdPlanArgs& a) {
         const int u0 = bu + iu - c, slot0 = bs + is - (c > 1 ? c : 0);
         if (c > 0 && (float)t > heavy_from * c) atomicAdd(&s_heavy, c);
         for (int i = 0; i < c; ++i)
-            a.units[u0 + i] = BwdUnit{block, (int)((long long)t * i / c), (int)((long long)t * (i + 1) / c), c > 1 ? (slot0 << 18 | i << 9 | c) : 0};
+            a.units[u0 + i] = unit_of(block, t, c, i, slot0);
         __syncthreads();
         if (tid == 255) {
             s_run[0] = bu + iu;
