@@ -1,0 +1,106 @@
+"""Metadata of small batches by one CTA, units and items that are chained in a CTA (needs a B200).
+
+Up to 64 blocks the metadata is one kernel, above it is two: a batch at the line gives the same results, bit for bit, as the same
+traces with one-token traces behind them.  Rows and whole key blocks (a workspace of the base size) are summed in the same order
+on both sides, so out, lse, dk and dv are equal; dq is added in the order of arrival, fp32, each term at most 2^-24 off."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2609_35750_b200 import binding as B
+from paper_2609_35750_b200 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def _pass(ev, cu, longest, ts, Hq, general=None):
+    q, k, v, do = ts
+    batch = len(cu) - 1
+    cud = torch.from_numpy(cu).cuda()
+    meta = B.kvs_mask_meta_keys(*general, cud, longest) if general else B.kvs_mask_meta(ev, cud, longest)
+    out, lse = B.kvs_attn_fwd(q, k, v, meta, batch, longest)
+    ws = torch.empty(-(-(256 + 4 * q.shape[0] * Hq) // 256) * 256, dtype=torch.uint8, device="cuda")
+    grads = B.kvs_attn_bwd(do, q, k, v, out, lse, meta, batch, longest, 0.0, B.GRAD_FP32, workspace=ws)
+    assert B.kvs_device_status(meta) == B.KVS_OK and B.kvs_device_status(ws) == B.KVS_OK
+    cls = B.kvs_mask_meta_export(meta, cu, q.shape[0], longest)
+    return (out, lse) + grads, cls
+
+
+@pytest.mark.parametrize("lens", [[8192], [8065], [1], [128] * 64, [127, 0, 129, 0, 0, 385, 1], [2048, 2049, 1, 3000], [1] * 62 + [129]])
+def test_one_cta_equals_two_kernels(lens):
+    Hq, Hkv, d = 2, 1, 64
+    r = np.random.default_rng(len(lens))
+    ev = np.concatenate([W.keep_last_k_evict_at(T, max(1, T // 16), r.integers(8, max(9, T // 8), size=T), 4) for T in lens if T])
+    more = lens + [1] * 65
+    total, all_tokens = sum(lens), sum(more)
+    ev = torch.from_numpy(np.concatenate([ev, np.full(65, 2 ** 31 - 1, dtype=np.int32)]).astype(np.int32)).cuda()
+    g = torch.Generator(device="cuda").manual_seed(total)
+    ts = [torch.randn((all_tokens, h, d), generator=g, device="cuda", dtype=torch.bfloat16) for h in (Hq, Hkv, Hkv, Hq)]
+    cu = np.concatenate([[0], np.cumsum(more)]).astype(np.int32)
+    small, cls = _pass(ev[:total].clone(), cu[:len(lens) + 1].copy(), max(lens), [t[:total].clone() for t in ts], Hq)
+    large, cls_l = _pass(ev, cu, max(lens), ts, Hq)
+    for a, b in zip(cls, cls_l):
+        assert np.array_equal(a, b[:len(a)])
+    for name, a, b in zip(("out", "lse", "dq", "dk", "dv"), small, large):
+        b = b[:, :total] if name == "lse" else b[:total]
+        if name == "dq":
+            assert (a - b).norm() <= 2.0 ** -24 * -(-max(lens) // 128) * max(1.0, b.norm().item()) * 4
+        else:
+            assert torch.equal(a, b), name
+
+
+@pytest.mark.parametrize("Hq,Hkv,d", [(4, 4, 64), (4, 2, 128)])
+def test_chained_units_with_key_blocks_that_nobody_sees(Hq, Hkv, d):
+    # 300 traces of 300: several units a CTA; every third key block is seen by no query (no tiles, zero gradients), single keys
+    # of others neither
+    T, n = 300, 300
+    r = np.random.default_rng(d)
+    first = np.tile(np.arange(T, dtype=np.int32), n)
+    evict = np.full(T * n, 2 ** 31 - 1, dtype=np.int32)
+    block = (np.arange(T * n) % T) // 128 + 3 * (np.arange(T * n) // T)
+    evict[(block % 3 == 1) & (r.random(3 * n) < 0.5)[block]] = 0
+    evict[(first % 128 != 0) & (r.random(T * n) < 0.1)] = 0
+    g = torch.Generator(device="cuda").manual_seed(d)
+    ts = [torch.randn((T * n, h, d), generator=g, device="cuda", dtype=torch.bfloat16) for h in (Hq, Hkv, Hkv, Hq)]
+    cu = np.arange(0, T * n + 1, T).astype(np.int32)
+    fd, ed = torch.from_numpy(first).cuda(), torch.from_numpy(evict).cuda()
+    (out, lse, dq, dk, dv), _ = _pass(None, cu, T, ts, Hq, (fd, ed))
+    gone = ed == 0
+    assert not dk[gone].any() and not dv[gone].any()
+    q, k, v, do = (t.double().view(n, T, -1, d) for t in ts)
+    i = torch.arange(T, device="cuda")
+    seen = (i[None, None] <= i[None, :, None]) & ~gone.view(n, 1, T)
+    k, v = k.repeat_interleave(Hq // Hkv, 2), v.repeat_interleave(Hq // Hkv, 2)
+    s = (torch.einsum("bihd,bjhd->bhij", q, k) * d ** -0.5).masked_fill(~seen[:, None], -float("inf"))
+    p = torch.softmax(s, 3)
+    o = torch.einsum("bhij,bjhd->bihd", p, v)
+    ds = p * (torch.einsum("bihd,bjhd->bhij", do, v) - (do * o).sum(3).transpose(1, 2)[..., None]) * d ** -0.5
+    fold = lambda t: t.view(n, T, Hkv, -1, d).sum(3)  # noqa: E731
+    want = (o, torch.einsum("bhij,bjhd->bihd", ds, k), fold(torch.einsum("bhij,bihd->bjhd", ds, q)), fold(torch.einsum("bhij,bihd->bjhd", p, do)))
+    for name, a, b in zip(("out", "dq", "dk", "dv"), (out, dq, dk, dv), want):
+        b = b.reshape(a.shape)
+        assert ((a - b).norm() / b.norm()) <= 5e-3, name          # bf16 operands: probabilities and score gradients to 8 bits
+
+
+@pytest.mark.parametrize("lens,Hq,Hkv,d", [([1], 2, 1, 64), ([300] * 80, 8, 2, 128), ([300] * 80, 6, 2, 64), ([2000, 130], 7, 1, 128)])
+def test_teacher_rows_are_merged_as_they_are_written(lens, Hq, Hkv, d):
+    # rows without an evicted key are the student's; against plain causal attention of the same kernel.  The student's part comes
+    # as bf16 (half a unit in the last place, 2^-9), the result is rounded once more.
+    r = np.random.default_rng(d)
+    ev = np.concatenate([W.keep_last_k_evict_at(T, max(1, T // 16), r.integers(8, max(9, T // 8), size=T), 4) for T in lens])
+    cu = torch.from_numpy(np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)).cuda()
+    g = torch.Generator(device="cuda").manual_seed(d)
+    q, k, v = (torch.randn((sum(lens), h, d), generator=g, device="cuda", dtype=torch.bfloat16) for h in (Hq, Hkv, Hkv))
+    evd = torch.from_numpy(ev).cuda()
+    ms, me = B.kvs_mask_meta(evd, cu, max(lens)), B.kvs_mask_meta_evicted(evd, cu, max(lens))
+    os, ls, ot, lt = B.kvs_attn_fwd_dual(q, k, v, ms, me, len(lens), max(lens))
+    full = B.kvs_mask_meta(torch.full_like(evd, 2 ** 31 - 1), cu, max(lens))
+    want, lse = B.kvs_attn_fwd(q, k, v, full, len(lens), max(lens))
+    plain, _ = B.kvs_attn_fwd(q, k, v, ms, len(lens), max(lens))
+    assert torch.equal(os, plain)
+    assert (lt - lse).abs().max() <= 2e-3
+    assert ((ot.float() - want.float()).norm() / want.float().norm()) <= 2.0 ** -8
+    at = np.concatenate([np.arange(T) for T in lens])
+    nothing = np.concatenate([np.arange(T) < e.min() for T, e in zip(lens, np.split(ev, np.cumsum(lens)[:-1]))])
+    rows = torch.from_numpy(np.nonzero(nothing)[0]).cuda()
+    assert len(at) == len(nothing) and torch.equal(ot[rows], os[rows])
