@@ -29,6 +29,7 @@ namespace kvs {
 
 constexpr int FWD_THREADS = 384;
 constexpr float RESCALE_THRESHOLD = 8.0f;
+constexpr int FWD_LATE = 2;     // chained: key blocks left of an item when the CTA asks for the next one
 constexpr int P_SPLIT = 96;     // keys of a tile whose probabilities are handed to the MMA warp early
 
 // an item of work: a query block of a pair of heads (or of a single one)
@@ -71,10 +72,12 @@ struct FwdParams {
 // loads and products while the softmax groups still write out the one before.  With a CTA per item the launch, the chain of
 // metadata loads, the set-up, the first loads and the write-out stand beside the tiles of the row, which counts where rows are
 // short; the loop over items costs registers that the long rows' tiles are faster with (see launch_fwd for the line).
+// The parameters are passed by value and not read in place (__grid_constant__): that costs the tile loop registers, 1 to 5 % of long
+// rows (24576 tokens of token-level eviction 5085 -> 5330 us).
 template <int D, bool CHAIN>
 __global__ void __launch_bounds__(FWD_THREADS, 1)
 fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
-           const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ MetaView mv, const __grid_constant__ FwdParams p) {
+           const __grid_constant__ CUtensorMap tm_v, MetaView mv, FwdParams p) {
     using L = FwdSmem<D>;
     constexpr int NBOX = D / 64;             // 64-column TMA boxes per tile row
     constexpr int BOX_BYTES = TILE * 128;    // 128 rows x 128 bytes
@@ -147,7 +150,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     auto bar_item = [&](int s) { return bars + 8 * (23 + s); };      // item written
     auto bar_itemfree = [&](int s) { return bars + 8 * (25 + s); };  // item read by the producer, MMA and 8 softmax warps
     const uint32_t bar_ask = bars + 8 * 28;                          // the launch control has answered
-    const uint32_t bar_started = bars + 8 * 29;                      // the MMA warp has begun an item
+    const uint32_t bar_late = bars + 8 * 29;                      // the MMA warp is near the end of an item
     auto put = [&](int slot, const FwdItem& it) {
         volatile FwdItem* dst = s_item + slot;
         dst->nlist = it.nlist;
@@ -199,7 +202,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         mbar_init(bar_xfree, 4);
         mbar_init(bar_x, 4);
         mbar_init(bar_ask, 1);
-        mbar_init(bar_started, 1);
+        mbar_init(bar_late, 1);
         fence_mbar_init();
     }
     if (!CHAIN && tid == 256) put(0, item_of(blockIdx.x, blockIdx.y));
@@ -320,9 +323,9 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
             }
         } else if (CHAIN && warp == 10) {
             // ================= work list =================
-            // The first item is the CTA's own; after it the CTAs that have not started yet, one at a time and only once the item
-            // before is under way, so that the last items still go to whoever is free.  The chain of metadata loads of an
-            // item lies beside the one before.
+            // The first item is the CTA's own; after it the CTAs that have not started yet, one at a time and only near the end of
+            // the item before, so that the last items still go to whoever is free (20 traces of 500 to 2000: 274 -> 271 us against
+            // asking at its start).  The chain of metadata loads of an item lies beside the one before.
             int x = blockIdx.x, y = blockIdx.y;
             bool ok = true;
             for (int r = 0, asked = 0;;) {
@@ -350,7 +353,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
                 }
                 __syncwarp();
                 if (!ok || *abort_flag) break;
-                mbar_wait(bar_started, r & 1, abort_flag, status);
+                mbar_wait(bar_late, r & 1, abort_flag, status);
                 ++r;
                 x = nblk;                                             // ask
             }
@@ -375,11 +378,15 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
                 int nlist, m, T, tok0, h0, ntile;
                 take(r, nlist, m, T, tok0, h0, ntile);
                 taken(r);
-                if (CHAIN) {
-                    if (lane == 0) mbar_arrive(bar_started);
-                    if (nlist < 0 || *abort_flag) break;
+                if (CHAIN && (nlist < 0 || *abort_flag)) break;
+                // the next item is asked for when this one has FWD_LATE key blocks left
+                auto near_end = [&](int i) {
+                    if (CHAIN && lane == 0 && (i + FWD_LATE == nlist || (i == 0 && nlist < FWD_LATE))) mbar_arrive(bar_late);
+                };
+                if (nlist == 0) {
+                    near_end(0);
+                    continue;
                 }
-                if (nlist == 0) continue;
                 const uint32_t r0 = ring;
                 ring += nlist;
                 mbar_wait(bar_q, q_items & 1, abort_flag, status);
@@ -421,6 +428,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
                     for (int i = 0; i < nlist; ++i) {
                         const int t = i & 1;
                         const uint32_t R = r0 + i;
+                        near_end(i);
                         issue_pv(t, R, i < 2, true);
                         if (leader) mma_commit(bar_vfree(R & 1));
                         if (i + 2 < nlist) {
@@ -439,6 +447,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
 #pragma unroll 1
                     for (int i = 0; i < nlist; ++i) {
                         const uint32_t R = r0 + i;
+                        near_end(i);
 #pragma unroll 1
                         for (int t = 0; t < 2; ++t) {
                             issue_pv(t, R, i == 0, t == 0);
