@@ -153,6 +153,9 @@ int make_tmap_f32_thd(CUtensorMap* map, const void* base, int total_tokens, int 
 // coordinates per instruction), 128-byte swizzle
 int make_tmap_rows(CUtensorMap* map, const void* base, int rows, int cols);
 int check_device_sm100();
+// kvs_attn_fwd over more keys of the same queries: merged with the result over the first ones
+int attn_fwd_merged(const void* q, const void* k, const void* v, const void* meta_buf, int batch, int total_tokens, int max_seqlen, int Hq, int Hkv,
+                    int head_dim, float softmax_scale, const void* first_out, const float* first_lse, void* out, float* lse, kvs_stream_t stream);
 
 // A refused call leaves no error behind: the runtime keeps the last one until it is asked for, and the next check after a
 // plain launch would report it.
@@ -498,6 +501,36 @@ struct RowStage {
             w.w = pack_bf16(__uint_as_float(r[e * 8 + 6]), __uint_as_float(r[e * 8 + 7]));
             *reinterpret_cast<uint4*>(row + (chunk(lane, i * 4 + e, COLS / 8) << 4)) = w;
         }
+    }
+    // as bf16 again
+    __device__ static __forceinline__ void get_bf16(const uint8_t* stage, int lane, int i, uint32_t (&w)[16]) {
+        const uint8_t* row = stage + lane * (COLS * 2);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const uint4 x = *reinterpret_cast<const uint4*>(row + (chunk(lane, i * 4 + e, COLS / 8) << 4));
+            w[e * 4] = x.x;
+            w[e * 4 + 1] = x.y;
+            w[e * 4 + 2] = x.z;
+            w[e * 4 + 3] = x.w;
+        }
+    }
+    // the first `rows` rows from memory
+    template <int BYTES>
+    __device__ static __forceinline__ void fetch(uint8_t* stage, int lane, const char* src, size_t stride, int rows) {
+        constexpr int CHUNKS = COLS * BYTES / 16, STEP = 32 / CHUNKS;
+        const int c = lane % CHUNKS;
+        uint4 w[32 / STEP];
+#pragma unroll
+        for (int r0 = 0; r0 < 32; r0 += STEP) {
+            const int r = r0 + lane / CHUNKS;
+            w[r0 / STEP] = r < rows ? *reinterpret_cast<const uint4*>(src + (size_t)r * stride * BYTES + c * 16) : make_uint4(0, 0, 0, 0);
+        }
+#pragma unroll
+        for (int r0 = 0; r0 < 32; r0 += STEP) {
+            const int r = r0 + lane / CHUNKS;
+            *reinterpret_cast<uint4*>(stage + r * (COLS * BYTES) + (chunk(r, c, CHUNKS) << 4)) = w[r0 / STEP];
+        }
+        __syncwarp();
     }
     // the piece's first `rows` rows to memory, `stride` elements of BYTES bytes apart
     template <int BYTES>

@@ -24,6 +24,7 @@
 // maximum until the running maximum exceeds it by more than 8 (base-2), so exp2 arguments stay
 // below 2^8 and the rescale of O in tensor memory is rare.
 #include "kvs_common.cuh"
+#include <type_traits>
 
 namespace kvs {
 
@@ -65,6 +66,8 @@ struct FwdParams {
     float scale_log2;   // softmax_scale * log2(e)
     __nv_bfloat16* out;
     float* lse;
+    const __nv_bfloat16* first_out;     // MERGE: the result over the other keys of the same queries, in the layout of out and lse
+    const float* first_lse;
 };
 
 
@@ -72,9 +75,12 @@ struct FwdParams {
 // loads and products while the softmax groups still write out the one before.  With a CTA per item the launch, the chain of
 // metadata loads, the set-up, the first loads and the write-out stand beside the tiles of the row, which counts where rows are
 // short; the loop over items costs registers that the long rows' tiles are faster with (see launch_fwd for the line).
+// MERGE: out and lse are those of attention over these keys and the ones that first_out and first_lse stand for (the teacher's of
+// self-distillation): the rows meet here, in fp32 and on their way out.  As a pass of its own the merge was bound by memory and
+// rounded this part to bf16 first: 3 traces of 9000 to 17000 tokens, 32 heads on 8, both forwards 4282 -> 4125 us.
 // The parameters are passed by value and not read in place (__grid_constant__): that costs the tile loop registers, 1 to 5 % of long
 // rows (24576 tokens of token-level eviction 5085 -> 5330 us).
-template <int D, bool CHAIN>
+template <int D, bool CHAIN, bool MERGE>
 __global__ void __launch_bounds__(FWD_THREADS, 1)
 fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
            const __grid_constant__ CUtensorMap tm_v, MetaView mv, FwdParams p) {
@@ -669,7 +675,19 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
                 ++singles;
             }
             if (!dual || t == 0) {
-                const float inv = (run_sum > 0.f && nlist > 0) ? 1.f / run_sum : 0.f;
+                float inv = (run_sum > 0.f && nlist > 0) ? 1.f / run_sum : 0.f;
+                float lse = ref_max * 0.6931471805599453f + logf(run_sum), w_first = 0.f;
+                if (MERGE) {
+                    const float other = valid ? p.first_lse[(size_t)h * p.total_tokens + tok0 + qi] : -INFINITY, mine = inv > 0.f ? lse : -INFINITY;
+                    const float top = fmaxf(other, mine);
+                    lse = -INFINITY;
+                    if (top > -INFINITY) {
+                        const float ea = __expf(other - top), eb = __expf(mine - top), sum = ea + eb;      // exp(-inf) = 0 for a part that saw no key
+                        w_first = ea / sum;
+                        inv *= eb / sum;
+                        lse = top + logf(sum);
+                    }
+                }
                 // Through shared memory to memory as whole rows: the whole row through the query tile, which no product reads any
                 // more, or, where the next item's comes there, in pieces of 64 bytes through memory of its own.
                 constexpr int COLS = CHAIN ? 32 : D;
@@ -682,7 +700,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
                     uint32_t r[32];
                     tmem_ld32(tmem_O + c * 32, r);
                     tmem_wait_ld();
-                    if (nlist == 0) {      // only a bad evict_at (already reported by the metadata pass) gets here
+                    if (nlist == 0) {      // a bad evict_at (already reported by the metadata pass), or nothing evicted yet
 #pragma unroll
                         for (int e = 0; e < 32; ++e) r[e] = 0u;
                     }
@@ -694,13 +712,26 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
                             r[e] = __float_as_uint(o);
                         }
                     }
+                    if (MERGE) {
+                        if (c % (COLS / 32) == 0)
+                            Rows::template fetch<2>(stage, lane, reinterpret_cast<const char*>(p.first_out + (orow - p.out) + (CHAIN ? c * 32 : 0)),
+                                                    (size_t)p.Hq * D, rows);
+                        uint32_t x[16];
+                        Rows::get_bf16(stage, lane, c % (COLS / 32), x);
 #pragma unroll
-                    for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) * inv);
+                        for (int e = 0; e < 16; ++e) {
+                            r[2 * e] = __float_as_uint(fmaf(__uint_as_float(x[e] << 16), w_first, __uint_as_float(r[2 * e]) * inv));
+                            r[2 * e + 1] = __float_as_uint(fmaf(__uint_as_float(x[e] & 0xffff0000u), w_first, __uint_as_float(r[2 * e + 1]) * inv));
+                        }
+                    } else {
+#pragma unroll
+                        for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) * inv);
+                    }
                     Rows::put_bf16(stage, lane, c % (COLS / 32), r);
                     if ((c + 1) % (COLS / 32) == 0)
                         Rows::template flush<2>(stage, lane, reinterpret_cast<char*>(orow + (CHAIN ? c * 32 : 0)), (size_t)p.Hq * D, rows);
                 }
-                if (valid) p.lse[(size_t)h * p.total_tokens + tok0 + qi] = ref_max * 0.6931471805599453f + logf(run_sum);
+                if (valid) p.lse[(size_t)h * p.total_tokens + tok0 + qi] = lse;
             }
             if (nlist > 0) {
                 tc_fence_before();
@@ -721,10 +752,10 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     }
 }
 
-template <int D, bool CHAIN>
+template <int D, bool CHAIN, bool MERGE>
 static int launch_fwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const MetaView& mv, const FwdParams& p,
                       int nb_cap, cudaStream_t st) {
-    auto kern = fwd_kernel<D, CHAIN>;
+    auto kern = fwd_kernel<D, CHAIN, MERGE>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem<D>::DYN_BYTES) != cudaSuccess) return cuda_refused();
     return launch_after(kern, dim3(nb_cap, p.heads, 1), FWD_THREADS, FwdSmem<D>::DYN_BYTES, st, tq, tk, tv, mv, p);
 }
@@ -751,7 +782,7 @@ namespace {
 // q_ts / kv_ts: elements between consecutive tokens of q and of k, v (0: tensors of their own)
 int fwd_impl(const void* q, const void* k, const void* v, long long q_ts, long long kv_ts, const void* meta_buf, int batch,
              int total_tokens, int max_seqlen, int Hq, int Hkv, int head_dim, float softmax_scale, void* out, float* lse,
-             kvs_stream_t stream) {
+             kvs_stream_t stream, const void* first_out = nullptr, const float* first_lse = nullptr) {
     if (batch < 0 || total_tokens < 0 || max_seqlen < 0 || Hq <= 0 || Hkv <= 0) return KVS_ERR_INVALID_ARG;
     if (head_dim != 64 && head_dim != 128) return KVS_ERR_UNSUPPORTED;
     if (Hq % Hkv != 0 || Hq > 65535) return KVS_ERR_UNSUPPORTED;
@@ -779,10 +810,16 @@ int fwd_impl(const void* q, const void* k, const void* v, long long q_ts, long l
     p.scale_log2 = s * 1.4426950408889634f;
     p.out = (__nv_bfloat16*)out;
     p.lse = lse;
+    p.first_out = (const __nv_bfloat16*)first_out;
+    p.first_lse = first_lse;
     cudaStream_t st = (cudaStream_t)stream;
-    if (chain_items(batch, total_tokens, L.nb_cap, p.heads))
-        return head_dim == 64 ? launch_fwd<64, true>(tq, tk, tv, mv, p, L.nb_cap, st) : launch_fwd<128, true>(tq, tk, tv, mv, p, L.nb_cap, st);
-    return head_dim == 64 ? launch_fwd<64, false>(tq, tk, tv, mv, p, L.nb_cap, st) : launch_fwd<128, false>(tq, tk, tv, mv, p, L.nb_cap, st);
+    const bool chain = chain_items(batch, total_tokens, L.nb_cap, p.heads);
+    auto launch = [&](auto dim) {
+        constexpr int D = decltype(dim)::value;
+        if (first_out) return chain ? launch_fwd<D, true, true>(tq, tk, tv, mv, p, L.nb_cap, st) : launch_fwd<D, false, true>(tq, tk, tv, mv, p, L.nb_cap, st);
+        return chain ? launch_fwd<D, true, false>(tq, tk, tv, mv, p, L.nb_cap, st) : launch_fwd<D, false, false>(tq, tk, tv, mv, p, L.nb_cap, st);
+    };
+    return head_dim == 64 ? launch(std::integral_constant<int, 64>()) : launch(std::integral_constant<int, 128>());
 }
 }  // namespace
 
@@ -800,4 +837,11 @@ extern "C" int kvs_attn_fwd_packed(const void* qkv, const void* meta_buf, int ba
     const char* base = (const char*)qkv;
     return fwd_impl(base, base + (size_t)Hq * head_dim * 2, base + (size_t)(Hq + Hkv) * head_dim * 2, ts, ts, meta_buf, batch,
                     total_tokens, max_seqlen, Hq, Hkv, head_dim, softmax_scale, out, lse, stream);
+}
+
+int kvs::attn_fwd_merged(const void* q, const void* k, const void* v, const void* meta_buf, int batch, int total_tokens, int max_seqlen, int Hq,
+                         int Hkv, int head_dim, float softmax_scale, const void* first_out, const float* first_lse, void* out, float* lse,
+                         kvs_stream_t stream) {
+    return fwd_impl(q, k, v, 0, 0, meta_buf, batch, total_tokens, max_seqlen, Hq, Hkv, head_dim, softmax_scale, out, lse, stream, first_out,
+                    first_lse);
 }
