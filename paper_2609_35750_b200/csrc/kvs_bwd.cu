@@ -13,6 +13,14 @@
 namespace kvs {
 
 constexpr int BWD_SMS = 148;
+// A batch whose Q, dO and fp32 dQ are larger than this is listed by trace (see bwd_plan): sorted by length throughout, a trace's
+// key blocks run far apart and its tiles come from memory again for each (96 traces of 60 to 900 tokens, 16 heads on 2: 2.7 GB
+// moved at 5.7 TB/s, 1.5 GB by trace).  Main kernel, by length -> by trace, us, 32 heads on 8: 200 traces of 300 tokens 1219 ->
+// 977, 96 of 60 to 900 (16 on 2) 480 -> 434, 60 of 100 to 2000 (28 on 4) 1409 -> 1302, 12 of 1500 to 12000 5216 -> 5126, 8 of
+// 8000 4771 -> 4712, 9 of 14000 with nothing evicted (16 on 2) 18.1 -> 17.6 ms.  Of fewer traces than eight an eighth is not to
+// be had for the end (3 of 14000: 11.5 -> 11.8 ms; 4 of 20000 without groups 6.9 -> 7.0 ms).
+constexpr long long BWD_L2_BYTES = 96ll << 20;
+constexpr int BWD_MANY_TRACES = 8, BWD_MOST_LATE = 6;
 constexpr uint32_t BWD_LATE = 3;              // tiles left of a unit when the CTA asks for the next one
 constexpr int BWD_MIN_UNIT = 4;             // tiles: a shorter unit is mostly its own start and end
 constexpr int BWD_MAX_SLOTS = 2 * BWD_SMS;  // slots of one CTA each for the dK and dV of cut items, over all KV heads
@@ -53,6 +61,7 @@ struct BwdPlanArgs {
     MetaView all, mv;                       // the batch the cut is chosen for; the (part of the) batch whose units are listed
     int all_batch, all_tokens, all_maxlen, batch, tokens, maxlen;
     int all_cap, cap;                       // key blocks that the two have room for
+    int by_trace;                           // the batch does not fit in L2: see BWD_L2_BYTES
     int pairs;                              // items are pairs of key blocks
     int G, all_Hkv, Hkv;
     int all_slots, slots;                   // slots there are, of an item's CTAs, over all KV heads
@@ -86,7 +95,7 @@ __device__ void bwd_plan(const BwdPlanArgs& a) {
     const int32_t* len = a.pairs ? a.mv.pair_len : a.mv.bwd_len;
     const int32_t* order = a.pairs ? a.mv.pair_order : a.mv.bwd_order;
     if (!meta_matches(all, a.all_batch, a.all_tokens, a.all_maxlen) || !meta_matches(part, a.batch, a.tokens, a.maxlen)) {
-        if (tid == 0) a.plan->n_units = a.plan->n_heavy = 0;
+        if (tid == 0) a.plan->n_units = a.plan->n_heavy = a.plan->n_apart = 0;
         return;
     }
     // this thread's first item, on its way while the candidates are set up (the arrays have room for `cap` entries, with or
@@ -172,6 +181,7 @@ __device__ void bwd_plan(const BwdPlanArgs& a) {
             a.plan->n_units = iu;
             a.plan->slots = is;
             a.plan->n_heavy = heavy;
+            a.plan->n_apart = iu - heavy;
         }
         return;
     }
@@ -230,45 +240,68 @@ __device__ void bwd_plan(const BwdPlanArgs& a) {
         __syncthreads();
         if ((long long)s_cut[0] * a.Hkv > a.slots) longest = most;
     }
-    // List the units, the items' order kept: prefix sums of the items' units and of their slots
-    for (int x0 = 0; x0 < n; x0 += 256) {
-        const int x = x0 + tid;
-        const int t = x >= n ? 0 : a.G * (x0 ? len[x] : len0), block = x >= n ? 0 : (x0 ? order[x] : order0);
-        const int c = x < n ? max((t + longest - 1) / longest, 1) : 0;
-        int iu = c, is = c > 1 ? c : 0;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int u = __shfl_up_sync(0xffffffffu, iu, o), s = __shfl_up_sync(0xffffffffu, is, o);
-            if (lane >= o) {
-                iu += u;
-                is += s;
+    // Where the traces do not fit in L2 together, all but `late` eighths of them come in the order of the batch, a head's units
+    // and then the next head's: key blocks of a trace run together and share its Q and dO tiles and the lines of its dQ.  The
+    // others come last, longest items first and of all heads together, as much work as it takes for all SMs to end together.
+    const float part_share = (float)(a.pairs ? part->pair_tiles : part->blk_tiles) * a.G * a.Hkv / sms;
+    const int late = a.by_trace ? (int)ceilf(8.f * (float)min(longest, most) / fmaxf(part_share, 1.f)) : 8;
+    const bool by_trace = late <= BWD_MOST_LATE;
+    auto is_late = [&](int block) { return ((a.mv.blk_trace[block] * late) & 7) < late; };        // evenly spread over the batch
+    // List the units, the items' order kept (by trace: a pass for either part): prefix sums of the items' units and of their slots
+    int n_apart = 0;
+    for (int pass = by_trace ? 0 : 1; pass < 2; ++pass) {
+        for (int x0 = 0; x0 < n; x0 += 256) {
+            const int x = x0 + tid;
+            int t = 0, block = 0;
+            bool listed = x < n;
+            if (listed && pass == 0) {
+                block = x;
+                t = max(a.mv.col_last[x] - a.mv.col_first[x] + 1, 0);
+                listed = !is_late(x);
+            } else if (listed) {
+                t = x0 ? len[x] : len0;
+                block = x0 ? order[x] : order0;
+                listed = !by_trace || is_late(block);
             }
+            t *= a.G;
+            const int c = listed ? max((t + longest - 1) / longest, 1) : 0;
+            int iu = c, is = c > 1 ? c : 0;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_up_sync(0xffffffffu, iu, o), s = __shfl_up_sync(0xffffffffu, is, o);
+                if (lane >= o) {
+                    iu += u;
+                    is += s;
+                }
+            }
+            if (lane == 31) {
+                s_scan[0][warp] = iu;
+                s_scan[1][warp] = is;
+            }
+            __syncthreads();
+            int bu = s_run[0], bs = s_run[1];
+            for (int w = 0; w < warp; ++w) {
+                bu += s_scan[0][w];
+                bs += s_scan[1][w];
+            }
+            const int u0 = bu + iu - c, slot0 = bs + is - (c > 1 ? c : 0);
+            if (c > 0 && (float)t > heavy_from * c) atomicAdd(&s_heavy, c);
+            for (int i = 0; i < c; ++i)
+                a.units[u0 + i] = unit_of(block, t, c, i, slot0);
+            __syncthreads();
+            if (tid == 255) {
+                s_run[0] = bu + iu;
+                s_run[1] = bs + is;
+            }
+            __syncthreads();
         }
-        if (lane == 31) {
-            s_scan[0][warp] = iu;
-            s_scan[1][warp] = is;
-        }
-        __syncthreads();
-        int bu = s_run[0], bs = s_run[1];
-        for (int w = 0; w < warp; ++w) {
-            bu += s_scan[0][w];
-            bs += s_scan[1][w];
-        }
-        const int u0 = bu + iu - c, slot0 = bs + is - (c > 1 ? c : 0);
-        if (c > 0 && (float)t > heavy_from * c) atomicAdd(&s_heavy, c);
-        for (int i = 0; i < c; ++i)
-            a.units[u0 + i] = unit_of(block, t, c, i, slot0);
-        __syncthreads();
-        if (tid == 255) {
-            s_run[0] = bu + iu;
-            s_run[1] = bs + is;
-        }
-        __syncthreads();
+        if (pass == 0) n_apart = s_run[0];
     }
     if (tid == 0) {
         a.plan->n_units = s_run[0];
         a.plan->slots = s_run[1];
-        a.plan->n_heavy = s_heavy;
+        a.plan->n_heavy = by_trace ? 0 : s_heavy;
+        a.plan->n_apart = by_trace ? n_apart : s_run[0] - s_heavy;
     }
 }
 
@@ -1018,6 +1051,7 @@ int bwd_impl(const void* dout, const void* q, const void* k, const void* v, long
         pa.tokens = total_tokens;
         pa.maxlen = p.max_seqlen;
         pa.pairs = pair;
+        pa.by_trace = !pair && whole.batch >= BWD_MANY_TRACES && (long long)total_tokens * Hq * head_dim * 8 > BWD_L2_BYTES;
         pa.G = Hq / Hkv;
         pa.all_Hkv = whole.Hkv;
         pa.Hkv = Hkv;

@@ -28,8 +28,9 @@ struct BwdWork {
 struct BwdPlan {
     int32_t n_units;
     int32_t slots;          // slots used per KV head
-    int32_t n_heavy;        // the first n_heavy units of ALL heads start first; after them one head's units, then the next head's
-    int32_t pad;
+    // Which unit a CTA takes: the first n_heavy units of ALL heads start first; then, of the next n_apart, one head's, the next
+    // head's, ...; then what is left, again of all heads together.
+    int32_t n_heavy, n_apart;
 };
 constexpr int BWD_MAX_CUT = 511;          // units of an item, and the unit's index, are 9 bits each
 
@@ -73,16 +74,16 @@ size_t bwd_cut_bytes(int total_tokens, int Hq, int head_dim);
 // The unit and KV head of CTA (or pair) x of a one-dimensional grid; false: there is none.  The CTAs without work come last.
 // A whole item has tile1 = -1: all of its list.
 __device__ __forceinline__ bool bwd_unit_of(const BwdParams& p, const int32_t* order, int n_items, int x, BwdUnit& unit, int& g) {
-    const int n = p.plan ? p.plan->n_units : n_items, heavy = p.plan ? p.plan->n_heavy : 0;
+    const int n = p.plan ? p.plan->n_units : n_items, heavy = p.plan ? p.plan->n_heavy : 0, apart = p.plan ? p.plan->n_apart : n;
     if (x >= n * p.Hkv) return false;
     int u;
-    if (x < heavy * p.Hkv) {
+    if (x < heavy * p.Hkv || x >= (heavy + apart) * p.Hkv) {
         u = x / p.Hkv;
         g = x % p.Hkv;
     } else {
         x -= heavy * p.Hkv;
-        u = heavy + x % (n - heavy);
-        g = x / (n - heavy);
+        u = heavy + x % apart;
+        g = x / apart;
     }
     unit = p.plan ? p.units[u] : BwdUnit{order[u], 0, -1, 0};
     return true;

@@ -10,6 +10,8 @@ import torch
 from paper_2609_35750_b200 import binding as B
 from paper_2609_35750_b200 import workloads as W
 
+from .test_bwd_units import _backward, _inputs, _same
+
 pytestmark = pytest.mark.gpu
 
 
@@ -104,3 +106,16 @@ def test_teacher_rows_are_merged_as_they_are_written(lens, Hq, Hkv, d):
     nothing = np.concatenate([np.arange(T) < e.min() for T, e in zip(lens, np.split(ev, np.cumsum(lens)[:-1]))])
     rows = torch.from_numpy(np.nonzero(nothing)[0]).cuda()
     assert len(at) == len(nothing) and torch.equal(ot[rows], os[rows])
+
+
+@pytest.mark.parametrize("lens,Hq,Hkv,d,rule", [
+    ([300] * 90, 8, 2, 128, "turns"), ([300, 129, 0, 1, 700] * 40, 4, 4, 128, "tokens"), ([2200] * 9, 12, 2, 64, "causal"), ([4000] + [333] * 40, 16, 1, 64, "turns"),
+])
+def test_units_listed_by_trace_equal_whole_items(lens, Hq, Hkv, d, rule):
+    # batches whose Q, dO and dQ do not fit in L2: most traces in the order of the batch, the others last.  Against whole items in
+    # the metadata's order; the bound is that of test_bwd_units
+    assert sum(lens) * Hq * d * 8 > 96 << 20
+    x = _inputs(lens, Hq, Hkv, d, rule)
+    out, lse, ref = _backward(x, lens, True)
+    _, _, got = _backward(x, lens, False, out, lse)
+    _same(got, ref, max(lens), Hq // Hkv)
