@@ -401,6 +401,16 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
     extern __shared__ uint8_t smem_raw[];
     const int z = blockIdx.x, g = blockIdx.y, s = blockIdx.z;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    pdl_wait();
+    decode_header(p);
+    const int n = min(max(p.n_tokens[s], 0), p.max_pages * p.page_size);    // never past the sequence's table
+    const int ps = p.page_size;
+    const int ppt = 128 / ps;                                   // pages per tile (PAGES)
+    const int ntiles = (n + 127) >> 7;
+    const int per = (ntiles + p.nsplit - 1) / p.nsplit;         // contiguous tiles per split
+    const int t_begin = min(z * per, ntiles), t_end = min(t_begin + per, ntiles);
+    const int my_tiles = t_end - t_begin;
+
     const uint32_t sraw = smem_u32(smem_raw);
     const uint32_t sbase = (sraw + 1023u) & ~1023u;
     uint8_t* sgen = smem_raw + (sbase - sraw);
@@ -427,10 +437,9 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
         mbar_init(bar_done, 1);
         fence_mbar_init();
     }
-    // What touches nothing but this CTA's shared memory lies beside the kernel before (an append as a rule).
     if (warp == 4) {
-        if (lane == 0) prefetch_tmap(&tm_k);
-        if (PAGES && lane == 1) prefetch_tmap(&tm_v);
+        tmem_alloc(smem_u32(s_tmem), 32);
+        tmem_relinquish();
     } else {
         // V starts as zeros (rows no page is loaded into must stay finite: their weight is 0, and 0 x NaN is NaN);
         // Q: rows 0..G-1 of the 16-row B operand, the rest zero; P^T: rows >= G stay zero for good
@@ -438,21 +447,6 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
         for (int i = tid; i < 32768 / 16; i += 128) reinterpret_cast<uint4*>(sgen + DtcSmem::OFF_V)[i] = zero4;
         for (int i = tid; i < 8192 / 16; i += 128) reinterpret_cast<uint4*>(sgen + DtcSmem::OFF_Q)[i] = zero4;
         named_bar_sync(1, 128);
-    }
-    pdl_wait();
-    decode_header(p);
-    const int n = min(max(p.n_tokens[s], 0), p.max_pages * p.page_size);    // never past the sequence's table
-    const int ps = p.page_size;
-    const int ppt = 128 / ps;                                   // pages per tile (PAGES)
-    const int ntiles = (n + 127) >> 7;
-    const int per = (ntiles + p.nsplit - 1) / p.nsplit;         // contiguous tiles per split
-    const int t_begin = min(z * per, ntiles), t_end = min(t_begin + per, ntiles);
-    const int my_tiles = t_end - t_begin;
-
-    if (warp == 4) {
-        tmem_alloc(smem_u32(s_tmem), 32);
-        tmem_relinquish();
-    } else {
         // Q row h, 16-byte chunk c (8 elements) of box b: physical chunk c ^ (h % 8) of the 128-byte row
         for (int i = tid; i < G * 16; i += 128) {
             const int h = i >> 4, c16 = i & 15, b = c16 >> 3, c = c16 & 7;
