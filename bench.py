@@ -465,7 +465,7 @@ def run_dual(args):
                       "config": {"workload": w.name, "tokens": w.total_tokens, "Hq": w.Hq, "Hkv": w.Hkv, "head_dim": w.d,
                                  "student_pairs": pairs_s, "teacher_pairs": pairs_t,
                                  "flops": "4*d*Hq*(student pairs + teacher pairs): the shared q k^T is counted once per stream"},
-                      "roofline": {"kernel": "fwd_kernel x2 + dual_merge_kernel", "bound": "tensor", "achieved": tf, "peak": float(peaks["bf16_tflops"]),
+                      "roofline": {"kernel": "fwd_kernel x2", "bound": "tensor", "achieved": tf, "peak": float(peaks["bf16_tflops"]),
                                    "unit": "TFLOP/s", "frac": tf / float(peaks["bf16_tflops"]), "traffic": None},
                       "dtype": "bf16", "data": "synthetic"}), flush=True)
 
