@@ -230,7 +230,7 @@ ArenaLayout arena_layout(int batch, int total_tokens, int max_seqlen, int Hq, in
     A.slot_tokens = (int)st;
     const size_t nq = (size_t)st * G * head_dim * 2, nkv = (size_t)st * head_dim * 2;
     const size_t gq = (size_t)st * G * head_dim * gsz, gkv = (size_t)st * head_dim * gsz;
-    A.meta_stride = align_up(kvs_mask_meta_bytes(batch, A.slot_tokens, max_seqlen), 256);
+    A.meta_stride = align_up(meta_layout(batch, A.slot_tokens, max_seqlen).least, 256);
     A.ws_bytes = bwd_base_bytes(A.slot_tokens, G, head_dim, grad_dtype);
     size_t o = 0;
     A.evict = o; o = align_up(o + (size_t)total_tokens * 4, 256);
@@ -238,7 +238,7 @@ ArenaLayout arena_layout(int batch, int total_tokens, int max_seqlen, int Hq, in
     A.sticky = o; o += 256;
     A.meta = o;  o += (size_t)A.ranges * A.meta_stride;
     // metadata of the whole batch, for the plan of the backward, where the ranges are parts of it
-    const size_t all = A.ranges > 1 ? align_up(kvs_mask_meta_bytes(batch, total_tokens, max_seqlen), 256) : 0;
+    const size_t all = A.ranges > 1 ? align_up(meta_layout(batch, total_tokens, max_seqlen).least, 256) : 0;
     A.meta_all = o; o += all;
     A.cu_all = o;   o = align_up(o + (A.ranges > 1 ? (size_t)(batch + 1) * 4 : 0), 256);
     A.cut = o;      o += bwd_cut_bytes(total_tokens, Hq, head_dim);     // one for all chunks: their backwards follow one another

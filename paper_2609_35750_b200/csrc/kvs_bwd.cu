@@ -618,7 +618,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
                 w.n_iter = -1;
                 BwdUnit unit;
                 if (ok && bwd_unit_of(p, mv.bwd_order, n_items, x, unit, w.g)) {
-                    const int4 me = mv.info[unit.block];
+                    const int4 me = block_info(mv, unit.block);
                     const int G = p.Hq / p.Hkv;
                     w.n = me.z;
                     w.tok0 = me.x;

@@ -152,7 +152,7 @@ bwd_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     {
         BwdUnit unit;
         if (!bwd_unit_of(p, mv.pair_order, mv.hdr->npair_total, blockIdx.x >> 1, unit, w.g)) return;
-        const int4 me = mv.info[unit.block];
+        const int4 me = block_info(mv, unit.block);
         const int G = p.Hq / p.Hkv, n0 = me.z;
         w.n = n0 + (int)rank;                           // this CTA's key block; past the trace when its block count is odd
         w.tok0 = me.x;

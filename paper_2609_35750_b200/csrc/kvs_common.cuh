@@ -30,13 +30,14 @@ struct MetaHeader {
     uint32_t rows_done;    // CTAs of the classification that are done
     int32_t blk_most, pair_most;        // query blocks of the longest key block, of the longest pair
     uint32_t blk_tiles, pair_tiles;     // their sums over all key blocks, over all pairs
+    int32_t has_info;                   // there was room for the blocks' info
 };
 
 // Byte offsets of the arrays inside meta_buf; a pure function of the three sizes so that
 // every entry point can recompute it.
 struct MetaLayout {
-    size_t blk_off, cls_off, seq_start, blk_trace, info, kmin, kmax, fmin, fmax, col_first, col_last, row_cnt, fwd_order, bwd_order, pair_order, bwd_len, pair_len, evict,
-        kfirst, tile_class, row_list, total;
+    size_t blk_off, cls_off, seq_start, blk_trace, kmin, kmax, fmin, fmax, col_first, col_last, row_cnt, fwd_order, bwd_order, pair_order, bwd_len, pair_len, evict,
+        kfirst, tile_class, row_list, least, info, total;
     int nb_cap;            // capacity in blocks
     size_t cls_cap;        // capacity in tiles
 };
@@ -61,7 +62,6 @@ __host__ __device__ inline MetaLayout meta_layout(int batch, int total_tokens, i
     L.cls_off = o;   o = align_up(o + sizeof(uint32_t) * (batch + 1), 256);
     L.seq_start = o; o = align_up(o + sizeof(int32_t) * (batch + 1), 256);
     L.blk_trace = o; o = align_up(o + sizeof(int32_t) * nb_cap, 256);
-    L.info = o;      o = align_up(o + 4 * sizeof(int32_t) * nb_cap, 256);
     L.kmin = o;      o = align_up(o + sizeof(int32_t) * nb_cap, 256);
     L.kmax = o;      o = align_up(o + sizeof(int32_t) * nb_cap, 256);
     L.fmin = o;      o = align_up(o + sizeof(int32_t) * nb_cap, 256);
@@ -78,6 +78,8 @@ __host__ __device__ inline MetaLayout meta_layout(int batch, int total_tokens, i
     L.kfirst = o;    o = align_up(o + sizeof(int32_t) * (size_t)(total_tokens > 0 ? total_tokens : 1), 256);
     L.tile_class = o; o = align_up(o + L.cls_cap, 256);
     L.row_list = o;  o = align_up(o + sizeof(uint16_t) * L.cls_cap, 256);
+    L.least = o;           // without the blocks' info, which a buffer of this size does without
+    L.info = o;      o = align_up(o + 4 * sizeof(int32_t) * nb_cap, 256);
     L.total = o;
     return L;
 }
@@ -89,7 +91,7 @@ struct MetaView {
     const uint32_t* cls_off;    // [batch+1] first tile of each trace's class matrix
     const int32_t* seq_start;   // [batch+1] copy of cu_seqlens
     const int32_t* blk_trace;   // [nblk] trace of a global block
-    const int4* info;           // [nblk] first token and length of the block's trace, block of the trace, first tile of its row
+    const int4* info;           // [nblk] see block_info
     const int32_t* kmin;        // [nblk] min / max over the block's key slots of the eviction step
     const int32_t* kmax;        // [nblk]
     const int32_t* fmin;        // [nblk] min / max over the block's key slots of the first query that may see the slot
@@ -194,6 +196,14 @@ __device__ __forceinline__ void set_status(int32_t* status, int code) { atomicCA
 __device__ __forceinline__ bool meta_matches(const MetaHeader* hdr, int batch, int total_tokens, int max_seqlen) {
     return hdr->magic == META_MAGIC && hdr->batch == batch && hdr->total_tokens == total_tokens &&
            hdr->max_seqlen == max_seqlen;
+}
+
+// First token and length of a block's trace, block of the trace, first tile of its row: one load, or a chain of them where the
+// buffer has no room for the entries.
+__device__ __forceinline__ int4 block_info(const MetaView& mv, int blk) {
+    if (mv.hdr->has_info) return mv.info[blk];
+    const int b = mv.blk_trace[blk], n = blk - mv.blk_off[b], tok0 = mv.seq_start[b], T = mv.seq_start[b + 1] - tok0;
+    return make_int4(tok0, T, n, (int)(mv.cls_off[b] + (uint32_t)n * (uint32_t)((T + TILE - 1) / TILE)));
 }
 
 // Query blocks that see key block `even` or, where the trace has one, the block after it (none: last < first).

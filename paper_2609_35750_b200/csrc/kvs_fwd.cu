@@ -109,7 +109,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     auto item_of = [&](int x, int y) {
         FwdItem it;
         const int gb = mv.fwd_order[x];
-        const int4 me = mv.info[gb];
+        const int4 me = block_info(mv, gb);
         it.nlist = mv.row_cnt[gb];
         it.tok0 = me.x;
         it.T = me.y;

@@ -182,6 +182,7 @@ meta_blocks_kernel(const int32_t* __restrict__ evict_at, const int32_t* __restri
         hdr->general = (key_first || complement) ? 1 : 0;
         hdr->npair_total = 0;
         hdr->rows_done = 0;
+        hdr->has_info = info != nullptr;
     }
     const int4 mine = s_mine[warp];
     if (blk0 + warp >= nblk || s_trace[warp] < 0) return;
@@ -190,7 +191,7 @@ meta_blocks_kernel(const int32_t* __restrict__ evict_at, const int32_t* __restri
     const BlockStat st = meta_block_stat(evict_at, key_first, complement, n, tok0, T, evict_copy, first_copy);
     if (lane == 0) {
         blk_trace[blk] = s_trace[warp];
-        info[blk] = mine;
+        if (info) info[blk] = mine;
         kmin[blk] = st.mn;
         kmax[blk] = st.mx;
         fmin[blk] = st.fmn;
@@ -319,7 +320,7 @@ __device__ void meta_order(int what, MetaHeader* hdr, const int32_t* blk_off, co
 // ---- kernel 2: one warp per query block row: classes and the compact non-empty list; the orders ----------------------
 // The first two CTAs sort the key blocks and the pairs, the others classify, and the last of those to finish sorts the rows.
 __global__ void __launch_bounds__(META_THREADS)
-meta_classify_kernel(MetaHeader* hdr, const int32_t* __restrict__ blk_off, const int32_t* __restrict__ blk_trace, const int4* __restrict__ info,
+meta_classify_kernel(MetaHeader* hdr, MetaView mv, const int32_t* __restrict__ blk_off, const int32_t* __restrict__ blk_trace,
                      const int32_t* __restrict__ kmin, const int32_t* __restrict__ kmax,
                      const int32_t* __restrict__ fmin, const int32_t* __restrict__ fmax, const int32_t* __restrict__ col_first,
                      const int32_t* __restrict__ col_last, uint8_t* tile_class, uint16_t* row_list, int32_t* row_cnt, int32_t* fwd_order,
@@ -335,7 +336,7 @@ meta_classify_kernel(MetaHeader* hdr, const int32_t* __restrict__ blk_off, const
     const int row = (blockIdx.x - 2) * META_WARPS + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (row < hdr->nblk_total) {
-        const int4 me = info[row];
+        const int4 me = block_info(mv, row);
         const int base = row - me.z;
         const size_t at = (uint32_t)me.w;
         const int count = meta_classify_row(me.z, me.y, kmin + base, kmax + base, fmin + base, fmax + base, tile_class + at, row_list + at);
@@ -360,7 +361,7 @@ meta_classify_kernel(MetaHeader* hdr, const int32_t* __restrict__ blk_off, const
 constexpr int META_SMALL = 64, META_SMALL_BATCH = 1024, META_SMALL_THREADS = 1024;
 __global__ void __launch_bounds__(META_SMALL_THREADS)
 meta_small_kernel(const int32_t* __restrict__ evict_at, const int32_t* __restrict__ key_first, int complement,
-                  const int32_t* __restrict__ cu_seqlens, int batch, int total_tokens, int max_seqlen, MetaView v, int nb_cap,
+                  const int32_t* __restrict__ cu_seqlens, int batch, int total_tokens, int max_seqlen, MetaView v, int has_info, int nb_cap,
                   unsigned long long cls_cap) {
     // per block: trace, block of the trace, first token and length of the trace, first tile of the row
     __shared__ int s_trace[META_SMALL], s_n[META_SMALL], s_tok0[META_SMALL], s_T[META_SMALL], s_at[META_SMALL];
@@ -427,7 +428,7 @@ meta_small_kernel(const int32_t* __restrict__ evict_at, const int32_t* __restric
         const BlockStat st = meta_block_stat(evict_at, key_first, complement, s_n[i], s_tok0[i], s_T[i], (int32_t*)v.evict, (int32_t*)v.kfirst);
         if (lane == 0) {
             ((int32_t*)v.blk_trace)[i] = s_trace[i];
-            ((int4*)v.info)[i] = make_int4(s_tok0[i], s_T[i], s_n[i], s_at[i]);
+            if (has_info) ((int4*)v.info)[i] = make_int4(s_tok0[i], s_T[i], s_n[i], s_at[i]);
             ((int32_t*)v.kmin)[i] = s_kmin[i] = st.mn;
             ((int32_t*)v.kmax)[i] = s_kmax[i] = st.mx;
             ((int32_t*)v.fmin)[i] = s_fmin[i] = st.fmn;
@@ -495,6 +496,7 @@ meta_small_kernel(const int32_t* __restrict__ evict_at, const int32_t* __restric
         h.general = (key_first || complement) ? 1 : 0;
         h.npair_total = items[ORDER_PAIRS];
         h.rows_done = 0;
+        h.has_info = has_info;
         h.blk_most = most[ORDER_COLS];
         h.pair_most = most[ORDER_PAIRS];
         h.blk_tiles = sum[ORDER_COLS];
@@ -553,20 +555,21 @@ int launch_mask_meta(const int32_t* key_evict, const int32_t* key_first, int com
     if ((long long)((max_seqlen + TILE - 1) / TILE) > 65535) return KVS_ERR_UNSUPPORTED;
     const MetaLayout L = meta_layout(batch, total_tokens, max_seqlen);
     if (L.cls_cap > 0xFFFFFFF0ull) return KVS_ERR_UNSUPPORTED;
-    if (meta_bytes < L.total) return KVS_ERR_WORKSPACE;
+    if (meta_bytes < L.least) return KVS_ERR_WORKSPACE;
+    const int has_info = meta_bytes >= L.total;
     cudaStream_t st = (cudaStream_t)stream;
     MetaView v = meta_view(meta_buf, L);
     if (L.nb_cap <= META_SMALL && batch <= META_SMALL_BATCH)
         return launch_after(meta_small_kernel, 1, META_SMALL_THREADS, 0, st, key_evict, key_first, complement, cu_seqlens, batch, total_tokens,
-                            max_seqlen, v, L.nb_cap, (unsigned long long)L.cls_cap);
+                            max_seqlen, v, has_info, L.nb_cap, (unsigned long long)L.cls_cap);
     const int grid = (L.nb_cap + META_WARPS - 1) / META_WARPS;
     const int rc = launch_after(meta_blocks_kernel, grid, META_THREADS, 0, st, key_evict, key_first, complement, cu_seqlens, batch, total_tokens,
                                 max_seqlen, v.hdr, (int32_t*)v.blk_off, (uint32_t*)v.cls_off, (int32_t*)v.seq_start, (int32_t*)v.blk_trace,
-                                (int4*)v.info, L.nb_cap, (unsigned long long)L.cls_cap, (int32_t*)v.kmin, (int32_t*)v.kmax, (int32_t*)v.fmin,
+                                has_info ? (int4*)v.info : nullptr, L.nb_cap, (unsigned long long)L.cls_cap, (int32_t*)v.kmin, (int32_t*)v.kmax, (int32_t*)v.fmin,
                                 (int32_t*)v.fmax, (int32_t*)v.col_first, (int32_t*)v.col_last, (int32_t*)v.row_cnt, (int32_t*)v.evict,
                                 (int32_t*)v.kfirst);
     if (rc != KVS_OK) return rc;
-    return launch_after(meta_classify_kernel, grid + 2, META_THREADS, 0, st, v.hdr, v.blk_off, v.blk_trace, v.info, v.kmin,
+    return launch_after(meta_classify_kernel, grid + 2, META_THREADS, 0, st, v.hdr, v, v.blk_off, v.blk_trace, v.kmin,
                         v.kmax, v.fmin, v.fmax, v.col_first, v.col_last, (uint8_t*)v.tile_class, (uint16_t*)v.row_list, (int32_t*)v.row_cnt,
                         (int32_t*)v.fwd_order, (int32_t*)v.bwd_order, (int32_t*)v.pair_order, (int32_t*)v.bwd_len, (int32_t*)v.pair_len);
 }

@@ -119,3 +119,23 @@ def test_units_listed_by_trace_equal_whole_items(lens, Hq, Hkv, d, rule):
     out, lse, ref = _backward(x, lens, True)
     _, _, got = _backward(x, lens, False, out, lse)
     _same(got, ref, max(lens), Hq // Hkv)
+
+
+@pytest.mark.parametrize("lens", [[1000, 1, 300], [300] * 40])
+def test_a_buffer_without_room_for_the_entries_of_the_blocks(lens):
+    # 16 bytes a block less, each array in whole 256 bytes: the same results by the tables of the traces; one byte less is refused
+    Hq, Hkv, d, total = 2, 1, 64, sum(lens)
+    ev, cu, q, k, v, do = _inputs(lens, Hq, Hkv, d, "turns")
+    blocks = min(len(lens) * -(-max(lens) // 128), total // 128 + len(lens))
+    least = B.kvs_mask_meta_bytes(len(lens), total, max(lens)) - -(-16 * blocks // 256) * 256
+    small = B.kvs_mask_meta(ev, cu, max(lens), torch.empty(least, dtype=torch.uint8, device="cuda"))
+    full = B.kvs_mask_meta(ev, cu, max(lens))
+    got = []
+    for meta in (small, full):
+        out, lse = B.kvs_attn_fwd(q, k, v, meta, len(lens), max(lens))
+        ws = torch.empty(-(-(256 + 4 * total * Hq) // 256) * 256, dtype=torch.uint8, device="cuda")
+        got.append((out, lse) + B.kvs_attn_bwd(do, q, k, v, out, lse, meta, len(lens), max(lens), 0.0, B.GRAD_FP32, workspace=ws))
+        assert B.kvs_device_status(meta) == B.KVS_OK
+    assert all(torch.equal(a, b) for i, (a, b) in enumerate(zip(*got)) if i != 2)           # dq is added in the order of arrival
+    with pytest.raises(B.KvsError):
+        B.kvs_mask_meta(ev, cu, max(lens), torch.empty(least - 1, dtype=torch.uint8, device="cuda"))
