@@ -22,7 +22,7 @@ constexpr int BWD_SMS = 148;
 constexpr long long BWD_L2_BYTES = 96ll << 20;
 constexpr int BWD_MANY_TRACES = 8, BWD_MOST_LATE = 6;
 constexpr uint32_t BWD_LATE = 3;              // tiles left of a unit when the CTA asks for the next one
-constexpr int BWD_MIN_UNIT = 4;             // tiles: a shorter unit is mostly its own start and end
+constexpr int BWD_MIN_UNIT = 2;             // tiles (4: main kernel of 1 x 1024 tokens, 4 heads, head_dim 64 22.1 -> 19.1 us with 2)
 constexpr int BWD_MAX_SLOTS = 2 * BWD_SMS;  // slots of one CTA each for the dK and dV of cut items, over all KV heads
 
 struct BwdWsLayout {
@@ -81,7 +81,8 @@ struct BwdPlanArgs {
 // 472 -> 454 us); and up to three waves take that many average units.
 // Main kernel, whole items -> cut, us: 1 trace of 1000 tokens with 16 heads on 2 154 -> 42; 4000 with 32 on 8 355 -> 180; 16000,
 // head_dim 64 1199 -> 748; 20 of 100 to 2000, head_dim 64 229 -> 161; 32768 with 28 on 4 (pairs) 5500 -> 4400.  Where nothing is
-// cut, the list and the registers of the slots cost 1 % at head_dim 64 and 9 % at 128 (96 of 60 to 900: 316 -> 319, 447 -> 494).
+// cut, the list and the registers of the slots cost 1 % at head_dim 64 and 9 % at 128 (96 of 60 to 900: 316 -> 319, 447 -> 494;
+// before units were chained).
 constexpr float BWD_UNIT_COST = 4.f, BWD_CUT_COST = 3.f;
 __device__ void bwd_plan(const BwdPlanArgs& a) {
     constexpr int NC = 8;
