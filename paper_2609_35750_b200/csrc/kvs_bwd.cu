@@ -15,7 +15,7 @@ namespace kvs {
 constexpr int BWD_SMS = 148;
 // A batch whose Q, dO and fp32 dQ are larger than this is listed by trace (see bwd_plan): sorted by length throughout, a trace's
 // key blocks run far apart and its tiles come from memory again for each (96 traces of 60 to 900 tokens, 16 heads on 2: 2.7 GB
-// moved at 5.7 TB/s, 1.5 GB by trace).  Main kernel, by length -> by trace, us, 32 heads on 8: 200 traces of 300 tokens 1219 ->
+// moved at 5.7 TB/s, 1.9 GB by trace).  Main kernel, by length -> by trace, us, 32 heads on 8: 200 traces of 300 tokens 1219 ->
 // 977, 96 of 60 to 900 (16 on 2) 480 -> 434, 60 of 100 to 2000 (28 on 4) 1409 -> 1302, 12 of 1500 to 12000 5216 -> 5126, 8 of
 // 8000 4771 -> 4712, 9 of 14000 with nothing evicted (16 on 2) 18.1 -> 17.6 ms.  Of fewer traces than eight an eighth is not to
 // be had for the end (3 of 14000: 11.5 -> 11.8 ms; 4 of 20000 without groups 6.9 -> 7.0 ms).
@@ -803,113 +803,113 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         float pv[64];
         uint32_t J = 0;                                         // tiles of the CTA so far
         for (int r = 0; take(r); ++r) {
-        const volatile BwdWork* work = s_work + (r & 1);
-        const uint32_t end = J + work->n_iter;
-        if (J == end) {                                         // a key block that no query sees: its gradients are zero
-            bwd_zero_rows<D>(p, work->tok0 + work->n * TILE, min(TILE, work->T - work->n * TILE), work->g, 256);
-            done(r);
-            continue;
-        }
-        // queries [my_first, my_end) of the trace see this key; nobody sees a slot past the trace
-        int my_end = 0, my_first = work->n * TILE + row;
-        if (my_first < work->T) {
-            const int at = work->tok0 + my_first;
-            my_end = min(mv.evict[at], work->T);
-            if (work->general) my_first = mv.kfirst[at];
-        }
-        int m = work->m_start;                             // query block of the tile of the next phase_p
-
-        auto phase_p = [&](uint32_t j) {        // P^T(j) = exp2(S^T * c - lse), masked
-            const int s = j & 1;
-            const int lo = my_first - (m * TILE + col0), hi = my_end - (m * TILE + col0);     // columns [lo, hi) see the key
-            m = (m == work->m_last) ? work->m_first : m + 1;       // read again, not kept: registers are short here
-            mbar_wait(bar_ldfull(s), (j >> 1) & 1, abort_flag, status);
-            mbar_wait(bar_s, j & 1, abort_flag, status);
-            tc_fence_after();
-            const float4* l4 = reinterpret_cast<const float4*>(sLse + s * TILE + col0);
-            uint32_t r0[32], r1[32];
-            tmem_ld32(tmem_S + lane_sel + col0, r0);
-            tmem_ld32(tmem_S + lane_sel + col0 + 32, r1);
-            tmem_wait_ld();
-            const float2 c2 = make_float2(p.scale_log2, p.scale_log2);
-#pragma unroll
-            for (int e4 = 0; e4 < 16; ++e4) {          // packed fp32x2 multiply-adds, then one ex2 per element
-                const float4 l = l4[e4];
-                const uint32_t* r = (e4 < 8) ? &r0[e4 * 4] : &r1[(e4 - 8) * 4];
-                const float2 x01 = __ffma2_rn(make_float2(__uint_as_float(r[0]), __uint_as_float(r[1])), c2, make_float2(l.x, l.y));
-                const float2 x23 = __ffma2_rn(make_float2(__uint_as_float(r[2]), __uint_as_float(r[3])), c2, make_float2(l.z, l.w));
-                pv[e4 * 4 + 0] = fast_exp2(x01.x);
-                pv[e4 * 4 + 1] = fast_exp2(x01.y);
-                pv[e4 * 4 + 2] = fast_exp2(x23.x);
-                pv[e4 * 4 + 3] = fast_exp2(x23.y);
+            const volatile BwdWork* work = s_work + (r & 1);
+            const uint32_t end = J + work->n_iter;
+            if (J == end) {                                         // a key block that no query sees: its gradients are zero
+                bwd_zero_rows<D>(p, work->tok0 + work->n * TILE, min(TILE, work->T - work->n * TILE), work->g, 256);
+                done(r);
+                continue;
             }
-            // Only the warps that hold a hidden pair pay for the mask, whatever the class of the tile (a loop of at most one
-            // pass: as an if, its 64 selects are predicated and issued for every tile)
-            const int masked = __any_sync(0xffffffffu, lo > 0 || hi < 64) ? 1 : 0;
+            // queries [my_first, my_end) of the trace see this key; nobody sees a slot past the trace
+            int my_end = 0, my_first = work->n * TILE + row;
+            if (my_first < work->T) {
+                const int at = work->tok0 + my_first;
+                my_end = min(mv.evict[at], work->T);
+                if (work->general) my_first = mv.kfirst[at];
+            }
+            int m = work->m_start;                             // query block of the tile of the next phase_p
+
+            auto phase_p = [&](uint32_t j) {        // P^T(j) = exp2(S^T * c - lse), masked
+                const int s = j & 1;
+                const int lo = my_first - (m * TILE + col0), hi = my_end - (m * TILE + col0);     // columns [lo, hi) see the key
+                m = (m == work->m_last) ? work->m_first : m + 1;       // read again, not kept: registers are short here
+                mbar_wait(bar_ldfull(s), (j >> 1) & 1, abort_flag, status);
+                mbar_wait(bar_s, j & 1, abort_flag, status);
+                tc_fence_after();
+                const float4* l4 = reinterpret_cast<const float4*>(sLse + s * TILE + col0);
+                uint32_t r0[32], r1[32];
+                tmem_ld32(tmem_S + lane_sel + col0, r0);
+                tmem_ld32(tmem_S + lane_sel + col0 + 32, r1);
+                tmem_wait_ld();
+                const float2 c2 = make_float2(p.scale_log2, p.scale_log2);
+#pragma unroll
+                for (int e4 = 0; e4 < 16; ++e4) {          // packed fp32x2 multiply-adds, then one ex2 per element
+                    const float4 l = l4[e4];
+                    const uint32_t* r = (e4 < 8) ? &r0[e4 * 4] : &r1[(e4 - 8) * 4];
+                    const float2 x01 = __ffma2_rn(make_float2(__uint_as_float(r[0]), __uint_as_float(r[1])), c2, make_float2(l.x, l.y));
+                    const float2 x23 = __ffma2_rn(make_float2(__uint_as_float(r[2]), __uint_as_float(r[3])), c2, make_float2(l.z, l.w));
+                    pv[e4 * 4 + 0] = fast_exp2(x01.x);
+                    pv[e4 * 4 + 1] = fast_exp2(x01.y);
+                    pv[e4 * 4 + 2] = fast_exp2(x23.x);
+                    pv[e4 * 4 + 3] = fast_exp2(x23.y);
+                }
+                // Only the warps that hold a hidden pair pay for the mask, whatever the class of the tile (a loop of at most one
+                // pass: as an if, its 64 selects are predicated and issued for every tile)
+                const int masked = __any_sync(0xffffffffu, lo > 0 || hi < 64) ? 1 : 0;
 #pragma unroll 1
-            for (int pass = 0; pass < masked; ++pass) {
-                const uint32_t seen0 = bit_range(lo, hi), seen1 = bit_range(lo - 32, hi - 32);
+                for (int pass = 0; pass < masked; ++pass) {
+                    const uint32_t seen0 = bit_range(lo, hi), seen1 = bit_range(lo - 32, hi - 32);
 #pragma unroll
-                for (int e = 0; e < 64; ++e) pv[e] = ((e < 32 ? seen0 : seen1) >> (e & 31) & 1u) ? pv[e] : 0.f;
-            }
-            uint32_t pk[32];
+                    for (int e = 0; e < 64; ++e) pv[e] = ((e < 32 ? seen0 : seen1) >> (e & 31) & 1u) ? pv[e] : 0.f;
+                }
+                uint32_t pk[32];
 #pragma unroll
-            for (int e = 0; e < 32; ++e) pk[e] = pack_bf16(pv[2 * e], pv[2 * e + 1]);
-            tmem_st32(tmem_S + lane_sel + col0, pk);       // 64 queries -> 32 packed columns at [col0, col0+32)
-            tmem_wait_st();
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar_p);
-        };
+                for (int e = 0; e < 32; ++e) pk[e] = pack_bf16(pv[2 * e], pv[2 * e + 1]);
+                tmem_st32(tmem_S + lane_sel + col0, pk);       // 64 queries -> 32 packed columns at [col0, col0+32)
+                tmem_wait_st();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar_p);
+            };
 
-        auto phase_ds = [&](uint32_t j) {       // dS^T(j) = P^T (scale dP^T - scale D)
-            const int s = j & 1;
-            mbar_wait(bar_dp, j & 1, abort_flag, status);
+            auto phase_ds = [&](uint32_t j) {       // dS^T(j) = P^T (scale dP^T - scale D)
+                const int s = j & 1;
+                mbar_wait(bar_dp, j & 1, abort_flag, status);
+                tc_fence_after();
+                const float4* d4 = reinterpret_cast<const float4*>(sDv + s * TILE + col0);
+                uint32_t r0[32], r1[32];
+                tmem_ld32(tmem_P + lane_sel + col0, r0);
+                tmem_ld32(tmem_P + lane_sel + col0 + 32, r1);
+                tmem_wait_ld();
+                uint32_t dk_[32];
+                const float2 sc2 = make_float2(p.scale, p.scale);
+#pragma unroll
+                for (int e4 = 0; e4 < 16; ++e4) {          // dS = P * (scale dP - scale D), two elements per instruction
+                    const float4 dd = d4[e4];
+                    const uint32_t* r = (e4 < 8) ? &r0[e4 * 4] : &r1[(e4 - 8) * 4];
+                    const float2 t01 = __ffma2_rn(make_float2(__uint_as_float(r[0]), __uint_as_float(r[1])), sc2, make_float2(dd.x, dd.y));
+                    const float2 t23 = __ffma2_rn(make_float2(__uint_as_float(r[2]), __uint_as_float(r[3])), sc2, make_float2(dd.z, dd.w));
+                    const float2 d01 = __fmul2_rn(make_float2(pv[e4 * 4 + 0], pv[e4 * 4 + 1]), t01);
+                    const float2 d23 = __fmul2_rn(make_float2(pv[e4 * 4 + 2], pv[e4 * 4 + 3]), t23);
+                    dk_[e4 * 2 + 0] = pack_bf16(d01.x, d01.y);
+                    dk_[e4 * 2 + 1] = pack_bf16(d23.x, d23.y);
+                }
+                // dS^T row -> shared memory, MN-major (queries contiguous), 128-byte swizzle: the 64 queries of
+                // this half are the 128-byte row `row` of block `half`; 16-byte chunk c sits at (c ^ (row % 8))
+#pragma unroll
+                for (int c = 0; c < 8; ++c)
+                    *reinterpret_cast<uint4*>(sDS_row + ((c ^ (row & 7)) << 4)) =
+                        make_uint4(dk_[c * 4], dk_[c * 4 + 1], dk_[c * 4 + 2], dk_[c * 4 + 3]);
+                fence_proxy_async();                     // dS visible to the tensor core's reads of shared memory
+                tc_fence_before();                       // orders this thread's reads of dP^T before the dQ MMA that overwrites it
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar_dss);
+            };
+
+            phase_p(J);
+            for (; J < end; ++J) {
+                phase_ds(J);
+                if (J + 1 < end) phase_p(J + 1);
+            }
+
+            // ---- epilogue: dK, dV of this key block, once every MMA has completed ----
+            mbar_wait(bar_qfree((end - 1) & 1), ((end - 1) >> 1) & 1, abort_flag, status);
             tc_fence_after();
-            const float4* d4 = reinterpret_cast<const float4*>(sDv + s * TILE + col0);
-            uint32_t r0[32], r1[32];
-            tmem_ld32(tmem_P + lane_sel + col0, r0);
-            tmem_ld32(tmem_P + lane_sel + col0 + 32, r1);
-            tmem_wait_ld();
-            uint32_t dk_[32];
-            const float2 sc2 = make_float2(p.scale, p.scale);
-#pragma unroll
-            for (int e4 = 0; e4 < 16; ++e4) {          // dS = P * (scale dP - scale D), two elements per instruction
-                const float4 dd = d4[e4];
-                const uint32_t* r = (e4 < 8) ? &r0[e4 * 4] : &r1[(e4 - 8) * 4];
-                const float2 t01 = __ffma2_rn(make_float2(__uint_as_float(r[0]), __uint_as_float(r[1])), sc2, make_float2(dd.x, dd.y));
-                const float2 t23 = __ffma2_rn(make_float2(__uint_as_float(r[2]), __uint_as_float(r[3])), sc2, make_float2(dd.z, dd.w));
-                const float2 d01 = __fmul2_rn(make_float2(pv[e4 * 4 + 0], pv[e4 * 4 + 1]), t01);
-                const float2 d23 = __fmul2_rn(make_float2(pv[e4 * 4 + 2], pv[e4 * 4 + 3]), t23);
-                dk_[e4 * 2 + 0] = pack_bf16(d01.x, d01.y);
-                dk_[e4 * 2 + 1] = pack_bf16(d23.x, d23.y);
-            }
-            // dS^T row -> shared memory, MN-major (queries contiguous), 128-byte swizzle: the 64 queries of
-            // this half are the 128-byte row `row` of block `half`; 16-byte chunk c sits at (c ^ (row % 8))
-#pragma unroll
-            for (int c = 0; c < 8; ++c)
-                *reinterpret_cast<uint4*>(sDS_row + ((c ^ (row & 7)) << 4)) =
-                    make_uint4(dk_[c * 4], dk_[c * 4 + 1], dk_[c * 4 + 2], dk_[c * 4 + 3]);
-            fence_proxy_async();                     // dS visible to the tensor core's reads of shared memory
-            tc_fence_before();                       // orders this thread's reads of dP^T before the dQ MMA that overwrites it
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar_dss);
-        };
-
-        phase_p(J);
-        for (; J < end; ++J) {
-            phase_ds(J);
-            if (J + 1 < end) phase_p(J + 1);
-        }
-
-        // ---- epilogue: dK, dV of this key block, once every MMA has completed ----
-        mbar_wait(bar_qfree((end - 1) & 1), ((end - 1) >> 1) & 1, abort_flag, status);
-        tc_fence_after();
-        // through the memory of dS, which nothing reads any more; the next unit's tiles are on their way into the others
-        bwd_epilogue<D>(p, work->cut, work->g, 1, 0, tmem_dK + lane_sel + half * HALF_D, tmem_dV + lane_sel + half * HALF_D, row, half,
-                        work->tok0 + work->n * TILE + quad * 32, work->T - work->n * TILE - quad * 32, sgen + L::OFF_DS + warp * 4096,
-                        reinterpret_cast<volatile int*>(sgen + L::OFF_MISC + 8));
-        done(r);
+            // through the memory of dS, which nothing reads any more; the next unit's tiles are on their way into the others
+            bwd_epilogue<D>(p, work->cut, work->g, 1, 0, tmem_dK + lane_sel + half * HALF_D, tmem_dV + lane_sel + half * HALF_D, row, half,
+                            work->tok0 + work->n * TILE + quad * 32, work->T - work->n * TILE - quad * 32, sgen + L::OFF_DS + warp * 4096,
+                            reinterpret_cast<volatile int*>(sgen + L::OFF_MISC + 8));
+            done(r);
         }
     }
     tc_fence_before();

@@ -1,6 +1,6 @@
 """Metadata of small batches by one CTA, units and items that are chained in a CTA (needs a B200).
 
-Up to 64 blocks the metadata is one kernel, above it is two: a batch at the line gives the same results, bit for bit, as the same
+Up to 64 blocks and 5120 tokens the metadata is one kernel, above it is two: a batch at the line gives the same results, bit for bit, as the same
 traces with one-token traces behind them.  Rows and whole key blocks (a workspace of the base size) are summed in the same order
 on both sides, so out, lse, dk and dv are equal; dq is added in the order of arrival, fp32, each term at most 2^-24 off."""
 import numpy as np
@@ -28,7 +28,7 @@ def _pass(ev, cu, longest, ts, Hq, general=None):
     return (out, lse) + grads, cls
 
 
-@pytest.mark.parametrize("lens", [[8192], [8065], [1], [128] * 64, [127, 0, 129, 0, 0, 385, 1], [2048, 2049, 1, 3000], [1] * 62 + [129]])
+@pytest.mark.parametrize("lens", [[5120], [5121], [4993], [1], [80] * 64, [80] * 63 + [81], [127, 0, 129, 0, 0, 385, 1], [1024, 1025, 1, 3000], [1] * 62 + [129]])
 def test_one_cta_equals_two_kernels(lens):
     Hq, Hkv, d = 2, 1, 64
     r = np.random.default_rng(len(lens))
