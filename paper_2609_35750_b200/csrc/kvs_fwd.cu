@@ -678,7 +678,8 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
                 float inv = (run_sum > 0.f && nlist > 0) ? 1.f / run_sum : 0.f;
                 float lse = ref_max * 0.6931471805599453f + logf(run_sum), w_first = 0.f;
                 if (MERGE) {
-                    const float other = valid ? p.first_lse[(size_t)h * p.total_tokens + tok0 + qi] : -INFINITY, mine = inv > 0.f ? lse : -INFINITY;
+                    // this part's is -inf where it saw no key and NaN where a score was one, and stays so
+                    const float other = valid ? p.first_lse[(size_t)h * p.total_tokens + tok0 + qi] : -INFINITY, mine = lse;
                     const float top = fmaxf(other, mine);
                     lse = -INFINITY;
                     if (top > -INFINITY) {

@@ -152,3 +152,27 @@ def test_dual_forward_growing_logits():
     q[:, :, 0] = 1.0
     k[:, :, 0] = (torch.arange(T, dtype=torch.float32) * 0.08).to(torch.bfloat16)[:, None]     # the maximum moves in every block
     _check_dual(w, (q, k, v, do))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("lens,Hq,Hkv,d", [([700], 4, 2, 128), ([700, 130], 3, 1, 64), ([700] + [300] * 80, 8, 2, 128)])     # the last: chained rows
+@pytest.mark.parametrize("what", [float("nan"), float("inf")])
+def test_a_nan_or_infinity_in_an_evicted_key_reaches_the_teacher(lens, Hq, Hkv, d, what):
+    # Key 40 of the first trace leaves at 200 and has a NaN or an infinity in one column.  Of the rows after that, a row whose
+    # score with it is NaN or +inf has no finite result in either of the teacher's outputs; a score of -inf is a key with weight 0.
+    from paper_2609_35750_b200 import binding as B
+    ev = np.full(sum(lens), int(W.INF), dtype=np.int32)
+    ev[:100] = 200
+    g = torch.Generator(device="cuda").manual_seed(11)
+    q, k, v = (torch.randn((sum(lens), h, d), generator=g, device="cuda", dtype=torch.bfloat16) for h in (Hq, Hkv, Hkv))
+    k[40, 0, 0] = what
+    evd, cu = torch.from_numpy(ev).cuda(), torch.from_numpy(np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)).cuda()
+    ms, me = B.kvs_mask_meta(evd, cu, max(lens)), B.kvs_mask_meta_evicted(evd, cu, max(lens))
+    os_, ls, ot, lt = B.kvs_attn_fwd_dual(q, k, v, ms, me, len(lens), max(lens))
+    heads = torch.arange(Hq, device="cuda") < Hq // Hkv                               # of the KV head with that key
+    bad = torch.zeros((Hq, sum(lens)), dtype=torch.bool, device="cuda")
+    bad[:, 200:lens[0]] = heads[:, None] & (q[200:lens[0], :, 0].T >= 0 if what > 0 else heads[:, None])
+    after = slice(200, None)
+    assert torch.equal(~torch.isfinite(lt[:, after]), bad[:, after])
+    assert torch.equal(~torch.isfinite(ot[after]).all(2).T, bad[:, after])
+    assert torch.isfinite(os_[after]).all() and torch.isfinite(ls[:, after]).all()    # the student no longer sees the key
