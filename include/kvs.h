@@ -219,7 +219,8 @@ int kvs_rope_qk(const void* q, const void* k, const int32_t* positions, const in
 
 /* Bytes of the backward workspace: row sums, fp32 dQ accumulator, status, and the plan and partial sums with which key blocks
  * with long walks are shared out among CTAs (37 MiB at most).  A workspace without room for the last part is accepted;
- * every key block is then one CTA's. */
+ * every key block is then one CTA's.  So is one with room for half of its slots or more, where a batch is so small that it
+ * has fewer than 37 MiB: the shortest share is then four tiles and not two. */
 size_t kvs_attn_bwd_workspace_bytes(int total_tokens, int Hq, int Hkv, int head_dim, int grad_dtype);
 
 /*
@@ -319,7 +320,8 @@ int kvs_host_chunk_plan(const int32_t* cu_seqlens_host, int batch, int total_tok
  * evict_at, cu_seqlens, q, k, v, dout to the device arena, runs mask metadata, forward and
  * backward, copies out, lse, dq, dk, dv back, and SYNCHRONISES the stream.  Host buffers
  * should be page-locked for the copies to be asynchronous.  arena: device memory the caller
- * provides, >= kvs_host_arena_bytes(...), 256-byte aligned.  Returns the device status.
+ * provides, >= kvs_host_arena_bytes(...), 256-byte aligned (less is accepted where the room for the backward's slots can
+ * be less, see kvs_attn_bwd_workspace_bytes).  Returns the device status.
  * The work is pipelined over chunks of (a contiguous range of traces, one KV-head group), which are
  * independent: while one chunk's forward and backward run, the next chunk's inputs are uploaded and
  * the previous chunk's results downloaded, on two internal streams that (with their events) are

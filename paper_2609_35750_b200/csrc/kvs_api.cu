@@ -216,7 +216,8 @@ struct ArenaLayout {
     size_t meta_stride, ws_bytes;
     int slots, ranges, slot_tokens;
 };
-ArenaLayout arena_layout(int batch, int total_tokens, int max_seqlen, int Hq, int Hkv, int head_dim, int grad_dtype) {
+// cut_less: an arena with less room for the slots of the backward (bwd_cut_bytes), which is accepted too
+ArenaLayout arena_layout(int batch, int total_tokens, int max_seqlen, int Hq, int Hkv, int head_dim, int grad_dtype, bool cut_less = false) {
     ArenaLayout A;
     const int G = Hq / Hkv;
     const size_t gsz = grad_dtype == KVS_GRAD_FP32 ? 4 : 2;
@@ -241,7 +242,7 @@ ArenaLayout arena_layout(int batch, int total_tokens, int max_seqlen, int Hq, in
     const size_t all = A.ranges > 1 ? align_up(meta_layout(batch, total_tokens, max_seqlen).least, 256) : 0;
     A.meta_all = o; o += all;
     A.cu_all = o;   o = align_up(o + (A.ranges > 1 ? (size_t)(batch + 1) * 4 : 0), 256);
-    A.cut = o;      o += bwd_cut_bytes(total_tokens, Hq, head_dim);     // one for all chunks: their backwards follow one another
+    A.cut = o;      o += bwd_cut_bytes(total_tokens, Hq, head_dim, cut_less);     // one for all chunks: their backwards follow one another
     A.slot0 = o;
     size_t t = 0;
     A.q = t;     t = align_up(t + nq, 256);
@@ -310,7 +311,9 @@ extern "C" int kvs_attn_fwd_bwd_host(const int32_t* evict_at_host, const int32_t
         const long long T = (long long)cu_seqlens_host[b + 1] - cu_seqlens_host[b];
         if (T < 0 || T > max_seqlen) return KVS_ERR_INVALID_ARG;
     }
-    const ArenaLayout A = arena_layout(batch, total_tokens, max_seqlen, Hq, Hkv, head_dim, grad_dtype);
+    ArenaLayout A = arena_layout(batch, total_tokens, max_seqlen, Hq, Hkv, head_dim, grad_dtype);
+    const bool cut_less = arena_bytes < A.total;
+    if (cut_less) A = arena_layout(batch, total_tokens, max_seqlen, Hq, Hkv, head_dim, grad_dtype, true);
     if (arena_bytes < A.total) return KVS_ERR_WORKSPACE;
     cudaStream_t st = (cudaStream_t)stream;
     char* a = (char*)arena;
@@ -356,7 +359,7 @@ extern "C" int kvs_attn_fwd_bwd_host(const int32_t* evict_at_host, const int32_t
                            meta, A.meta_stride, stream);
         if (rc != KVS_OK) return rc;
     }
-    BwdWhole whole = {a + A.meta, batch, total_tokens, max_seqlen, Hkv, a + A.cut};
+    BwdWhole whole = {a + A.meta, batch, total_tokens, max_seqlen, Hkv, a + A.cut, cut_less};
     if (A.ranges > 1) {
         whole.meta_buf = a + A.meta_all;
         KVS_CK(cudaMemcpyAsync(a + A.cu_all, cu_seqlens_host, (size_t)(batch + 1) * 4, cudaMemcpyHostToDevice, st));

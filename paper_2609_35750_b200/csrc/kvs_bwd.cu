@@ -22,7 +22,9 @@ constexpr int BWD_SMS = 148;
 constexpr long long BWD_L2_BYTES = 96ll << 20;
 constexpr int BWD_MANY_TRACES = 8, BWD_MOST_LATE = 6;
 constexpr uint32_t BWD_LATE = 3;              // tiles left of a unit when the CTA asks for the next one
-constexpr int BWD_MIN_UNIT = 2;             // tiles (4: main kernel of 1 x 1024 tokens, 4 heads, head_dim 64 22.1 -> 19.1 us with 2)
+// Tiles of the shortest unit (4 -> 2: main kernel of 1 x 1024 tokens, 4 heads, head_dim 64 22.1 -> 19.1 us).  The shorter it is, the
+// more slots a small batch asks for; a buffer that was sized for units of four is accepted and keeps to them.
+constexpr int BWD_MIN_UNIT = 2, BWD_MIN_UNIT_LESS = 4;
 constexpr int BWD_MAX_SLOTS = 2 * BWD_SMS;  // slots of one CTA each for the dK and dV of cut items, over all KV heads
 
 struct BwdWsLayout {
@@ -32,7 +34,7 @@ struct BwdWsLayout {
     int slots, unit_cap;                    // slots of one CTA; entries of the unit list
 };
 
-__host__ __device__ inline BwdWsLayout bwd_ws_layout(int total_tokens, int Hq, int head_dim, int grad_dtype) {
+inline BwdWsLayout bwd_ws_layout(int total_tokens, int Hq, int head_dim, int grad_dtype, int min_unit = BWD_MIN_UNIT) {
     BwdWsLayout L;
     size_t o = align_up(sizeof(WsHeader), 256);
     L.dvec = o;
@@ -40,10 +42,10 @@ __host__ __device__ inline BwdWsLayout bwd_ws_layout(int total_tokens, int Hq, i
     L.dq_acc = o;
     if (grad_dtype == KVS_GRAD_BF16) o = align_up(o + sizeof(float) * (size_t)total_tokens * Hq * head_dim, 256);
     L.base = o;
-    // An item of t tiles cut into units of at least BWD_MIN_UNIT tiles has at most 2 t / BWD_MIN_UNIT of them, and all items
+    // An item of t tiles cut into units of at least min_unit tiles has at most 2 t / min_unit of them, and all items
     // of a batch have at most Hq nb (nb + 1) / 2 tiles (one trace, nothing evicted).
     const long long nb = ((long long)total_tokens + TILE - 1) / TILE;
-    const long long most = Hq * nb * (nb + 1) / BWD_MIN_UNIT;
+    const long long most = Hq * nb * (nb + 1) / min_unit;
     L.slots = (int)(most < BWD_MAX_SLOTS ? most : BWD_MAX_SLOTS);
     // key blocks of a batch: short traces have more than total / 128; beyond 4096 more the items are not cut
     L.unit_cap = (int)((total_tokens < nb + 4096 ? total_tokens : nb + 4096) + L.slots);
@@ -65,6 +67,7 @@ struct BwdPlanArgs {
     int pairs;                              // items are pairs of key blocks
     int G, all_Hkv, Hkv;
     int all_slots, slots;                   // slots there are, of an item's CTAs, over all KV heads
+    int min_unit;                           // tiles of the shortest unit
     BwdPlan* plan;                          // nullptr: none is wanted
     BwdUnit* units;
     int32_t* arrived;
@@ -112,7 +115,7 @@ __device__ void bwd_plan(const BwdPlanArgs& a) {
     const float frac[NC] = {0.25f, 0.5f, 0.75f, 1.0f, 1.25f, 1.6f, 2.2f, 0.f};
 #pragma unroll
     for (int k = 0; k < NC; ++k) {
-        const float l = fmaxf(ceilf(share * frac[k]), (float)max(BWD_MIN_UNIT, (most + BWD_MAX_CUT - 1) / BWD_MAX_CUT));
+        const float l = fmaxf(ceilf(share * frac[k]), (float)max(a.min_unit, (most + BWD_MAX_CUT - 1) / BWD_MAX_CUT));
         cand[k] = (k == NC - 1 || l > (float)most) ? most : (int)l;
     }
     // What a warp makes of the candidates' numbers (lane k: those of candidate k): the longest unit, and from which length on
@@ -953,8 +956,8 @@ extern "C" size_t kvs_attn_bwd_workspace_bytes(int total_tokens, int Hq, int Hkv
 size_t kvs::bwd_base_bytes(int total_tokens, int Hq, int head_dim, int grad_dtype) {
     return bwd_ws_layout(total_tokens, Hq, head_dim, grad_dtype).base;
 }
-size_t kvs::bwd_cut_bytes(int total_tokens, int Hq, int head_dim) {
-    const BwdWsLayout L = bwd_ws_layout(total_tokens, Hq, head_dim, KVS_GRAD_FP32);
+size_t kvs::bwd_cut_bytes(int total_tokens, int Hq, int head_dim, bool less) {
+    const BwdWsLayout L = bwd_ws_layout(total_tokens, Hq, head_dim, KVS_GRAD_FP32, less ? BWD_MIN_UNIT_LESS : BWD_MIN_UNIT);
     return L.total - L.base;
 }
 
@@ -991,13 +994,15 @@ int bwd_impl(const void* dout, const void* q, const void* k, const void* v, long
         return KVS_ERR_ALIGNMENT;
     if (((uintptr_t)lse & 3) != 0 || ((uintptr_t)workspace & 255) != 0 || ((uintptr_t)meta_buf & 255) != 0) return KVS_ERR_ALIGNMENT;
     if (softmax_scale < 0.f || softmax_scale != softmax_scale) return KVS_ERR_INVALID_ARG;
-    const BwdWsLayout W = bwd_ws_layout(total_tokens, Hq, head_dim, grad_dtype);
+    const BwdWhole whole = part_of ? *part_of : BwdWhole{meta_buf, batch, total_tokens, max_seqlen, Hkv, nullptr, false};
+    const bool less = whole.cut_buf ? whole.cut_less : workspace_bytes < bwd_ws_layout(total_tokens, Hq, head_dim, grad_dtype).total;
+    const int min_unit = less ? BWD_MIN_UNIT_LESS : BWD_MIN_UNIT;
+    const BwdWsLayout W = bwd_ws_layout(total_tokens, Hq, head_dim, grad_dtype, min_unit);
     if (workspace_bytes < W.base) return KVS_ERR_WORKSPACE;
     int rc = check_device_sm100();
     if (rc != KVS_OK) return rc;
     const MetaLayout L = meta_layout(batch, total_tokens, max_seqlen);
     const MetaView mv = meta_view(meta_buf, L);
-    const BwdWhole whole = part_of ? *part_of : BwdWhole{meta_buf, batch, total_tokens, max_seqlen, Hkv, nullptr};
     const bool pair = use_pairs(whole.batch, whole.total_tokens, Hq / Hkv, head_dim);
     const int q_rows = pair ? TILE / 2 : TILE;       // rows of the boxes of q, dout and dq
     CUtensorMap tq, tk, tv, tdo, tdq;
@@ -1056,8 +1061,9 @@ int bwd_impl(const void* dout, const void* q, const void* k, const void* v, long
         pa.G = Hq / Hkv;
         pa.all_Hkv = whole.Hkv;
         pa.Hkv = Hkv;
-        pa.all_slots = bwd_ws_layout(whole.total_tokens, whole.Hkv * pa.G, head_dim, grad_dtype).slots / ctas;
+        pa.all_slots = bwd_ws_layout(whole.total_tokens, whole.Hkv * pa.G, head_dim, grad_dtype, min_unit).slots / ctas;
         pa.slots = slots;
+        pa.min_unit = min_unit;
         pa.plan = (BwdPlan*)(cut + W.plan);
         pa.units = (BwdUnit*)(cut + W.units);
         pa.arrived = (int32_t*)(cut + W.arrived);

@@ -62,13 +62,15 @@ struct BwdWhole {
     const void* meta_buf;
     int batch, total_tokens, max_seqlen, Hkv;
     void* cut_buf;
+    bool cut_less;          // which of the two sizes of bwd_cut_bytes it has
 };
 int bwd_of_chunk(const BwdWhole& whole, const void* dout, const void* q, const void* k, const void* v, const void* out, const float* lse,
                  const void* meta_buf, int batch, int total_tokens, int max_seqlen, int Hq, int Hkv, int head_dim, float softmax_scale,
                  int grad_dtype, void* dq, void* dk, void* dv, void* workspace, size_t workspace_bytes, kvs_stream_t stream);
-// workspace bytes of a backward: what it needs without cutting items (status, row sums, fp32 dQ accumulator), and the rest
+// workspace bytes of a backward: what it needs without cutting items (status, row sums, fp32 dQ accumulator), and the rest (`less`:
+// with the fewer slots of longer units)
 size_t bwd_base_bytes(int total_tokens, int Hq, int head_dim, int grad_dtype);
-size_t bwd_cut_bytes(int total_tokens, int Hq, int head_dim);
+size_t bwd_cut_bytes(int total_tokens, int Hq, int head_dim, bool less);
 
 #ifdef __CUDACC__
 // The unit and KV head of CTA (or pair) x of a one-dimensional grid; false: there is none.  The CTAs without work come last.
