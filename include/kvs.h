@@ -301,6 +301,13 @@ int kvs_device_status(const void* meta_or_workspace, kvs_stream_t stream);
 int kvs_selftest_bounded_wait(int32_t* status_word, int expected_arrivals, long long limit_clocks,
                               kvs_stream_t stream);
 
+/*
+ * Self-test of a bounded wait that lasts for several steps of others: half of a group of 128 threads waits for a
+ * barrier that completes at once, half for one that completes after 3 step_clocks, with the limit of `tiles` steps, which
+ * is (tiles + 1) step_clocks.  words (device int32[2]): the status as above, and how many threads went on.  0 <= tiles <= 16, step_clocks at most 2e8.
+ */
+int kvs_selftest_group_wait(int32_t* words, int tiles, long long step_clocks, kvs_stream_t stream);
+
 /* Bytes of device arena needed by kvs_attn_fwd_bwd_host for these dims. */
 size_t kvs_host_arena_bytes(int batch, int total_tokens, int max_seqlen,
                             int Hq, int Hkv, int head_dim, int grad_dtype);

@@ -56,6 +56,7 @@ SIGNATURES = {
                                   ctypes.POINTER(ctypes.c_void_p), _vp]),
     "kvs_device_status": (_i, [_vp, _vp]),
     "kvs_selftest_bounded_wait": (_i, [_vp, _i, ctypes.c_longlong, _vp]),
+    "kvs_selftest_group_wait": (_i, [_vp, _i, ctypes.c_longlong, _vp]),
     "kvs_cache_free_list_bytes": (_sz, [_i]),
     "kvs_cache_init": (_i, [_vp, _i, _vp]),
     "kvs_cache_append": (_i, [_vp, _vp, _vp, _i, _i, _i, _i, _i, _i, _vp, _vp, _vp, _vp, _vp, _vp]),
@@ -332,6 +333,13 @@ def kvs_selftest_bounded_wait(expected_arrivals: int, limit_clocks: int, stream=
     _check(load().kvs_selftest_bounded_wait(word.data_ptr(), expected_arrivals, limit_clocks, _stream(stream)),
            "kvs_selftest_bounded_wait")
     return int(word.item())
+
+
+def kvs_selftest_group_wait(tiles: int, step_clocks: int, stream=None) -> Tuple[int, int]:
+    """Runs the self-test of a group's decision after a wait; returns (status, threads that went on)."""
+    words = torch.zeros(2, dtype=torch.int32, device="cuda")
+    _check(load().kvs_selftest_group_wait(words.data_ptr(), tiles, step_clocks, _stream(stream)), "kvs_selftest_group_wait")
+    return tuple(words.tolist())
 
 
 def kvs_host_arena_bytes(batch, total_tokens, max_seqlen, Hq, Hkv, head_dim, grad_dtype) -> int:

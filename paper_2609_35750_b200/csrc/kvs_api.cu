@@ -137,6 +137,44 @@ extern "C" int kvs_selftest_bounded_wait(int32_t* status_word, int expected_arri
     return cudaGetLastError() == cudaSuccess ? KVS_OK : KVS_ERR_CUDA;
 }
 
+// ---- self-test of a wait for several steps --------------------------------------------------
+namespace kvs {
+// Warps 0 and 1 of a group of four wait for a barrier that completes at once, warps 2 and 3 for one that the fifth warp arrives
+// at after 3 `step_clocks`, with the limit of `tiles` steps.
+__global__ void selftest_group_kernel(int32_t* words, int tiles, long long step_clocks) {
+    __shared__ __align__(8) unsigned long long s_bar[2];
+    __shared__ int s_abort;
+    const int warp = threadIdx.x >> 5;
+    if (threadIdx.x == 0) {
+        s_abort = 0;
+        for (int i = 0; i < 2; ++i) mbar_init(smem_u32(&s_bar[i]), 1);
+        fence_mbar_init();
+    }
+    __syncthreads();
+    if (warp == 4) {
+        if (threadIdx.x == 128) {
+            mbar_arrive(smem_u32(&s_bar[0]));
+            const long long t0 = clock64();
+            while (clock64() - t0 < 3 * step_clocks) {}
+            mbar_arrive(smem_u32(&s_bar[1]));
+        }
+    } else {
+        mbar_wait_limit(smem_u32(&s_bar[warp >> 1]), 0, &s_abort, words, wait_limit_of(step_clocks, tiles));
+        const bool mine = !*(volatile int*)&s_abort;
+        if (mine) atomicAdd(words + 1, 1);
+    }
+    __syncthreads();
+}
+}  // namespace kvs
+
+extern "C" int kvs_selftest_group_wait(int32_t* words, int tiles, long long step_clocks, kvs_stream_t stream) {
+    if (!words || tiles < 0 || tiles > 16 || step_clocks <= 0 || step_clocks > 200000000LL) return KVS_ERR_INVALID_ARG;
+    cudaStream_t st = (cudaStream_t)stream;
+    if (cudaMemsetAsync(words, 0, 2 * sizeof(int32_t), st) != cudaSuccess) return KVS_ERR_CUDA;
+    selftest_group_kernel<<<1, 160, 0, st>>>(words, tiles, step_clocks);
+    return cudaGetLastError() == cudaSuccess ? KVS_OK : KVS_ERR_CUDA;
+}
+
 // ---- whole path from host buffers ------------------------------------------------------------
 // The work is cut into chunks of (a contiguous range of traces, one KV head with its G query heads): chunks are
 // independent in the forward and the backward, so while chunk c computes, the inputs of chunk c+1 arrive and

@@ -601,11 +601,11 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
             // The first one is the CTA's own; after it units of CTAs of the grid that have not started, asked for a few tiles
             // before the end of the one before: what is asked for and found (about 3 us) lies beside those tiles, and the last
             // units still go to whoever is free first.
-            int x = blockIdx.x;
+            int x = blockIdx.x, tiles = 0;                // of the unit before
             bool ok = true;
             for (int r = 0; ; ++r) {
                 if (r > 0) {
-                    mbar_wait(bar_late, (r - 1) & 1, abort_flag, status);
+                    mbar_wait_limit(bar_late, (r - 1) & 1, abort_flag, status, wait_limit_of(WAIT_LIMIT_CLOCKS, tiles));
                     if (*abort_flag) break;               // nothing is asked for that would not be waited for
                     if (lane == 0) {
                         mbar_expect_tx(bar_ask, 16);
@@ -642,6 +642,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
                 }
                 const int slot = r & 1;
                 if (r >= 2) mbar_wait(bar_workfree(slot), ((r >> 1) + 1) & 1, abort_flag, status);
+                tiles = w.n_iter;
                 if (lane == 0) {
                     volatile int* dst = reinterpret_cast<volatile int*>(s_work + slot);
                     const int* src = reinterpret_cast<const int*>(&w);

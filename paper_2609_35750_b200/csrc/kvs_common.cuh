@@ -293,6 +293,8 @@ __device__ __forceinline__ void mbar_wait_limit(uint32_t bar, uint32_t parity, v
 __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int32_t* status) {
     mbar_wait_limit(bar, parity, abort_flag, status, WAIT_LIMIT_CLOCKS);
 }
+// The limit of a wait that lasts as long as `tiles` steps of other warps, each of which has a wait of `step_clocks` at most
+__device__ __forceinline__ long long wait_limit_of(long long step_clocks, int tiles) { return step_clocks * (tiles + 1ll); }
 
 // Programmatic dependent launch: a kernel started by launch_after() may get its CTAs while the kernel before it in the stream
 // still runs its last ones.  It calls pdl_wait() before it touches memory, which returns once that kernel is complete and its

@@ -84,3 +84,12 @@ def test_pairs_equal_single_ctas(T, rule):
     _, _, ref = _backward(y, [T, 1], True)
     _same(got, [t[:T] for t in ref], T, Hq // Hkv)
     _same(whole, [t[:T] for t in ref], T, Hq // Hkv)
+
+
+@pytest.mark.parametrize("tiles", [0, 8])
+def test_a_wait_for_several_steps_has_their_limit(tiles):
+    # a barrier that completes after 3 steps of 0.01 s: the limit of 9 steps is kept, that of one runs out
+    status, went_on = B.kvs_selftest_group_wait(tiles, 20_000_000)
+    assert (status, went_on == 128) == ((B.KVS_OK, True) if tiles else (B.KVS_ERR_TIMEOUT, False))
+    with pytest.raises(B.KvsError):
+        B.kvs_selftest_group_wait(17, 1000)
