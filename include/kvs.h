@@ -302,9 +302,10 @@ int kvs_selftest_bounded_wait(int32_t* status_word, int expected_arrivals, long 
                               kvs_stream_t stream);
 
 /*
- * Self-test of a bounded wait that lasts for several steps of others: half of a group of 128 threads waits for a
+ * Self-test of what warps that work as a group do after a bounded wait: half of a group of 128 threads waits for a
  * barrier that completes at once, half for one that completes after 3 step_clocks, with the limit of `tiles` steps, which
- * is (tiles + 1) step_clocks.  words (device int32[2]): the status as above, and how many threads went on.  0 <= tiles <= 16, step_clocks at most 2e8.
+ * is (tiles + 1) step_clocks.  words (device int32[2]): the status as above, and how many threads went on: all 128, or
+ * none where the wait ran out (tiles < 2).  0 <= tiles <= 16, step_clocks at most 2e8.
  */
 int kvs_selftest_group_wait(int32_t* words, int tiles, long long step_clocks, kvs_stream_t stream);
 

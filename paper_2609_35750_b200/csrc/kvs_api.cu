@@ -137,10 +137,10 @@ extern "C" int kvs_selftest_bounded_wait(int32_t* status_word, int expected_arri
     return cudaGetLastError() == cudaSuccess ? KVS_OK : KVS_ERR_CUDA;
 }
 
-// ---- self-test of a wait for several steps --------------------------------------------------
+// ---- self-test of a group's decision after a wait --------------------------------------------------
 namespace kvs {
 // Warps 0 and 1 of a group of four wait for a barrier that completes at once, warps 2 and 3 for one that the fifth warp arrives
-// at after 3 `step_clocks`, with the limit of `tiles` steps.
+// at after 3 `step_clocks`, with the limit of `tiles` steps.  The four go on together (and meet again) or not at all.
 __global__ void selftest_group_kernel(int32_t* words, int tiles, long long step_clocks) {
     __shared__ __align__(8) unsigned long long s_bar[2];
     __shared__ int s_abort;
@@ -161,7 +161,11 @@ __global__ void selftest_group_kernel(int32_t* words, int tiles, long long step_
     } else {
         mbar_wait_limit(smem_u32(&s_bar[warp >> 1]), 0, &s_abort, words, wait_limit_of(step_clocks, tiles));
         const bool mine = !*(volatile int*)&s_abort;
-        if (mine) atomicAdd(words + 1, 1);
+        __syncwarp();
+        if (group_all(1, 128, mine)) {
+            named_bar_sync(1, 128);
+            atomicAdd(words + 1, 1);
+        }
     }
     __syncthreads();
 }

@@ -516,10 +516,17 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *s_tmem_base;
-    // The r-th unit of the CTA; false: there is none.  A role reads what it needs of it and arrives at the end of it.
-    auto take = [&](int r) {
+    // The r-th unit of the CTA; false: there is none, or a wait gave up.  A role reads what it needs of it and arrives at the end
+    // of it; the warps of a role take it together or not at all.
+    auto taken = [&](int r) {
         mbar_wait(bar_work(r & 1), (r >> 1) & 1, abort_flag, status);
         return s_work[r & 1].n_iter >= 0 && !*abort_flag;
+    };
+    auto take = [&](int r) { return (bool)__all_sync(0xffffffffu, taken(r)); };
+    auto take_together = [&](int r, int id, int threads) {
+        const bool mine = taken(r);
+        __syncwarp();
+        return group_all(id, threads, mine);
     };
     auto done = [&](int r) {
         __syncwarp();
@@ -642,6 +649,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
                 }
                 const int slot = r & 1;
                 if (r >= 2) mbar_wait(bar_workfree(slot), ((r >> 1) + 1) & 1, abort_flag, status);
+                if (*abort_flag) break;                   // the slot may still be read: no role may see another length of its unit
                 tiles = w.n_iter;
                 if (lane == 0) {
                     volatile int* dst = reinterpret_cast<volatile int*>(s_work + slot);
@@ -651,7 +659,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
                     mbar_arrive(bar_work(slot));
                 }
                 __syncwarp();
-                if (w.n_iter < 0 || *abort_flag) break;
+                if (w.n_iter < 0) break;
             }
         } else if (warp == 13) {
             // ================= MMA issuer (all lanes walk the loop, one elected lane issues) =================
@@ -748,7 +756,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         const uint32_t lane_sel = (uint32_t)(quad * 32) << 16;
         uint8_t* stg_row = sgen + L::OFF_STG + row * 128;
         uint32_t J = 0;                                         // tiles of the CTA so far
-        for (int r = 0; take(r); ++r) {
+        for (int r = 0; take_together(r, 1, 128); ++r) {
             const volatile BwdWork* work = s_work + (r & 1);
             const int tok0 = work->tok0, m_first = work->m_first, m_last = work->m_last;
             const uint32_t end = J + work->n_iter;
@@ -806,7 +814,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         uint8_t* sDS_row = sgen + L::OFF_DS + half * BOX_BYTES + row * 128;
         float pv[64];
         uint32_t J = 0;                                         // tiles of the CTA so far
-        for (int r = 0; take(r); ++r) {
+        for (int r = 0; take_together(r, 2, 256); ++r) {
             const volatile BwdWork* work = s_work + (r & 1);
             const uint32_t end = J + work->n_iter;
             if (J == end) {                                         // a key block that no query sees: its gradients are zero

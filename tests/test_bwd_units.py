@@ -86,10 +86,11 @@ def test_pairs_equal_single_ctas(T, rule):
     _same(whole, [t[:T] for t in ref], T, Hq // Hkv)
 
 
-@pytest.mark.parametrize("tiles", [0, 8])
-def test_a_wait_for_several_steps_has_their_limit(tiles):
-    # a barrier that completes after 3 steps of 0.01 s: the limit of 9 steps is kept, that of one runs out
-    status, went_on = B.kvs_selftest_group_wait(tiles, 20_000_000)
-    assert (status, went_on == 128) == ((B.KVS_OK, True) if tiles else (B.KVS_ERR_TIMEOUT, False))
+@pytest.mark.parametrize("tiles,went_on", [(0, 0), (8, 128)])
+def test_warps_of_a_group_go_on_together_after_a_wait(tiles, went_on):
+    # Two of four warps are through their wait at once, the others after 3 steps: with the limit of 9 steps all go on, with that of
+    # one step (0.01 s) the wait runs out and none does, although two had seen no reason to stop.
+    status = B.KVS_OK if went_on else B.KVS_ERR_TIMEOUT
+    assert B.kvs_selftest_group_wait(tiles, 20_000_000) == (status, went_on)
     with pytest.raises(B.KvsError):
         B.kvs_selftest_group_wait(17, 1000)
