@@ -90,10 +90,24 @@ kvs_stream_t stream_of(PyObject* stream) {
     if (PyErr_Occurred()) throw Raised();
     return (kvs_stream_t)p;
 }
-at::Tensor bytes(size_t n, const at::Tensor& like) { return at::empty({(int64_t)n}, like.options().dtype(at::kByte)); }
+// Allocations, like calls into the library, are made without the interpreter lock: the allocator may wait for the device.
+struct Unlocked {
+    PyThreadState* state = PyEval_SaveThread();
+    ~Unlocked() { PyEval_RestoreThread(state); }
+};
+at::Tensor empty(at::IntArrayRef sizes, const at::Tensor& like, at::ScalarType dtype) {
+    Unlocked u;
+    return at::empty(sizes, like.options().dtype(dtype));
+}
+at::Tensor bytes(size_t n, const at::Tensor& like) { return empty({(int64_t)n}, like, at::kByte); }
 // the tensor given, or a new one
 at::Tensor out_of(PyObject* o, const char* name, at::IntArrayRef sizes, const at::Tensor& like, at::ScalarType dtype) {
-    return given(o) ? tensor(o, name) : at::empty(sizes, like.options().dtype(dtype));
+    return given(o) ? tensor(o, name) : empty(sizes, like, dtype);
+}
+at::Tensor out_of(PyObject* o, const char* name, const at::Tensor& like) {
+    if (given(o)) return tensor(o, name);
+    Unlocked u;
+    return at::empty_like(like);
 }
 
 void check(int code, const char* where) {
@@ -105,13 +119,14 @@ void check(int code, const char* where) {
     }
     throw Raised();
 }
-// a call into the library, without the interpreter lock
+// a call into the library
 template <typename F>
 void call(const char* where, F f) {
     int rc;
-    Py_BEGIN_ALLOW_THREADS
-    rc = f();
-    Py_END_ALLOW_THREADS
+    {
+        Unlocked u;
+        rc = f();
+    }
     check(rc, where);
 }
 PyObject* wrap(const at::Tensor& t, PyObject* o) {
@@ -168,7 +183,7 @@ PyObject* attn_fwd(PyObject* const* a) {
     const int total = (int)q.size(0), Hq = (int)q.size(1), d = (int)q.size(2), Hkv = (int)size1(k, "k");
     const int batch = whole(a[4]), max_seqlen = whole(a[5]);
     const float scale = real(a[6]);
-    const at::Tensor out = given(a[7]) ? tensor(a[7], "out") : at::empty_like(q);
+    const at::Tensor out = out_of(a[7], "out", q);
     const at::Tensor lse = out_of(a[8], "lse", {Hq, total}, q, F32);
     void *pq = address(q, "q", BF16), *pk = address(k, "k", BF16), *pv = address(v, "v", BF16), *pm = address(meta, "meta_buf", U8),
          *po = address(out, "out", BF16);
@@ -201,8 +216,8 @@ PyObject* attn_fwd_dual(PyObject* const* a) {
     const int total = (int)q.size(0), Hq = (int)q.size(1), d = (int)q.size(2), Hkv = (int)size1(k, "k");
     const int batch = whole(a[5]), max_seqlen = whole(a[6]);
     const float scale = real(a[7]);
-    const at::Tensor os = given(a[8]) ? tensor(a[8], "out_student") : at::empty_like(q), ls = out_of(a[9], "lse_student", {Hq, total}, q, F32),
-                     ot = given(a[10]) ? tensor(a[10], "out_teacher") : at::empty_like(q), lt = out_of(a[11], "lse_teacher", {Hq, total}, q, F32);
+    const at::Tensor os = out_of(a[8], "out_student", q), ls = out_of(a[9], "lse_student", {Hq, total}, q, F32),
+                     ot = out_of(a[10], "out_teacher", q), lt = out_of(a[11], "lse_teacher", {Hq, total}, q, F32);
     void *pq = address(q, "q", BF16), *pk = address(k, "k", BF16), *pv = address(v, "v", BF16), *pms = address(ms, "meta_student", U8),
          *pme = address(me, "meta_evicted", U8), *pos = address(os, "out_student", BF16), *pot = address(ot, "out_teacher", BF16);
     float *pls = (float*)address(ls, "lse_student", F32), *plt = (float*)address(lt, "lse_teacher", F32);
@@ -261,7 +276,7 @@ PyObject* attn_bwd_packed(PyObject* const* a) {
 // (src, perm, dst, inverse, stream)
 PyObject* permute_rows(PyObject* const* a) {
     const at::Tensor &src = tensor(a[0], "src"), &perm = tensor(a[1], "perm");
-    const at::Tensor dst = given(a[2]) ? tensor(a[2], "dst") : at::empty_like(src);
+    const at::Tensor dst = out_of(a[2], "dst", src);
     const int inverse = PyObject_IsTrue(a[3]);
     if (inverse < 0) throw Raised();
     if (src.dim() < 1) value_error("%s must have a leading dimension", "src");
@@ -294,7 +309,7 @@ PyObject* rope_qk(PyObject* const* a) {
         if (given(a[i])) {
             const at::Tensor& t = tensor(a[i], names[i]);
             heads[i] = (int)size1(t, names[i]);
-            out[i] = given(a[6 + i]) ? tensor(a[6 + i], names[2 + i]) : at::empty_like(t);
+            out[i] = out_of(a[6 + i], names[2 + i], t);
             p[i] = address(t, names[i], must);
             p[2 + i] = address(out[i], names[2 + i], must);
         } else if (given(a[6 + i])) {
@@ -341,7 +356,7 @@ PyObject* decode(PyObject* const* a) {
     int splits = whole(a[2]);
     if (splits <= 0) splits = lib.kvs_decode_num_splits(S, Hkv, whole(a[6]));
     const at::Tensor ws = given(a[5]) ? tensor(a[5], "workspace") : bytes(lib.kvs_decode_workspace_bytes(S, Hq, d, splits), q);
-    const at::Tensor out = given(a[3]) ? tensor(a[3], "out") : at::empty_like(q), lse = out_of(a[4], "lse", {S, Hq}, q, F32);
+    const at::Tensor out = out_of(a[3], "out", q), lse = out_of(a[4], "lse", {S, Hq}, q, F32);
     const void* pq = address(q, "q", BF16);
     void *po = address(out, "out", BF16), *pw = address(ws, "workspace", U8);
     float* pl = (float*)address(lse, "lse", F32);

@@ -1,4 +1,7 @@
 """The native calls of the binding refuse what the path does not take, as Python errors (no GPU needed)."""
+import threading
+import time
+
 import pytest
 import torch
 
@@ -28,3 +31,32 @@ def test_wrong_arguments_are_python_errors():
         B.kvs_attn_fwd(CPU["q"][0], CPU["q"], CPU["q"], CPU["q"], 1, 4)              # two dimensions
     with pytest.raises(ValueError, match="heads"):
         B.kvs_attn_fwd_packed(CPU["q"], CPU["q"], 1, 4, 2, 1)
+
+
+def test_other_threads_run_while_outputs_are_allocated():
+    # An allocation may wait (for the device, or as here for 500 MB to be filled); it is refused afterwards for being on the host
+    total = 1 << 21
+    evict = torch.ones(total, dtype=torch.int32)
+    cu = torch.tensor([0, total], dtype=torch.int32)
+    ticks, stop = [0], threading.Event()
+
+    def tick():
+        while not stop.is_set():
+            ticks[0] += 1
+            time.sleep(1e-3)
+
+    B.load()
+    thread = threading.Thread(target=tick)
+    before = torch.are_deterministic_algorithms_enabled()
+    torch.use_deterministic_algorithms(True)                  # new tensors are filled
+    thread.start()
+    try:
+        t0, n0 = time.perf_counter(), ticks[0]
+        with pytest.raises(ValueError, match="CUDA"):
+            B.kvs_mask_meta(evict, cu, total)
+        took, n = time.perf_counter() - t0, ticks[0] - n0
+    finally:
+        torch.use_deterministic_algorithms(before)
+        stop.set()
+        thread.join()
+    assert took > 0.02 and n >= took / 0.02, (took, n)        # a tick takes a millisecond; held up, there are at most two
