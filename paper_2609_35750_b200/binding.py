@@ -82,8 +82,8 @@ class KvsError(RuntimeError):
 
 
 def load() -> ctypes.CDLL:
-    """Loads libkvs.so and the native calls (built by paper_2609_35750_b200.build).  Raises if either is absent."""
-    global _lib, _native
+    """Loads libkvs.so (built by paper_2609_35750_b200.build).  Raises if absent."""
+    global _lib
     if _lib is None:
         path = LIB_PATH
         if not os.path.exists(path):
@@ -94,10 +94,19 @@ def load() -> ctypes.CDLL:
             fn = getattr(lib, name)
             fn.restype = res
             fn.argtypes = args
+        _lib = lib
+    return _lib
+
+
+def _calls():
+    """The native calls, loaded by the first function that needs them: the size queries and the chunk plan do not."""
+    global _native
+    if _native is None:
+        lib = load()
         native = importlib.import_module("._kvs_native", __package__)
         native.bind({name: ctypes.cast(getattr(lib, name), ctypes.c_void_p).value for name in SIGNATURES}, KvsError)
-        _lib, _native = lib, native
-    return _lib
+        _native = native
+    return _native
 
 
 def strerror(code: int) -> str:
@@ -149,15 +158,13 @@ def kvs_evict_at_from_events(events: torch.Tensor, cu_seqlens: torch.Tensor, tot
 def kvs_mask_meta(evict_at: torch.Tensor, cu_seqlens: torch.Tensor, max_seqlen: int,
                   meta_buf: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """evict_at int32 [Ttot], cu_seqlens int32 [batch+1] (device).  Returns meta_buf (uint8)."""
-    load()
-    return _native.mask_meta(0, None, evict_at, cu_seqlens, max_seqlen, meta_buf, stream)
+    return _calls().mask_meta(0, None, evict_at, cu_seqlens, max_seqlen, meta_buf, stream)
 
 
 def kvs_mask_meta_keys(key_first: torch.Tensor, key_evict: torch.Tensor, cu_seqlens: torch.Tensor, max_seqlen: int,
                        meta_buf: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """Metadata for key slots with their own visibility interval [key_first, key_evict) (int32 [Ttot], device)."""
-    load()
-    return _native.mask_meta(1, key_first, key_evict, cu_seqlens, max_seqlen, meta_buf, stream)
+    return _calls().mask_meta(1, key_first, key_evict, cu_seqlens, max_seqlen, meta_buf, stream)
 
 
 def kvs_reorder_keys(evict_at: torch.Tensor, cu_seqlens: torch.Tensor, max_seqlen: int, window: int, perm=None, key_first=None,
@@ -176,8 +183,7 @@ def kvs_reorder_keys(evict_at: torch.Tensor, cu_seqlens: torch.Tensor, max_seqle
 
 def kvs_permute_rows(src: torch.Tensor, perm: torch.Tensor, dst: Optional[torch.Tensor] = None, inverse: bool = False, stream=None):
     """dst[s] = src[perm[s]] (inverse False) or dst[perm[s]] = src[s] (inverse True) along the leading dimension."""
-    load()
-    return _native.permute_rows(src, perm, dst, inverse, stream)
+    return _calls().permute_rows(src, perm, dst, inverse, stream)
 
 
 def kvs_mask_meta_export(meta_buf: torch.Tensor, cu_seqlens_host, total_tokens: int, max_seqlen: int, stream=None):
@@ -198,46 +204,40 @@ def kvs_mask_meta_export(meta_buf: torch.Tensor, cu_seqlens_host, total_tokens: 
 def kvs_attn_fwd(q, k, v, meta_buf, batch: int, max_seqlen: int, softmax_scale: float = 0.0,
                  out: Optional[torch.Tensor] = None, lse: Optional[torch.Tensor] = None, stream=None):
     """q [Ttot,Hq,d], k, v [Ttot,Hkv,d] bf16 (device).  Returns (out bf16 [Ttot,Hq,d], lse fp32 [Hq,Ttot])."""
-    load()
-    return _native.attn_fwd(q, k, v, meta_buf, batch, max_seqlen, softmax_scale, out, lse, stream)
+    return _calls().attn_fwd(q, k, v, meta_buf, batch, max_seqlen, softmax_scale, out, lse, stream)
 
 
 def kvs_mask_meta_evicted(key_evict: torch.Tensor, cu_seqlens: torch.Tensor, max_seqlen: int,
                           meta_buf: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """Metadata for the keys the eviction mask no longer shows (visible from their eviction step on)."""
-    load()
-    return _native.mask_meta(2, None, key_evict, cu_seqlens, max_seqlen, meta_buf, stream)
+    return _calls().mask_meta(2, None, key_evict, cu_seqlens, max_seqlen, meta_buf, stream)
 
 
 def kvs_attn_fwd_dual(q, k, v, meta_student, meta_evicted, batch: int, max_seqlen: int, softmax_scale: float = 0.0,
                       out_student=None, lse_student=None, out_teacher=None, lse_teacher=None, stream=None):
     """Student (eviction mask) and teacher (every key seen or evicted: the full causal context) forward.
     Returns (out_student, lse_student, out_teacher, lse_teacher)."""
-    load()
-    return _native.attn_fwd_dual(q, k, v, meta_student, meta_evicted, batch, max_seqlen, softmax_scale, out_student, lse_student,
-                                 out_teacher, lse_teacher, stream)
+    return _calls().attn_fwd_dual(q, k, v, meta_student, meta_evicted, batch, max_seqlen, softmax_scale, out_student, lse_student,
+                                  out_teacher, lse_teacher, stream)
 
 
 def kvs_attn_fwd_packed(qkv, meta_buf, batch: int, max_seqlen: int, Hq: int, Hkv: int, softmax_scale: float = 0.0,
                         out=None, lse=None, stream=None):
     """qkv bf16 [Ttot, Hq + 2 Hkv, d] (q heads, k heads, v heads).  Returns (out [Ttot,Hq,d], lse [Hq,Ttot])."""
-    load()
-    return _native.attn_fwd_packed(qkv, meta_buf, batch, max_seqlen, Hq, Hkv, softmax_scale, out, lse, stream)
+    return _calls().attn_fwd_packed(qkv, meta_buf, batch, max_seqlen, Hq, Hkv, softmax_scale, out, lse, stream)
 
 
 def kvs_attn_bwd_packed(dout, qkv, out, lse, meta_buf, batch: int, max_seqlen: int, Hq: int, Hkv: int, softmax_scale: float = 0.0,
                         grad_dtype: int = GRAD_FP32, dqkv=None, workspace=None, stream=None):
     """Returns dqkv [Ttot, Hq + 2 Hkv, d] (bf16 or fp32): dq, dk, dv in the head order of qkv."""
-    load()
-    return _native.attn_bwd_packed(dout, qkv, out, lse, meta_buf, batch, max_seqlen, Hq, Hkv, softmax_scale, grad_dtype, dqkv, workspace, stream)
+    return _calls().attn_bwd_packed(dout, qkv, out, lse, meta_buf, batch, max_seqlen, Hq, Hkv, softmax_scale, grad_dtype, dqkv, workspace, stream)
 
 
 def kvs_rope_qk(q, k, cu_seqlens=None, positions=None, theta_base: float = 10000.0, inverse: bool = False, q_out=None, k_out=None,
                 stream=None):
     """Rotary embedding of q and/or k (bf16 or fp32, [Ttot, H, d]); inverse=True applies the transposed rotation (for
     gradients).  positions int32 [Ttot] or None for the trace-local index (cu_seqlens then required).  Returns (q_out, k_out)."""
-    load()
-    return _native.rope_qk(q, k, cu_seqlens, positions, theta_base, inverse, q_out, k_out, stream)
+    return _calls().rope_qk(q, k, cu_seqlens, positions, theta_base, inverse, q_out, k_out, stream)
 
 
 def kvs_host_chunk_plan(cu_seqlens, max_seqlen: int, Hkv: int):
@@ -263,9 +263,8 @@ def kvs_attn_bwd(dout, q, k, v, out, lse, meta_buf, batch: int, max_seqlen: int,
     """Returns (dq, dk, dv) in bf16 or fp32 according to grad_dtype.  main_events: two timing
     events (already recorded once, so that their handles exist) to be recorded around the
     main kernel; this routes through kvs_attn_bwd_ex."""
-    load()
     if main_events is None:
-        return _native.attn_bwd(dout, q, k, v, out, lse, meta_buf, batch, max_seqlen, softmax_scale, grad_dtype, dq, dk, dv, workspace, stream)
+        return _calls().attn_bwd(dout, q, k, v, out, lse, meta_buf, batch, max_seqlen, softmax_scale, grad_dtype, dq, dk, dv, workspace, stream)
     total, Hq, d = q.shape
     Hkv = k.shape[1]
     gdt = torch.float32 if grad_dtype == GRAD_FP32 else torch.bfloat16
@@ -382,9 +381,8 @@ class PagedCache:
         _check(load().kvs_cache_init(self.free_list.data_ptr(), num_pages, _stream(None)), "kvs_cache_init")
 
     def append(self, k_new: torch.Tensor, v_new: torch.Tensor, active: Optional[torch.Tensor] = None, stream=None) -> None:
-        load()
-        _native.cache_append(k_new, v_new, active, self.num_seqs, self.Hkv, self.d, self.page_size, self.max_pages, self.num_pages,
-                             self.block_table, self.n_tokens, self.free_list, self.k_cache, self.v_cache, stream)
+        _calls().cache_append(k_new, v_new, active, self.num_seqs, self.Hkv, self.d, self.page_size, self.max_pages, self.num_pages,
+                              self.block_table, self.n_tokens, self.free_list, self.k_cache, self.v_cache, stream)
 
     def evict(self, ranges: torch.Tensor, stream=None) -> None:
         """ranges int32 [n, 3] rows (sequence, first_page_slot, n_pages) (device)."""
@@ -402,6 +400,5 @@ class PagedCache:
     def decode(self, q: torch.Tensor, softmax_scale: float = 0.0, num_splits: int = 0, out=None, lse=None, workspace=None,
                max_tokens: Optional[int] = None, stream=None):
         """q bf16 [num_seqs, Hq, d] -> (out bf16 [num_seqs, Hq, d], lse fp32 [num_seqs, Hq])."""
-        load()
-        return _native.decode(q, softmax_scale, num_splits, out, lse, workspace, max_tokens or self.max_pages * self.page_size, self.Hkv,
-                              self.page_size, self.max_pages, self.num_pages, self.block_table, self.n_tokens, self.k_cache, self.v_cache, stream)
+        return _calls().decode(q, softmax_scale, num_splits, out, lse, workspace, max_tokens or self.max_pages * self.page_size, self.Hkv,
+                               self.page_size, self.max_pages, self.num_pages, self.block_table, self.n_tokens, self.k_cache, self.v_cache, stream)

@@ -60,3 +60,17 @@ def test_other_threads_run_while_outputs_are_allocated():
         stop.set()
         thread.join()
     assert took > 0.02 and n >= took / 0.02, (took, n)        # a tick takes a millisecond; held up, there are at most two
+
+
+def test_host_only_functions_do_without_the_native_calls(monkeypatch):
+    def absent(name, package=None):
+        raise ImportError(name)
+
+    monkeypatch.setattr(B, "_lib", None)
+    monkeypatch.setattr(B, "_native", None)
+    monkeypatch.setattr(B.importlib, "import_module", absent)
+    assert B.kvs_mask_meta_bytes(1, 1024, 1024) > 0 and B.strerror(0) == "ok"
+    assert B.kvs_attn_bwd_workspace_bytes(1024, 4, 4, 64, B.GRAD_BF16) > 0 and B.kvs_host_arena_bytes(1, 1024, 1024, 4, 4, 64, B.GRAD_BF16) > 0
+    assert B.kvs_host_chunk_plan([0, 5, 9], 5, 1) == [(0, 1), (1, 2)]
+    with pytest.raises(ImportError):
+        B.kvs_mask_meta(CPU["evict"], CPU["cu"], 4)
