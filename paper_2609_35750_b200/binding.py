@@ -8,11 +8,13 @@ the tensors are not on a CUDA device the calls raise.
 from __future__ import annotations
 
 import ctypes
-import importlib
+import importlib.util
 import os
 from typing import Optional, Tuple
 
 import torch
+
+from .build import native_path
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libkvs.so")
@@ -103,7 +105,12 @@ def _calls():
     global _native
     if _native is None:
         lib = load()
-        native = importlib.import_module("._kvs_native", __package__)
+        path = native_path()
+        if not os.path.exists(path):
+            raise FileNotFoundError(f"{path} not found: build it with `python -m paper_2609_35750_b200.build`")
+        spec = importlib.util.spec_from_file_location(f"{__package__}._kvs_native", path)
+        native = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(native)
         native.bind({name: ctypes.cast(getattr(lib, name), ctypes.c_void_p).value for name in SIGNATURES}, KvsError)
         _native = native
     return _native

@@ -1,4 +1,4 @@
-"""Builds libkvs.so (the C-ABI library, nvcc for sm_100a) and _kvs_native.so (the native calls of the binding, g++) in-tree.
+"""Builds libkvs.so (the C-ABI library, nvcc for sm_100a) and the extension module _kvs_native (the native calls of the binding, g++) in-tree.
 
     python -m paper_2609_35750_b200.build [--force]
 """
@@ -7,12 +7,12 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 LIB = os.path.join(HERE, "libkvs.so")
-NATIVE = os.path.join(HERE, "_kvs_native.so")
 NATIVE_SOURCE = os.path.join(CSRC, "kvs_native.cpp")
 SOURCES = ["kvs_api.cu", "kvs_meta.cu", "kvs_fwd.cu", "kvs_fwd_dual.cu", "kvs_bwd.cu", "kvs_bwd_pair.cu", "kvs_bwd_noalloc.cu", "kvs_decode.cu", "kvs_rope.cu"]
 HEADERS = [os.path.join(CSRC, "kvs_common.cuh"), os.path.join(CSRC, "kvs_bwd.cuh"), os.path.join(INCLUDE, "kvs.h")]
@@ -27,15 +27,20 @@ def _nvcc() -> str:
     return "nvcc"
 
 
-def native_command() -> list:
-    import sysconfig
+def native_path() -> str:
+    """The module depends on Python's and torch's binary interface: both versions are in its name, so that one compiled against
+    others is neither up to date nor loaded."""
+    import torch
+    return os.path.join(HERE, f"_kvs_native-{torch.__version__}{sysconfig.get_config_var('EXT_SUFFIX')}")
 
+
+def native_command() -> list:
     import torch
     from torch.utils.cpp_extension import include_paths, library_paths
     cuda = os.path.dirname(os.path.dirname(_nvcc())) if os.path.sep in _nvcc() else "/usr/local/cuda"
     dirs = include_paths() + [sysconfig.get_paths()["include"], os.path.join(cuda, "include"), INCLUDE]
     return (["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch.compiled_with_cxx11_abi()] +
-            ["-I" + d for d in dirs] + [NATIVE_SOURCE, "-o", NATIVE] + ["-L" + d for d in library_paths()] +
+            ["-I" + d for d in dirs] + [NATIVE_SOURCE, "-o", native_path()] + ["-L" + d for d in library_paths()] +
             ["-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda"])
 
 
@@ -45,7 +50,7 @@ def _older(target: str, deps: list) -> bool:
 
 def needs_build() -> bool:
     return (_older(LIB, [os.path.join(CSRC, s) for s in SOURCES] + HEADERS) or
-            _older(NATIVE, [NATIVE_SOURCE, os.path.join(INCLUDE, "kvs.h")]))
+            _older(native_path(), [NATIVE_SOURCE, os.path.join(INCLUDE, "kvs.h")]))
 
 
 def build(force: bool = False, verbose: bool = False) -> str:

@@ -6,6 +6,7 @@ import pytest
 import torch
 
 from paper_2609_35750_b200 import binding as B
+from paper_2609_35750_b200 import build
 
 CPU = {"evict": torch.ones(4, dtype=torch.int32), "cu": torch.tensor([0, 4], dtype=torch.int32), "q": torch.zeros((4, 2, 64), dtype=torch.bfloat16)}
 
@@ -63,14 +64,19 @@ def test_other_threads_run_while_outputs_are_allocated():
 
 
 def test_host_only_functions_do_without_the_native_calls(monkeypatch):
-    def absent(name, package=None):
-        raise ImportError(name)
-
     monkeypatch.setattr(B, "_lib", None)
     monkeypatch.setattr(B, "_native", None)
-    monkeypatch.setattr(B.importlib, "import_module", absent)
+    monkeypatch.setattr(B, "native_path", lambda: "/nowhere/_kvs_native.so")
     assert B.kvs_mask_meta_bytes(1, 1024, 1024) > 0 and B.strerror(0) == "ok"
     assert B.kvs_attn_bwd_workspace_bytes(1024, 4, 4, 64, B.GRAD_BF16) > 0 and B.kvs_host_arena_bytes(1, 1024, 1024, 4, 4, 64, B.GRAD_BF16) > 0
     assert B.kvs_host_chunk_plan([0, 5, 9], 5, 1) == [(0, 1), (1, 2)]
-    with pytest.raises(ImportError):
+    with pytest.raises(FileNotFoundError):
+        B.kvs_mask_meta(CPU["evict"], CPU["cu"], 4)
+
+
+def test_a_module_built_against_another_torch_is_not_used(monkeypatch):
+    monkeypatch.setattr(torch, "__version__", "0.0.1")
+    monkeypatch.setattr(B, "_native", None)
+    assert build.needs_build()
+    with pytest.raises(FileNotFoundError, match="0.0.1"):
         B.kvs_mask_meta(CPU["evict"], CPU["cu"], 4)
