@@ -8,6 +8,7 @@
 
 #include <ATen/ATen.h>
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/DynamicTypes.h>
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
@@ -61,9 +62,7 @@ void* address(const at::Tensor& t, const char* name, at::ScalarType dtype) {
     if (!t.is_cuda()) value_error("%s must be a CUDA tensor (there is no CPU path)", name);
     if (!t.is_contiguous()) value_error("%s must be contiguous", name);
     if (t.scalar_type() != dtype) {
-        PyErr_Format(PyExc_ValueError, "%s must be torch.%s, got torch.%s", name,
-                     dtype == at::kBFloat16 ? "bfloat16" : dtype == at::kFloat ? "float32" : dtype == at::kInt ? "int32" : "uint8",
-                     t.scalar_type() == at::kBFloat16 ? "bfloat16" : at::toString(t.scalar_type()));
+        PyErr_Format(PyExc_ValueError, "%s must be %S, got %S", name, torch::getTHPDtype(dtype), torch::getTHPDtype(t.scalar_type()));
         throw Raised();
     }
     return t.mutable_data_ptr();
@@ -279,7 +278,10 @@ PyObject* permute_rows(PyObject* const* a) {
     const at::Tensor dst = out_of(a[2], "dst", src);
     const int inverse = PyObject_IsTrue(a[3]);
     if (inverse < 0) throw Raised();
-    if (src.dim() < 1) value_error("%s must have a leading dimension", "src");
+    if (src.dim() < 1) {
+        PyErr_SetString(PyExc_IndexError, "src must have a leading dimension");
+        throw Raised();
+    }
     const long long n = src.size(0), row_bytes = (long long)(src.numel() / (n > 0 ? n : 1)) * (long long)src.element_size();
     if (!src.is_cuda() || !src.is_contiguous() || !dst.is_contiguous() || dst.sizes() != src.sizes() || dst.scalar_type() != src.scalar_type())
         value_error("%s must be contiguous CUDA tensors of the same shape and dtype", "src and dst");

@@ -32,6 +32,19 @@ def test_wrong_arguments_are_python_errors():
         B.kvs_attn_fwd(CPU["q"][0], CPU["q"], CPU["q"], CPU["q"], 1, 4)              # two dimensions
     with pytest.raises(ValueError, match="heads"):
         B.kvs_attn_fwd_packed(CPU["q"], CPU["q"], 1, 4, 2, 1)
+    with pytest.raises(IndexError):
+        B.kvs_permute_rows(torch.zeros(()), CPU["cu"])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype", [torch.int64, torch.float16, torch.float64, torch.bool, torch.uint8])
+def test_a_wrong_dtype_is_named_as_torch_names_it(dtype):
+    cu = CPU["cu"].cuda()
+    with pytest.raises(ValueError, match=f"^evict_at must be torch.int32, got {dtype}$"):
+        B.kvs_mask_meta(torch.ones(4, dtype=dtype, device="cuda"), cu, 4)
+    q = torch.zeros((4, 2, 64), dtype=dtype, device="cuda")
+    with pytest.raises(ValueError, match=f"^q must be torch.bfloat16, got {dtype}$"):
+        B.kvs_attn_fwd(q, q, q, torch.zeros(1 << 16, dtype=torch.uint8, device="cuda"), 1, 4)
 
 
 def test_other_threads_run_while_outputs_are_allocated():
