@@ -299,6 +299,10 @@ PyObject* rope_qk(PyObject* const* a) {
     dims(ref, 3, given(a[0]) ? "q" : "k");
     const int total = (int)ref.size(0), d = (int)ref.size(2);
     const at::ScalarType dt = ref.scalar_type();
+    if (dt != BF16 && dt != F32) {
+        PyErr_Format(PyExc_ValueError, "%s must be torch.bfloat16 or torch.float32, got %S", given(a[0]) ? "q" : "k", torch::getTHPDtype(dt));
+        throw Raised();
+    }
     const float theta = real(a[4]);
     const int inverse = PyObject_IsTrue(a[5]);
     if (inverse < 0) throw Raised();
@@ -306,16 +310,15 @@ PyObject* rope_qk(PyObject* const* a) {
     at::Tensor out[2];
     void* p[4] = {nullptr, nullptr, nullptr, nullptr};
     int heads[2] = {0, 0};
-    const at::ScalarType must = dt == F32 ? F32 : dt;
     for (int i = 0; i < 2; ++i) {
         if (given(a[i])) {
             const at::Tensor& t = tensor(a[i], names[i]);
             heads[i] = (int)size1(t, names[i]);
             out[i] = out_of(a[6 + i], names[2 + i], t);
-            p[i] = address(t, names[i], must);
-            p[2 + i] = address(out[i], names[2 + i], must);
+            p[i] = address(t, names[i], dt);
+            p[2 + i] = address(out[i], names[2 + i], dt);
         } else if (given(a[6 + i])) {
-            p[2 + i] = address(tensor(a[6 + i], names[2 + i]), names[2 + i], must);
+            p[2 + i] = address(tensor(a[6 + i], names[2 + i]), names[2 + i], dt);
         }
     }
     const int32_t* pos = given(a[3]) ? (const int32_t*)address(tensor(a[3], "positions"), "positions", I32) : nullptr;

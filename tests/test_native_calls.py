@@ -93,3 +93,13 @@ def test_a_module_built_against_another_torch_is_not_used(monkeypatch):
     assert build.needs_build()
     with pytest.raises(FileNotFoundError, match="0.0.1"):
         B.kvs_mask_meta(CPU["evict"], CPU["cu"], 4)
+
+
+@pytest.mark.parametrize("dtype", [torch.float16, torch.float64, torch.int32])
+def test_rope_refuses_what_it_does_not_rotate(dtype):
+    # found before the device is asked for; halves used to be rotated as if their bits were bfloat16
+    x = torch.zeros((4, 2, 64), dtype=dtype)
+    with pytest.raises(ValueError, match=f"^q must be torch.bfloat16 or torch.float32, got {dtype}$"):
+        B.kvs_rope_qk(x, None, CPU["cu"])
+    with pytest.raises(ValueError, match=f"^k must be torch.bfloat16 or torch.float32, got {dtype}$"):
+        B.kvs_rope_qk(None, x, CPU["cu"])
