@@ -113,10 +113,10 @@ __device__ __forceinline__ void bwd_zero_rows(const BwdParams& p, int tok, int r
 // Epilogue of the 256 compute threads: thread (row, half) has the columns [half * D/2, +D/2) of its row of dK and dV in
 // tensor memory.  A whole item goes straight to memory (`tok`: first token of this warp's 32 rows, `rows`: how many of them the
 // trace has; `stage`: 4 KB of shared memory of this warp's own).  A unit of a cut item writes them to its slot; the item's last unit
-// adds the slots up in order.  `ctas`: CTAs per item, `cta`: this one's index.
-template <int D>
+// adds the slots up in order.  `ctas`: CTAs per item, `cta`: this one's index; `meet`: a barrier of the 256 threads.
+template <int D, typename Meet>
 __device__ __forceinline__ void bwd_epilogue(const BwdParams& p, int cut, int g, int ctas, int cta, uint32_t tmem_dk, uint32_t tmem_dv, int row,
-                                             int half, int tok, int rows, uint8_t* stage, volatile int* s_last) {
+                                             int half, int tok, int rows, uint8_t* stage, volatile int* s_last, Meet meet) {
     constexpr int CH = D / 64;              // 32-column pieces per thread and tensor
     const int lane = threadIdx.x & 31;
     const size_t elem = (size_t)tok * (size_t)p.dkv_ts + (size_t)g * D + half * (D / 2);
@@ -160,9 +160,9 @@ __device__ __forceinline__ void bwd_epilogue(const BwdParams& p, int cut, int g,
         }
     }
     __threadfence();
-    named_bar_sync(2, 256);
+    meet();
     if (threadIdx.x == 0) *s_last = atomicAdd(&p.arrived[slot0 * 2 + cta], 1) == count - 1;
-    named_bar_sync(2, 256);
+    meet();
     if (!*s_last) return;
     __threadfence();
 #pragma unroll

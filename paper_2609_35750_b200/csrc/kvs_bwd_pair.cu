@@ -601,7 +601,7 @@ bwd_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         // through the memory of K and V, which nothing reads any more
         bwd_epilogue<D>(p, work->cut, g, 2, (int)rank, tmem_dK + lane_sel + half * 64, tmem_dV + lane_sel + half * 64, row, half,
                         tok0 + n * TILE + quad * 32, T - n * TILE - quad * 32, sgen + L::OFF_K + warp * 4096,
-                        reinterpret_cast<volatile int*>(sgen + L::OFF_MISC + 8));
+                        reinterpret_cast<volatile int*>(sgen + L::OFF_MISC + 8), [] { named_bar_sync(2, 256); });
     }
     tc_fence_before();
     __syncthreads();
