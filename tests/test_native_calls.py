@@ -103,3 +103,57 @@ def test_rope_refuses_what_it_does_not_rotate(dtype):
         B.kvs_rope_qk(x, None, CPU["cu"])
     with pytest.raises(ValueError, match=f"^k must be torch.bfloat16 or torch.float32, got {dtype}$"):
         B.kvs_rope_qk(None, x, CPU["cu"])
+
+
+@pytest.mark.gpu
+def test_calls_go_to_the_stream_that_is_given():
+    # the current stream is busy for a second meanwhile; results of the given one are there before that, and equal
+    Hq, Hkv, d, T = 4, 2, 64, 300
+    g = torch.Generator(device="cuda").manual_seed(0)
+    rnd = lambda *shape: torch.randn(shape, generator=g, device="cuda", dtype=torch.bfloat16)  # noqa: E731
+    q, k, v, do, qkv = rnd(T, Hq, d), rnd(T, Hkv, d), rnd(T, Hkv, d), rnd(T, Hq, d), rnd(T, Hq + 2 * Hkv, d)
+    ev = (torch.arange(T, device="cuda") + 100).int()
+    first, perm, cu = torch.arange(T, device="cuda").int(), torch.arange(T - 1, -1, -1, device="cuda").int(), torch.tensor([0, T], device="cuda").int()
+    kn, vn, qn = rnd(2, Hkv, d), rnd(2, Hkv, d), rnd(2, Hq, d)
+    size = B.kvs_mask_meta_bytes(1, T, T)
+    workspace = torch.zeros(B.kvs_attn_bwd_workspace_bytes(T, Hq, Hkv, d, B.GRAD_FP32), dtype=torch.uint8, device="cuda")
+    scratch = torch.zeros(1 << 22, dtype=torch.uint8, device="cuda")
+    caches = [B.PagedCache(4, 16, 2, 2, Hkv, d) for _ in range(2)]
+
+    def buffers():
+        new = lambda like, dtype=None: torch.full_like(like, -1, dtype=dtype)  # noqa: E731
+        lse = lambda: torch.full((Hq, T), -1.0, device="cuda")  # noqa: E731
+        return dict(meta=[torch.zeros(size, dtype=torch.uint8, device="cuda") for _ in range(3)], fwd=[new(q), lse()], packed=[new(q), lse()],
+                    dual=[new(q), lse(), new(q), lse()], bwd=[new(t, torch.float32) for t in (q, k, v)], dqkv=[new(qkv, torch.float32)],
+                    rows=[new(k)], rope=[new(q), new(k)], decode=[new(qn), torch.full((2, Hq), -1.0, device="cuda")])
+
+    def calls(b, cache, stream):
+        m = b["meta"]
+        B.kvs_mask_meta(ev, cu, T, m[0], stream=stream)
+        B.kvs_mask_meta_evicted(ev, cu, T, m[1], stream=stream)
+        B.kvs_mask_meta_keys(first, ev, cu, T, m[2], stream=stream)
+        B.kvs_attn_fwd(q, k, v, m[2], 1, T, 0.0, *b["fwd"], stream=stream)
+        B.kvs_attn_fwd_packed(qkv, m[0], 1, T, Hq, Hkv, 0.0, *b["packed"], stream=stream)
+        B.kvs_attn_fwd_dual(q, k, v, m[0], m[1], 1, T, 0.0, *b["dual"], stream=stream)
+        B.kvs_attn_bwd(do, q, k, v, *b["fwd"], m[2], 1, T, 0.0, B.GRAD_FP32, *b["bwd"], workspace, stream=stream)
+        B.kvs_attn_bwd_packed(do, qkv, *b["packed"], m[0], 1, T, Hq, Hkv, 0.0, B.GRAD_FP32, *b["dqkv"], workspace, stream=stream)
+        B.kvs_permute_rows(k, perm, b["rows"][0], True, stream=stream)
+        B.kvs_rope_qk(q, k, cu, q_out=b["rope"][0], k_out=b["rope"][1], stream=stream)
+        cache.append(kn, vn, stream=stream)
+        cache.decode(qn, 0.0, 1, *b["decode"], scratch, stream=stream)
+
+    want, got, side = buffers(), buffers(), torch.cuda.Stream()
+    calls(want, caches[0], None)
+    torch.cuda.synchronize()
+    torch.cuda._sleep(1 << 31)
+    busy = torch.cuda.Event()
+    busy.record()
+    calls(got, caches[1], side)
+    with torch.cuda.stream(side):
+        copies = {n: [t.cpu() for t in x] for n, x in got.items() if n != "meta"}
+    assert not busy.query()
+    torch.cuda.synchronize()
+    for n, x in copies.items():
+        for a, b in zip(x, want[n]):
+            # dq: two key blocks and more are added in the order of arrival, in fp32
+            assert torch.allclose(a.float(), b.cpu().float(), rtol=0, atol=1e-5 if n in ("bwd", "dqkv") else 0), n

@@ -10,7 +10,7 @@ import torch
 from paper_2609_35750_b200 import binding as B
 from paper_2609_35750_b200 import workloads as W
 
-from .test_bwd_units import _backward, _inputs, _same
+from .test_bwd_units import _backward, _base_bytes, _inputs, _same
 
 pytestmark = pytest.mark.gpu
 
@@ -119,6 +119,41 @@ def test_units_listed_by_trace_equal_whole_items(lens, Hq, Hkv, d, rule):
     out, lse, ref = _backward(x, lens, True)
     _, _, got = _backward(x, lens, False, out, lse)
     _same(got, ref, max(lens), Hq // Hkv)
+
+
+@pytest.mark.parametrize("at", [0, 5, 150])
+def test_one_long_trace_among_short_ones(at):
+    # listed by trace: no units of all heads first, and some of them last.  The long trace at a place where it comes last, in the
+    # order of the batch, and at its end
+    Hq, Hkv, d = 32, 8, 128
+    lens = [200] * at + [2000] + [200] * (150 - at)
+    x = _inputs(lens, Hq, Hkv, d, "causal")
+    out, lse, ref = _backward(x, lens, True)
+    ev, cu, q, k, v, do = x
+    meta = B.kvs_mask_meta(ev, cu, max(lens))
+    ws = torch.zeros(B.kvs_attn_bwd_workspace_bytes(sum(lens), Hq, Hkv, d, B.GRAD_FP32), dtype=torch.uint8, device="cuda")
+    got = B.kvs_attn_bwd(do, q, k, v, out, lse, meta, len(lens), max(lens), 0.0, B.GRAD_FP32, workspace=ws)
+    assert B.kvs_device_status(ws) == B.KVS_OK
+    units, _, first, apart = ws[_base_bytes(sum(lens), Hq):][:16].view(torch.int32).tolist()          # the plan's header
+    assert first == 0 and 0 < apart < units
+    _same(got, ref, max(lens), Hq // Hkv)
+
+
+def test_a_short_range_of_a_host_batch_by_pairs():
+    # two ranges of one trace each; the second one's metadata is made by one CTA, and with a mean of 17000 tokens its keys are
+    # taken by CTA pairs, which go by the tables of pairs of key blocks
+    lens, Hq, Hkv, d = [30000, 4000], 8, 4, 128
+    ev, cu, q, k, v, do = x = _inputs(lens, Hq, Hkv, d, "turns")
+    assert B.kvs_host_chunk_plan(cu.cpu(), max(lens), Hkv) == [(0, 1), (1, 2)]
+    out, lse, ref = _backward(x, lens, False)
+    pin = lambda t: t.cpu().pin_memory()  # noqa: E731
+    room = lambda t, dtype: torch.full(t.shape, float("nan"), dtype=dtype).pin_memory()  # noqa: E731
+    o = [room(out, out.dtype), room(lse, lse.dtype)] + [room(t, torch.float32) for t in (q, k, v)]
+    arena = torch.empty(B.kvs_host_arena_bytes(2, sum(lens), max(lens), Hq, Hkv, d, B.GRAD_FP32), dtype=torch.uint8, device="cuda")
+    B.kvs_attn_fwd_bwd_host(pin(ev), pin(cu), pin(q), pin(k), pin(v), pin(do), max(lens), 0.0, B.GRAD_FP32, *o, arena)
+    assert torch.equal(o[0], out.cpu()) and torch.equal(o[1], lse.cpu())
+    assert torch.equal(o[3], ref[1].cpu()) and torch.equal(o[4], ref[2].cpu())
+    _same([t.cuda() for t in o[2:]], ref, max(lens), Hq // Hkv)
 
 
 @pytest.mark.parametrize("lens", [[1000, 1, 300], [300] * 40])
