@@ -22,8 +22,10 @@ constexpr int BWD_SMS = 148;
 constexpr long long BWD_L2_BYTES = 96ll << 20;
 constexpr int BWD_MANY_TRACES = 8, BWD_MOST_LATE = 6;
 constexpr uint32_t BWD_LATE = 3;              // tiles left of a unit when the CTA asks for the next one
-// Tiles of the shortest unit (4 -> 2: main kernel of 1 x 1024 tokens, 4 heads, head_dim 64 22.1 -> 19.1 us).  The shorter it is, the
-// more slots a small batch asks for; a buffer that was sized for units of four is accepted and keeps to them.
+// Tiles of the shortest unit: 2 (1 x 1024 tokens, 4 heads, head_dim 64: main kernel 21.5 us with 4, 19.5 with 2), but as many as make
+// four units of the longest item, up to 4: an item's last unit reads the slots of all, 1.6 us each at head_dim 128 (16 heads on 2,
+// 1 x 600 tokens 35.8 us with 4, 44.0 with 2; 1 x 1000 43.0, 50.1).  The shorter the unit, the more slots a small batch asks for; a
+// buffer that was sized for units of four is accepted and keeps to them.
 constexpr int BWD_MIN_UNIT = 2, BWD_MIN_UNIT_LESS = 4;
 constexpr int BWD_MAX_SLOTS = 2 * BWD_SMS;  // slots of one CTA each for the dK and dV of cut items, over all KV heads
 
@@ -111,11 +113,12 @@ __device__ void bwd_plan(const BwdPlanArgs& a) {
     const int sms = a.pairs ? BWD_SMS / 2 : BWD_SMS;
     const float share = (float)(a.pairs ? all->pair_tiles : all->blk_tiles) * a.G * a.all_Hkv / sms;          // tiles per SM or pair
     for (int i = tid; i < a.arrived_n; i += 256) a.arrived[i] = 0;
+    const int min_unit = max(a.min_unit, min(most / 4, BWD_MIN_UNIT_LESS));
     int cand[NC];
     const float frac[NC] = {0.25f, 0.5f, 0.75f, 1.0f, 1.25f, 1.6f, 2.2f, 0.f};
 #pragma unroll
     for (int k = 0; k < NC; ++k) {
-        const float l = fmaxf(ceilf(share * frac[k]), (float)max(a.min_unit, (most + BWD_MAX_CUT - 1) / BWD_MAX_CUT));
+        const float l = fmaxf(ceilf(share * frac[k]), (float)max(min_unit, (most + BWD_MAX_CUT - 1) / BWD_MAX_CUT));
         cand[k] = (k == NC - 1 || l > (float)most) ? most : (int)l;
     }
     // What a warp makes of the candidates' numbers (lane k: those of candidate k): the longest unit, and from which length on

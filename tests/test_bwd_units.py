@@ -94,3 +94,18 @@ def test_warps_of_a_group_go_on_together_after_a_wait(tiles, went_on):
     assert B.kvs_selftest_group_wait(tiles, 20_000_000) == (status, went_on)
     with pytest.raises(B.KvsError):
         B.kvs_selftest_group_wait(17, 1000)
+
+
+@pytest.mark.parametrize("T,Hq,Hkv,d,longest", [(600, 16, 2, 128, 4), (1000, 16, 2, 128, 4), (384, 16, 4, 64, 3), (1024, 4, 4, 64, 2), (300, 2, 2, 128, 3)])
+def test_short_items_are_cut_into_few_units(T, Hq, Hkv, d, longest):
+    # an item's last unit adds up the slots of all of them: units of fewer than four tiles only where four of them are an item
+    x = _inputs([T], Hq, Hkv, d, "causal")
+    out, lse, ref = _backward(x, [T], True)
+    ev, cu, q, k, v, do = x
+    meta = B.kvs_mask_meta(ev, cu, T)
+    ws = torch.zeros(B.kvs_attn_bwd_workspace_bytes(T, Hq, Hkv, d, B.GRAD_FP32), dtype=torch.uint8, device="cuda")
+    got = B.kvs_attn_bwd(do, q, k, v, out, lse, meta, 1, T, 0.0, B.GRAD_FP32, workspace=ws)
+    _same(got, ref, T, Hq // Hkv)
+    plan = ws[_base_bytes(T, Hq):]
+    units = plan[256:][:16 * plan[:4].view(torch.int32).item()].view(torch.int32).view(-1, 4)          # key block, first tile, end, slots
+    assert (units[:, 2] - units[:, 1]).max().item() == longest
