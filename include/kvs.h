@@ -86,7 +86,8 @@ int kvs_evict_at_from_events(const int32_t* events, int n_events, const int32_t*
  * ascending list of its non-empty key blocks and, per key block, the last query block that
  * sees it, and keeps a copy of evict_at and cu_seqlens, so meta_buf is self-contained and
  * may be reused by every layer and head that shares (evict_at, cu_seqlens).
- * max_seqlen must be >= the longest trace.  meta_bytes >= kvs_mask_meta_bytes(...).
+ * max_seqlen must be >= the longest trace.  meta_bytes >= kvs_mask_meta_bytes(...); a buffer without the
+ * last 16 bytes a block of it is accepted too (the kernels then look up what these entries hold).
  */
 int kvs_mask_meta(const int32_t* evict_at, const int32_t* cu_seqlens,
                   int batch, int total_tokens, int max_seqlen,

@@ -21,7 +21,10 @@ constexpr int BWD_SMS = 148;
 // be had for the end (3 of 14000: 11.5 -> 11.8 ms; 4 of 20000 without groups 6.9 -> 7.0 ms).
 constexpr long long BWD_L2_BYTES = 96ll << 20;
 constexpr int BWD_MANY_TRACES = 8, BWD_MOST_LATE = 6;
-constexpr uint32_t BWD_LATE = 3;              // tiles left of a unit when the CTA asks for the next one
+// Tiles left of a unit when the CTA asks for the next one.  Main kernel, us, with 1, 2, 3, 5, 8 (32 heads on 8): 200 traces of 300 tokens
+// 953, 945, 945, 947, 970; 20 of 500 to 2000 552, 548, 548, 548, 550; 123 of 270, 16 on 4, head_dim 64 199.7, 197.6, 197.6, 197.6,
+// 201.7: earlier takes units from CTAs that are free before, with 1 they are waited for.
+constexpr uint32_t BWD_LATE = 3;
 // Tiles of the shortest unit: 2 (1 x 1024 tokens, 4 heads, head_dim 64: main kernel 21.5 us with 4, 19.5 with 2), but as many as make
 // four units of the longest item, up to 4: an item's last unit reads the slots of all, 1.6 us each at head_dim 128 (16 heads on 2,
 // 1 x 600 tokens 35.8 us with 4, 44.0 with 2; 1 x 1000 43.0, 50.1).  The shorter the unit, the more slots a small batch asks for; a
@@ -87,7 +90,8 @@ struct BwdPlanArgs {
 // Main kernel, whole items -> cut, us: 1 trace of 1000 tokens with 16 heads on 2 154 -> 42; 4000 with 32 on 8 355 -> 180; 16000,
 // head_dim 64 1199 -> 748; 20 of 100 to 2000, head_dim 64 229 -> 161; 32768 with 28 on 4 (pairs) 5500 -> 4400.  Where nothing is
 // cut, the list and the registers of the slots cost 1 % at head_dim 64 and 9 % at 128 (96 of 60 to 900: 316 -> 319, 447 -> 494;
-// before units were chained).
+// before units were chained).  BWD_UNIT_COST of 2, 4, 6 with chained units, us: 96 of 60 to 900 401, 401, 427; 20 of 500 to 2000, 1 x 1000
+// (16 on 2), 1 x 4000, 20 x 550 at head_dim 64 the same.
 constexpr float BWD_UNIT_COST = 4.f, BWD_CUT_COST = 3.f;
 __device__ void bwd_plan(const BwdPlanArgs& a) {
     constexpr int NC = 8;
@@ -249,7 +253,8 @@ __device__ void bwd_plan(const BwdPlanArgs& a) {
     }
     // Where the traces do not fit in L2 together, all but `late` eighths of them come in the order of the batch, a head's units
     // and then the next head's: key blocks of a trace run together and share its Q and dO tiles and the lines of its dQ.  The
-    // others come last, longest items first and of all heads together, as much work as it takes for all SMs to end together.
+    // others come last, longest items first and of all heads together: as much work as it takes for all SMs to end together, where
+    // the traces' lengths have nothing to do with their places in the batch (eighths of the traces, not of the tiles).
     const float part_share = (float)(a.pairs ? part->pair_tiles : part->blk_tiles) * a.G * a.Hkv / sms;
     const int late = a.by_trace ? (int)ceilf(8.f * (float)min(longest, most) / fmaxf(part_share, 1.f)) : 8;
     const bool by_trace = late <= BWD_MOST_LATE;

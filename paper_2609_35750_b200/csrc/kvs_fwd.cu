@@ -30,7 +30,9 @@ namespace kvs {
 
 constexpr int FWD_THREADS = 384;
 constexpr float RESCALE_THRESHOLD = 8.0f;
-constexpr int FWD_LATE = 2;     // chained: key blocks left of an item when the CTA asks for the next one
+// Chained: key blocks left of an item when the CTA asks for the next one.  Forward, us, with 1, 2, 4: 131 traces of 500 tokens, 32 heads
+// on 8, 524.5, 524.5, 530; 96 of 480, 16 on 2, 204.1, 204.5, 206.4; 32 of 2000 708, 709, 702.
+constexpr int FWD_LATE = 2;
 constexpr int P_SPLIT = 96;     // keys of a tile whose probabilities are handed to the MMA warp early
 
 // an item of work: a query block of a pair of heads (or of a single one)

@@ -6,10 +6,10 @@
 // evicted before the query.  Attention over a union of disjoint key sets is the merge of the attention
 // over each: with lse = log(e^lse_a + e^lse_b),  out = e^(lse_a - lse) out_a + e^(lse_b - lse) out_b.
 // So the teacher costs one more forward over the EVICTED keys only (metadata for key slots that become
-// visible at their eviction step and stay, kvs_mask_meta_evicted) and one streaming merge: every
-// (query, key) pair of a FULL or EMPTY tile is scored once for both streams, only tiles that are PARTIAL
-// for the student are visited by both passes.  Both passes run the forward kernel as it is (two query
-// heads of a group share every K/V tile).  A fused kernel with both accumulators of one head in tensor
+// visible at their eviction step and stay, kvs_mask_meta_evicted), which reads the student's rows and merges
+// them with its own as it writes them (MERGE in kvs_fwd.cu): every (query, key) pair of a FULL or EMPTY tile
+// is scored once for both streams, only tiles that are PARTIAL for the student are visited by both passes.
+// Both passes are the forward kernel (two query heads of a group share every K/V tile).  A fused kernel with both accumulators of one head in tensor
 // memory was measured first: 512 columns hold S twice and the two outputs of ONE head, so a CTA cannot
 // keep two query tiles in flight, its eight softmax warps move through load / maximum / exponentials /
 // store in lockstep and the special-function unit idles half the time; it was slower than two plain

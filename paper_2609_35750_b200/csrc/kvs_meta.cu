@@ -1,5 +1,5 @@
 // Mask metadata: per key block min/max of evict_at, per-tile class, per-row lists, launch orders.
-// Integer work only, bound by latency: two kernels on the caller's stream, no host synchronisation.
+// Integer work only, bound by latency: two kernels on the caller's stream, or one for small batches, no host synchronisation.
 #include "kvs_common.cuh"
 
 namespace kvs {
@@ -359,7 +359,7 @@ meta_classify_kernel(MetaHeader* hdr, MetaView mv, const int32_t* __restrict__ b
 // between the input and the tables stays in shared memory of one CTA of 32 warps, and an item's place in an order is counted,
 // not sorted for (the same order: by bucket, then by index).  It is slower where the one CTA
 // has much to read and write: see launch_mask_meta.
-constexpr int META_SMALL = 64, META_SMALL_TOKENS = 5120, META_SMALL_BATCH = 1024, META_SMALL_THREADS = 1024;
+constexpr int META_SMALL = 64, META_SMALL_TOKENS = 5120, META_SMALL_THREADS = 1024;
 __global__ void __launch_bounds__(META_SMALL_THREADS)
 meta_small_kernel(const int32_t* __restrict__ evict_at, const int32_t* __restrict__ key_first, int complement,
                   const int32_t* __restrict__ cu_seqlens, int batch, int total_tokens, int max_seqlen, MetaView v, int has_info, int nb_cap,
@@ -562,7 +562,7 @@ int launch_mask_meta(const int32_t* key_evict, const int32_t* key_first, int com
     MetaView v = meta_view(meta_buf, L);
     // Two kernels -> one, us: 1 x 1024 tokens 7.8 -> 4.6, 6 of 120 to 627 6.3 -> 5.1, 20 of 50 to 380 8.8 -> 7.2, 1 x 4096 7.9 -> 6.9;
     // 20 x 380 8.7 -> 8.6, 60 x 128 8.3 -> 8.9, 2 x 4000 8.2 -> 9.3, 1 x 8192 8.5 -> 11.4: the tokens decide.
-    if (L.nb_cap <= META_SMALL && total_tokens <= META_SMALL_TOKENS && batch <= META_SMALL_BATCH)
+    if (L.nb_cap <= META_SMALL && total_tokens <= META_SMALL_TOKENS)
         return launch_after(meta_small_kernel, 1, META_SMALL_THREADS, 0, st, key_evict, key_first, complement, cu_seqlens, batch, total_tokens,
                             max_seqlen, v, has_info, L.nb_cap, (unsigned long long)L.cls_cap);
     const int grid = (L.nb_cap + META_WARPS - 1) / META_WARPS;
