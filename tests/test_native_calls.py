@@ -48,7 +48,7 @@ def test_a_wrong_dtype_is_named_as_torch_names_it(dtype):
 
 
 def test_other_threads_run_while_outputs_are_allocated():
-    # An allocation may wait (for the device, or as here for 500 MB to be filled); it is refused afterwards for being on the host
+    # An allocation may wait (for the device, or as here for 800 MB to be filled); it is refused afterwards for being on the host
     total = 1 << 21
     evict = torch.ones(total, dtype=torch.int32)
     cu = torch.tensor([0, total], dtype=torch.int32)
@@ -73,7 +73,7 @@ def test_other_threads_run_while_outputs_are_allocated():
         torch.use_deterministic_algorithms(before)
         stop.set()
         thread.join()
-    assert took > 0.02 and n >= took / 0.02, (took, n)        # a tick takes a millisecond; held up, there are at most two
+    assert n >= took / 0.02, (took, n)        # a tick takes a millisecond; held up, there are two at most (of 0.1 s)
 
 
 def test_host_only_functions_do_without_the_native_calls(monkeypatch):
